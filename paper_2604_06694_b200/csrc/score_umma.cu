@@ -1032,7 +1032,13 @@ cudaError_t launch_score_umma_cap(const Shape& sh, const ReqDesc* h_reqs, const 
   args.wait_cycles = score_wait_cycles();
   const int q_bytes = args.q_rows * d * 2, stage = kTileKeys * d * 2;
   const int room = kSmemLimit - 1024 - static_cast<int>(sizeof(Small)) - q_bytes;
-  args.n_stages = room / stage < kMaxStages ? room / stage : kMaxStages;
+  // An even number of stages: the tiles alternate between the two MMA threads, and with an even ring a stage always holds
+  // tiles of the same thread, which therefore sees every phase of the stage's barrier. With five stages (head_dim 128
+  // and up to 128 query rows) a thread saw every second phase only: waiting for phase n while the other thread's tile, in
+  // phase n - 1, had not landed yet, it took the end of phase n - 2, which has the same parity, for its own, read a
+  // stage that was still being filled and handed it back. Copies seldom land out of order, so this took thousands of
+  // launches to show, as a launch failure.
+  args.n_stages = (room / stage < kMaxStages ? room / stage : kMaxStages) & ~1;
   const size_t smem = 1024 + static_cast<size_t>(q_bytes) + static_cast<size_t>(args.n_stages) * stage + sizeof(Small);
 
   // Tensor maps are kernel arguments, CAP requests' worth per launch: one pack per run of CAP requests. They depend
