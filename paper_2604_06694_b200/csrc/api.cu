@@ -1012,9 +1012,7 @@ int audiokv_hit_score(audiokv_ctx* ctx, const float* attn, int32_t n_steps, int3
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Launch ln{s, &ctx->launches, &ctx->prof};
-  // the status word is the first thing in the workspace, whatever plan the context holds
-  e = launch_hit_score(attn, n_steps, n_heads, row_stride, row_len, span, top_k, hit_counts, s_hit,
-                       reinterpret_cast<int*>(ctx->ws), ln);
+  e = launch_hit_score(attn, n_steps, n_heads, row_stride, row_len, span, top_k, hit_counts, s_hit, ln);
   return e == cudaSuccess ? AUDIOKV_OK : cuda_fail(ctx, e);
 }
 

@@ -250,7 +250,7 @@ cudaError_t launch_gather(const Shape& sh, const ReqDesc* d_reqs, const int32_t*
 
 // hit_score.cu: offline head score. counts: int32 [n_heads] (cleared here, then the hit totals).
 cudaError_t launch_hit_score(const float* attn, int n_steps, int n_heads, int64_t row_stride, const int32_t* row_len,
-                             const int32_t* span, int top_k, int32_t* counts, float* s_hit, int* status, Launch ln);
+                             const int32_t* span, int top_k, int32_t* counts, float* s_hit, Launch ln);
 
 // spread.cu: histogram of the kept prefix tokens over n_bins stretches of each request's prefix (hist int32
 // [n_req][n_bins], cleared here) and its summaries (stats fp32 [n_req][2]: balance, peak).

@@ -1,0 +1,46 @@
+"""The head-score kernel at the row shapes where its paths part ways: rows shorter than a warp's worth of 16-byte pieces,
+remainders before and after them, rows longer than what a block holds in registers, top_k around the limit of the
+list, and rows of so many equal values that the list overflows. Counts are whole numbers: they equal the oracle's."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2604_06694_b200 import build as akv_build
+    akv_build.build()
+    from paper_2604_06694_b200 import binding
+    return binding
+
+
+@pytest.mark.parametrize("lens,K", [((1, 2, 31, 65), 1), ((66, 127, 128, 129, 133), 64), ((1025, 1026, 1027), 65),
+                                    ((8191, 8192, 8193, 9001), 24), ((20011, 16384), 8), ((5000,), 63)])
+@pytest.mark.parametrize("kind", ["softmax", "steps"])
+def test_hit_score_row_shapes(B, lens, K, kind):
+    rng = np.random.default_rng(sum(lens) + K)
+    H, width = 7, max(lens) + 1                     # an odd stride in places: rows start off the 16-byte grid
+    attn = np.zeros((len(lens), H, width), dtype=np.float32)
+    span = np.zeros((len(lens), 2), dtype=np.int32)
+    for t, L in enumerate(lens):
+        x = rng.standard_normal((H, L))
+        if kind == "steps":                         # a handful of distinct values: ties decide by index
+            x = np.round(x)
+        attn[t, :, :L] = np.exp(x) / L
+        span[t] = (L // 4, min(L - 1, L // 4 + 40))
+    row_len = np.array(lens, dtype=np.int32)
+    prob = B.Problem(B.AUDIOKV_BF16, 1, 4, 4, 64, [64], 8, (0, 0, 0, 0), (0, 64, 0))
+    ctx = B.Context(prob)
+    counts = torch.full((H,), -1, dtype=torch.int32, device="cuda")
+    s = torch.full((H,), float("nan"), device="cuda")
+    B.audiokv_hit_score(ctx, torch.from_numpy(attn).cuda(), torch.from_numpy(row_len).cuda(),
+                        torch.from_numpy(span).cuda(), K, counts, s)
+    torch.cuda.synchronize()
+    want_s, want = oracle.hit_score(attn, row_len, span, K)
+    assert np.array_equal(counts.cpu().numpy(), want)
+    assert np.array_equal(s.cpu().numpy(), want_s.astype(np.float32))
+    assert ctx.last_device_status() == 0
