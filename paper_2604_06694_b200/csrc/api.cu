@@ -15,7 +15,6 @@ using namespace akv;
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr int kSssSmemComplex = 25600;  // 200 KB of float2: the largest work buffer kept in shared memory
 constexpr int kSlabKeys = 256;          // keys per slab of the softmax statistics (two K tiles of the tensor-core kernel)
 constexpr int kMaxRows = 1024;          // W * G
 constexpr int kMaxHeadsPerReq = 2048;
@@ -149,6 +148,9 @@ bool same_plan(const Plan& pl, const audiokv_params* p) {
   return true;
 }
 
+// What a smoothing block can have in dynamic shared memory, in float2: 227 KB less what it uses beside it.
+int sss_room() { return (232448 - sss_static_smem()) / static_cast<int>(sizeof(float2)); }
+
 // Radix sequence for a complex length N: primes 11..127 first (descending), then 7, 5, 3, 4s, 2.
 // Returns false when N has a prime factor above 127.
 bool factor_len(int N, FftSeq* sq) {
@@ -160,7 +162,7 @@ bool factor_len(int N, FftSeq* sq) {
     ++twos;
   }
   std::vector<int> odd;
-  for (int q = 3; q <= 127 && rest > 1; q += 2)
+  for (int q = 3; q <= kMaxPrime && rest > 1; q += 2)
     while (rest % q == 0) {
       odd.push_back(q);
       rest /= q;
@@ -176,10 +178,23 @@ bool factor_len(int N, FftSeq* sq) {
   return true;
 }
 
-// float2 slots of shared memory a plan's block needs: the work buffer, and with tables N (W_N) + N/2 + 1 (post) + N/4 + 1 (positions)
-int sss_smem_complex(const FftPlan& fp, bool with_tables) {
-  const int len = sss_padded(fp.bluestein ? fp.M : fp.N);
-  return len + (with_tables ? fp.N + fp.N / 2 + 1 + fp.N / 4 + 1 : 0);
+// Rough cost of a transform, in arbitrary units: index arithmetic, shared-memory traffic and butterflies of the small
+// radices are much alike per pass; a prime radix is a p x p product.
+double seq_cost(const FftSeq& sq) {
+  double c = 0.5;
+  for (int i = 0; i < sq.n_pass; ++i) c += sq.radix[i] > 13 ? 1.5 + sq.radix[i] / 20.0 : 1.0;
+  return c * sq.N;
+}
+
+// Places for the matrices of a sequence's prime radices.
+void seq_tables(FftSeq* sq, int64_t* table_len) {
+  sq->base = *table_len = (*table_len + 1) & ~int64_t(1);  // matrices and filters are read as float4
+  int off = 0;
+  for (int i = 0; i < sq->n_pass; ++i) {
+    sq->mat[i] = off;
+    if (sq->radix[i] > 13) off += (sq->radix[i] - 1) / 2 * fft_mat_cols(sq->radix[i]);
+  }
+  *table_len += off;
 }
 
 void build_fft_plan(int n, FftPlan* fp, int64_t* table_len) {
@@ -188,11 +203,7 @@ void build_fft_plan(int n, FftPlan* fp, int64_t* table_len) {
   fp->packed = (n % 2 == 0) ? 1 : 0;
   fp->N = fp->packed ? n / 2 : n;
   const int N = fp->N;
-  int buf_len = N;
-  if (factor_len(N, &fp->seq)) {
-    fp->bluestein = 0;
-    fp->M = 0;
-  } else {
+  if (!factor_len(N, &fp->seq)) {
     fp->bluestein = 1;
     // An odd real length is transformed at full complex length N = n, but only bins 0 .. (n-1)/2 are wanted (the rest
     // mirror them) and only those go back into the inverse: differences between input and output indices then span
@@ -212,32 +223,31 @@ void build_fft_plan(int n, FftPlan* fp, int64_t* table_len) {
             }
     fp->M = M;
     factor_len(M, &fp->seq);
-    buf_len = M;
   }
-  fp->in_smem = sss_padded(buf_len) <= kSssSmemComplex ? 1 : 0;
-  fp->g_pass = 0;
+  const int len = fp->seq.N;
+  fp->root_mult = fp->packed && !fp->bluestein ? 2 : 1;  // an even n's post-twiddles are roots of order 2N
+  fp->root_count = root_entries(len * fp->root_mult);
+  fp->root_count2 = fp->bluestein ? root_entries(2 * N) : 0;
+  const int room = sss_room() - 2 * (fp->root_count + fp->root_count2);  // for the work buffer
+  fp->in_smem = sss_slots(len) <= room ? 1 : 0;
   if (!fp->in_smem) {
-    // leading passes on the global buffer until a block and its twiddles (padded(len) + len slots) fit on chip
-    int len = buf_len;
-    while (fp->g_pass < fp->seq.n_pass && sss_padded(len) + len > kSssSmemComplex) len /= fp->seq.radix[fp->g_pass++];
+    // leading passes on the global buffer until a block fits on chip; then as many blocks at a time as fit
+    const int cap = (room - 4) / 273 * 256;  // sss_slots(cap) <= room
+    int blk = len;
+    while (fp->g_pass < fp->seq.n_pass && blk > cap) blk /= fp->seq.radix[fp->g_pass++];
+    fp->chunk = cap / blk * blk;
   }
-  // a direct transform also keeps its tables on chip when buffer + W_N + post-twiddles + uint16 positions fit
-  fp->tabs_smem = (!fp->bluestein && fp->in_smem && N < 65536 && sss_smem_complex(*fp, true) <= kSssSmemComplex) ? 1 : 0;
-  fp->seq.tw_offset = *table_len;
-  *table_len += fp->seq.N;
-  if (fp->packed) {
-    fp->post_offset = *table_len;
-    *table_len += N / 2 + 1;
-  }
+  fp->root_at = sss_slots(fp->in_smem ? len : fp->chunk);
+  fp->root_offset = *table_len = (*table_len + 1) & ~int64_t(1);
+  *table_len += 2 * (fp->root_count + fp->root_count2);
+  seq_tables(&fp->seq, table_len);
   if (!fp->bluestein) {
+    fp->wide_pos = N > 65536 ? 1 : 0;
     fp->pos_offset = *table_len;
-    *table_len += (N + 1) / 2;  // N int32 entries
-  }
-  if (fp->bluestein) {
-    fp->chirp_offset = *table_len;
-    *table_len += N;
-    fp->filter_offset = *table_len;
-    *table_len += fp->M;
+    *table_len += (N / 2 + 1) * (1 + fp->wide_pos) / 2 + 1;
+  } else {
+    fp->filter_offset = *table_len = (*table_len + 1) & ~int64_t(1);
+    *table_len += fp->M;  // even
     if (fp->half) {
       fp->filter2_offset = *table_len;
       *table_len += fp->M;
@@ -415,6 +425,7 @@ int build_plan(const audiokv_params* p, Plan* pl) {
     if (it == plan_of.end()) {
       FftPlan fp;
       build_fft_plan(d.P, &fp, &pl->table_len);
+      fp.id = static_cast<int>(pl->fft.size());
       pl->fft.push_back(fp);
       it = plan_of.emplace(d.P, static_cast<int>(pl->fft.size()) - 1).first;
     }
@@ -431,11 +442,7 @@ int build_plan(const audiokv_params* p, Plan* pl) {
     // a ragged batch with a few expensive lengths (chirp-z in global scratch) does not leave them to one block.
     auto cost = [&](int u) -> double {
       const FftPlan& fp = pl->fft[pl->reqs[u / sh.heads_per_req].fft_plan];
-      const double len = fp.bluestein ? fp.M : fp.N;
-      double c = len * (fp.bluestein ? 4.0 : 1.0) * (fp.in_smem ? 1.0 : 6.0);
-      for (int i = 0; i < fp.seq.n_pass; ++i)
-        if (fp.seq.radix[i] > 19) c += static_cast<double>(fp.seq.N) * fp.seq.radix[i] / 8.0;  // O(p N) prime pass
-      return c;
+      return seq_cost(fp.seq) * (fp.bluestein ? 2.0 : 1.0) * (fp.in_smem ? 1.0 : 1.5) + 8.0 * fp.n;
     };
     std::vector<int32_t> by_cost(sh.total_heads);
     for (int u = 0; u < sh.total_heads; ++u) by_cost[u] = u;
@@ -447,21 +454,12 @@ int build_plan(const audiokv_params* p, Plan* pl) {
       pl->sss_order[static_cast<size_t>(tier) * g + ((tier & 1) ? g - 1 - j : j)] = by_cost[i];
     }
   }
-  int smem_c = 2;
+  int smem_c = 64;
   pl->scratch_per_block = 0;
   for (const FftPlan& fp : pl->fft) {
-    const int len = fp.bluestein ? fp.M : fp.N;
-    if (fp.in_smem) {
-      const int need = sss_smem_complex(fp, fp.tabs_smem != 0);
-      smem_c = need > smem_c ? need : smem_c;
-    }
-    else {
-      pl->scratch_per_block = len > pl->scratch_per_block ? len : pl->scratch_per_block;
-      int blk = len;
-      for (int i = 0; i < fp.g_pass; ++i) blk /= fp.seq.radix[i];
-      const int need = sss_padded(blk) + blk;
-      smem_c = need > smem_c ? need : smem_c;
-    }
+    const int need = fp.root_at + 2 * (fp.root_count + fp.root_count2);
+    smem_c = need > smem_c ? need : smem_c;
+    if (!fp.in_smem) pl->scratch_per_block = fp.seq.N > pl->scratch_per_block ? fp.seq.N : pl->scratch_per_block;
   }
   pl->sss_smem = static_cast<size_t>(smem_c) * sizeof(float2);
 
@@ -537,7 +535,7 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream) {
       return cuda_fail(ctx, e);
     Launch ln{stream, &ctx->launches, &ctx->prof};
     e = launch_fft_tables(static_cast<int>(pl.fft.size()), reinterpret_cast<float2*>(ctx->ws + pl.lay.tables),
-                          reinterpret_cast<const FftPlan*>(ctx->ws + pl.lay.plans), ln);
+                          reinterpret_cast<const FftPlan*>(ctx->ws + pl.lay.plans), pl.sss_smem, ln);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     // The host waits until the plan is resident (once per shape): calls that follow, on any stream or inside a
     // capture, then need no ordering against the upload.

@@ -61,15 +61,20 @@ __device__ __forceinline__ int find_req(const ReqDesc* __restrict__ reqs, int n_
 }
 
 // ---- FFT plans -------------------------------------------------------------------------
-constexpr int kMaxRadices = 20;
+constexpr int kMaxRadices = 20;   // passes of one transform
+constexpr int kMaxPrime = 127;    // largest radix of a pass; lengths with a larger prime factor go through a chirp-z
+constexpr int kSssThreads = 512;  // threads of a smoothing block: 128 registers each
 
-// How one complex transform of length N is carried out (Stockham passes over `radix`).
+// How one complex transform of length N is carried out: in-place passes, forward in the order of the list (decimation
+// in frequency, natural order in, digit-reversed order out), inverse in the opposite order.
 struct FftSeq {
   int32_t N;
   int32_t n_pass;
   int32_t radix[kMaxRadices];
-  int64_t tw_offset;  // float2 index of W_N^t, t in [0, N), inside the table area
+  int32_t mat[kMaxRadices];  // radices above 13: (cos, sin)(2 pi s c / p), [s = 1 .. H][c = 0 .. fft_mat_cols - 1], from `base`
+  int64_t base;              // float2 index of the first of these matrices inside the table area
 };
+__host__ __device__ inline int fft_mat_cols(int p) { return ((p - 1) / 2 + 1 + 7) / 8 * 8; }
 
 // Plan for a real sequence of length n (one per distinct prefix length in the batch).
 struct FftPlan {
@@ -80,19 +85,24 @@ struct FftPlan {
   int32_t half;      // bluestein, not packed (odd n): only bins 0 .. (n-1)/2 are computed and fed back, M >= N + (N-1)/2
   int32_t M;         // convolution length (bluestein only)
   int32_t in_smem;   // 1: the work buffer fits in shared memory
-  int32_t tabs_smem; // 1: twiddles, post-twiddles and bin positions are staged in shared memory after the buffer
-  int32_t g_pass;    // not in_smem: leading passes that run on the global buffer; the rest runs block by block in shared memory
+  int32_t g_pass;    // not in_smem: leading passes that run on the global buffer
+  int32_t chunk;     // not in_smem: elements brought into shared memory at a time for the other passes
+  int32_t wide_pos;  // slots of bins as pairs of 32 bits (N > 65536), else of 16
+  int32_t id;        // index of this plan
+  int32_t root_at;   // where the roots of unity (double2) go in shared memory, in float2, behind the work buffer
+  int32_t root_mult; // order of the first table of roots / length of the passes
+  int32_t root_count, root_count2;  // entries of the first table, and of the second (chirp-z: order 2N)
+  int32_t reserved;
   FftSeq seq;        // passes for length N (direct) or M (bluestein)
-  int64_t chirp_offset;   // float2 index of c_j = exp(-i pi j^2 / N), j in [0, N)      (bluestein)
+  int64_t root_offset;    // float2 index of the tables of roots
   int64_t filter_offset;  // float2 index of FFT_M of the wrapped conjugate chirp / M    (bluestein)
   int64_t filter2_offset; // half: the same for the inverse direction's wrap (few inputs, all outputs)
-  int64_t post_offset;    // float2 index of exp(-2 pi i k / n), k in [0, N/2]           (packed)
-  int64_t pos_offset;     // float2 index of an int32 table: slot of bin k after the forward passes (direct)
+  int64_t pos_offset;     // float2 index of the slots of bins k and N - k after the forward passes, k in [0, N/2] (direct)
 };
 
-
-// float2 slots of a shared-memory work buffer of `len` elements: element i sits at i + (i >> 4) (see SkewBuf in sss.cu)
-__host__ __device__ inline int sss_padded(int len) { return len + (len >> 4) + 1; }
+// float2 slots of a shared-memory work buffer of `len` elements (see SmemBuf in sss.cu), and of everything a plan wants there
+__host__ __device__ inline int sss_slots(int len) { return (len + (len >> 4) + (len >> 8) + 2) & ~1; }
+__host__ __device__ inline int root_entries(int order) { return 256 + (order - 1) / 256 + 1; }
 
 // SMs of the current device, asked once per device (grids of the bandwidth-bound kernels are sized by it).
 inline int device_sm_count() {
@@ -221,7 +231,9 @@ cudaError_t launch_score_umma(const Shape& sh, const ReqDesc* h_reqs, const Scor
                               int head_end = -1, ScoreMapCache* cache = nullptr, uint64_t plan_id = 0, bool beside = false);
 
 // sss.cu
-cudaError_t launch_fft_tables(int n_plans, float2* d_tables, const FftPlan* d_plans, Launch ln);
+int sss_static_smem();  // bytes of shared memory a smoothing block uses beside its work buffer
+// smem_bytes: the dynamic shared memory launch_sss is given for these plans.
+cudaError_t launch_fft_tables(int n_plans, float2* d_tables, const FftPlan* d_plans, size_t smem_bytes, Launch ln);
 // order: n_order head indices (or -1); block b takes entries b, b + grid, ... ; a null order stands for the n_order heads
 // first_head, first_head + 1, ... . smoothed may be null when budgets, cu_kept and kept_idx are given: the kernel then goes on to the
 // top-k selection of each head from the smoothed scores it holds on chip (step 4a of the pass).

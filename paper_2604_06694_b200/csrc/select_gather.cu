@@ -6,13 +6,16 @@
 namespace akv {
 namespace {
 
-// One block per head: the head's keys staged once in shared memory when they fit, then select_topk.
+constexpr int kSelThreads = 1024;
+
+// One block per head: the head's keys staged once in shared memory when they fit, then select_entries.
 __global__ void __launch_bounds__(kSelThreads, 1)
 select_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const float* __restrict__ smoothed,
               const int32_t* __restrict__ budgets, const int32_t* __restrict__ cu_kept,
               int32_t* __restrict__ kept_idx, int smem_keys, int* __restrict__ status) {
-  extern __shared__ uint32_t skeys[];
+  extern __shared__ uint32_t skeys[];  // smem_keys keys, then the masks and prefix sums of the longest head
   __shared__ SelectSmem ssm;
+  __shared__ uint32_t s_min, s_max;
 
   for (int u = blockIdx.x; u < sh.total_heads; u += gridDim.x) {
     const int r = u / sh.heads_per_req;
@@ -25,14 +28,35 @@ select_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const float* __restric
       k = k < 0 ? 0 : P;
     }
     const bool staged = P <= smem_keys;
+    if (threadIdx.x == 0) {
+      s_min = 0xffffffffu;
+      s_max = 0u;
+    }
     __syncthreads();
-    if (staged)
-      for (int j = threadIdx.x; j < P; j += kSelThreads) skeys[j] = score_key(s[j]);
+    uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll 4
+    for (int j = threadIdx.x; j < P; j += kSelThreads) {
+      const uint32_t key = score_key(s[j]);
+      if (staged) skeys[j] = key;
+      lo = min(lo, key);
+      hi = max(hi, key);
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0) {
+      atomicMin(&s_min, lo);
+      atomicMax(&s_max, hi);
+    }
     __syncthreads();
+    uint32_t* words = skeys + smem_keys;
+    int* pre = reinterpret_cast<int*>(words) + select_words(P, false);
+    int32_t* out = kept_idx + cu_kept[u];
     if (staged)
-      select_topk([&](int j) -> uint32_t { return skeys[j]; }, P, W, k, kept_idx + cu_kept[u], &ssm, status);
+      select_entries<kSelThreads, false>([&](int j) { return make_float2(__uint_as_float(skeys[j]), 0.f); }, P, P, W, k,
+                                         s_min, s_max, out, &ssm, words, pre, status);
     else
-      select_topk([&](int j) -> uint32_t { return score_key(s[j]); }, P, W, k, kept_idx + cu_kept[u], &ssm, status);
+      select_entries<kSelThreads, false>([&](int j) { return make_float2(__uint_as_float(score_key(s[j])), 0.f); }, P, P,
+                                         W, k, s_min, s_max, out, &ssm, words, pre, status);
   }
 }
 
@@ -101,8 +125,8 @@ gather_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const int32_t* __restr
 
 cudaError_t launch_select(const Shape& sh, const ReqDesc* d_reqs, const float* smoothed, const int32_t* budgets,
                           const int32_t* cu_kept, int32_t* kept_idx, int max_P, int* status, Launch ln) {
-  const int smem_keys = max_P <= 48 * 1024 ? max_P : 48 * 1024;
-  const size_t smem = static_cast<size_t>(smem_keys) * sizeof(uint32_t);
+  const int smem_keys = max_P <= 40 * 1024 ? max_P : 40 * 1024;
+  const size_t smem = (static_cast<size_t>(smem_keys) + 2 * select_words(max_P, false)) * sizeof(uint32_t);
   cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int max_grid = device_sm_count() * 4;

@@ -2,19 +2,30 @@
 //
 // A real sequence of even length n is packed into a complex one of length N = n/2
 // (odd n: length N = n with zero imaginary part). The complex transform is an in-place
-// mixed-radix decimation-in-frequency FFT (radices 2 to 19 one butterfly per thread, larger primes up
-// to 127 as paired O(p^2) sums, one output pair of one butterfly per task); its output is left in digit-reversed order and addressed through
-// pos(k), and the inverse is the matching decimation-in-time chain, so no reordering pass
-// and no second buffer is needed. Lengths with a larger prime factor go through a chirp-z
-// (Bluestein) convolution of power-of-two length M >= 2N - 1 built from the same passes.
-// The work buffer lives in shared memory when it fits, else in a per-block global scratch.
+// mixed-radix decimation-in-frequency FFT: radices 2 to 13 one butterfly per thread, larger primes
+// as a product with the p x p cosine and sine matrices, register-tiled. Its output is left in digit-reversed order
+// and addressed through a table, and the inverse is the matching decimation-in-time chain, so no reordering pass
+// and no second buffer is needed. Lengths with a large prime factor go through a chirp-z
+// (Bluestein) convolution of a length M >= 2N - 1 made of small radices.
+// The work buffer lives in shared memory when it fits. A longer one lies in a per-block global scratch (it stays in
+// L2): the first pass, and the last of the inverse, run there; after it the transform falls apart into contiguous
+// blocks, which are brought into shared memory a chunk at a time for everything in between.
+//
+// What bounds it: a head is a chain of short phases with a barrier between them, each a few thousand cycles of
+// shared-memory traffic and index arithmetic on one SM; HBM sees only the scores coming in and the indices going out.
+// So the block reads the scores once into shared memory, 512 threads keep eight or more independent accesses in
+// flight each (128 registers; the earlier 1024 threads with 64 registers spent more cycles on the barriers and on
+// radix-4 passes than on arithmetic), every access to shared memory is a compile-time LDS / STS through a swizzle
+// that keeps the power-of-two strides of the passes and the digit-reversed reads of the spectrum off the same banks,
+// and twiddles come from per-pass tables whose reads are contiguous over the threads.
 #include "common.cuh"
 #include "select.cuh"
 
 namespace akv {
 namespace {
 
-constexpr int kSssThreads = kSelThreads;  // 1024: select_topk runs in the same block
+constexpr int kT = kSssThreads;
+constexpr int kWarps = kT / 32;
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
@@ -29,63 +40,160 @@ __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2
 __device__ __forceinline__ float2 mul_i(float2 a) { return make_float2(-a.y, a.x); }    // i * a
 __device__ __forceinline__ float2 mul_mi(float2 a) { return make_float2(a.y, -a.x); }   // -i * a
 
-// The work buffer of a transform. In shared memory element i lives at i + (i >> 4): the passes of an in-place
-// transform read with power-of-two strides (and the late ones with strides of a few elements between
-// neighbouring threads), which without the skew puts many lanes on the same banks. sh = 31 switches the skew
-// off (global scratch, tables).
-struct SkewBuf {
+// ---- work buffers ------------------------------------------------------------------------
+// Shared memory: element e sits at e + e / 16 + e / 256. Sixteen float2 are one turn of the banks: neighbours come out on
+// different banks, so do the power-of-two strides of late passes, and the two divisors together keep the strides of the
+// digit-reversed reads of the spectrum apart to a few. (An exclusive-or of the low four bits with the next twelve
+// has fewer conflicts still, but six operations per access instead of four; a radix-8 pass has sixteen accesses.)
+extern __shared__ __align__(16) float2 g_sbuf[];
+struct SmemBuf {
+  static __device__ __forceinline__ int slot(int e) { return e + (e >> 4) + (e >> 8); }
+  __device__ __forceinline__ float2 ld(int e) const { return g_sbuf[slot(e)]; }
+  __device__ __forceinline__ void st(int e, float2 v) const { g_sbuf[slot(e)] = v; }
+};
+struct GlobBuf {
   float2* p;
-  int sh;
-  int off;
-  __device__ __forceinline__ float2& operator[](int i) const {
-    const int e = off + i;
-    return p[e + (e >> sh)];
-  }
-  __device__ __forceinline__ SkewBuf operator+(int d) const { return SkewBuf{p, sh, off + d}; }
+  __device__ __forceinline__ float2 ld(int e) const { return p[e]; }
+  __device__ __forceinline__ void st(int e, float2 v) const { p[e] = v; }
 };
 
-// cos / sin of 2 pi t / R for the odd radices handled per thread.
+// The n scores of a head as transform entries: entry m = tokens 2m and 2m + 1 (packed) or token m and zero.
+struct Scores {
+  const float* x;
+  bool packed, pairs;  // pairs: packed, and the head starts on an 8-byte boundary
+  __device__ __forceinline__ float2 pair(int m) const { return *reinterpret_cast<const float2*>(x + 2 * m); }
+  __device__ __forceinline__ float2 single(int m) const {
+    const int j = packed ? 2 * m : m;
+    const float v = x[j], w = x[packed ? j + 1 : j];
+    return make_float2(v, packed ? w : 0.f);
+  }
+  __device__ __forceinline__ float2 entry(int m) const { return pairs ? pair(m) : single(m); }
+};
+
+// Loops of the block over [0, n). An access to L2 takes some 700 cycles from here, and with 16 warps on the SM it is
+// the number of accesses in flight that decides the time of every phase: get(i) is therefore issued for U elements
+// before the first use(i, value), with no branch in between (a branch, even a uniform one, keeps the compiler from
+// moving the loads of one element above the use of another: the sweep that reads a head's 32736 scores took 23 k cycles
+// that way, 32 round trips one after another).
+template <int U, class Get, class Use>
+__device__ __forceinline__ void batched(int n, Get get, Use use) {
+  batched_loop<kT, U>(n, get, use);
+}
+
+// use(m, entry m) for every entry of the head's scores.
+template <int U, class Use>
+__device__ __forceinline__ void for_entries(const Scores& sc, int n, Use use) {
+  if (sc.pairs) batched<U>(n, [&](int m) { return sc.pair(m); }, use);
+  else batched<U>(n, [&](int m) { return sc.single(m); }, use);
+}
+
+// Roots of unity e^{-2 pi i e / Q} of one order Q, 0 <= e < Q: the product, in double precision, of two table entries in
+// shared memory, 256 fine ones and Q / 256 coarse ones, rounded once. Every twiddle, chirp and post-twiddle of a head
+// comes from here, and is the correctly rounded value that a table of all Q of them would hold.
+// (Tables of whole passes in global memory were tried first: all blocks then read the same lines at the same time, and
+// L2 delivered 6 bytes per clock and SM: one sweep over 15840 twiddles took 23 k cycles, more than the
+// butterflies it belonged to. A table of all Q in shared memory fits beside the shorter buffers only. Products of
+// single-precision entries are twice as fast, but off by an ulp or two, and the selection behind the transform sees
+// the last bit: with attention sinks every other rounding of the transform moves a token across the threshold in 5 % of the
+// heads at n = 16352.)
+__device__ __forceinline__ double2 zmul(double2 a, double2 b) { return make_double2(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x)); }
+__device__ __forceinline__ float2 rounded(double2 a) { return make_float2(static_cast<float>(a.x), static_cast<float>(a.y)); }
+struct Roots {
+  int at;    // where the fine entries lie in g_sbuf, in float2 (even); the coarse ones follow
+  int mult;  // order of the table / order asked for
+  __device__ __forceinline__ double2 exact(int e) const {
+    const double2* tab = reinterpret_cast<const double2*>(g_sbuf + at);
+    e *= mult;
+    return zmul(tab[e & 255], tab[256 + (e >> 8)]);
+  }
+  __device__ __forceinline__ float2 operator()(int e) const { return rounded(exact(e)); }
+};
+
+// ---- shared state ------------------------------------------------------------------------
+constexpr int kDirectBins = 12;
+constexpr int kDirectRows = 128;  // entries per thread the table covers: even n up to 131072, odd n up to 65535
+
+// First bins of the spectrum without a transform (see direct_bins).
+struct DirectSmem {
+  float2 tab[kDirectRows][kDirectBins];     // tab[i][k] = w_k^{a kT i}
+  float2 part[kWarps][kDirectBins];         // per warp: bins 1 .. kDirectBins - 1
+  double energy[kDirectBins];               // |F_k|^2 as it counts towards the cumulative energy
+  double tot[3];                            // F_0 (= sum x), the energy threshold rho E, the margin of a decision
+  float2 bin[kDirectBins];                  // F_k
+  int kstar;                                // stage 1: k*, -1: left to the transform, -2: the bins decide
+  int k_hi;                                 // last bin to evaluate; after stage 3: k* or -1
+};
+
+constexpr int kMaxChunks = 2 * (65536 / 64 + 1);  // energy sums: 32 bins each, from both ends of the spectrum
+constexpr int kPreInts = 832;                     // prefix sums of the selection, for a buffer in shared memory
+
+struct SssShared {
+  FftPlan pl;
+  // the head at hand; kept here and not in registers, which the passes want all to themselves
+  const float* x;
+  float* y;
+  float2* g;
+  int32_t *out, *kstar_out;
+  int k_keep;
+  double sums[3];      // sum x, sum x^2, alternating sum
+  int kstar;
+  int loaded;          // plan whose roots lie in shared memory
+  uint32_t kmin, kmax;
+  int pre[kPreInts];
+  alignas(16) union {  // never alive at the same time
+    DirectSmem ds;
+    double energy[kMaxChunks];
+    SelectSmem sel;
+  };
+};
+__shared__ __align__(16) SssShared S;
+
+// While a pass runs none of the union is alive: a prime pass stages rows of its matrix there.
+constexpr int kPassScratch = sizeof(double) * kMaxChunks / sizeof(float4);
+__device__ __forceinline__ float4* pass_scratch() { return reinterpret_cast<float4*>(S.energy); }
+
+// ---- passes ------------------------------------------------------------------------------
+// cos / sin of 2 pi t / R, 0 <= t < R, for the odd radices handled in registers (t is a compile-time constant at every use).
 template <int R>
-__device__ __forceinline__ float rcos(int t) {
-  if (R == 3) return t == 0 ? 1.f : -0.5f;
-  if (R == 5) return t == 0 ? 1.f : (t == 1 || t == 4) ? 0.30901699437494745f : -0.8090169943749475f;
-  if (R == 7)
-    return t == 0 ? 1.f
-                  : (t == 1 || t == 6) ? 0.6234898018587336f
-                                       : (t == 2 || t == 5) ? -0.2225209339563144f : -0.9009688679024191f;
-  return 0.f;
+__device__ __forceinline__ constexpr float rcos(int t) {
+  constexpr float c3[2] = {1.f, -0.5f};
+  constexpr float c5[3] = {1.f, 0.30901699437494745f, -0.8090169943749475f};
+  constexpr float c7[4] = {1.f, 0.6234898018587336f, -0.2225209339563144f, -0.9009688679024191f};
+  constexpr float c11[6] = {1.f, 0.84125353283118121f, 0.41541501300188644f, -0.142314838273285f, -0.65486073394528499f,
+                            -0.95949297361449737f};
+  constexpr float c13[7] = {1.f, 0.88545602565320991f, 0.56806474673115592f, 0.12053668025532301f,
+                            -0.35460488704253545f, -0.74851074817110119f, -0.97094181742605201f};
+  const int i = 2 * t > R ? R - t : t;
+  return R == 3 ? c3[i < 2 ? i : 0] : R == 5 ? c5[i < 3 ? i : 0] : R == 7 ? c7[i < 4 ? i : 0] : R == 11 ? c11[i < 6 ? i : 0] : c13[i];
 }
 template <int R>
-__device__ __forceinline__ float rsin(int t) {
-  if (R == 3) return t == 0 ? 0.f : t == 1 ? 0.8660254037844386f : -0.8660254037844386f;
-  if (R == 5)
-    return t == 0 ? 0.f
-                  : t == 1 ? 0.9510565162951535f
-                           : t == 2 ? 0.5877852522924731f : t == 3 ? -0.5877852522924731f : -0.9510565162951535f;
-  if (R == 7)
-    return t == 0 ? 0.f
-                  : t == 1 ? 0.7818314824680298f
-                           : t == 2 ? 0.9749279121818236f
-                                    : t == 3 ? 0.4338837391175581f
-                                             : t == 4 ? -0.4338837391175581f
-                                                      : t == 5 ? -0.9749279121818236f : -0.7818314824680298f;
-  return 0.f;
+__device__ __forceinline__ constexpr float rsin(int t) {
+  constexpr float s3[2] = {0.f, 0.8660254037844386f};
+  constexpr float s5[3] = {0.f, 0.9510565162951535f, 0.5877852522924731f};
+  constexpr float s7[4] = {0.f, 0.7818314824680298f, 0.9749279121818236f, 0.4338837391175581f};
+  constexpr float s11[6] = {0.f, 0.54064081745559756f, 0.90963199535451833f, 0.9898214418809328f, 0.75574957435425827f,
+                            0.28173255684142967f};
+  constexpr float s13[7] = {0.f, 0.46472317204376851f, 0.82298386589365635f, 0.99270887409805397f, 0.93501624268541483f,
+                            0.66312265824079519f, 0.23931566428755768f};
+  const int i = 2 * t > R ? R - t : t;
+  const float v = R == 3 ? s3[i < 2 ? i : 0] : R == 5 ? s5[i < 3 ? i : 0] : R == 7 ? s7[i < 4 ? i : 0] : R == 11 ? s11[i < 6 ? i : 0] : s13[i];
+  return 2 * t > R ? -v : v;
 }
 
 // In-register DFT of R points: X_c = sum_s v_s exp(-/+ 2 pi i s c / R)  (INV: plus sign).
 template <int R, bool INV>
-__device__ __forceinline__ void dft_small(float2* v) {
-  if (R == 2) {
-    float2 a = v[0], b = v[1];
+__device__ __forceinline__ void dft_small(float2 (&v)[R]) {
+  auto rot = [](float2 a) { return INV ? mul_i(a) : mul_mi(a); };  // times exp(-/+ i pi / 2)
+  if constexpr (R == 2) {
+    const float2 a = v[0], b = v[1];
     v[0] = cadd(a, b);
     v[1] = csub(a, b);
-  } else if (R == 4) {
-    float2 t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]), t2 = cadd(v[1], v[3]), t3 = csub(v[1], v[3]);
+  } else if constexpr (R == 4) {
+    const float2 t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]), t2 = cadd(v[1], v[3]), t3 = rot(csub(v[1], v[3]));
     v[0] = cadd(t0, t2);
     v[2] = csub(t0, t2);
-    float2 r = INV ? mul_i(t3) : mul_mi(t3);
-    v[1] = cadd(t1, r);
-    v[3] = csub(t1, r);
+    v[1] = cadd(t1, t3);
+    v[3] = csub(t1, t3);
   } else {
     constexpr int H = (R - 1) / 2;
     float2 p[H + 1], q[H + 1];
@@ -94,7 +202,7 @@ __device__ __forceinline__ void dft_small(float2* v) {
       p[s] = cadd(v[s], v[R - s]);
       q[s] = csub(v[s], v[R - s]);
     }
-    float2 v0 = v[0];
+    const float2 v0 = v[0];
     float2 sum = v0;
 #pragma unroll
     for (int s = 1; s <= H; ++s) sum = cadd(sum, p[s]);
@@ -111,447 +219,243 @@ __device__ __forceinline__ void dft_small(float2* v) {
         B.y = fmaf(q[s].y, ss, B.y);
       }
       // forward: X_c = A - i B, X_{R-c} = A + i B; inverse: the other way round
-      float2 iB = mul_i(B);
+      const float2 iB = mul_i(B);
       v[c] = INV ? cadd(A, iB) : csub(A, iB);
       v[R - c] = INV ? csub(A, iB) : cadd(A, iB);
     }
   }
 }
 
-// One in-place pass of radix R over sub-transforms of length ns (thread per butterfly).
+// v[c] times w1^c (INV: times its conjugate), c = 1 .. R - 1; the powers are formed in double precision and rounded each.
+template <int R, bool INV>
+__device__ __forceinline__ void twiddle(float2 (&v)[R], double2 w1) {
+  double2 w = w1;
+#pragma unroll
+  for (int c = 1; c < R; ++c) {
+    const float2 r = rounded(w);
+    v[c] = INV ? cmulc(v[c], r) : cmul(v[c], r);
+    if (c + 1 < R) w = zmul(w, w1);
+  }
+}
+
+// t / m for t < 2^32 / m by a multiplication: magic = ceil(2^32 / m). (t m <= (length / R)^2 < 2^32 for every pass.)
+struct FastDiv {
+  uint32_t m, magic;
+  __device__ __forceinline__ explicit FastDiv(int d) : m(d), magic(d > 1 ? 0xffffffffu / static_cast<uint32_t>(d) + 1u : 0u) {}
+  __device__ __forceinline__ int div(int t) const { return m > 1 ? static_cast<int>(__umulhi(static_cast<uint32_t>(t), magic)) : t; }
+};
+
+// One in-place pass of radix R over `total` elements that fall into sub-transforms of length ns (thread per butterfly).
 // Forward (decimation in frequency): DFT_R, then multiply output c by W_ns^{j c}.
 // Inverse (decimation in time): multiply input c by W_ns^{-j c}, then inverse DFT_R.
-template <int R, bool INV>
-__device__ __forceinline__ void pass_small(SkewBuf buf, int N, int ns, const float2* tw) {
-  const int m = ns / R, step = N / ns, nb = N / R;
-  for (int t = threadIdx.x; t < nb; t += kSssThreads) {
-    const int b = t / m, j = t - b * m;
-    const SkewBuf p = buf + (b * ns + j);
+// `in` and `out` are the same buffer, or two views of it (the element is then moved on the way).
+template <int R, bool INV, class In, class Out>
+__device__ __forceinline__ void pass_small(const In& in, const Out& out, int total, int ns, int N, const Roots& root) {
+  const int m = ns / R, nb = total / R, step = N / ns;
+  const FastDiv dm(m);
+#pragma unroll 1
+  for (int t = threadIdx.x; t < nb; t += kT) {
+    const int b = dm.div(t), j = t - b * m;
+    const int e0 = b * ns + j;
     float2 v[R];
 #pragma unroll
-    for (int s = 0; s < R; ++s) v[s] = p[s * m];
-    if (!INV) {
-      dft_small<R, false>(v);
-      if (m > 1) {
+    for (int s = 0; s < R; ++s) v[s] = in.ld(e0 + s * m);
+    if (INV && m > 1) twiddle<R, true>(v, root.exact(j * step));
+    dft_small<R, INV>(v);
+    if (!INV && m > 1) twiddle<R, false>(v, root.exact(j * step));
 #pragma unroll
-        for (int c = 1; c < R; ++c) v[c] = cmul(v[c], tw[j * c * step]);
-      }
-    } else {
-      if (m > 1) {
-#pragma unroll
-        for (int c = 1; c < R; ++c) v[c] = cmulc(v[c], tw[j * c * step]);
-      }
-      dft_small<R, true>(v);
-    }
-#pragma unroll
-    for (int s = 0; s < R; ++s) p[s * m] = v[s];
+    for (int s = 0; s < R; ++s) out.st(e0 + s * m, v[s]);
   }
   __syncthreads();
 }
 
-// cos / sin of 2 pi t / R for the odd radices handled by one thread per butterfly with streamed outputs.
-template <int R>
-__device__ __forceinline__ float ocos(int t) {
-  if (R == 11) {
-    switch (t) {
-      case 0: return 1.0f;
-      case 1: return 0.84125353283118121f;
-      case 2: return 0.41541501300188644f;
-      case 3: return -0.142314838273285f;
-      case 4: return -0.65486073394528499f;
-      case 5: return -0.95949297361449737f;
-      case 6: return -0.95949297361449748f;
-      case 7: return -0.65486073394528521f;
-      case 8: return -0.14231483827328523f;
-      case 9: return 0.41541501300188605f;
-      case 10: return 0.84125353283118121f;
-    }
-  }
-  if (R == 13) {
-    switch (t) {
-      case 0: return 1.0f;
-      case 1: return 0.88545602565320991f;
-      case 2: return 0.56806474673115592f;
-      case 3: return 0.12053668025532301f;
-      case 4: return -0.35460488704253545f;
-      case 5: return -0.74851074817110119f;
-      case 6: return -0.97094181742605201f;
-      case 7: return -0.97094181742605212f;
-      case 8: return -0.7485107481711013f;
-      case 9: return -0.3546048870425359f;
-      case 10: return 0.1205366802553232f;
-      case 11: return 0.56806474673115481f;
-      case 12: return 0.88545602565321002f;
-    }
-  }
-  if (R == 17) {
-    switch (t) {
-      case 0: return 1.0f;
-      case 1: return 0.93247222940435581f;
-      case 2: return 0.73900891722065909f;
-      case 3: return 0.44573835577653831f;
-      case 4: return 0.092268359463302016f;
-      case 5: return -0.27366299007208289f;
-      case 6: return -0.60263463637925629f;
-      case 7: return -0.85021713572961399f;
-      case 8: return -0.98297309968390179f;
-      case 9: return -0.98297309968390179f;
-      case 10: return -0.8502171357296141f;
-      case 11: return -0.60263463637925718f;
-      case 12: return -0.27366299007208311f;
-      case 13: return 0.092268359463302432f;
-      case 14: return 0.4457383557765377f;
-      case 15: return 0.73900891722065853f;
-      case 16: return 0.93247222940435581f;
-    }
-  }
-  if (R == 19) {
-    switch (t) {
-      case 0: return 1.0f;
-      case 1: return 0.94581724170063464f;
-      case 2: return 0.78914050939639357f;
-      case 3: return 0.54694815812242692f;
-      case 4: return 0.24548548714079924f;
-      case 5: return -0.082579345472332269f;
-      case 6: return -0.40169542465296942f;
-      case 7: return -0.67728157162574087f;
-      case 8: return -0.87947375120648896f;
-      case 9: return -0.98636130340272232f;
-      case 10: return -0.98636130340272243f;
-      case 11: return -0.8794737512064893f;
-      case 12: return -0.6772815716257411f;
-      case 13: return -0.40169542465296904f;
-      case 14: return -0.082579345472332741f;
-      case 15: return 0.24548548714079879f;
-      case 16: return 0.54694815812242659f;
-      case 17: return 0.78914050939639391f;
-      case 18: return 0.94581724170063464f;
-    }
-  }
-  return 0.f;
-}
-template <int R>
-__device__ __forceinline__ float osin(int t) {
-  if (R == 11) {
-    switch (t) {
-      case 0: return 0.0f;
-      case 1: return 0.54064081745559756f;
-      case 2: return 0.90963199535451833f;
-      case 3: return 0.9898214418809328f;
-      case 4: return 0.75574957435425827f;
-      case 5: return 0.28173255684142967f;
-      case 6: return -0.28173255684142939f;
-      case 7: return -0.75574957435425816f;
-      case 8: return -0.98982144188093268f;
-      case 9: return -0.90963199535451855f;
-      case 10: return -0.54064081745559744f;
-    }
-  }
-  if (R == 13) {
-    switch (t) {
-      case 0: return 0.0f;
-      case 1: return 0.46472317204376851f;
-      case 2: return 0.82298386589365635f;
-      case 3: return 0.99270887409805397f;
-      case 4: return 0.93501624268541483f;
-      case 5: return 0.66312265824079519f;
-      case 6: return 0.23931566428755768f;
-      case 7: return -0.23931566428755743f;
-      case 8: return -0.66312265824079497f;
-      case 9: return -0.93501624268541472f;
-      case 10: return -0.99270887409805397f;
-      case 11: return -0.82298386589365702f;
-      case 12: return -0.4647231720437684f;
-    }
-  }
-  if (R == 17) {
-    switch (t) {
-      case 0: return 0.0f;
-      case 1: return 0.36124166618715292f;
-      case 2: return 0.67369564364655721f;
-      case 3: return 0.89516329135506234f;
-      case 4: return 0.99573417629503447f;
-      case 5: return 0.96182564317281904f;
-      case 6: return 0.7980172272802396f;
-      case 7: return 0.52643216287735606f;
-      case 8: return 0.18374951781657037f;
-      case 9: return -0.18374951781657012f;
-      case 10: return -0.52643216287735584f;
-      case 11: return -0.79801722728023894f;
-      case 12: return -0.96182564317281904f;
-      case 13: return -0.99573417629503447f;
-      case 14: return -0.89516329135506256f;
-      case 15: return -0.67369564364655776f;
-      case 16: return -0.36124166618715303f;
-    }
-  }
-  if (R == 19) {
-    switch (t) {
-      case 0: return 0.0f;
-      case 1: return 0.32469946920468346f;
-      case 2: return 0.61421271268966782f;
-      case 3: return 0.83716647826252855f;
-      case 4: return 0.96940026593933037f;
-      case 5: return 0.99658449300666985f;
-      case 6: return 0.9157733266550574f;
-      case 7: return 0.73572391067313181f;
-      case 8: return 0.47594739303707367f;
-      case 9: return 0.16459459028073403f;
-      case 10: return -0.16459459028073378f;
-      case 11: return -0.47594739303707312f;
-      case 12: return -0.73572391067313159f;
-      case 13: return -0.91577332665505762f;
-      case 14: return -0.99658449300666985f;
-      case 15: return -0.96940026593933049f;
-      case 16: return -0.83716647826252877f;
-      case 17: return -0.61421271268966737f;
-      case 18: return -0.32469946920468373f;
-    }
-  }
-  return 0.f;
-}
-
-// One in-place pass of an odd radix R in {11, 13, 17, 19}: one thread per butterfly. The inputs are folded into
-// P_s = a_s + a_{R-s}, Q_s = a_s - a_{R-s} (kept in registers); outputs c and R - c come from the same
-// real-by-complex products, X_c = A -/+ iB with A = a_0 + sum_s P_s cos(2 pi s c / R), B = sum_s Q_s sin(2 pi s c / R),
-// and are written back as soon as they are complete.
-template <int R, bool INV>
-__device__ __noinline__ void pass_odd(SkewBuf buf, int N, int ns, const float2* tw) {
-  constexpr int H = (R - 1) / 2;
-  const int m = ns / R, step = N / ns, nb = N / R;
-  for (int t = threadIdx.x; t < nb; t += kSssThreads) {
-    const int b = t / m, j = t - b * m;
-    const SkewBuf p = buf + (b * ns + j);
-    const float2 v0 = p[0];
-    float2 P[H], Q[H];
-    float2 sum = v0;
+// The same pass for an odd prime radix p, 17 <= p <= kMaxPrime. With inputs s and p - s folded into P_s = a_s + a_{p-s}
+// and Q_s = a_s - a_{p-s}, outputs c and p - c come from the same real-by-complex sums, X_c = A_c -/+ i B_c,
+// A_c = a_0 + sum_s P_s cos(2 pi s c / p), B_c = sum_s Q_s sin(2 pi s c / p): a product of a small matrix with as many
+// columns as there are butterflies. A thread computes a tile of TO outputs x TC butterflies in registers: per s it reads TC
+// values of P and of Q and TO (cos, sin) pairs, the latter the same for most of a warp and staged in shared memory, for 4 TO TC
+// FMAs. 8 x 2 where that gives enough tiles to go round, 2 x 1 for few butterflies (which are latency: a length of 7 x 167
+// has 44 tiles of 8 x 2, two warps' worth). The folding sweep (inverse) and the write-back (forward) carry the
+// pass twiddles. (An earlier version gave a thread 5 outputs of one butterfly and looked the cosines up by (s c mod p): the
+// radix-73 pass of N = 8176 took 45-55 k cycles, seven loads and their index arithmetic for every 20 FMAs.)
+template <bool INV, class Buf, int TO, int TC>
+__device__ __forceinline__ void prime_product(const Buf& buf, int ns, int p, int m, int nb, int step, const Roots& root,
+                                              const float2* __restrict__ mat) {
+  const int H = (p - 1) / 2, Cp = fft_mat_cols(p);
+  const FastDiv dm(m);
+  const int n_ct = Cp / TO;                 // tiles of outputs
+  const int tiles = (nb + TC - 1) / TC;     // tiles of butterflies
+  const int n_round = (tiles * n_ct + kT - 1) / kT;
+  const int per_round = min((tiles + n_round - 1) / n_round, kT / n_ct);  // rounds of equal size
+  float4* s_mat = pass_scratch();
+  const int s_rows = min(H, kPassScratch / (Cp / 2));  // matrix rows staged at a time
+  int staged = -1;
+  for (int p0 = 0; p0 < tiles; p0 += per_round) {
+    const int np = min(per_round, tiles - p0);
+    const int ct = static_cast<int>(threadIdx.x) / np;  // neighbouring threads: the same outputs of neighbouring butterflies
+    const int jt = p0 + static_cast<int>(threadIdx.x) - ct * np;
+    const bool live = ct < n_ct;
+    int e[TC], j[TC];
+    float2 A[TC][TO], B[TC][TO];
 #pragma unroll
-    for (int sI = 1; sI <= H; ++sI) {
-      float2 x = p[sI * m], y = p[(R - sI) * m];
-      if (INV && m > 1) {
-        x = cmulc(x, tw[j * sI * step]);
-        y = cmulc(y, tw[j * (R - sI) * step]);
+    for (int h = 0; h < TC; ++h) {
+      const int col = min(TC * jt + h, nb - 1), b = dm.div(col);
+      j[h] = col - b * m;
+      e[h] = b * ns + j[h];
+#pragma unroll
+      for (int i = 0; i < TO; ++i) {
+        A[h][i] = buf.ld(e[h]);
+        B[h][i] = make_float2(0.f, 0.f);
       }
-      P[sI - 1] = cadd(x, y);
-      Q[sI - 1] = csub(x, y);
-      sum = cadd(sum, P[sI - 1]);
     }
-    p[0] = sum;
-#pragma unroll
-    for (int c = 1; c <= H; ++c) {
-      float2 A = v0, B = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int sI = 1; sI <= H; ++sI) {
-        const float cc = ocos<R>((sI * c) % R), ss = osin<R>((sI * c) % R);
-        A.x = fmaf(P[sI - 1].x, cc, A.x);
-        A.y = fmaf(P[sI - 1].y, cc, A.y);
-        B.x = fmaf(Q[sI - 1].x, ss, B.x);
-        B.y = fmaf(Q[sI - 1].y, ss, B.y);
+    for (int s0 = 0; s0 < H; s0 += s_rows) {
+      const int rows = min(s_rows, H - s0);
+      if (staged != s0) {
+        __syncthreads();
+        const float4* src = reinterpret_cast<const float4*>(mat + s0 * Cp);
+        batched<4>(rows * (Cp / 2), [&](int t) { return __ldg(src + t); }, [&](int t, float4 v) { s_mat[t] = v; });
+        staged = s0;
+        __syncthreads();
       }
-      const float2 iB = mul_i(B);
-      float2 xc = INV ? cadd(A, iB) : csub(A, iB);
-      float2 xq = INV ? csub(A, iB) : cadd(A, iB);
-      if (!INV && m > 1) {
-        xc = cmul(xc, tw[j * c * step]);
-        xq = cmul(xq, tw[j * (R - c) * step]);
-      }
-      p[c * m] = xc;
-      p[(R - c) * m] = xq;
-    }
-  }
-  __syncthreads();
-}
-
-// The same pass for an odd prime radix p, 23 <= p <= 127 (11 to 19 have pass_odd). A length-p DFT is O(p^2); pairing
-// inputs s and p - s (P = a_s + a_{p-s}, Q = a_s - a_{p-s}) gives outputs c and p - c from the
-// same real-by-complex products: X_c = A -/+ iB, A = a_0 + sum_s P_s cos(2 pi s c / p),
-// B = sum_s Q_s sin(2 pi s c / p); c = 0 is the plain sum. One task = one butterfly and kPrimeOut
-// consecutive c in [0, (p-1)/2]; consecutive threads take consecutive butterflies of the same c, so
-// the data reads are contiguous and the cos/sin reads are broadcasts. A thread keeps the results of
-// its (at most kPrimeTasks) tasks in registers until every task of the round has read its inputs.
-// The pass twiddles are applied in a sweep of their own (inverse: before, forward: with the
-// write-back).
-constexpr int kPrimeTasks = 1;  // tasks per thread and round (two were tried: the second slot is mostly empty and costs registers)
-constexpr int kPrimeOut = 5;    // consecutive c per task: the folded inputs P_s, Q_s are formed once for all of them
-
-template <bool INV>
-__device__ __noinline__ void pass_prime(SkewBuf buf, int N, int ns, int p, const float2* tw,
-                                        float2* cs /* smem [128]: (cos, sin) of 2 pi t / p */) {
-  __syncthreads();
-  for (int t = threadIdx.x; t < p; t += kSssThreads) {
-    const float2 w = tw[t * (N / p)];
-    cs[t] = make_float2(w.x, -w.y);
-  }
-  const int m = ns / p, step = N / ns, nb = N / p, H = (p - 1) / 2;
-  if (INV && m > 1) {
-    // element e = b ns + s m + j gets W_ns^{-j s}
-    for (int e = threadIdx.x; e < N; e += kSssThreads) {
-      const int r = e % ns, sI = r / m, j = r - sI * m;
-      if (sI > 0 && j > 0) buf[e] = cmulc(buf[e], tw[j * sI * step]);
-    }
-  }
-  __syncthreads();
-  const int n_chunks = (H + kPrimeOut) / kPrimeOut;  // chunks of c over [0, H]
-  const int per_round = max(1, (kPrimeTasks * kSssThreads) / n_chunks);  // butterflies per round
-  for (int b0 = 0; b0 < nb; b0 += per_round) {
-    const int nbr = min(per_round, nb - b0);
-    const int n_task = nbr * n_chunks;
-    float2 A[kPrimeTasks][kPrimeOut], B[kPrimeTasks][kPrimeOut];
+      if (live) {
+        const float4* w4 = s_mat + ct * (TO / 2);
+#pragma unroll 2
+        for (int s = s0 + 1; s <= s0 + rows; ++s) {
+          float2 P[TC], Q[TC];
 #pragma unroll
-    for (int i = 0; i < kPrimeTasks; ++i) {
-      const int q = threadIdx.x + kSssThreads * i;
-#pragma unroll
-      for (int o = 0; o < kPrimeOut; ++o) A[i][o] = B[i][o] = make_float2(0.f, 0.f);
-      if (q < n_task) {
-        const int chunk = q / nbr;
-        const int t = b0 + q - chunk * nbr;
-        const int b = t / m, j = t - b * m;
-        const SkewBuf base = buf + (b * ns + j);
-        const float2 a0 = base[0];
-        int idx[kPrimeOut];
-#pragma unroll
-        for (int o = 0; o < kPrimeOut; ++o) {
-          A[i][o] = a0;
-          idx[o] = chunk * kPrimeOut + o;  // (s c) mod p at s = 1; c <= H + kPrimeOut - 1 < p
-        }
-        for (int sI = 1; sI <= H; ++sI) {
-          const float2 x = base[sI * m], y = base[(p - sI) * m];
-          const float2 P = cadd(x, y), Q = csub(x, y);
-#pragma unroll
-          for (int o = 0; o < kPrimeOut; ++o) {
-            const float2 w = cs[idx[o]];
-            A[i][o].x = fmaf(P.x, w.x, A[i][o].x);
-            A[i][o].y = fmaf(P.y, w.x, A[i][o].y);
-            B[i][o].x = fmaf(Q.x, w.y, B[i][o].x);
-            B[i][o].y = fmaf(Q.y, w.y, B[i][o].y);
-            idx[o] += chunk * kPrimeOut + o;
-            if (idx[o] >= p) idx[o] -= p;
+          for (int h = 0; h < TC; ++h) {
+            P[h] = buf.ld(e[h] + s * m);
+            Q[h] = buf.ld(e[h] + (p - s) * m);
           }
-        }
-      }
-    }
-    __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kPrimeTasks; ++i) {
-      const int q = threadIdx.x + kSssThreads * i;
-      if (q < n_task) {
-        const int chunk = q / nbr;
-        const int t = b0 + q - chunk * nbr;
-        const int b = t / m, j = t - b * m;
-        const SkewBuf base = buf + (b * ns + j);
+          for (int i = 0; i < TO; i += 2) {
+            const float4 w = w4[i >> 1];  // (cos, sin) of outputs i and i + 1
 #pragma unroll
-        for (int o = 0; o < kPrimeOut; ++o) {
-          const int c = chunk * kPrimeOut + o;
-          if (c == 0) {
-            base[0] = A[i][o];
-          } else if (c <= H) {
-            const float2 iB = mul_i(B[i][o]);
-            float2 xc = INV ? cadd(A[i][o], iB) : csub(A[i][o], iB);
-            float2 xq = INV ? csub(A[i][o], iB) : cadd(A[i][o], iB);
-            if (!INV && m > 1) {
-              xc = cmul(xc, tw[j * c * step]);
-              xq = cmul(xq, tw[j * (p - c) * step]);
+            for (int h = 0; h < TC; ++h) {
+              A[h][i].x = fmaf(P[h].x, w.x, A[h][i].x);
+              A[h][i].y = fmaf(P[h].y, w.x, A[h][i].y);
+              B[h][i].x = fmaf(Q[h].x, w.y, B[h][i].x);
+              B[h][i].y = fmaf(Q[h].y, w.y, B[h][i].y);
+              A[h][i + 1].x = fmaf(P[h].x, w.z, A[h][i + 1].x);
+              A[h][i + 1].y = fmaf(P[h].y, w.z, A[h][i + 1].y);
+              B[h][i + 1].x = fmaf(Q[h].x, w.w, B[h][i + 1].x);
+              B[h][i + 1].y = fmaf(Q[h].y, w.w, B[h][i + 1].y);
             }
-            base[c * m] = xc;
-            base[(p - c) * m] = xq;
           }
+          w4 += Cp / 2;
         }
       }
     }
-    __syncthreads();
+    __syncthreads();  // every thread of the round has read its inputs
+    if (live) {
+#pragma unroll
+      for (int h = 0; h < TC; ++h) {
+        if (TC * jt + h >= nb) continue;
+#pragma unroll
+        for (int i = 0; i < TO; ++i) {
+          const int c = ct * TO + i;
+          if (c > H) continue;
+          if (c == 0) {
+            buf.st(e[h], A[h][i]);
+            continue;
+          }
+          const float2 iB = mul_i(B[h][i]);
+          float2 xc = INV ? cadd(A[h][i], iB) : csub(A[h][i], iB), xq = INV ? csub(A[h][i], iB) : cadd(A[h][i], iB);
+          if (!INV && m > 1) {
+            xc = cmul(xc, root(j[h] * c * step));
+            xq = cmul(xq, root(j[h] * (p - c) * step));
+          }
+          buf.st(e[h] + c * m, xc);
+          buf.st(e[h] + (p - c) * m, xq);
+        }
+      }
+    }
+  }
+  __syncthreads();
+}
+template <bool INV, class Buf>
+__device__ __noinline__ void pass_prime(const Buf buf, int total, int ns, int N, int p, const Roots root,
+                                        const float2* __restrict__ mat) {
+  const int m = ns / p, nb = total / p, H = (p - 1) / 2, step = N / ns;
+  const FastDiv dm(m), dn(nb);
+#pragma unroll 2
+  for (int t = threadIdx.x; t < nb * H; t += kT) {
+    const int s = dn.div(t) + 1, col = t - (s - 1) * nb;
+    const int b = dm.div(col), j = col - b * m;
+    const int e0 = b * ns + j + s * m, e1 = b * ns + j + (p - s) * m;
+    float2 x = buf.ld(e0), y = buf.ld(e1);
+    if (INV && m > 1) {
+      x = cmulc(x, root(j * s * step));
+      y = cmulc(y, root(j * (p - s) * step));
+    }
+    buf.st(e0, cadd(x, y));
+    buf.st(e1, csub(x, y));
+  }
+  if (nb * fft_mat_cols(p) >= 16 * 160) prime_product<INV, Buf, 8, 2>(buf, ns, p, m, nb, step, root, mat);
+  else prime_product<INV, Buf, 2, 1>(buf, ns, p, m, nb, step, root, mat);
+}
+
+// Pass i of a sequence, on `total` elements whose sub-transforms have length ns.
+template <bool INV, class Buf>
+__device__ __forceinline__ void one_pass(const Buf& buf, int total, int ns, const FftSeq& sq, int i, const Roots& root,
+                                         const float2* __restrict__ tables) {
+  const int N = sq.N;
+  switch (sq.radix[i]) {
+    case 4: pass_small<4, INV>(buf, buf, total, ns, N, root); break;
+    case 2: pass_small<2, INV>(buf, buf, total, ns, N, root); break;
+    case 3: pass_small<3, INV>(buf, buf, total, ns, N, root); break;
+    case 5: pass_small<5, INV>(buf, buf, total, ns, N, root); break;
+    case 7: pass_small<7, INV>(buf, buf, total, ns, N, root); break;
+    case 11: pass_small<11, INV>(buf, buf, total, ns, N, root); break;
+    case 13: pass_small<13, INV>(buf, buf, total, ns, N, root); break;
+    default: pass_prime<INV, Buf>(buf, total, ns, N, sq.radix[i], root, tables + sq.base + sq.mat[i]); break;
+  }
+}
+// Passes [i0, i1) of a transform, forward in order or inverse in reverse order, on a buffer of `total` elements; ns:
+// length of the sub-transforms at pass i0.
+template <class Buf>
+__device__ __noinline__ void passes_fwd(const Buf buf, int total, int ns, const FftSeq& sq, int i0, int i1, const Roots root,
+                                        const float2* __restrict__ tables) {
+#pragma unroll 1
+  for (int i = i0; i < i1; ++i) {
+    one_pass<false>(buf, total, ns, sq, i, root, tables);
+    ns /= sq.radix[i];
+  }
+}
+template <class Buf>
+__device__ __noinline__ void passes_inv(const Buf buf, int total, int ns, const FftSeq& sq, int i0, int i1, const Roots root,
+                                        const float2* __restrict__ tables) {
+  for (int i = i0; i < i1; ++i) ns /= sq.radix[i];
+#pragma unroll 1
+  for (int i = i1 - 1; i >= i0; --i) {
+    ns *= sq.radix[i];
+    one_pass<true>(buf, total, ns, sq, i, root, tables);
   }
 }
 
+// A direct transform of a buffer in global memory: the first g passes couple elements that lie far apart and run on the
+// global buffer; after them the transform falls apart into contiguous blocks of length len, of which `chunk` elements'
+// worth at a time go through shared memory for the remaining passes. The inverse runs the steps backwards.
 template <bool INV>
-__device__ __forceinline__ void one_pass(SkewBuf buf, int N, int ns, int r, const float2* tw, float2* wp) {
-  switch (r) {
-    case 2: pass_small<2, INV>(buf, N, ns, tw); break;
-    case 3: pass_small<3, INV>(buf, N, ns, tw); break;
-    case 4: pass_small<4, INV>(buf, N, ns, tw); break;
-    case 5: pass_small<5, INV>(buf, N, ns, tw); break;
-    case 7: pass_small<7, INV>(buf, N, ns, tw); break;
-    case 11: pass_odd<11, INV>(buf, N, ns, tw); break;
-    case 13: pass_odd<13, INV>(buf, N, ns, tw); break;
-    case 17: pass_odd<17, INV>(buf, N, ns, tw); break;
-    case 19: pass_odd<19, INV>(buf, N, ns, tw); break;
-    default: pass_prime<INV>(buf, N, ns, r, tw, wp); break;
+__device__ __noinline__ void fft_big(float2* g, const FftPlan& pl, const Roots root, const float2* __restrict__ tables) {
+  const FftSeq& sq = pl.seq;
+  const GlobBuf gb{g};
+  const SmemBuf sb;
+  int len = sq.N;
+  for (int i = 0; i < pl.g_pass; ++i) len /= sq.radix[i];
+  if (!INV) passes_fwd(gb, sq.N, sq.N, sq, 0, pl.g_pass, root, tables);
+  for (int c0 = 0; c0 < sq.N; c0 += pl.chunk) {
+    const int n = min(pl.chunk, sq.N - c0);
+    batched<8>(n, [&](int t) { return g[c0 + t]; }, [&](int t, float2 v) { sb.st(t, v); });
+    __syncthreads();
+    if (!INV) passes_fwd(sb, n, len, sq, pl.g_pass, sq.n_pass, root, tables);
+    else passes_inv(sb, n, len, sq, pl.g_pass, sq.n_pass, root, tables);
+    for (int t = threadIdx.x; t < n; t += kT) g[c0 + t] = sb.ld(t);
+    __syncthreads();
   }
+  if (INV) passes_inv(gb, sq.N, sq.N, sq, 0, pl.g_pass, root, tables);
 }
 
-// Forward transform, natural order in, digit-reversed order out (see seq_pos).
-// tw: W_N^t = exp(-2 pi i t / N), t in [0, N); in shared or global memory.
-__device__ __noinline__ void fft_dif(SkewBuf buf, const FftSeq& sq, const float2* tw, float2* wp) {
-  int ns = sq.N;
-  for (int i = 0; i < sq.n_pass; ++i) {
-    one_pass<false>(buf, sq.N, ns, sq.radix[i], tw, wp);
-    ns /= sq.radix[i];
-  }
-}
-// Inverse (unnormalised, sign +), digit-reversed order in, natural order out.
-__device__ __noinline__ void fft_dit_inv(SkewBuf buf, const FftSeq& sq, const float2* tw, float2* wp) {
-  int ns = 1;
-  for (int i = sq.n_pass - 1; i >= 0; --i) {
-    ns *= sq.radix[i];
-    one_pass<true>(buf, sq.N, ns, sq.radix[i], tw, wp);
-  }
-}
-// The same two transforms for a buffer in global memory that is too long for shared memory. The first g passes
-// of the forward transform couple elements that lie far apart and run on the global buffer; after them the
-// transform falls apart into F = r_1 ... r_g contiguous blocks of length len = N / F, each of which is brought
-// into shared memory (with its own twiddles W_len^t = W_N^{t F}) for the remaining passes. The inverse runs the
-// steps backwards. Every element then makes g + 1 round trips to global memory instead of one per pass.
-__device__ __noinline__ void fft_dif_big(SkewBuf gbuf, const FftSeq& sq, int g, const float2* tw, float2* wp,
-                                         float2* sbuf) {
-  int ns = sq.N;
-  for (int i = 0; i < g; ++i) {
-    one_pass<false>(gbuf, sq.N, ns, sq.radix[i], tw, wp);
-    ns /= sq.radix[i];
-  }
-  const int len = ns, F = sq.N / len;
-  const SkewBuf sb{sbuf, 4, 0};
-  float2* s_tw = sbuf + sss_padded(len);
-  __syncthreads();
-  for (int t = threadIdx.x; t < len; t += kSssThreads) s_tw[t] = tw[t * F];
-  for (int blk = 0; blk < F; ++blk) {
-    __syncthreads();
-    for (int t = threadIdx.x; t < len; t += kSssThreads) sb[t] = gbuf[blk * len + t];
-    __syncthreads();
-    int ns2 = len;
-    for (int i = g; i < sq.n_pass; ++i) {
-      one_pass<false>(sb, len, ns2, sq.radix[i], s_tw, wp);
-      ns2 /= sq.radix[i];
-    }
-    for (int t = threadIdx.x; t < len; t += kSssThreads) gbuf[blk * len + t] = sb[t];
-  }
-  __syncthreads();
-}
-__device__ __noinline__ void fft_dit_inv_big(SkewBuf gbuf, const FftSeq& sq, int g, const float2* tw, float2* wp,
-                                             float2* sbuf) {
-  int len = sq.N;
-  for (int i = 0; i < g; ++i) len /= sq.radix[i];
-  const int F = sq.N / len;
-  const SkewBuf sb{sbuf, 4, 0};
-  float2* s_tw = sbuf + sss_padded(len);
-  __syncthreads();
-  for (int t = threadIdx.x; t < len; t += kSssThreads) s_tw[t] = tw[t * F];
-  for (int blk = 0; blk < F; ++blk) {
-    __syncthreads();
-    for (int t = threadIdx.x; t < len; t += kSssThreads) sb[t] = gbuf[blk * len + t];
-    __syncthreads();
-    int ns2 = 1;
-    for (int i = sq.n_pass - 1; i >= g; --i) {
-      ns2 *= sq.radix[i];
-      one_pass<true>(sb, len, ns2, sq.radix[i], s_tw, wp);
-    }
-    for (int t = threadIdx.x; t < len; t += kSssThreads) gbuf[blk * len + t] = sb[t];
-  }
-  __syncthreads();
-  int ns = len;
-  for (int i = g - 1; i >= 0; --i) {
-    ns *= sq.radix[i];
-    one_pass<true>(gbuf, sq.N, ns, sq.radix[i], tw, wp);
-  }
-}
 // Where the forward transform leaves bin k.
 __device__ __forceinline__ int seq_pos(const FftSeq& sq, int k) {
   int len = sq.N, p = 0;
@@ -565,102 +469,168 @@ __device__ __forceinline__ int seq_pos(const FftSeq& sq, int k) {
   return p;
 }
 
-// Chirp-z: buf[0..n_in) holds y (natural order; entries from n_in on count as zero) on entry and bins 0..n_out-1
-// of DFT_N(y) (natural order) on exit. `filt` is the transformed wrapped chirp that fits this pair of ranges: the
-// plan's filter for n_in = n_out = N, and for a half plan the filter (N in, (N+1)/2 out) or filter2 ((N+1)/2 in,
-// N out). CONJ: conjugate on the way in and out, which turns the forward transform into the unnormalised inverse.
-template <bool CONJ>
-__device__ __forceinline__ void bluestein(SkewBuf buf, const FftPlan& pl, const float2* tables, float2* wp, float2* sbuf,
-                                          int n_in, int n_out, const float2* filt) {
-  const float2* chirp = tables + pl.chirp_offset;
-  const int M = pl.M;
-  for (int j = threadIdx.x; j < M; j += kSssThreads) {
-    float2 v = make_float2(0.f, 0.f);
-    if (j < n_in) {
-      v = buf[j];
-      if (CONJ) v = cconj(v);
-      v = cmul(v, __ldg(chirp + j));
-    }
-    buf[j] = v;
+// ---- chirp-z -----------------------------------------------------------------------------
+// The last forward pass of a convolution (radix R, no twiddles), the product with the transformed filter and the first
+// inverse pass work on the same R neighbours: one sweep in registers does all three.
+template <int R>
+__device__ __forceinline__ void pass_filter(int total, const float2* __restrict__ filt) {
+  const SmemBuf sb;
+  struct Piece {
+    float4 f[R / 2];
+  };
+  const float4* f4 = reinterpret_cast<const float4*>(filt);  // filters start on 16-byte boundaries
+  batched<4>(total / R,
+             [&](int t) {
+               Piece p;
+#pragma unroll
+               for (int s = 0; s < R / 2; ++s) p.f[s] = __ldg(f4 + R / 2 * t + s);
+               return p;
+             },
+             [&](int t, const Piece& p) {
+               float2 v[R];
+#pragma unroll
+               for (int s = 0; s < R; ++s) v[s] = sb.ld(R * t + s);
+               dft_small<R, false>(v);
+#pragma unroll
+               for (int s = 0; s < R / 2; ++s) {
+                 v[2 * s] = cmul(v[2 * s], make_float2(p.f[s].x, p.f[s].y));
+                 v[2 * s + 1] = cmul(v[2 * s + 1], make_float2(p.f[s].z, p.f[s].w));
+               }
+               dft_small<R, true>(v);
+#pragma unroll
+               for (int s = 0; s < R; ++s) sb.st(R * t + s, v[s]);
+             });
+  __syncthreads();
+}
+__device__ __forceinline__ void apply_filter(const FftSeq& sq, int total, const float2* __restrict__ filt) {
+  if (sq.radix[sq.n_pass - 1] == 4) pass_filter<4>(total, filt);
+  else pass_filter<2>(total, filt);  // convolution lengths are multiples of 4
+}
+
+// The chirp e^{-i pi j^2 / N} = e^{-2 pi i (j^2 mod 2N) / 2N}, j < N.
+struct Chirp {
+  Roots root;  // of order 2N
+  uint32_t two_n, magic;
+  __device__ __forceinline__ Chirp(const Roots& r, int N) : root(r), two_n(2 * N), magic(0xffffffffu / (2u * N)) {}
+  __device__ __forceinline__ float2 operator()(int j) const {
+    const uint64_t q = static_cast<uint64_t>(j) * static_cast<uint64_t>(j);  // j < 2^17
+    // the quotient from the upper bits is short by a little; the remainder is put right
+    uint32_t r = static_cast<uint32_t>(q) - __umulhi(static_cast<uint32_t>(q >> 4), magic) * 16u * two_n;
+    while (r >= 16u * two_n) r -= 16u * two_n;
+    r -= __umulhi(r, magic) * two_n;
+    while (r >= two_n) r -= two_n;
+    return root(static_cast<int>(r));
   }
+};
+
+// Views of the global buffer at the two ends of a long convolution: the chirp goes on with the first pass's reads and off
+// with the last pass's writes. conj: conjugate on the way in and out, which turns the forward transform into the
+// unnormalised inverse.
+struct ChirpIn {
+  Scores sc;
+  const float2* g;  // null: the head's scores
+  Chirp chirp;
+  int n_in;
+  bool conj;
+  __device__ __forceinline__ float2 ld(int e) const {
+    if (e >= n_in) return make_float2(0.f, 0.f);
+    float2 v = g ? g[e] : sc.entry(e);
+    if (conj) v = cconj(v);
+    return cmul(v, chirp(e));
+  }
+};
+struct ChirpOut {
+  float2* g;
+  Chirp chirp;
+  int n_out;
+  bool conj;
+  __device__ __forceinline__ void st(int e, float2 v) const {
+    if (e >= n_out) return;
+    v = cmul(v, chirp(e));
+    g[e] = conj ? cconj(v) : v;
+  }
+};
+template <bool INV, class In, class Out>
+__device__ __noinline__ void end_pass(const In in, const Out out, const FftSeq& sq, const Roots root) {
+  const int M = sq.N;
+  switch (sq.radix[0]) {  // convolution lengths are made of 7, 5, 3 and 2
+    case 7: pass_small<7, INV>(in, out, M, M, M, root); break;
+    case 5: pass_small<5, INV>(in, out, M, M, M, root); break;
+    case 3: pass_small<3, INV>(in, out, M, M, M, root); break;
+    default: pass_small<4, INV>(in, out, M, M, M, root); break;
+  }
+}
+
+// Chirp-z: entries [0, n_in) (natural order; the rest counts as zero) in, bins 0..n_out-1 of DFT_N (natural order) out.
+// `filt` is the transformed wrapped chirp that fits this pair of ranges: the plan's filter for n_in = n_out = N, and for
+// a half plan the filter (N in, (N+1)/2 out) or filter2 ((N+1)/2 in, N out). Short: the work buffer in shared memory.
+// Long: scratch g; from_scores: the input is read from the scores. root: of order M; rootn: of order 2N.
+template <bool CONJ>
+__device__ __forceinline__ void chirp_z_smem(const FftPlan& pl, const Roots& root, const Roots& rootn,
+                                             const float2* __restrict__ tables, int n_in, int n_out,
+                                             const float2* __restrict__ filt) {
+  const SmemBuf sb;
+  const Chirp chirp(rootn, pl.N);
+  const int M = pl.M, last = pl.seq.n_pass - 1;
+#pragma unroll 2
+  for (int j = threadIdx.x; j < n_in; j += kT) {
+    const float2 v = sb.ld(j);
+    sb.st(j, cmul(CONJ ? cconj(v) : v, chirp(j)));
+  }
+  for (int j = n_in + threadIdx.x; j < M; j += kT) sb.st(j, make_float2(0.f, 0.f));
   __syncthreads();
-  if (pl.in_smem) fft_dif(buf, pl.seq, tables + pl.seq.tw_offset, wp);
-  else fft_dif_big(buf, pl.seq, pl.g_pass, tables + pl.seq.tw_offset, wp, sbuf);
-  for (int j = threadIdx.x; j < M; j += kSssThreads) buf[j] = cmul(buf[j], __ldg(filt + j));
-  __syncthreads();
-  if (pl.in_smem) fft_dit_inv(buf, pl.seq, tables + pl.seq.tw_offset, wp);
-  else fft_dit_inv_big(buf, pl.seq, pl.g_pass, tables + pl.seq.tw_offset, wp, sbuf);
-  for (int j = threadIdx.x; j < n_out; j += kSssThreads) {
-    float2 v = cmul(buf[j], __ldg(chirp + j));
-    buf[j] = CONJ ? cconj(v) : v;
+  passes_fwd(sb, M, M, pl.seq, 0, last, root, tables);
+  apply_filter(pl.seq, M, filt);
+  passes_inv(sb, M, M, pl.seq, 0, last, root, tables);
+#pragma unroll 2
+  for (int j = threadIdx.x; j < n_out; j += kT) {
+    const float2 v = cmul(sb.ld(j), chirp(j));
+    sb.st(j, CONJ ? cconj(v) : v);
   }
   __syncthreads();
 }
+__device__ __noinline__ void chirp_z_big(const Scores sc, bool from_scores, bool conj, float2* g, const FftPlan& pl, const Roots root,
+                                         const Roots rootn, const float2* __restrict__ tables, int n_in, int n_out,
+                                         const float2* __restrict__ filt) {
+  const FftSeq& sq = pl.seq;
+  const Chirp chirp(rootn, pl.N);
+  const int M = pl.M, last = sq.n_pass - 1;
+  const SmemBuf sb;
+  const GlobBuf gb{g};
+  int len = M;
+  for (int i = 0; i < pl.g_pass; ++i) len /= sq.radix[i];
+  end_pass<false>(ChirpIn{sc, from_scores ? nullptr : g, chirp, n_in, conj}, gb, sq, root);
+  passes_fwd(gb, M, M / sq.radix[0], sq, 1, pl.g_pass, root, tables);
+  for (int c0 = 0; c0 < M; c0 += pl.chunk) {
+    const int n = min(pl.chunk, M - c0);
+    batched<8>(n, [&](int t) { return g[c0 + t]; }, [&](int t, float2 v) { sb.st(t, v); });
+    __syncthreads();
+    passes_fwd(sb, n, len, sq, pl.g_pass, last, root, tables);
+    apply_filter(sq, n, filt + c0);
+    passes_inv(sb, n, len, sq, pl.g_pass, last, root, tables);
+    for (int t = threadIdx.x; t < n; t += kT) g[c0 + t] = sb.ld(t);
+    __syncthreads();
+  }
+  passes_inv(gb, M, M / sq.radix[0], sq, 1, pl.g_pass, root, tables);
+  end_pass<true>(gb, ChirpOut{g, chirp, n_out, conj}, sq, root);
+}
 
-__device__ __forceinline__ double block_sum(double v, double* red /* smem [32] */) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  double t = red[lane];  // kSssThreads / 32 == 32 warps
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
-}
-
-// Exclusive prefix of v over the block's threads (by thread index).
-__device__ __forceinline__ double block_excl_scan(double v, double* red /* smem [32] */) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    double t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
-  }
-  __syncthreads();
-  if (lane == 31) red[warp] = inc;
-  __syncthreads();
-  double wsum = red[lane];
-  double winc = wsum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    double t = __shfl_up_sync(0xffffffffu, winc, o);
-    if (lane >= o) winc += t;
-  }
-  double wexcl = __shfl_sync(0xffffffffu, winc - wsum, warp);
-  return wexcl + inc - v;
+  return v;
 }
 
 // ---- low cut-offs without a transform ---------------------------------------------------------------------------
-// Attention scores are positive, so their mean usually carries most of the energy and k* is a handful of bins. The
-// block then evaluates those bins directly, O(n (k* + T)) operations instead of two transforms of n points: the
-// total energy comes from Parseval's identity (sum of squares in fp64), the first kDirectBins bins from their
-// definition. The shortcut is taken only when those bins decide k* with a clear margin and k* + T lies inside them;
-// otherwise the transform path decides.
-constexpr int kDirectBins = 12;
-constexpr int kDirectRows = 64;  // entries per thread the table covers: even n up to 131072, odd n up to 65535
-constexpr int kDirectRegs = 8;   // entries per thread held in registers
-
-// Entry m = t + kSssThreads i of thread t holds token m (odd n) or tokens 2m and 2m + 1 (even n): token j = a m + b.
-// With w_k = e^{-2 pi i k / n},  w_k^j = w_k^{a t} * w_k^b * w_k^{a kSssThreads i}: the first factor is a power of one
+// Attention scores are positive, so where a head attends evenly their mean carries most of the energy and k* is a
+// handful of bins. The block then evaluates those bins directly, O(n (k* + T)) operations instead of two transforms of
+// n points: the total energy comes from Parseval's identity (sum of squares in fp64), the first kDirectBins bins from
+// their definition. The shortcut is taken only when those bins decide k* with a clear margin and k* + T lies inside
+// them; otherwise the transform path decides.
+// Entry m = t + kT i of thread t holds token m (odd n) or tokens 2m and 2m + 1 (even n): token j = a m + b.
+// With w_k = e^{-2 pi i k / n},  w_k^j = w_k^{a t} * w_k^b * w_k^{a kT i}: the first factor is a power of one
 // rotation per thread, the second a power of one rotation per head, the third comes from a table of
-// rows x kDirectBins entries built once per head. A bin then costs one shared-memory read and two FMAs per token.
-// The code is kept short on purpose: it runs once per head and launch, mostly from a cold instruction cache; for the
-// same reason it is inlined into the kernel, next to the code that runs before and after it (out of line the
-// benchmark's smoothing kernel took 29.2 instead of 28.1 us, at L = 32768 62.5 instead of 58.0).
-struct DirectSmem {
-  float2 tab[kDirectRows][kDirectBins];          // tab[i][k] = w_k^{a kSssThreads i}
-  float2 part[kSssThreads / 32][kDirectBins];    // per warp: bins 1 .. kDirectBins - 1
-  double sums[kSssThreads / 32][3];              // per warp: sum x, sum x^2, alternating sum
-  double energy[kDirectBins];                    // |F_k|^2 as it counts towards the cumulative energy
-  double tot[3];                                 // F_0 (= sum x), the energy threshold rho E, the margin of a decision
-  float2 bin[kDirectBins];                       // F_k
-  int kstar;                                     // stage 1: k*, -1: left to the transform, -2: the bins decide
-  int k_hi;                                      // last bin to evaluate; after stage 3: k* or -1
-};
-
+// rows x kDirectBins entries built once per head. A bin then costs one read of the table and two FMAs per token.
 // e^{-2 pi i (j k mod n) / n}: the product is reduced exactly in integers, the angle then lies in [-pi, pi] where the
 // fast sine and cosine are good to 5e-7.
 __device__ __forceinline__ float2 unit_root(int j, int k, int n, float inv_n, float two_pi_over_n) {
@@ -692,7 +662,7 @@ __device__ __forceinline__ DirectGeom direct_geom(int n, bool packed) {
   DirectGeom g;
   g.a = packed ? 2 : 1;
   g.M = n / g.a;
-  g.rows = (g.M + kSssThreads - 1) / kSssThreads;
+  g.rows = (g.M + kT - 1) / kT;
   // one accurate rotation per thread, w_1^t; w_1 is the ratio of two neighbours' and w_1^{2t} its square
   const float2 w = unit_root_exact(threadIdx.x, n);
   const float2 w_l0 = make_float2(__shfl_sync(0xffffffffu, w.x, 0), __shfl_sync(0xffffffffu, w.y, 0));
@@ -702,140 +672,96 @@ __device__ __forceinline__ DirectGeom direct_geom(int n, bool packed) {
   return g;
 }
 
-// x: the n scores of the head (rows <= kDirectRows); T: bins of the cosine band. Returns k* (and leaves the bins in
-// ds->bin and the table in ds->tab) or -1 when the transform has to decide.
-__device__ __forceinline__ int direct_cutoff(const float* __restrict__ x, int n, bool packed, const DirectGeom& g, int smooth_mode,
-                                         float rho, float kappa, int T, DirectSmem* ds) {
+// Stage 1, from three sums over the block (s[0] = sum x, s[1] = sum x^2, s[2] = alternating sum; one thread): the mean
+// bin F_0 and, by Parseval, the total over the bins 0 .. floor(n/2). Often that settles the cut-off at bin 0, and only
+// the T bins of the cosine band are needed; it also tells the heads for which the other eleven bins are not worth
+// evaluating (a matter of time only: both paths compute the same function): a spectrum without a strong low end
+// would have to hold the missing energy there in an eighth of what lies outside the mean.
+__device__ __forceinline__ void direct_stage1(const double* s, int n, int smooth_mode, float rho, float kappa, int T, DirectSmem* ds) {
+  const int Kb = n / 2;
+  const double F0 = s[0], FN = s[2];
+  const double total = 0.5 * (static_cast<double>(n) * s[1] + F0 * F0 + ((n & 1) ? 0.0 : FN * FN));
+  const bool no_mean = smooth_mode == AUDIOKV_SMOOTH_ENERGY_NO_MEAN;
+  const double rest = fmax(total - F0 * F0, 0.0), whole = no_mean ? rest : total;
+  const double thr = static_cast<double>(rho) * whole;
+  // The rotations are good to about 1e-6, so a bin's energy is off by up to 2e-6 |F_k| F_0: a decision is taken
+  // here only when it is clear of the threshold by several times the sum of that over the bins.
+  const double margin = 1e-5 * (whole + fabs(F0) * static_cast<double>(sqrtf(static_cast<float>(rest))));
+  int ks = -2, k_hi = kDirectBins - 1;  // -2: the bins have to decide
+  if (smooth_mode == AUDIOKV_SMOOTH_FIXED_FRACTION) {
+    ks = static_cast<int>(floor(static_cast<double>(kappa) * Kb));
+  } else if (!(whole > 0.0)) {
+    ks = -1;
+  } else if (!no_mean && F0 * F0 >= thr + margin) {
+    ks = 0;
+  } else if ((no_mean ? 0.0 : F0 * F0) + 0.125 * rest < thr) {
+    ks = -1;
+  }
+  if (ks >= 0) {
+    k_hi = ks + T;
+    if (k_hi >= kDirectBins || k_hi >= Kb) ks = -1;
+  }
+  ds->tot[0] = F0;
+  ds->tot[1] = thr;
+  ds->tot[2] = margin;
+  ds->bin[0] = make_float2(static_cast<float>(F0), 0.f);
+  ds->energy[0] = no_mean ? 0.0 : F0 * F0;
+  ds->k_hi = k_hi;
+  ds->kstar = ks;
+}
+
+// Stages 2 and 3, where stage 1 did not send the head to the transform. entry(m): the head's scores. Returns k* (and
+// leaves the bins in ds->bin and the table in ds->tab) or -1 when the transform has to decide.
+template <class Entry>
+__device__ __forceinline__ int direct_bins(Entry entry, int n, bool packed, const DirectGeom& g, int T, DirectSmem* ds) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __syncthreads();  // ds may still be read by the head before
   {
     const float inv_n = 1.f / static_cast<float>(n), tpn = 6.283185307179586f * inv_n;
-    for (int e = threadIdx.x; e < g.rows * kDirectBins; e += kSssThreads) {
+    for (int e = threadIdx.x; e < g.rows * kDirectBins; e += kT) {
       const int i = e / kDirectBins, k = e - i * kDirectBins;
-      ds->tab[i][k] = unit_root(g.a * kSssThreads * i, k, n, inv_n, tpn);
-    }
-  }
-  // the thread's first entries stay in registers; the plain, squared and alternating sums are kept in fp64
-  float x0[kDirectRegs], x1[kDirectRegs];
-  double sx = 0.0, sxx = 0.0, salt = 0.0;
-#pragma unroll
-  for (int i = 0; i < kDirectRegs; ++i) {
-    const int m = threadIdx.x + kSssThreads * i;
-    x0[i] = m < g.M ? x[g.a * m] : 0.f;
-    x1[i] = (packed && m < g.M) ? x[g.a * m + 1] : 0.f;
-  }
-  const bool even_entry = packed || (threadIdx.x & 1) == 0;  // kSssThreads is even: all of a thread's tokens m alike
-#pragma unroll
-  for (int i = 0; i < kDirectRegs; ++i) {
-    const double d0 = static_cast<double>(x0[i]), d1 = static_cast<double>(x1[i]);
-    sx += d0 + d1;
-    sxx = fma(d0, d0, fma(d1, d1, sxx));
-    salt += even_entry ? d0 - d1 : -d0;
-  }
-  for (int i = kDirectRegs; i < g.rows; ++i) {
-    const int m = threadIdx.x + kSssThreads * i;
-    if (m >= g.M) break;
-    const double d0 = static_cast<double>(x[g.a * m]), d1 = packed ? static_cast<double>(x[g.a * m + 1]) : 0.0;
-    sx += d0 + d1;
-    sxx = fma(d0, d0, fma(d1, d1, sxx));
-    salt += even_entry ? d0 - d1 : -d0;
-  }
-#pragma unroll 1
-  for (int q = 0; q < 3; ++q) {
-    double val = q == 0 ? sx : (q == 1 ? sxx : salt);
-    for (int o = 16; o > 0; o >>= 1) val += __shfl_xor_sync(0xffffffffu, val, o);
-    if (lane == 0) ds->sums[warp][q] = val;
-  }
-  __syncthreads();  // the table and the warps' sums are complete
-  // Stage 1, from the three sums alone (warp 0): the mean bin F_0 and, by Parseval, the total over the bins
-  // 0 .. floor(n/2). Often that settles the cut-off at bin 0, and only the T bins of the cosine band are needed; it
-  // also tells a head whose mean holds less than half of the energy asked for, which is left to the transform at once
-  // (a matter of time only: both paths compute the same function).
-  if (warp == 0) {
-    double t[3];
-#pragma unroll 1
-    for (int q = 0; q < 3; ++q) {
-      double v = ds->sums[lane][q];
-#pragma unroll 1
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      t[q] = v;
-    }
-    if (lane == 0) {
-      const int Kb = n / 2;
-      const double F0 = t[0], FN = t[2];
-      const double total = 0.5 * (static_cast<double>(n) * t[1] + F0 * F0 + ((n & 1) ? 0.0 : FN * FN));
-      const bool no_mean = smooth_mode == AUDIOKV_SMOOTH_ENERGY_NO_MEAN;
-      const double rest = fmax(total - F0 * F0, 0.0), whole = no_mean ? rest : total;
-      const double thr = static_cast<double>(rho) * whole;
-      // The rotations are good to about 1e-6, so a bin's energy is off by up to 2e-6 |F_k| F_0: a decision is taken
-      // here only when it is clear of the threshold by several times the sum of that over the bins.
-      const double margin = 1e-5 * (whole + fabs(F0) * static_cast<double>(sqrtf(static_cast<float>(rest))));
-      int ks = -2, k_hi = kDirectBins - 1;  // -2: the bins have to decide
-      if (smooth_mode == AUDIOKV_SMOOTH_FIXED_FRACTION) {
-        ks = static_cast<int>(floor(static_cast<double>(kappa) * Kb));
-      } else if (!(whole > 0.0)) {
-        ks = -1;
-      } else if (!no_mean) {
-        if (F0 * F0 >= thr + margin) ks = 0;
-        else if (F0 * F0 < 0.5 * thr) ks = -1;
-      }
-      if (ks >= 0) {
-        k_hi = ks + T;
-        if (k_hi >= kDirectBins || k_hi >= Kb) ks = -1;
-      }
-      ds->tot[0] = F0;
-      ds->tot[1] = thr;
-      ds->tot[2] = margin;
-      ds->bin[0] = make_float2(static_cast<float>(F0), 0.f);
-      ds->energy[0] = no_mean ? 0.0 : F0 * F0;
-      ds->k_hi = k_hi;
-      ds->kstar = ks;
+      ds->tab[i][k] = unit_root(g.a * kT * i, k, n, inv_n, tpn);
     }
   }
   __syncthreads();
-  if (ds->kstar == -1) return -1;
   const int k_hi = ds->k_hi;
-  // Stage 2: bins 1 .. k_hi from their definition
+  // bins 1 .. k_hi from their definition, four at a time
   float2 pk = make_float2(1.f, 0.f), vk = pk;
 #pragma unroll 1
-  for (int k = 1; k <= k_hi; ++k) {
-    pk = cmul(pk, g.wt);  // w_k^{a t}
-    vk = cmul(vk, g.v);   // w_k
-    float2 A0 = make_float2(0.f, 0.f), A1 = A0;  // at most 64 entries per thread: their sums stay in fp32
+  for (int k0 = 1; k0 <= k_hi; k0 += 4) {
+    float2 A0[4], A1[4];  // at most 128 entries per thread: their sums stay in fp32
 #pragma unroll
-    for (int i = 0; i < kDirectRegs; ++i) {
-      if (i < g.rows) {
-        const float2 tb = ds->tab[i][k];
-        A0.x = fmaf(x0[i], tb.x, A0.x);
-        A0.y = fmaf(x0[i], tb.y, A0.y);
-        A1.x = fmaf(x1[i], tb.x, A1.x);
-        A1.y = fmaf(x1[i], tb.y, A1.y);
+    for (int q = 0; q < 4; ++q) A0[q] = A1[q] = make_float2(0.f, 0.f);
+    batched<4>(g.M, entry, [&](int m, float2 x) {
+      const float2* tb = &ds->tab[m / kT][0];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 t = tb[min(k0 + q, kDirectBins - 1)];
+        A0[q].x = fmaf(x.x, t.x, A0[q].x);
+        A0[q].y = fmaf(x.x, t.y, A0[q].y);
+        A1[q].x = fmaf(x.y, t.x, A1[q].x);
+        A1[q].y = fmaf(x.y, t.y, A1[q].y);
       }
+    });
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      pk = cmul(pk, g.wt);  // w_k^{a t}
+      vk = cmul(vk, g.v);   // w_k
+      float2 F = A0[q];
+      if (packed) F = cadd(F, cmul(A1[q], vk));
+      F = cmul(F, pk);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        F.x += __shfl_xor_sync(0xffffffffu, F.x, o);
+        F.y += __shfl_xor_sync(0xffffffffu, F.y, o);
+      }
+      if (lane == 0 && k0 + q <= k_hi) ds->part[warp][k0 + q] = F;
     }
-    for (int i = kDirectRegs; i < g.rows; ++i) {
-      const int m = threadIdx.x + kSssThreads * i;
-      if (m >= g.M) break;
-      const float2 tb = ds->tab[i][k];
-      const float xa = x[g.a * m], xb = packed ? x[g.a * m + 1] : 0.f;
-      A0.x = fmaf(xa, tb.x, A0.x);
-      A0.y = fmaf(xa, tb.y, A0.y);
-      A1.x = fmaf(xb, tb.x, A1.x);
-      A1.y = fmaf(xb, tb.y, A1.y);
-    }
-    if (packed) A0 = cadd(A0, cmul(A1, vk));
-    float2 F = cmul(A0, pk);
-    for (int o = 16; o > 0; o >>= 1) {
-      F.x += __shfl_xor_sync(0xffffffffu, F.x, o);
-      F.y += __shfl_xor_sync(0xffffffffu, F.y, o);
-    }
-    if (lane == 0) ds->part[warp][k] = F;
   }
   __syncthreads();
-  // warp k adds up bin k over the warps' parts (lane w reads warp w's). (Rolled loops: this runs once, and
-  // straight-line code costs more in instruction fetches than its arithmetic takes.)
+  // warp k adds up bin k over the warps' parts (lane w reads warp w's)
   if (warp >= 1 && warp <= k_hi) {
-    float2 t = ds->part[lane][warp];
-#pragma unroll 1
+    float2 t = lane < kWarps ? ds->part[lane][warp] : make_float2(0.f, 0.f);
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
       t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
@@ -870,17 +796,18 @@ __device__ __forceinline__ int direct_cutoff(const float* __restrict__ x, int n,
 }
 
 // The residual mix of every token from the masked bins c_k = mask_k F_k (1 up to k*, raised cosine over the T bins
-// after it): y_j = alpha (1/n) [c_0 + 2 sum_k Re(c_k conj(w_k^j))] + (1 - alpha) x_j, written to y (when given) and,
-// for the selection, left in buf as order-preserving keys in the layout the transform path leaves them (even n: the
-// keys of tokens 2m, 2m + 1 in element m).
-__device__ __forceinline__ void direct_apply(const float* __restrict__ x, float* y, int n, bool packed, const DirectGeom& g, int kstar,
-                                          int T, float al, bool sel, SkewBuf buf, const DirectSmem* ds) {
+// after it): y_j = alpha (1/n) [c_0 + 2 sum_k Re(c_k conj(w_k^j))] + (1 - alpha) x_j. emit(m, x, y) gets the scores and
+// the results of entry m.
+template <class Entry, class Emit>
+__device__ __forceinline__ void direct_apply(Entry entry, Emit emit, int n, bool packed, const DirectGeom& g, int kstar, int T, float al, const DirectSmem* ds) {
+  constexpr int kRows = 8;
   const float om = 1.f - al, c0 = ds->bin[0].x, inv_n = 1.f / static_cast<float>(n);
   const float band = 3.14159265358979f / static_cast<float>(T + 1);
-  for (int i0 = 0; i0 < g.rows; i0 += kDirectRegs) {
-    float acc0[kDirectRegs], acc1[kDirectRegs];
+#pragma unroll 1
+  for (int i0 = 0; i0 < g.rows; i0 += kRows) {
+    float acc0[kRows], acc1[kRows];
 #pragma unroll
-    for (int ii = 0; ii < kDirectRegs; ++ii) acc0[ii] = acc1[ii] = 0.f;
+    for (int ii = 0; ii < kRows; ++ii) acc0[ii] = acc1[ii] = 0.f;
     float2 pk = make_float2(1.f, 0.f), vk = pk;
 #pragma unroll 1
     for (int k = 1; k <= kstar + T; ++k) {
@@ -890,354 +817,513 @@ __device__ __forceinline__ void direct_apply(const float* __restrict__ x, float*
       const float2 g0 = cscale(cmulc(ds->bin[k], pk), mask);  // c_k conj(w_k^{a t})
       const float2 g1 = cmulc(g0, vk);
 #pragma unroll
-      for (int ii = 0; ii < kDirectRegs; ++ii) {
-        if (i0 + ii < g.rows) {
-          const float2 tb = ds->tab[i0 + ii][k];
-          acc0[ii] = fmaf(g0.x, tb.x, fmaf(g0.y, tb.y, acc0[ii]));  // Re(g conj(tb))
-          acc1[ii] = fmaf(g1.x, tb.x, fmaf(g1.y, tb.y, acc1[ii]));
-        }
+      for (int ii = 0; ii < kRows; ++ii) {
+        const float2 tb = ds->tab[min(i0 + ii, kDirectRows - 1)][k];
+        acc0[ii] = fmaf(g0.x, tb.x, fmaf(g0.y, tb.y, acc0[ii]));  // Re(g conj(tb))
+        acc1[ii] = fmaf(g1.x, tb.x, fmaf(g1.y, tb.y, acc1[ii]));
       }
     }
 #pragma unroll
-    for (int ii = 0; ii < kDirectRegs; ++ii) {
-      const int m = threadIdx.x + kSssThreads * (i0 + ii);
+    for (int ii = 0; ii < kRows; ++ii) {
+      const int m = threadIdx.x + kT * (i0 + ii);
       if (m < g.M) {
-        if (packed) {
-          const float y0 = fmaf(al, fmaf(2.f, acc0[ii], c0) * inv_n, om * x[2 * m]);
-          const float y1 = fmaf(al, fmaf(2.f, acc1[ii], c0) * inv_n, om * x[2 * m + 1]);
-          if (y) {
-            y[2 * m] = y0;
-            y[2 * m + 1] = y1;
-          }
-          if (sel) buf[m] = make_float2(__uint_as_float(score_key(y0)), __uint_as_float(score_key(y1)));
-        } else {
-          const float ym = fmaf(al, fmaf(2.f, acc0[ii], c0) * inv_n, om * x[m]);
-          if (y) y[m] = ym;
-          if (sel) buf[m].x = __uint_as_float(score_key(ym));
-        }
+        const float2 x = entry(m);
+        emit(m, make_float2(fmaf(al, fmaf(2.f, acc0[ii], c0) * inv_n, om * x.x),
+                            fmaf(al, fmaf(2.f, acc1[ii], c0) * inv_n, om * x.y)));
       }
     }
   }
 }
 
-__global__ void __launch_bounds__(kSssThreads, 1)
+// ---- the kernel --------------------------------------------------------------------------
+__device__ __forceinline__ Scores scores_of_head() {
+  const bool packed = S.pl.packed != 0;
+  return Scores{S.x, packed, packed && (reinterpret_cast<uintptr_t>(S.x) & 7) == 0};
+}
+
+// The first `count` entries of the plan's tables of roots, into shared memory.
+__device__ __forceinline__ void load_roots(const FftPlan& pl, const float2* __restrict__ tables, int count) {
+  const float4* src = reinterpret_cast<const float4*>(tables + pl.root_offset);
+  float4* dst = reinterpret_cast<float4*>(g_sbuf + pl.root_at);
+  batched<2>(count, [&](int t) { return __ldg(src + t); }, [&](int t, float4 v) { dst[t] = v; });
+}
+
+// A work buffer of either kind, for the steps around the transforms.
+template <bool BIG>
+struct Work {
+  float2* g;
+  __device__ __forceinline__ float2 ld(int e) const {
+    if constexpr (BIG) return g[e];
+    else return SmemBuf().ld(e);
+  }
+  __device__ __forceinline__ void st(int e, float2 v) const {
+    if constexpr (BIG) g[e] = v;
+    else SmemBuf().st(e, v);
+  }
+};
+
+// Smoothing of one head by transforms: the entries of `sc` (BIG = false: already in the buffer) become the masked
+// spectrum's inverse in the buffer, natural order; *inv_scale is what that still has to be multiplied with.
+template <bool BIG>
+__device__ __noinline__ void transform_head(const Shape& sh, const float2* __restrict__ tables) {
+  const FftPlan& pl = S.pl;
+  float2* g = S.g;
+  const Scores sc = scores_of_head();
+  const Work<BIG> buf{g};
+  const int n = pl.n, N = pl.N, Kb = n / 2;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool packed = pl.packed != 0, direct = pl.bluestein == 0, half = pl.half != 0;
+  // the slots of bins k and N - k after the forward passes: in order for a chirp-z, else from the plan
+  const uint32_t* __restrict__ rec = reinterpret_cast<const uint32_t*>(tables + pl.pos_offset);
+  auto slots_of = [&](int k) -> uint2 {
+    if (!direct) return make_uint2(k, k == 0 ? 0 : N - k);
+    if (pl.wide_pos) return make_uint2(__ldg(rec + 2 * k), __ldg(rec + 2 * k + 1));
+    const uint32_t r = __ldg(rec + k);
+    return make_uint2(r & 0xffffu, r >> 16);
+  };
+  const Roots root{pl.root_at, pl.root_mult};                              // of the passes
+  const Roots rootn{direct ? pl.root_at : pl.root_at + 2 * pl.root_count, 1};  // of order 2N (odd n, direct: not used)
+  if (S.loaded != pl.id) {
+    load_roots(pl, tables, pl.root_count + pl.root_count2);
+    __syncthreads();
+    if (threadIdx.x == 0) S.loaded = pl.id;
+  }
+
+  // 1. forward complex transform; bin k then sits at pos(k)
+  if constexpr (BIG) {
+    if (direct) {
+      for_entries<8>(sc, N, [&](int m, float2 v) { g[m] = v; });
+      __syncthreads();
+      fft_big<false>(g, pl, root, tables);
+    } else {
+      chirp_z_big(sc, true, false, g, pl, root, rootn, tables, N, half ? Kb + 1 : N, tables + pl.filter_offset);
+    }
+  } else {
+    if (direct) passes_fwd(SmemBuf(), N, N, pl.seq, 0, pl.seq.n_pass, root, tables);
+    else chirp_z_smem<false>(pl, root, rootn, tables, N, half ? Kb + 1 : N, tables + pl.filter_offset);
+  }
+
+  // 2. The spectrum of the real sequence and the cut-off, the smallest k with E(k) = sum_{i<=k} |F_i|^2 >= rho E(Kb) (fp64).
+  //    E(Kb) is known from the sums over the scores (Parseval), so the bins are gone through in ascending order and only
+  //    until the threshold is reached; what lies above the cut-off and its band is masked away unseen.
+  //    packed: Z is turned into F pairwise in place (the slot of bin 0 holds (F_0, F_N), both real). Energies are summed by
+  //    chunks of 32 neighbouring bins (one warp's share): chunk i of the low bins at energy[i], chunk i of their partners
+  //    N - k, which count downwards, at energy[2 nc - 1 - i]. After every 64 chunks each warp looks where the sum stands.
+  const bool no_mean = sh.smooth_mode == AUDIOKV_SMOOTH_ENERGY_NO_MEAN;  // variant: bin 0 adds no energy
+  const int n_low = packed ? N / 2 + 1 : Kb + 1;
+  const int nc = (n_low + 31) / 32, n_chunk = packed ? 2 * nc : nc;
+  auto sq_abs = [](float2 f) -> double { return fma(static_cast<double>(f.x), static_cast<double>(f.x), static_cast<double>(f.y) * f.y); };
+  // the spectrum's bins k and N - k from the two values of the packed transform. Bin 0 and the middle bin of an even N are
+  // their own partners; the formulas give them what they should (bin 0: F_0 and F_N).
+  auto split = [&](int k, float2 a, float2 b, float2& fk, float2& fq) {
+    const float2 zq = cconj(b);
+    const float2 E = cscale(cadd(a, zq), 0.5f), T = cmul(mul_mi(cscale(csub(a, zq), 0.5f)), rootn(k));
+    fk = cadd(E, T);
+    fq = cconj(csub(E, T));
+  };
+  int kc = 0;  // packed: bins k < kc (and their partners) have been split
+  if (sh.smooth_mode == AUDIOKV_SMOOTH_FIXED_FRACTION) {
+    // variant: the cut-off sits at a fixed fraction of the spectrum, no energies needed
+    if (threadIdx.x == 0) S.kstar = min(static_cast<int>(floor(static_cast<double>(sh.smooth_kappa) * Kb)), Kb);
+  } else {
+    const double F0 = S.sums[0], FN = S.sums[2];
+    const double total = 0.5 * (static_cast<double>(n) * S.sums[1] + F0 * F0 + ((n & 1) ? 0.0 : FN * FN));
+    // rho = 1 asks for everything: the two ways of summing may differ by rounding, so no bin short of the last will do
+    const double thr = sh.rho < 1.f ? static_cast<double>(sh.rho) * (no_mean ? fmax(total - F0 * F0, 0.0) : total) : INFINITY;
+    constexpr int U = 4;
+    static_assert(U * kWarps == 64, "two chunks per lane and round");
+    double run = 0.0;
+    int chunk = -1;  // the chunk that crosses the threshold, and the sum before it
+#pragma unroll 1
+    for (int c0 = 0; c0 < n_chunk && chunk < 0; c0 += U * kWarps) {
+      if (c0 < nc) {
+        uint2 at[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) at[q] = slots_of(min(32 * (c0 + q * kWarps + warp) + lane, n_low - 1));
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+          const int c = c0 + q * kWarps + warp, k = 32 * c + lane;
+          double el = 0.0, eh = 0.0;
+          if (k < n_low) {
+            float2 fk = buf.ld(at[q].x);
+            if (packed) {
+              float2 fq;
+              split(k, fk, buf.ld(at[q].y), fk, fq);
+              buf.st(at[q].x, k == 0 ? make_float2(fk.x, fq.x) : fk);
+              if (k > 0) buf.st(at[q].y, fq);
+              eh = 2 * k == N ? 0.0 : sq_abs(fq);
+            }
+            el = k == 0 && no_mean ? 0.0 : sq_abs(fk);
+          }
+          // both sums in one tree: the lower half of the warp goes on with the low bins, the upper half with the others
+          const double ol = __shfl_xor_sync(0xffffffffu, el, 16), oh = __shfl_xor_sync(0xffffffffu, eh, 16);
+          double v = (lane & 16) ? eh + oh : el + ol;
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (c < nc) {
+            if (lane == 0) S.energy[c] = v;
+            if (lane == 16 && packed) S.energy[2 * nc - 1 - c] = v;
+          }
+        }
+        kc = min(n_low, 32 * (c0 + U * kWarps));
+        __syncthreads();
+      }
+      // chunks c0 .. c0 + 63: in the last round of the low bins the chunks of the upper bins follow at once
+      const int ca = c0 + 2 * lane;
+      const double ea = ca < n_chunk && (ca < nc || c0 + U * kWarps > nc) ? S.energy[ca] : 0.0;
+      const double eb = ca + 1 < n_chunk && (ca + 1 < nc || c0 + U * kWarps > nc) ? S.energy[ca + 1] : 0.0;
+      double inc = ea + eb;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      const uint32_t hit = __ballot_sync(0xffffffffu, run + inc >= thr);
+      if (hit) {
+        const int at_lane = __ffs(hit) - 1;
+        const double before = run + __shfl_sync(0xffffffffu, inc - (ea + eb), at_lane);
+        const double first = __shfl_sync(0xffffffffu, ea, at_lane);
+        const bool second = !(before + first >= thr);
+        chunk = min(c0 + 2 * at_lane + (second ? 1 : 0), n_chunk - 1);
+        run = second ? before + first : before;
+      } else {
+        run += __shfl_sync(0xffffffffu, inc, 31);
+      }
+    }
+    if (warp == 0) {
+      int ks = Kb;
+      if (chunk >= 0) {
+        // the chunk's bins in ascending order, one per lane
+        const bool upper = packed && chunk >= nc;
+        const int k = upper ? N - (32 * (2 * nc - 1 - chunk) + 31 - lane) : 32 * chunk + lane;
+        const bool in = upper ? (k >= N - N / 2 && 2 * k != N && k <= N) : k < n_low;
+        double e = 0.0;
+        if (in) {
+          if (packed && (k == N || k == 0)) {
+            const float2 f = buf.ld(0);
+            e = k == N ? static_cast<double>(f.y) * f.y : no_mean ? 0.0 : static_cast<double>(f.x) * f.x;
+          } else if (!(k == 0 && no_mean)) {
+            const uint2 at = slots_of(upper ? N - k : k);
+            e = sq_abs(buf.ld(upper ? at.y : at.x));
+          }
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const double t = __shfl_up_sync(0xffffffffu, e, o);
+          if (lane >= o) e += t;
+        }
+        const uint32_t hit = __ballot_sync(0xffffffffu, in && run + e >= thr);
+        const uint32_t any = __ballot_sync(0xffffffffu, in);
+        const int at_lane = hit ? __ffs(hit) - 1 : 31 - __clz(any | 1u);  // rounding of the two sums: the chunk's last bin
+        ks = min(max(__shfl_sync(0xffffffffu, k, at_lane), 0), Kb);
+      }
+      if (lane == 0) S.kstar = ks;
+    }
+  }
+  __syncthreads();
+  const int kstar = S.kstar;
+
+  // 3. mask (1 up to k*, raised-cosine tail of T bins, 0 beyond) and back to the packed transform
+  const int T = sh.transition_bins, k_hi = kstar + min(T, n);  // last bin that is not masked away
+  auto weight = [&](int k) -> float {
+    if (k <= kstar) return 1.f;
+    if (k <= k_hi) return 0.5f * (1.f + cospif(static_cast<float>(k - kstar) / static_cast<float>(T + 1)));
+    return 0.f;
+  };
+  if (packed) {
+    batched<4>(n_low, slots_of, [&](int k, uint2 at) {
+      float2 ok = make_float2(0.f, 0.f), oq = ok;
+      if (k <= k_hi) {  // else its partner, further up, is masked away as well
+        float2 fk = buf.ld(at.x), fq = buf.ld(at.y);
+        if (k >= kc) {
+          split(k, fk, fq, fk, fq);
+        } else if (k == 0) {
+          fq = make_float2(fk.y, 0.f);
+          fk.y = 0.f;
+        }
+        fk = cscale(fk, weight(k));
+        fq = cconj(cscale(fq, weight(N - k)));
+        const float2 E = cscale(cadd(fk, fq), 0.5f), O = cmulc(cscale(csub(fk, fq), 0.5f), rootn(k));
+        ok = cadd(E, mul_i(O));
+        oq = cconj(csub(E, mul_i(O)));
+      }
+      buf.st(at.x, ok);
+      if (k > 0) buf.st(at.y, oq);
+    });
+  } else if (half) {
+    // bins 0 .. Kb alone go back: x_j = (2 / N) Re sum_{k <= Kb} h_k e^{+2 pi i j k / N}, h_0 = F_0 / 2, h_k = F_k
+    for (int k = threadIdx.x; k <= Kb; k += kT) buf.st(k, cscale(buf.ld(k), k == 0 ? 0.5f * weight(0) : weight(k)));
+  } else {
+    batched<4>(Kb + 1, slots_of, [&](int k, uint2 at) {
+      const float w = weight(k);
+      buf.st(at.x, cscale(buf.ld(at.x), w));
+      if (k > 0) buf.st(at.y, cscale(buf.ld(at.y), w));
+    });
+  }
+  __syncthreads();
+
+  // 4. inverse complex transform (unnormalised), natural order out
+  if constexpr (BIG) {
+    if (direct) fft_big<true>(g, pl, root, tables);
+    else chirp_z_big(sc, false, true, g, pl, root, rootn, tables, half ? Kb + 1 : N, N, tables + (half ? pl.filter2_offset : pl.filter_offset));
+  } else {
+    if (direct) passes_inv(SmemBuf(), N, N, pl.seq, 0, pl.seq.n_pass, root, tables);
+    else chirp_z_smem<true>(pl, root, rootn, tables, half ? Kb + 1 : N, N, tables + (half ? pl.filter2_offset : pl.filter_offset));
+  }
+}
+
+// Top-k of the keys in the work buffer. Bit masks and their prefix sums: over the histogram and in S.pre when the buffer
+// is on chip, else in the idle dynamic area.
+template <bool BIG, bool PAIR>
+__device__ __noinline__ void select_head(int window, int* status) {
+  const Work<BIG> buf{S.g};
+  const int N = S.pl.N;
+  uint32_t* words = BIG ? reinterpret_cast<uint32_t*>(g_sbuf) : reinterpret_cast<uint32_t*>(S.sel.hist);
+  int* pre = BIG ? reinterpret_cast<int*>(g_sbuf) + select_words(N, PAIR) : S.pre;
+  select_entries<kT, PAIR>([&](int m) -> float2 { return buf.ld(m); }, N, S.pl.n, window, S.k_keep, S.kmin, S.kmax, S.out,
+                           &S.sel, words, pre, status);
+}
+
+// One head from its scores to its smoothed scores and, with `sel`, its kept tokens.
+template <bool BIG>
+__device__ __noinline__ void smooth_head(const Shape& sh, const float2* __restrict__ tables, bool sel, int* status) {
+  const FftPlan& pl = S.pl;
+  const Work<BIG> buf{S.g};
+  const int n = pl.n, N = pl.N;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool packed = pl.packed != 0;
+
+  // The scores go into the buffer (or stay where they are when it is not on chip); plain, squared and alternating
+  // sums are taken on the way, in fp64.
+  double sx = 0.0, sxx = 0.0, salt = 0.0;
+  {
+    const bool even_entry = packed || (threadIdx.x & 1) == 0;  // kT is even: all of a thread's tokens m alike
+    const Scores sc = scores_of_head();
+    for_entries<8>(sc, N, [&](int m, float2 v) {
+      if (!BIG) buf.st(m, v);
+      const double d0 = static_cast<double>(v.x), d1 = static_cast<double>(v.y);
+      sx += d0 + d1;
+      sxx = fma(d0, d0, fma(d1, d1, sxx));
+      salt += even_entry ? d0 - d1 : -d0;
+    });
+  }
+  sx = warp_sum(sx);
+  sxx = warp_sum(sxx);
+  salt = warp_sum(salt);
+  if (threadIdx.x == 0) {
+    S.kmin = 0xffffffffu;
+    S.kmax = 0u;
+  }
+  double* part = S.energy;  // [3][kWarps]
+  if (lane == 0) {
+    part[warp] = sx;
+    part[kWarps + warp] = sxx;
+    part[2 * kWarps + warp] = salt;
+  }
+  __syncthreads();
+  if (warp < 3) {
+    const double v = warp_sum(lane < kWarps ? part[warp * kWarps + lane] : 0.0);
+    if (lane == 0) S.sums[warp] = v;
+  }
+  __syncthreads();
+
+  // A low cut-off is settled from the first few bins of the spectrum, without a transform.
+  const bool direct_ok = n >= 4 * kDirectBins && N <= kDirectRows * kT;
+  int kd = -1;
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+  auto emit = [&](int m, float2 v) {  // entry m's smoothed scores: to memory, and as keys into the buffer
+    const int j = packed ? 2 * m : m;
+    if (float* y = S.y) {
+      y[j] = v.x;
+      if (packed) y[j + 1] = v.y;
+    }
+    if (sel) {
+      const uint32_t a = score_key(v.x), b = packed ? score_key(v.y) : a;
+      kmin = min(kmin, min(a, b));
+      kmax = max(kmax, max(a, b));
+      buf.st(m, make_float2(__uint_as_float(a), __uint_as_float(b)));
+    }
+  };
+  if (direct_ok) {
+    if (threadIdx.x == 0) direct_stage1(S.sums, n, sh.smooth_mode, sh.rho, sh.smooth_kappa, sh.transition_bins, &S.ds);
+    __syncthreads();
+    if (S.ds.kstar != -1) {
+      const DirectGeom dg = direct_geom(n, packed);
+      auto entry = [&](int m) -> float2 {
+        if constexpr (BIG) return scores_of_head().entry(m);
+        else return buf.ld(m);
+      };
+      kd = direct_bins(entry, n, packed, dg, sh.transition_bins, &S.ds);
+      if (kd >= 0) direct_apply(entry, emit, n, packed, dg, kd, sh.transition_bins, sh.alpha, &S.ds);
+    }
+    __syncthreads();  // S.ds makes room for the energies
+  }
+  if (kd >= 0) {
+    if (threadIdx.x == 0 && S.kstar_out) *S.kstar_out = kd;
+  } else {
+    transform_head<BIG>(sh, tables);
+    if (threadIdx.x == 0 && S.kstar_out) *S.kstar_out = S.kstar;
+    // residual mix
+    const float inv = (pl.half ? 2.f : 1.f) / static_cast<float>(N), al = sh.alpha, om = 1.f - sh.alpha;
+    const Scores sc = scores_of_head();
+    for_entries<8>(sc, N, [&](int m, float2 v) {
+      const float2 z = buf.ld(m);
+      emit(m, make_float2(fmaf(al, z.x * inv, om * v.x), fmaf(al, z.y * inv, om * v.y)));
+    });
+  }
+  if (!sel) return;
+  // top-k of the smoothed scores, straight from the work buffer
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if (lane == 0) {
+    atomicMin(&S.kmin, kmin);
+    atomicMax(&S.kmax, kmax);
+  }
+  __syncthreads();
+  if (packed) select_head<BIG, true>(sh.window, status);
+  else select_head<BIG, false>(sh.window, status);
+}
+
+__global__ void __launch_bounds__(kT, 1)
 sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict__ plans,
            const float2* __restrict__ tables, const float* scores, float* smoothed /* may alias scores */,
            int32_t* __restrict__ kstar_out, float2* __restrict__ scratch, int64_t scratch_per_block,
            const int32_t* __restrict__ order, int n_order, int first_head, const int32_t* __restrict__ budgets,
            const int32_t* __restrict__ cu_kept, int32_t* __restrict__ kept_idx, int* __restrict__ status) {
-  extern __shared__ __align__(16) float2 sbuf[];
-  __shared__ FftPlan pl;
-  __shared__ float2 wp[128];
-  __shared__ double red[32];
-  __shared__ int s_kstar;
-  __shared__ SelectSmem ssm;
-  __shared__ DirectSmem dsm;
   // Launched as a programmatic dependent: the block is brought in while the kernel before it drains, reads its plan
   // (written when the plan was made, not by the kernels of the pass), and waits for that kernel only where it first
   // touches the scores.
   chain_release();
   bool waited = false;
+  if (threadIdx.x == 0) S.loaded = -1;
+  const bool sel = budgets != nullptr;
 
-  int loaded_plan = -1;  // plan whose tables sit in shared memory
   for (int slot = blockIdx.x; slot < n_order; slot += gridDim.x) {
     const int u = order ? order[slot] : first_head + slot;  // no list: heads first_head, first_head + 1, ...
     if (u < 0) continue;
     const int r = u / sh.heads_per_req;
     const ReqDesc rq = reqs[r];
     __syncthreads();
-    if (threadIdx.x == 0) {
-      pl = plans[rq.fft_plan];
-      s_kstar = 0x7fffffff;
+    {
+      const int* src = reinterpret_cast<const int*>(plans + rq.fft_plan);
+      for (int i = threadIdx.x; i < static_cast<int>(sizeof(FftPlan) / 4); i += kT) reinterpret_cast<int*>(&S.pl)[i] = src[i];
     }
-    __syncthreads();
-    const int n = pl.n, N = pl.N, Kb = n / 2;
-    const SkewBuf buf = pl.in_smem ? SkewBuf{sbuf, 4, 0}
-                                   : SkewBuf{scratch + static_cast<int64_t>(blockIdx.x) * scratch_per_block, 31, 0};
-    const float* x = scores + rq.score_offset + static_cast<int64_t>(u - rq.head_base) * rq.P;
-    float* y = smoothed ? smoothed + rq.score_offset + static_cast<int64_t>(u - rq.head_base) * rq.P : nullptr;
-
+    const int64_t base = rq.score_offset + static_cast<int64_t>(u - rq.head_base) * rq.P;
+    const int P = rq.P, W = sh.window;
     if (!waited) {
       chain_wait();
       waited = true;
     }
+    if (threadIdx.x == 0) {
+      S.x = scores + base;
+      S.y = smoothed ? smoothed + base : nullptr;
+      S.g = scratch + static_cast<int64_t>(blockIdx.x) * scratch_per_block;
+      S.kstar_out = kstar_out ? kstar_out + u : nullptr;
+      if (sel) {
+        int k = budgets[u] - W;
+        if (k < 0 || k > P) {
+          atomicExch(status, AUDIOKV_EDEVICE);
+          k = k < 0 ? 0 : P;
+        }
+        S.k_keep = k;
+        S.out = kept_idx + cu_kept[u];
+      }
+    }
+    __syncthreads();
     if (sh.smooth_mode >= AUDIOKV_SMOOTH_AVG_POOL) {
       // Variant: local pooling instead of the spectral filter. The sequence is staged first (scores and smoothed
       // may be the same array), pooled over |i - j| <= pool_kernel / 2 (average: zero padding counts in the
       // divisor; maximum: padding never wins), mixed with alpha and written out; the selection then reads it back.
-      float* st = pl.in_smem ? reinterpret_cast<float*>(sbuf)
-                             : reinterpret_cast<float*>(scratch + static_cast<int64_t>(blockIdx.x) * scratch_per_block);
-      loaded_plan = -1;
-      for (int j = threadIdx.x; j < n; j += kSssThreads) st[j] = x[j];
+      const int n = P;
+      const float* x = S.x;
+      float* y = S.y;
+      float* st = S.pl.in_smem ? reinterpret_cast<float*>(g_sbuf) : reinterpret_cast<float*>(S.g);
+      if (threadIdx.x == 0) {
+        S.kmin = 0xffffffffu;
+        S.kmax = 0u;
+      }
+#pragma unroll 4
+      for (int j = threadIdx.x; j < n; j += kT) st[j] = x[j];
       __syncthreads();
       const int hw = sh.pool_kernel / 2;
       const bool is_max = sh.smooth_mode == AUDIOKV_SMOOTH_MAX_POOL;
       const float inv_pool = 1.f / static_cast<float>(sh.pool_kernel), al = sh.alpha, om = 1.f - sh.alpha;
-      for (int j = threadIdx.x; j < n; j += kSssThreads) {
+      uint32_t kmin = 0xffffffffu, kmax = 0u;
+      for (int j = threadIdx.x; j < n; j += kT) {
         const int lo = max(0, j - hw), hi = min(n - 1, j + hw);
         float acc = is_max ? -INFINITY : 0.f;
         for (int i = lo; i <= hi; ++i) acc = is_max ? fmaxf(acc, st[i]) : acc + st[i];
         const float pooled = is_max ? acc : acc * inv_pool;
-        if (y) y[j] = fmaf(al, pooled, om * st[j]);
+        const float v = fmaf(al, pooled, om * st[j]);
+        if (y) y[j] = v;
+        kmin = min(kmin, score_key(v));
+        kmax = max(kmax, score_key(v));
       }
-      if (threadIdx.x == 0 && kstar_out) kstar_out[u] = 0;
-      __syncthreads();
-      if (budgets != nullptr) {
-        const int P = rq.P, W = sh.window;
-        int k = budgets[u] - W;
-        if (k < 0 || k > P || y == nullptr) {
+      if (threadIdx.x == 0 && S.kstar_out) *S.kstar_out = 0;
+      if (sel) {
+        if (y == nullptr) {
           if (threadIdx.x == 0) atomicExch(status, AUDIOKV_EDEVICE);
-          k = k < 0 ? 0 : (k > P ? P : k);
+          continue;
         }
-        if (y) select_topk([&](int j) -> uint32_t { return score_key(y[j]); }, P, W, k, kept_idx + cu_kept[u], &ssm, status);
+        kmin = __reduce_min_sync(0xffffffffu, kmin);
+        kmax = __reduce_max_sync(0xffffffffu, kmax);
+        if ((threadIdx.x & 31) == 0) {
+          atomicMin(&S.kmin, kmin);
+          atomicMax(&S.kmax, kmax);
+        }
+        __syncthreads();  // the staged sequence makes room for the masks; y is complete
+        int* words = reinterpret_cast<int*>(g_sbuf);
+        select_entries<kT, false>([&](int j) -> float2 { return make_float2(__uint_as_float(score_key(y[j])), 0.f); }, n, P, W,
+                                  S.k_keep, S.kmin, S.kmax, S.out, &S.sel, reinterpret_cast<uint32_t*>(words),
+                                  words + select_words(n, false), status);
       }
       continue;
     }
-
-    const bool sel = budgets != nullptr;
-    // A low cut-off is settled from the first few bins of the spectrum, without a transform (see direct_cutoff).
-    const bool direct_ok = n >= 4 * kDirectBins && N <= kDirectRows * kSssThreads;
-    DirectGeom dg;
-    if (direct_ok) dg = direct_geom(n, pl.packed != 0);
-    const int kd = direct_ok ? direct_cutoff(x, n, pl.packed != 0, dg, sh.smooth_mode, sh.rho, sh.smooth_kappa,
-                                             sh.transition_bins, &dsm)
-                             : -1;
-    if (kd >= 0) {
-      if (threadIdx.x == 0 && kstar_out) kstar_out[u] = kd;
-      direct_apply(x, y, n, pl.packed != 0, dg, kd, sh.transition_bins, sh.alpha, sel, buf, &dsm);
-    } else {
-    // Tables of a direct transform that fit beside the work buffer are staged in shared memory once per plan:
-    // the passes read twiddles with data-dependent strides, which from global memory costs a round trip each.
-    const float2* tw = tables + pl.seq.tw_offset;
-    const float2* post = tables + pl.post_offset;
-    const int* pos_tab = reinterpret_cast<const int*>(tables + pl.pos_offset);  // where the forward pass left each bin
-    const uint16_t* s_pos = nullptr;
-    if (pl.tabs_smem) {
-      float2* s_tw = sbuf + sss_padded(N);
-      float2* s_post = s_tw + N;
-      uint16_t* sp = reinterpret_cast<uint16_t*>(s_post + N / 2 + 1);
-      if (loaded_plan != rq.fft_plan) {
-        for (int t = threadIdx.x; t < N; t += kSssThreads) {
-          s_tw[t] = __ldg(tw + t);
-          sp[t] = static_cast<uint16_t>(__ldg(pos_tab + t));
-        }
-        if (pl.packed)
-          for (int t = threadIdx.x; t <= N / 2; t += kSssThreads) s_post[t] = __ldg(post + t);
-        loaded_plan = rq.fft_plan;
-      }
-      tw = s_tw;
-      post = s_post;
-      s_pos = sp;
-    } else {
-      loaded_plan = -1;  // this head's work buffer (or its blocks) may run over the staged tables
-    }
-    // 1. load (packed: z_m = x_2m + i x_2m+1)
-    if (pl.packed) {
-      for (int m = threadIdx.x; m < N; m += kSssThreads) buf[m] = make_float2(x[2 * m], x[2 * m + 1]);
-    } else {
-      for (int m = threadIdx.x; m < N; m += kSssThreads) buf[m] = make_float2(x[m], 0.f);
-    }
-    __syncthreads();
-
-    // 2. forward complex transform; bin k then sits at POS(k)
-    if (pl.bluestein)
-      bluestein<false>(buf, pl, tables, wp, sbuf, N, pl.half ? Kb + 1 : N, tables + pl.filter_offset);
-    else if (pl.in_smem)
-      fft_dif(buf, pl.seq, tw, wp);
-    else
-      fft_dif_big(buf, pl.seq, pl.g_pass, tw, wp, sbuf);
-    const bool direct = !pl.bluestein;
-#define POS(k) (direct ? (s_pos ? static_cast<int>(s_pos[(k)]) : __ldg(pos_tab + (k))) : (k))
-
-    // 3. packed: turn Z into the real sequence's spectrum F, pairwise in place.
-    //    Slot of bin 0 holds (F_0, F_N), both real.
-    if (pl.packed) {
-      for (int k = threadIdx.x; k <= N / 2; k += kSssThreads) {
-        if (k == 0) {
-          float2 z = buf[0];
-          buf[0] = make_float2(z.x + z.y, z.x - z.y);
-        } else if (2 * k == N) {
-          const int pk = POS(k);
-          buf[pk] = cconj(buf[pk]);
-        } else {
-          const int pk = POS(k), pq = POS(N - k);
-          float2 zk = buf[pk], zq = cconj(buf[pq]);
-          float2 E = cscale(cadd(zk, zq), 0.5f);
-          float2 O = mul_mi(cscale(csub(zk, zq), 0.5f));
-          float2 T = cmul(O, post[k]);
-          buf[pk] = cadd(E, T);
-          buf[pq] = cconj(csub(E, T));
-        }
-      }
-      __syncthreads();
-    }
-
-    // 4. cumulative energy E(k) = sum_{i<=k} |F_i|^2 in fp64, and the smallest k with E(k) >= rho E(Kb)
-    const int nbins = Kb + 1;
-    const int per = (nbins + kSssThreads - 1) / kSssThreads;
-    const int k0 = min(nbins, static_cast<int>(threadIdx.x) * per), k1 = min(nbins, k0 + per);
-    const bool no_mean = sh.smooth_mode == AUDIOKV_SMOOTH_ENERGY_NO_MEAN;  // variant: bin 0 adds no energy
-    auto energy = [&](int k) -> double {
-      if (k == 0 && no_mean) return 0.0;
-      if (pl.packed) {
-        if (k == 0) return static_cast<double>(buf[0].x) * buf[0].x;
-        if (k == N) return static_cast<double>(buf[0].y) * buf[0].y;
-      }
-      float2 f = buf[POS(k)];
-      return static_cast<double>(f.x) * f.x + static_cast<double>(f.y) * f.y;
-    };
-    if (sh.smooth_mode == AUDIOKV_SMOOTH_FIXED_FRACTION) {
-      // variant: the cut-off sits at a fixed fraction of the spectrum, no energies needed
-      if (threadIdx.x == 0) s_kstar = static_cast<int>(floor(static_cast<double>(sh.smooth_kappa) * Kb));
-    } else {
-    // each thread owns `per` consecutive bins; up to 8 of their energies stay in registers for the second look
-    double ecache[8];
-    double local = 0.0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      ecache[i] = k0 + i < k1 ? energy(k0 + i) : 0.0;
-      local += ecache[i];
-    }
-    for (int k = k0 + 8; k < k1; ++k) local += energy(k);
-    const double before = block_excl_scan(local, red);
-    const double total = block_sum(local, red);
-    const double thr = static_cast<double>(sh.rho) * total;
-    {
-      double run = before;
-      bool found = false;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        if (!found && k0 + i < k1) {
-          run += ecache[i];
-          if (run >= thr) {
-            atomicMin(&s_kstar, k0 + i);
-            found = true;
-          }
-        }
-      }
-      for (int k = k0 + 8; k < k1 && !found; ++k) {
-        run += energy(k);
-        if (run >= thr) {
-          atomicMin(&s_kstar, k);
-          found = true;
-        }
-      }
-    }
-    }
-    __syncthreads();
-    const int kstar = min(s_kstar, Kb);
-    if (threadIdx.x == 0 && kstar_out) kstar_out[u] = kstar;
-
-    // 5. mask (1 up to k*, raised-cosine tail of T bins, 0 beyond) and the inverse of step 3
-    const int T = sh.transition_bins;
-    auto weight = [&](int k) -> float {
-      if (k <= kstar) return 1.f;
-      if (k <= kstar + T) return 0.5f * (1.f + cospif(static_cast<float>(k - kstar) / static_cast<float>(T + 1)));
-      return 0.f;
-    };
-    if (pl.packed) {
-      for (int k = threadIdx.x; k <= N / 2; k += kSssThreads) {
-        if (k == 0) {
-          float2 f = buf[0];
-          const float f0 = f.x * weight(0), fN = f.y * weight(N);
-          buf[0] = make_float2(0.5f * (f0 + fN), 0.5f * (f0 - fN));
-        } else if (2 * k == N) {
-          const int pk = POS(k);
-          buf[pk] = cscale(cconj(buf[pk]), weight(k));
-        } else {
-          const int pk = POS(k), pq = POS(N - k);
-          float2 fk = cscale(buf[pk], weight(k)), fq = cconj(cscale(buf[pq], weight(N - k)));
-          float2 E = cscale(cadd(fk, fq), 0.5f);
-          float2 Tt = cscale(csub(fk, fq), 0.5f);
-          float2 O = cmulc(Tt, post[k]);
-          float2 iO = mul_i(O);
-          buf[pk] = cadd(E, iO);
-          buf[pq] = cconj(csub(E, iO));
-        }
-      }
-    } else if (pl.half) {
-      // bins 0 .. Kb alone go back: x_j = (2 / N) Re sum_{k <= Kb} h_k e^{+2 pi i j k / N}, h_0 = F_0 / 2, h_k = F_k
-      for (int k = threadIdx.x; k <= Kb; k += kSssThreads) buf[k] = cscale(buf[k], k == 0 ? 0.5f * weight(0) : weight(k));
-    } else {
-      for (int k = threadIdx.x; k < N; k += kSssThreads) {
-        const int kk = k <= Kb ? k : N - k;
-        const int pk = POS(k);
-        buf[pk] = cscale(buf[pk], weight(kk));
-      }
-    }
-    __syncthreads();
-
-    // 6. inverse complex transform (unnormalised), natural order out
-    if (pl.bluestein)
-      bluestein<true>(buf, pl, tables, wp, sbuf, pl.half ? Kb + 1 : N, N,
-                      tables + (pl.half ? pl.filter2_offset : pl.filter_offset));
-    else if (pl.in_smem)
-      fft_dit_inv(buf, pl.seq, tw, wp);
-    else
-      fft_dit_inv_big(buf, pl.seq, pl.g_pass, tw, wp, sbuf);
-#undef POS
-
-    // 7. residual mix. `smoothed` (optional) gets the result; when budgets are given the result
-    //    also stays in the work buffer, as order-preserving keys, for the selection below.
-    const float inv = (pl.half ? 2.f : 1.f) / static_cast<float>(N), al = sh.alpha, om = 1.f - sh.alpha;
-    // packed: the keys of tokens 2m and 2m+1 replace element m; otherwise the key of token m goes to the real part of element m
-    if (pl.packed) {
-      for (int m = threadIdx.x; m < N; m += kSssThreads) {
-        float2 z = buf[m];
-        const float x0 = x[2 * m], x1 = x[2 * m + 1];
-        const float y0 = fmaf(al, z.x * inv, om * x0), y1 = fmaf(al, z.y * inv, om * x1);
-        if (y) {
-          y[2 * m] = y0;
-          y[2 * m + 1] = y1;
-        }
-        if (sel) buf[m] = make_float2(__uint_as_float(score_key(y0)), __uint_as_float(score_key(y1)));
-      }
-    } else {
-      for (int m = threadIdx.x; m < N; m += kSssThreads) {
-        const float ym = fmaf(al, buf[m].x * inv, om * x[m]);
-        if (y) y[m] = ym;
-        if (sel) buf[m].x = __uint_as_float(score_key(ym));
-      }
-    }
-    }  // transform path
-    if (sel) {
-      // 8. top-k of the smoothed scores, straight from the work buffer
-      const int P = rq.P, W = sh.window;
-      int k = budgets[u] - W;
-      if (k < 0 || k > P) {
-        if (threadIdx.x == 0) atomicExch(status, AUDIOKV_EDEVICE);
-        k = k < 0 ? 0 : P;
-      }
-      __syncthreads();
-      if (pl.packed)
-        select_topk([&](int j) -> uint32_t { const float2 e = buf[j >> 1]; return __float_as_uint((j & 1) ? e.y : e.x); }, P, W, k,
-                    kept_idx + cu_kept[u], &ssm, status);
-      else
-        select_topk([&](int j) -> uint32_t { return __float_as_uint(buf[j].x); }, P, W, k, kept_idx + cu_kept[u], &ssm, status);
-    }
+    if (S.pl.in_smem) smooth_head<false>(sh, tables, sel, status);
+    else smooth_head<true>(sh, tables, sel, status);
   }
 }
 
 // ---- tables ---------------------------------------------------------------------------
+__device__ __forceinline__ float2 root_of_unity(int64_t num, int den) {  // exp(-2 pi i num / den)
+  double s, c;
+  sincospi(2.0 * static_cast<double>(num % den) / den, &s, &c);
+  return make_float2(static_cast<float>(c), static_cast<float>(-s));
+}
+
 __global__ void fft_table_kernel(const FftPlan* __restrict__ plans, int n_plans, float2* __restrict__ tables) {
-  const FftPlan pl = plans[blockIdx.y];
+  const FftPlan& pl = plans[blockIdx.y];
   const int gid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
-  const int Nt = pl.seq.N;
-  for (int t = gid; t < Nt; t += gsz) {
-    double s, c;
-    sincospi(2.0 * t / Nt, &s, &c);
-    tables[pl.seq.tw_offset + t] = make_float2(static_cast<float>(c), static_cast<float>(-s));
+  // roots: 256 fine entries and the coarse ones, of the order the passes want and, for a chirp-z, of order 2N
+  for (int t = gid; t < pl.root_count + pl.root_count2; t += gsz) {
+    const bool second = t >= pl.root_count;
+    const int i = second ? t - pl.root_count : t, order = second ? 2 * pl.N : pl.seq.N * pl.root_mult;
+    double sn, cs;
+    sincospi(2.0 * static_cast<double>(i < 256 ? i : (i - 256) * 256) / order, &sn, &cs);
+    reinterpret_cast<double2*>(tables + pl.root_offset)[t] = make_double2(cs, -sn);
   }
-  if (pl.packed) {
-    for (int k = gid; k <= pl.N / 2; k += gsz) {
-      double s, c;
-      sincospi(2.0 * k / pl.n, &s, &c);
-      tables[pl.post_offset + k] = make_float2(static_cast<float>(c), static_cast<float>(-s));
+  for (int i = 0; i < pl.seq.n_pass; ++i) {
+    const int R = pl.seq.radix[i];
+    if (R > 13) {
+      const int H = (R - 1) / 2, Cp = fft_mat_cols(R);
+      for (int t = gid; t < H * Cp; t += gsz) {
+        const int s = t / Cp + 1, c = t - (s - 1) * Cp;
+        const float2 w = root_of_unity(static_cast<int64_t>(s) * c, R);
+        tables[pl.seq.base + pl.seq.mat[i] + t] = make_float2(w.x, -w.y);  // (cos, sin)
+      }
     }
   }
   if (!pl.bluestein) {
-    int* pos_tab = reinterpret_cast<int*>(tables + pl.pos_offset);
-    for (int k = gid; k < pl.N; k += gsz) pos_tab[k] = seq_pos(pl.seq, k);
+    uint32_t* rec = reinterpret_cast<uint32_t*>(tables + pl.pos_offset);
+    for (int k = gid; k <= pl.N / 2; k += gsz) {
+      const uint32_t a = seq_pos(pl.seq, k), b = seq_pos(pl.seq, k == 0 ? 0 : pl.N - k);
+      if (pl.wide_pos) {
+        rec[2 * k] = a;
+        rec[2 * k + 1] = b;
+      } else {
+        rec[k] = a | b << 16;
+      }
+    }
   }
   if (pl.bluestein) {
     const int N = pl.N, M = pl.M;
@@ -1254,46 +1340,55 @@ __global__ void fft_table_kernel(const FftPlan* __restrict__ plans, int n_plans,
       return make_float2(static_cast<float>(c), static_cast<float>(s));
     };
     for (int j = gid; j < M; j += gsz) {
-      if (j < N) {
-        const float2 b = chirp_at(j);
-        tables[pl.chirp_offset + j] = make_float2(b.x, -b.y);
-      }
       // position j holds difference +j inside the positive support, difference -(M - j) inside the negative one
       // (they never collide: M is at least their total length), zero in between
-      auto wrapped = [&](int pos, int neg) -> float2 {
-        if (j < pos) return chirp_at(j);
-        if (M - j < neg) return chirp_at(M - j);
-        return make_float2(0.f, 0.f);
-      };
+      const int d = j < N ? j : M - j;
+      const float2 b = d < N ? chirp_at(d) : make_float2(0.f, 0.f), zero = make_float2(0.f, 0.f);
+      const float2 bn = j < N && M - j < N ? chirp_at(M - j) : b;  // the value on the negative side, should j lie there
+      auto wrapped = [&](int pos, int neg) -> float2 { return j < pos ? b : M - j < neg ? bn : zero; };
       tables[pl.filter_offset + j] = wrapped(pos_f, neg_f);
       if (pl.half) tables[pl.filter2_offset + j] = wrapped(pos_i, neg_i);
     }
   }
 }
 
-// Transforms each chirp-z filter in place (global memory) and folds in the 1/M of the inverse.
-__global__ void __launch_bounds__(kSssThreads, 1)
+// Transforms each chirp-z filter in place and folds in the 1/M of the inverse: one block per plan and filter.
+__global__ void __launch_bounds__(kT, 1)
 fft_filter_kernel(const FftPlan* __restrict__ plans, float2* __restrict__ tables) {
-  __shared__ FftPlan pl;
-  __shared__ float2 wp[128];
-  if (threadIdx.x == 0) pl = plans[blockIdx.x];
+  const FftPlan& pl = S.pl;
+  for (int i = threadIdx.x; i < static_cast<int>(sizeof(FftPlan) / 4); i += kT)
+    reinterpret_cast<int*>(&S.pl)[i] = reinterpret_cast<const int*>(plans + blockIdx.x)[i];
   __syncthreads();
-  if (!pl.bluestein) return;
-  for (int which = 0; which < (pl.half ? 2 : 1); ++which) {
-    float2* f = tables + (which ? pl.filter2_offset : pl.filter_offset);
+  if (!pl.bluestein || (blockIdx.y == 1 && !pl.half)) return;
+  const Roots root{pl.root_at, pl.root_mult};
+  load_roots(pl, tables, pl.root_count);
+  __syncthreads();
+  float2* f = tables + (blockIdx.y ? pl.filter2_offset : pl.filter_offset);
+  const float inv = 1.f / static_cast<float>(pl.M);
+  if (pl.in_smem) {
+    const SmemBuf sb;
+    batched<8>(pl.M, [&](int j) { return f[j]; }, [&](int j, float2 v) { sb.st(j, v); });
     __syncthreads();
-    fft_dif(SkewBuf{f, 31, 0}, pl.seq, tables + pl.seq.tw_offset, wp);
-    const float inv = 1.f / static_cast<float>(pl.M);
-    for (int j = threadIdx.x; j < pl.M; j += kSssThreads) f[j] = cscale(f[j], inv);
+    passes_fwd(sb, pl.M, pl.M, pl.seq, 0, pl.seq.n_pass, root, tables);
+#pragma unroll 4
+    for (int j = threadIdx.x; j < pl.M; j += kT) f[j] = cscale(sb.ld(j), inv);
+  } else {
+    fft_big<false>(f, pl, root, tables);
+#pragma unroll 4
+    for (int j = threadIdx.x; j < pl.M; j += kT) f[j] = cscale(f[j], inv);
   }
 }
 
 }  // namespace
 
-cudaError_t launch_fft_tables(int n_plans, float2* d_tables, const FftPlan* d_plans, Launch ln) {
+int sss_static_smem() { return static_cast<int>(sizeof(SssShared)); }
+
+cudaError_t launch_fft_tables(int n_plans, float2* d_tables, const FftPlan* d_plans, size_t smem_bytes, Launch ln) {
   fft_table_kernel<<<dim3(32, n_plans), 256, 0, ln.stream>>>(d_plans, n_plans, d_tables);
   ln.done("fft_table");
-  fft_filter_kernel<<<n_plans, kSssThreads, 0, ln.stream>>>(d_plans, d_tables);
+  cudaError_t e = cudaFuncSetAttribute(fft_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+  if (e != cudaSuccess) return e;
+  fft_filter_kernel<<<dim3(n_plans, 2), kT, smem_bytes, ln.stream>>>(d_plans, d_tables);
   ln.done("fft_filter");
   return cudaGetLastError();
 }
@@ -1305,7 +1400,7 @@ cudaError_t launch_sss(const Shape& sh, const ReqDesc* d_reqs, const FftPlan* d_
                        Launch ln) {
   cudaError_t e = cudaFuncSetAttribute(sss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   if (e != cudaSuccess) return e;
-  e = launch_chained(sss_kernel, dim3(grid), dim3(kSssThreads), smem_bytes, ln.stream, sh, d_reqs, d_plans, d_tables, scores,
+  e = launch_chained(sss_kernel, dim3(grid), dim3(kT), smem_bytes, ln.stream, sh, d_reqs, d_plans, d_tables, scores,
                      smoothed, kstar, scratch, scratch_per_block, order, n_order, first_head, budgets, cu_kept, kept_idx,
                      status);
   ln.done(budgets ? "sss_select" : "sss");
