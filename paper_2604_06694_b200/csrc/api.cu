@@ -23,7 +23,7 @@ constexpr int kHostChunks = 8;          // the host-buffer call evicts one reque
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {  // byte offsets inside the workspace
-  size_t status, reqs, plans, tables, units, ctas, order, stats, fft_scratch, scores, kstar, aux, end;
+  size_t status, reqs, plans, tables, units, ctas, order, stats, exps, fft_scratch, scores, kstar, aux, end;
 };
 
 struct Plan {
@@ -43,6 +43,7 @@ struct Plan {
   int64_t scores_len = 0;
   int max_L = 0, max_P = 0;
   int n_slab = 0;
+  int64_t exps_len = 0;         // floats
   int sss_grid = 0;
   size_t sss_smem = 0;
   int64_t scratch_per_block = 0;  // float2 elements
@@ -474,9 +475,14 @@ int build_plan(const audiokv_params* p, Plan* pl) {
   L.order = off;       off = align_up(off + sizeof(int32_t) * pl->sss_order.size());
   {
     // softmax statistics: [head][slab][row] for the FMA kernels, [head][part][group][row] for the tensor-core ones
-    const size_t slots = std::max<size_t>(pl->n_slab, static_cast<size_t>(pl->score_parts) * score_stat_sets());
-    L.stats = off;     off = align_up(off + sizeof(float2) * static_cast<size_t>(sh.total_heads) * slots * sh.window * sh.group);
+    const int rows = sh.window * sh.group;
+    size_t entries = static_cast<size_t>(sh.total_heads) * std::max<size_t>(pl->n_slab, static_cast<size_t>(pl->score_parts) * score_stat_sets()) * rows;
+    // the FMA kernels keep a chunk's exponentials when they are the ones that score (see score_simt.cu)
+    pl->exps_len = score_umma_takes(sh) ? 0 : score_simt_exps_len(sh.total_heads, pl->max_L, rows);
+    entries = std::max(entries, static_cast<size_t>(pl->exps_len / score_simt_tile_keys()));
+    L.stats = off;     off = align_up(off + sizeof(float2) * entries);
   }
+  L.exps = off;        off = align_up(off + sizeof(float) * static_cast<size_t>(pl->exps_len));
   L.fft_scratch = off; off = align_up(off + sizeof(float2) * static_cast<size_t>(pl->scratch_per_block) * pl->sss_grid);
   L.scores = off;      off = align_up(off + sizeof(float) * static_cast<size_t>(pl->scores_len));
   L.kstar = off;       off = align_up(off + sizeof(int32_t) * static_cast<size_t>(sh.total_heads));
@@ -579,7 +585,8 @@ int do_score(audiokv_ctx* ctx, const void* q, const void* k, float* scores, cuda
     // fp32 inputs (which must not be rounded to TF32), a GQA group above 256 query heads, or strides the copy
     // engine cannot take; audiokv_last_score_path tells the caller which route ran
     ctx->score_path = 2;
-    e = launch_score_simt(pl.sh, d_reqs(ctx), q, k, scores, stats, pl.n_slab, kSlabKeys, ln);
+    float* exps = pl.exps_len ? reinterpret_cast<float*>(ctx->ws + pl.lay.exps) : nullptr;
+    e = launch_score_simt(pl.sh, d_reqs(ctx), q, k, scores, stats, pl.n_slab, kSlabKeys, exps, pl.exps_len, pl.max_L, ln);
   }
   return e == cudaSuccess ? AUDIOKV_OK : cuda_fail(ctx, e);
 }

@@ -1,33 +1,32 @@
 // Importance scores on the fp32 FMA pipe, for any element type.
 //
-// This is the path for fp32 inputs (which must not be rounded to TF32) and the
-// fallback for shapes the tensor-core kernels do not take. Two sweeps over the keys:
-//   sweep 1  per (head, key slab): running max and sum of exp2 of every window row,
-//   sweep 2  per (head, key slab): merge the slabs' statistics, then for every prefix
-//            key sum exp2(z - max - log2 sum) over the rows.
+// This is the path for fp32 inputs (which must not be rounded to TF32) and the fallback for shapes the tensor-core kernels
+// do not take. A column sum mixes rows with different normalisers, which are known only when every key has been seen.
+//
+// What bounds it: the FMAs of Q K^T, 26.3 GFLOP for 28 layers of the 7B shape at 4096 keys, 0.35 ms of the fp32 pipe if
+// they are done once. So where there is room they are done once: the product kernel writes exp2(z - m) of its tile, m the
+// row's maximum over the tile's keys, and (m, sum) per row; a merge gives every row c = -(max + log2 sum) over all keys;
+// the sum kernel adds exp2(m + c) exp2(z - m) over the rows of every key, a stream at memory speed. Heads go through in
+// chunks of up to 128 MB of exponentials. A head too long for the chunk's room, and the entry point with fixed
+// scratch, run the product twice: statistics, merge, column sums.
+// The product is a register-tiled matrix product: 64 keys x 64, 112 or 128 query rows a block of 128 threads, 8 x 4, 7 or 8
+// logits a thread, panels of 32 dimensions through three stages of asynchronous copies, two blocks an SM. A logit is kept as
+// a pair, the sums over its even and its odd dimensions, so that packed FMAs take their operands as they lie in shared
+// memory: per four dimensions a thread reads 8 + 7 16-byte pieces (15 cycles of shared memory a warp) for 112 packed FMAs. (With
+// scalar FMAs on 8 x 7 single sums the pipe was 49 % busy, held up by dispatch stalls of three-operand reads: 139 us for
+// a chunk of 16 heads at 4096 keys.) The 64 x 64 tiles of 4 x 4 logits that were here first, with the tile's logits through
+// shared memory and the product done twice, took 1487 + 1234 us on that shape.
 // Logits are kept in base 2 (scale * log2 e folded into one multiply).
 #include "common.cuh"
 
 namespace akv {
 namespace {
 
-constexpr int kTile = 64;      // keys per tile and rows per row chunk
-constexpr int kThreads = 256;  // 16 x 16 threads, 4 x 4 logits each
-
-template <typename T>
-__device__ __forceinline__ float4 load4(const T* p);
-template <>
-__device__ __forceinline__ float4 load4<float>(const float* p) {
-  return *reinterpret_cast<const float4*>(p);
-}
-template <>
-__device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
-  uint2 raw = *reinterpret_cast<const uint2*>(p);
-  __nv_bfloat162 a = *reinterpret_cast<__nv_bfloat162*>(&raw.x);
-  __nv_bfloat162 b = *reinterpret_cast<__nv_bfloat162*>(&raw.y);
-  float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
-  return make_float4(fa.x, fa.y, fb.x, fb.y);
-}
+constexpr int kKeys = 64;            // keys per tile
+constexpr int kTileThreads = 128;    // 8 x 16 threads: keys x rows
+constexpr int kThreads = 256;        // of the merge and the sum kernel
+constexpr int kPanel = 32;     // dimensions per stage
+constexpr int kStages = 3;
 
 struct HeadCoord {
   int r, l, h;
@@ -41,189 +40,378 @@ __device__ __forceinline__ HeadCoord head_coord(const Shape& sh, int u) {
   return c;
 }
 
-// Stages `kTile` rows of D elements as fp32 into smem (row stride D + 4); rows >= n_valid are zero.
-template <typename T, int D, typename RowPtr>
-__device__ __forceinline__ void stage_rows(float* smem, int n_valid, RowPtr row_ptr) {
-  constexpr int C4 = D / 4;
-  for (int idx = threadIdx.x; idx < kTile * C4; idx += kThreads) {
-    int row = idx / C4, c4 = idx - row * C4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (row < n_valid) v = load4<T>(row_ptr(row) + c4 * 4);
-    *reinterpret_cast<float4*>(smem + row * (D + 4) + c4 * 4) = v;
-  }
+// A panel row in shared memory: 32 elements and 16 bytes of padding, which puts eight neighbouring rows' 16-byte pieces
+// on different banks.
+template <typename T>
+struct PanelRow {
+  static constexpr int kBytes = kPanel * static_cast<int>(sizeof(T)) + 16;
+};
+typedef unsigned long long f32x2;
+struct Piece {
+  f32x2 lo, hi;  // dimensions t, t + 1 and t + 2, t + 3
+};
+__device__ __forceinline__ f32x2 pair_of(uint32_t a, uint32_t b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float pair_sum(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a + b;
+}
+__device__ __forceinline__ Piece piece(const unsigned char* row, int t, float) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(row + t * 4);
+  return Piece{v.x, v.y};
+}
+__device__ __forceinline__ Piece piece(const unsigned char* row, int t, __nv_bfloat16) {
+  const uint2 raw = *reinterpret_cast<const uint2*>(row + t * 2);
+  return Piece{pair_of(raw.x << 16, raw.x & 0xffff0000u), pair_of(raw.y << 16, raw.y & 0xffff0000u)};
+}
+// 16 bytes to shared memory without passing through registers; zeros when `ok` is false (nothing is read then).
+__device__ __forceinline__ void copy16(void* dst, const void* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src),
+               "r"(ok ? 16 : 0)
+               : "memory");
 }
 
-// acc[a][b] = <Q row ty + 16 a, K row tx + 16 b>
-template <int D>
-__device__ __forceinline__ void tile_dot(const float* Qs, const float* Ks, int ty, int tx, float acc[4][4]) {
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-#pragma unroll 4
-  for (int t = 0; t < D; t += 4) {
-    float4 qv[4], kv[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) qv[a] = *reinterpret_cast<const float4*>(Qs + (ty + 16 * a) * (D + 4) + t);
-#pragma unroll
-    for (int b = 0; b < 4; ++b) kv[b] = *reinterpret_cast<const float4*>(Ks + (tx + 16 * b) * (D + 4) + t);
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        acc[a][b] = fmaf(qv[a].x, kv[b].x, acc[a][b]);
-        acc[a][b] = fmaf(qv[a].y, kv[b].y, acc[a][b]);
-        acc[a][b] = fmaf(qv[a].z, kv[b].z, acc[a][b]);
-        acc[a][b] = fmaf(qv[a].w, kv[b].w, acc[a][b]);
-      }
-  }
+enum { kStore = 0, kStats = 1, kColsum = 2 };
+
+constexpr int tile_smem_bytes(int rpt, int esize) {
+  return kStages * (kKeys + 16 * rpt) * (kPanel * esize + 16) + (kKeys + 16 * rpt) * static_cast<int>(sizeof(long long));
 }
 
-// SWEEP = 1: row statistics; SWEEP = 2: column sums.
-template <typename T, int D, int SWEEP>
-__global__ void __launch_bounds__(kThreads) score_simt_kernel(Shape sh, const ReqDesc* __restrict__ reqs,
-                                                              const T* __restrict__ q, const T* __restrict__ k,
-                                                              float* __restrict__ scores, float2* __restrict__ stats,
-                                                              int n_slab, int slab_keys) {
-  extern __shared__ __align__(16) float smem[];
-  float* Qs = smem;
-  float* Ks = Qs + kTile * (D + 4);
-  float* Zt = Ks + kTile * (D + 4);      // [kTile][kTile + 1]
-  float* rowA = Zt + kTile * (kTile + 1);  // sweep 1: running max; sweep 2: max + log2 sum
-  float* rowB = rowA + sh.window * sh.group;  // sweep 1: running sum; sweep 2: partial column sums [4][kTile]
+// MODE kStore: one tile of keys per slab; its exponentials and row statistics. kStats: row statistics of a slab. kColsum: column
+// sums of a slab's prefix keys, the rows' c given (see merge_kernel). Heads u0, u0 + 1, ...; statistics of head u at u - u0.
+template <typename T, int D, int RPT, int MODE>
+__global__ void __launch_bounds__(kTileThreads, 2)
+score_tile_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const T* __restrict__ q, const T* __restrict__ k,
+                  float* __restrict__ scores, float2* __restrict__ stats, float* __restrict__ exps, int n_slab, int slab_keys,
+                  int u0) {
+  constexpr int kRows = 16 * RPT, kRowBytes = PanelRow<T>::kBytes, kStage = (kKeys + kRows) * kRowBytes;
+  constexpr int kPieces = kPanel * static_cast<int>(sizeof(T)) / 16;  // 16-byte pieces of a panel row
+  extern __shared__ __align__(16) unsigned char smem[];
+  long long* off = reinterpret_cast<long long*>(smem + kStages * kStage);  // element offsets of the tile's rows, -1: zeros
 
-  const int u = blockIdx.x / n_slab, slab = blockIdx.x - u * n_slab;  // one block per (head, slab), heads outermost
+  chain_release();
+  chain_wait();  // the request table may be the work of the kernel before
+  const int uc = blockIdx.x / n_slab, slab = blockIdx.x - uc * n_slab, u = u0 + uc;
   const HeadCoord hc = head_coord(sh, u);
   const ReqDesc rq = reqs[hc.r];
   const int R = sh.window * sh.group, G = sh.group;
-  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+  const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;  // this thread's rows ty + 16 a and keys tx + 8 b
   const int j0 = slab * slab_keys;
-  const int j_end = SWEEP == 1 ? rq.L : rq.P;  // sweep 2 only needs the prefix keys
-  const int j1 = min(j_end, j0 + slab_keys);
-  float2* my_stats = stats + (static_cast<int64_t>(u) * n_slab + slab) * R;
-
+  const int j1 = min(MODE == kColsum ? rq.P : rq.L, j0 + slab_keys);  // column sums: prefix keys only
+  float2* my_stats = stats + (static_cast<int64_t>(uc) * n_slab + slab) * R;
   const T* kbase = k + hc.l * sh.kv_stride_layer + hc.h * sh.kv_stride_head;  // the token term: kv_token_offset
   const T* qbase = q + rq.q_offset + hc.l * sh.q_stride_layer + static_cast<int64_t>(hc.h) * G * sh.q_stride_head;
 
-  if (SWEEP == 1) {
-    for (int r = threadIdx.x; r < R; r += kThreads) {
-      rowA[r] = -INFINITY;
-      rowB[r] = 0.f;
-    }
-  } else {
-    const float2* hs = stats + static_cast<int64_t>(u) * n_slab * R;
-    for (int r = threadIdx.x; r < R; r += kThreads) {
-      float M = -INFINITY;
-      for (int s = 0; s < n_slab; ++s) M = fmaxf(M, hs[static_cast<int64_t>(s) * R + r].x);
-      float Z = 0.f;
-      for (int s = 0; s < n_slab; ++s) {
-        float2 st = hs[static_cast<int64_t>(s) * R + r];
-        if (st.y > 0.f) Z += st.y * exp2f(st.x - M);
+  // acc[a][b] = <Q row rc + ty + 16 a, K row kt + tx + 8 b>
+  auto product = [&](float (&acc)[RPT][8], int kt, int rc) {
+    __syncthreads();  // the panels and offsets of the product before are free
+    for (int i = threadIdx.x; i < kKeys + kRows; i += kTileThreads) {
+      long long o = -1;
+      if (i < kKeys) {
+        if (kt + i < j1) o = kv_token_offset(sh, rq, hc.r, kt + i);
+      } else {
+        const int rr = rc + i - kKeys;
+        if (rr < R) o = rr / G * sh.q_stride_tok + rr % G * sh.q_stride_head;
       }
-      rowA[r] = M + log2f(Z);
+      off[i] = o;
     }
-  }
-  __syncthreads();
-
-  for (int kt = j0; kt < j1; kt += kTile) {
-    const int nk = min(kTile, j1 - kt);
-    stage_rows<T, D>(Ks, nk, [&](int row) { return kbase + kv_token_offset(sh, rq, hc.r, kt + row); });
-    float colsum = 0.f;  // sweep 2, threads 0..63
-    for (int rc = 0; rc < R; rc += kTile) {
-      const int nr = min(kTile, R - rc);
-      __syncthreads();  // Qs, Zt free
-      stage_rows<T, D>(Qs, nr, [&](int row) {
-        int rr = rc + row;
-        int i = rr / G, g = rr - i * G;
-        return qbase + i * sh.q_stride_tok + g * sh.q_stride_head;
-      });
-      __syncthreads();
-      float acc[4][4];
-      tile_dot<D>(Qs, Ks, ty, tx, acc);
+    __syncthreads();
+    auto load = [&](int p) {  // panel p into stage p % kStages
+      unsigned char* st = smem + p % kStages * kStage;
+#pragma unroll 4
+      for (int i = threadIdx.x; i < (kKeys + kRows) * kPieces; i += kTileThreads) {
+        const int row = i / kPieces, c = i - row * kPieces;
+        const long long o = off[row];
+        const T* src = (row < kKeys ? kbase : qbase) + (o < 0 ? 0 : o) + p * kPanel + c * (16 / static_cast<int>(sizeof(T)));
+        copy16(st + row * kRowBytes + c * 16, src, o >= 0);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    f32x2 sum[RPT][8];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const int row = ty + 16 * a, rr = rc + row;
-        const int i = rr / G;
+    for (int a = 0; a < RPT; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int key = tx + 16 * b, j = kt + key;
-          float z = acc[a][b] * sh.scale_log2e;
-          if (SWEEP == 1) {
-            bool ok = rr < R && key < nk && j <= rq.P + i;
-            Zt[row * (kTile + 1) + key] = ok ? z : -INFINITY;
-          } else {
-            bool ok = rr < R && key < nk;
-            Zt[row * (kTile + 1) + key] = ok ? exp2f(z - rowA[rr < R ? rr : 0]) : 0.f;
+      for (int b = 0; b < 8; ++b) sum[a][b] = 0ull;
+    constexpr int kPanels = D / kPanel;
+    load(0);
+    load(1);
+#pragma unroll 1
+    for (int p = 0; p < kPanels; ++p) {
+      if (p + 1 < kPanels) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();  // panel p is complete; everybody is done with panel p - 1
+      if (p + 2 < kPanels) load(p + 2);
+      const unsigned char* st = smem + p % kStages * kStage;
+      const unsigned char* kr = st + tx * kRowBytes;
+      const unsigned char* qr = st + (kKeys + ty) * kRowBytes;
+#pragma unroll(sizeof(T) == 4 ? 2 : 1)
+      for (int t = 0; t < kPanel; t += 4) {
+        Piece kv[8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) kv[b] = piece(kr + 8 * b * kRowBytes, t, T());
+#pragma unroll
+        for (int a = 0; a < RPT; ++a) {
+          const Piece qv = piece(qr + 16 * a * kRowBytes, t, T());
+#pragma unroll
+          for (int b = 0; b < 8; ++b) {
+            sum[a][b] = fma2(qv.lo, kv[b].lo, sum[a][b]);
+            sum[a][b] = fma2(qv.hi, kv[b].hi, sum[a][b]);
           }
         }
       }
+    }
+#pragma unroll
+    for (int a = 0; a < RPT; ++a)
+#pragma unroll
+      for (int b = 0; b < 8; ++b) acc[a][b] = pair_sum(sum[a][b]);
+  };
+  float acc[RPT][8];
+  if constexpr (MODE == kColsum) {
+    const float2* hs = stats + static_cast<int64_t>(uc) * n_slab * R;  // c of row r: .y of the head's first slab
+    for (int kt = j0; kt < j1; kt += kKeys) {
+      float col[8];
+#pragma unroll
+      for (int b = 0; b < 8; ++b) col[b] = 0.f;
+      for (int rc = 0; rc < R; rc += kRows) {
+        product(acc, kt, rc);
+#pragma unroll
+        for (int a = 0; a < RPT; ++a) {
+          const int rr = rc + ty + 16 * a;
+          const float c = rr < R ? hs[rr].y : -INFINITY;
+#pragma unroll
+          for (int b = 0; b < 8; ++b) col[b] += exp2f(fmaf(acc[a][b], sh.scale_log2e, c));
+        }
+      }
+      __syncthreads();  // the panels make room for the sums of the 16 thread rows
+      float* red = reinterpret_cast<float*>(smem);
+#pragma unroll
+      for (int b = 0; b < 8; ++b) red[ty * kKeys + tx + 8 * b] = col[b];
       __syncthreads();
-      if (SWEEP == 1) {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int row = warp; row < nr; row += kThreads / 32) {
-          float z0 = Zt[row * (kTile + 1) + lane], z1 = Zt[row * (kTile + 1) + lane + 32];
-          float m = fmaxf(z0, z1);
+      if (threadIdx.x < kKeys && kt + static_cast<int>(threadIdx.x) < j1) {
+        float s = 0.f;
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-          if (m > -INFINITY) {
-            const float m_old = rowA[rc + row];
-            const float m_new = fmaxf(m_old, m);
-            float e = exp2f(z0 - m_new) + exp2f(z1 - m_new);
+        for (int y = 0; y < 16; ++y) s += red[y * kKeys + threadIdx.x];
+        scores[rq.score_offset + (static_cast<int64_t>(hc.l) * sh.n_kv_heads + hc.h) * rq.P + kt + threadIdx.x] = s;
+      }
+    }
+  } else {
+    for (int rc = 0; rc < R; rc += kRows) {
+      float m[RPT], Z[RPT];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-            if (lane == 0) {
-              rowB[rc + row] = rowB[rc + row] * exp2f(m_old - m_new) + e;
-              rowA[rc + row] = m_new;
+      for (int a = 0; a < RPT; ++a) {
+        m[a] = -INFINITY;
+        Z[a] = 0.f;
+      }
+      for (int kt = j0; kt < j1; kt += kKeys) {
+        product(acc, kt, rc);
+#pragma unroll
+        for (int a = 0; a < RPT; ++a) {
+          const int rr = rc + ty + 16 * a;
+          const int last = min(j1 - 1, rq.P + rr / G) - kt;  // last visible key of this row in the tile
+          float top = -INFINITY;
+#pragma unroll
+          for (int b = 0; b < 8; ++b) {
+            acc[a][b] = tx + 8 * b <= last ? acc[a][b] * sh.scale_log2e : -INFINITY;
+            top = fmaxf(top, acc[a][b]);
+          }
+          if (MODE == kStore) {  // one reference for the row's keys of the tile
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+          }
+          const float ref = fmaxf(m[a], top);
+          const float safe = ref == -INFINITY ? 0.f : ref;  // nothing visible yet: the exponentials are zeros
+          float s = 0.f;
+#pragma unroll
+          for (int b = 0; b < 8; ++b) {
+            acc[a][b] = exp2f(acc[a][b] - safe);
+            s += acc[a][b];
+          }
+          Z[a] = Z[a] * exp2f(m[a] - safe) + s;
+          m[a] = ref;
+        }
+        if (MODE == kStore) {
+          float* e = exps + ((static_cast<int64_t>(uc) * n_slab + slab) * R) * kKeys;
+#pragma unroll
+          for (int a = 0; a < RPT; ++a) {
+            const int rr = rc + ty + 16 * a;
+            if (rr < R) {
+#pragma unroll
+              for (int b = 0; b < 8; ++b) e[static_cast<int64_t>(rr) * kKeys + tx + 8 * b] = acc[a][b];
             }
           }
         }
-      } else {
-        const int key = threadIdx.x & 63, part = threadIdx.x >> 6;
-        float sacc = 0.f;
+      }
 #pragma unroll
-        for (int rr = 0; rr < 16; ++rr) sacc += Zt[(part * 16 + rr) * (kTile + 1) + key];
-        rowB[part * kTile + key] = sacc;
-        __syncthreads();
-        if (threadIdx.x < kTile)
-          colsum += (rowB[threadIdx.x] + rowB[kTile + threadIdx.x]) + (rowB[2 * kTile + threadIdx.x] + rowB[3 * kTile + threadIdx.x]);
+      for (int a = 0; a < RPT; ++a) {
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+          const float mo = __shfl_xor_sync(0xffffffffu, m[a], o), zo = __shfl_xor_sync(0xffffffffu, Z[a], o);
+          const float mn = fmaxf(m[a], mo), safe = mn == -INFINITY ? 0.f : mn;
+          Z[a] = Z[a] * exp2f(m[a] - safe) + zo * exp2f(mo - safe);
+          m[a] = mn;
+        }
+        const int rr = rc + ty + 16 * a;
+        if (tx == 0 && rr < R) my_stats[rr] = make_float2(m[a], Z[a]);
       }
     }
-    if (SWEEP == 2 && threadIdx.x < nk) {
-      scores[rq.score_offset + (static_cast<int64_t>(hc.l) * sh.n_kv_heads + hc.h) * rq.P + kt + threadIdx.x] = colsum;
-    }
-    __syncthreads();  // Ks free
-  }
-  if (SWEEP == 1) {
-    __syncthreads();
-    for (int r = threadIdx.x; r < R; r += kThreads) my_stats[r] = make_float2(rowA[r], rowB[r]);
   }
 }
 
+// c = -(max + log2 sum) of every row over its head's slabs, into .y of the row's entry of the first slab (whose sum is no
+// longer needed; its maximum stays). One block per 32 rows of a head: eight warps share the slabs.
+__global__ void __launch_bounds__(kThreads) merge_kernel(float2* __restrict__ stats, int n_slab, int R) {
+  __shared__ float2 part[8][32];
+  chain_release();
+  chain_wait();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r = blockIdx.y * 32 + lane;
+  float2* hs = stats + static_cast<int64_t>(blockIdx.x) * n_slab * R;
+  float M = -INFINITY, Z = 0.f;
+  auto add = [&](float2 st) {
+    if (!(st.y > 0.f)) return;
+    const float mn = fmaxf(M, st.x);
+    Z = Z * exp2f(M - mn) + st.y * exp2f(st.x - mn);
+    M = mn;
+  };
+  if (r < R) {
+#pragma unroll 4
+    for (int s = warp; s < n_slab; s += 8) add(hs[static_cast<int64_t>(s) * R + r]);
+  }
+  part[warp][lane] = make_float2(M, Z);
+  __syncthreads();
+  if (warp == 0 && r < R) {
+    for (int w = 1; w < 8; ++w) add(part[w][lane]);
+    hs[r].y = -(M + log2f(Z));
+  }
+}
+
+// Column sums from the stored exponentials: one block per tile. Half a warp reads one row (256 bytes) at a time.
+__global__ void __launch_bounds__(kThreads)
+colsum_kernel(Shape sh, const ReqDesc* __restrict__ reqs, float* __restrict__ scores, const float2* __restrict__ stats,
+              const float* __restrict__ exps, int n_slab, int u0) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float* f = reinterpret_cast<float*>(smem);                   // [R] factor of every row
+  constexpr int kHalves = kThreads / 16;
+  __shared__ float4 red[kHalves][16];
+  chain_release();
+  chain_wait();
+  const int uc = blockIdx.x / n_slab, slab = blockIdx.x - uc * n_slab, u = u0 + uc;
+  const HeadCoord hc = head_coord(sh, u);
+  const ReqDesc rq = reqs[hc.r];
+  const int R = sh.window * sh.group, j0 = slab * kKeys;
+  const int lane = threadIdx.x & 15, half = threadIdx.x >> 4;
+  if (j0 >= rq.P) return;
+  const float2* hs = stats + static_cast<int64_t>(uc) * n_slab * R;
+  const float4* e = reinterpret_cast<const float4*>(exps + (static_cast<int64_t>(uc) * n_slab + slab) * R * kKeys) + lane;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 v[8];
+  auto fetch = [&](int r0) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __ldcs(e + static_cast<int64_t>(min(r0 + i * kHalves, R - 1)) * (kKeys / 4));
+  };
+  fetch(half);  // the first rows run beside the factors' loads
+  for (int r = threadIdx.x; r < R; r += kThreads) f[r] = exp2f(hs[static_cast<int64_t>(slab) * R + r].x + hs[r].y);
+  __syncthreads();
+  for (int r0 = half; r0 < R;) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float w = r0 + i * kHalves < R ? f[r0 + i * kHalves] : 0.f;
+      s.x = fmaf(v[i].x, w, s.x);
+      s.y = fmaf(v[i].y, w, s.y);
+      s.z = fmaf(v[i].z, w, s.z);
+      s.w = fmaf(v[i].w, w, s.w);
+    }
+    r0 += 8 * kHalves;
+    if (r0 < R) fetch(r0);
+  }
+  red[half][lane] = s;
+  __syncthreads();
+  if (threadIdx.x < kKeys && j0 + static_cast<int>(threadIdx.x) < rq.P) {
+    const float* col = reinterpret_cast<const float*>(red) + threadIdx.x;
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < kHalves; ++w) t += col[w * kKeys];
+    scores[rq.score_offset + (static_cast<int64_t>(hc.l) * sh.n_kv_heads + hc.h) * rq.P + j0 + threadIdx.x] = t;
+  }
+}
+
+template <typename T, int D, int RPT, int MODE>
+cudaError_t launch_tile(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
+                        float* exps, int n_slab, int slab_keys, int u0, int heads, Launch ln) {
+  auto kern = score_tile_kernel<T, D, RPT, MODE>;
+  const int smem = tile_smem_bytes(RPT, static_cast<int>(sizeof(T)));
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  e = launch_chained(kern, dim3(static_cast<unsigned>(n_slab) * heads), dim3(kTileThreads), smem, ln.stream, sh, d_reqs,
+                     static_cast<const T*>(q), static_cast<const T*>(k), scores, stats, exps, n_slab, slab_keys, u0);
+  ln.done(MODE == kStore ? "score_simt_exps" : MODE == kStats ? "score_simt_stats" : "score_simt_colsum");
+  return e;
+}
+
+template <typename T, int D, int RPT>
+cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
+                         int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln) {
+  const int R = sh.window * sh.group, n_tile = (max_L + kKeys - 1) / kKeys;
+  const int64_t per_head = static_cast<int64_t>(n_tile) * R * kKeys;
+  const bool store = exps != nullptr && per_head <= exps_len;
+  const int slabs = store ? n_tile : n_slab;
+  const int64_t room = store ? exps_len / per_head : 0x7fffffffLL / slabs;
+  const int chunk = static_cast<int>(room < sh.total_heads ? room : sh.total_heads);
+  cudaError_t e = cudaSuccess;
+  for (int u0 = 0; u0 < sh.total_heads && e == cudaSuccess; u0 += chunk) {
+    const int heads = sh.total_heads - u0 < chunk ? sh.total_heads - u0 : chunk;
+    if (store) e = launch_tile<T, D, RPT, kStore>(sh, d_reqs, q, k, scores, stats, exps, slabs, kKeys, u0, heads, ln);
+    else e = launch_tile<T, D, RPT, kStats>(sh, d_reqs, q, k, scores, stats, exps, slabs, slab_keys, u0, heads, ln);
+    if (e != cudaSuccess) return e;
+    e = launch_chained(merge_kernel, dim3(heads, (R + 31) / 32), dim3(kThreads), 0, ln.stream, stats, slabs, R);
+    ln.done("score_simt_merge");
+    if (e != cudaSuccess) return e;
+    if (store) {
+      e = launch_chained(colsum_kernel, dim3(static_cast<unsigned>(slabs) * heads), dim3(kThreads), sizeof(float) * R, ln.stream, sh,
+                         d_reqs, scores, stats, exps, slabs, u0);
+      ln.done("score_simt_colsum");
+    } else {
+      e = launch_tile<T, D, RPT, kColsum>(sh, d_reqs, q, k, scores, stats, exps, slabs, slab_keys, u0, heads, ln);
+    }
+  }
+  return e;
+}
+
+// Rows per thread: the tile height that leaves the fewest padding rows, the larger one on a tie.
 template <typename T, int D>
-cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores,
-                         float2* stats_ws, int n_slab, int slab_keys, Launch ln) {
+cudaError_t launch_rows(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
+                        int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln) {
   const int R = sh.window * sh.group;
-  const int rows_extra = R > 4 * kTile ? R : 4 * kTile;
-  size_t smem = sizeof(float) * (2 * kTile * (D + 4) + kTile * (kTile + 1) + R + rows_extra);
-  auto k1 = score_simt_kernel<T, D, 1>;
-  auto k2 = score_simt_kernel<T, D, 2>;
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  if (static_cast<int64_t>(n_slab) * sh.total_heads > 0x7fffffffLL) return cudaErrorNotSupported;
-  dim3 grid(static_cast<unsigned>(n_slab) * static_cast<unsigned>(sh.total_heads));
-  k1<<<grid, kThreads, smem, ln.stream>>>(sh, d_reqs, (const T*)q, (const T*)k, scores, stats_ws, n_slab, slab_keys);
-  ln.done("score_simt_stats");
-  k2<<<grid, kThreads, smem, ln.stream>>>(sh, d_reqs, (const T*)q, (const T*)k, scores, stats_ws, n_slab, slab_keys);
-  ln.done("score_simt_colsum");
-  return cudaGetLastError();
+  auto padded = [R](int rows) { return (R + rows - 1) / rows * rows; };
+  if (R <= 64) return launch_typed<T, D, 4>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln);
+  if (padded(112) < padded(128)) return launch_typed<T, D, 7>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln);
+  return launch_typed<T, D, 8>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln);
 }
 
 }  // namespace
 
+int64_t score_simt_exps_len(int total_heads, int max_L, int rows) {
+  constexpr int64_t kRoom = (128LL << 20) / sizeof(float);
+  const int64_t per_head = static_cast<int64_t>((max_L + kKeys - 1) / kKeys) * kKeys * rows;
+  if (per_head > kRoom) return 0;
+  const int64_t heads = kRoom / per_head < total_heads ? kRoom / per_head : total_heads;
+  // chunks of equal size
+  const int64_t n_chunks = (total_heads + heads - 1) / heads;
+  return (total_heads + n_chunks - 1) / n_chunks * per_head;
+}
+int score_simt_tile_keys() { return kKeys; }
+
 cudaError_t launch_score_simt(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores,
-                              float2* stats_ws, int n_slab, int slab_keys, Launch ln) {
-#define AKV_CASE(T, D) return launch_typed<T, D>(sh, d_reqs, q, k, scores, stats_ws, n_slab, slab_keys, ln)
+                              float2* stats_ws, int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln) {
+#define AKV_CASE(T, D) return launch_rows<T, D>(sh, d_reqs, q, k, scores, stats_ws, n_slab, slab_keys, exps, exps_len, max_L, ln)
   if (sh.dtype == AUDIOKV_F32) {
     if (sh.head_dim == 64) AKV_CASE(float, 64);
     if (sh.head_dim == 128) AKV_CASE(float, 128);
@@ -367,6 +555,6 @@ extern "C" int audiokv_score_noalloc(int device, const audiokv_params* p, const 
   // Sweep 1 writes every statistics entry that sweep 2 reads, so nothing has to start at zero.
   cudaError_t e = launch_score_simt(sh, static_cast<const ReqDesc*>(base), q_win, k, scores,
                                     reinterpret_cast<float2*>(static_cast<unsigned char*>(base) + kNoAllocTableBytes),
-                                    n_slab, kSlabKeys, ln);
+                                    n_slab, kSlabKeys, nullptr, 0, max_L, ln);
   return e == cudaSuccess ? AUDIOKV_OK : AUDIOKV_ECUDA;
 }

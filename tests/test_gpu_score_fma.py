@@ -1,0 +1,91 @@
+"""The fp32 scoring kernels at the sizes where they can go wrong: key tiles of 64 and their remainders, every height of the row
+tile and its remainders, requests of different lengths in one launch, both element types, and both routes: exponentials
+kept (chunks of heads), and the product done twice (a head too long to be kept; the entry point with fixed scratch).
+
+Bound: a logit is a sum of d products in fp32, off by at most d 2^-24 of sum_t |q_t k_t| scale, about 0.64 sqrt(d) for normal
+q and k; half as much again for the fluctuation of that sum, and twice (the row's normaliser is as far off). The exponentials
+and the sums over at most 1024 rows add 2^-19."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2604_06694_b200 import workloads as wl
+from helpers import oracle_scores, rel_err, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2604_06694_b200 import build as akv_build
+    akv_build.build()
+    from paper_2604_06694_b200 import binding
+    return binding
+
+
+def _bound(d):
+    return 2 * 1.5 * d * 2.0 ** -24 * 0.64 * np.sqrt(d) + 2.0 ** -19
+
+
+def _check(w, g):
+    assert np.isfinite(g).all()
+    off = 0
+    for r in range(len(w.spec.seq_lens)):
+        o, _ = oracle_scores(w, r)
+        gr = g[off:off + o.size].reshape(o.shape)
+        off += o.size
+        for l in range(o.shape[0]):
+            for h in range(o.shape[1]):
+                assert rel_err(gr[l, h], o[l, h]) <= _bound(w.spec.head_dim), (r, l, h)
+    assert off == g.size
+
+
+# (window, query heads per KV head): W * G = 1, 15, 16, 63, 64, 65, 112, 113, 128, 129, 224, 225, 1024
+ROWS = [(1, 1), (5, 3), (16, 1), (9, 7), (32, 2), (13, 5), (16, 7), (113, 1), (32, 4), (43, 3), (32, 7), (45, 5), (128, 8)]
+
+
+@pytest.mark.parametrize("W,G", ROWS)
+@pytest.mark.parametrize("d", [64, 128, 256])
+def test_score_f32_rows(B, W, G, d):
+    lens = [W + 1, W + 63, W + 64, 65, 128, 129, 300]
+    lens = [max(W + 1, L) for L in lens]
+    w = wl.generate(wl.WorkloadSpec("fma", "f32", 1, 2 * G, 2, d, lens, [0.8] * len(lens), 0, window=W), seed=W * G + d)
+    prob = B.Problem.from_workload(w)
+    ctx = B.Context(prob)
+    scores = torch.full((B.audiokv_scores_len(prob),), float("nan"), device="cuda")
+    B.audiokv_score(ctx, prob, to_dev(w, w.q), to_dev(w, w.k), scores)
+    torch.cuda.synchronize()
+    assert ctx.last_score_path() == "fma" and ctx.last_device_status() == 0
+    _check(w, scores.cpu().numpy())
+
+
+def test_score_f32_chunks_of_heads(B):
+    """Seven heads of 13 MB of exponentials each fit the room of one launch; forty take several."""
+    w = wl.generate(wl.WorkloadSpec("fma", "f32", 10, 28, 4, 64, [3700], [0.8], 0, window=32), seed=4)
+    prob = B.Problem.from_workload(w)
+    ctx = B.Context(prob)
+    scores = torch.full((B.audiokv_scores_len(prob),), float("nan"), device="cuda")
+    B.audiokv_score(ctx, prob, to_dev(w, w.q), to_dev(w, w.k), scores)
+    torch.cuda.synchronize()
+    _check(w, scores.cpu().numpy())
+
+
+def test_score_f32_head_too_long_to_keep(B):
+    """W * G = 1024 and 33000 keys: 135 MB of exponentials for one head, so the product is done twice."""
+    w = wl.generate(wl.WorkloadSpec("fma", "f32", 1, 8, 1, 64, [33000], [0.8], 0, window=128), seed=6)
+    prob = B.Problem.from_workload(w)
+    ctx = B.Context(prob)
+    scores = torch.full((B.audiokv_scores_len(prob),), float("nan"), device="cuda")
+    B.audiokv_score(ctx, prob, to_dev(w, w.q), to_dev(w, w.k), scores)
+    torch.cuda.synchronize()
+    _check(w, scores.cpu().numpy())
+
+
+@pytest.mark.parametrize("dtype,W,G,d", [("f32", 32, 7, 128), ("bf16", 32, 7, 128), ("bf16", 9, 7, 64), ("bf16", 33, 4, 256)])
+def test_score_noalloc_tiles(B, dtype, W, G, d):
+    w = wl.generate(wl.WorkloadSpec("fma", dtype, 2, 2 * G, 2, d, [W + 1, 511, 512, 513, 1100], [0.8] * 5, 0, window=W), seed=9)
+    prob = B.Problem.from_workload(w)
+    scores = torch.full((B.audiokv_scores_len(prob),), float("nan"), device="cuda")
+    B.audiokv_score_noalloc(prob, to_dev(w, w.q), to_dev(w, w.k), scores)
+    torch.cuda.synchronize()
+    _check(w, scores.cpu().numpy())
