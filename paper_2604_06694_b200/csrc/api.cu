@@ -478,8 +478,8 @@ int build_plan(const audiokv_params* p, Plan* pl) {
     const int rows = sh.window * sh.group;
     size_t entries = static_cast<size_t>(sh.total_heads) * std::max<size_t>(pl->n_slab, static_cast<size_t>(pl->score_parts) * score_stat_sets()) * rows;
     // the FMA kernels keep a chunk's exponentials when they are the ones that score (see score_simt.cu)
-    pl->exps_len = score_umma_takes(sh) ? 0 : score_simt_exps_len(sh.total_heads, pl->max_L, rows);
-    entries = std::max(entries, static_cast<size_t>(pl->exps_len / score_simt_tile_keys()));
+    pl->exps_len = score_umma_takes(sh) ? 0 : score_simt_exps_len(sh.total_heads, pl->max_L, rows, sh.head_dim);
+    entries = std::max(entries, static_cast<size_t>(pl->exps_len / score_simt_tile_keys(sh.head_dim)));
     L.stats = off;     off = align_up(off + sizeof(float2) * entries);
   }
   L.exps = off;        off = align_up(off + sizeof(float) * static_cast<size_t>(pl->exps_len));

@@ -9,24 +9,25 @@
 // the sum kernel adds exp2(m + c) exp2(z - m) over the rows of every key, a stream at memory speed. Heads go through in
 // chunks of up to 128 MB of exponentials. A head too long for the chunk's room, and the entry point with fixed
 // scratch, run the product twice: statistics, merge, column sums.
-// The product is a register-tiled matrix product: 64 keys x 64, 112 or 128 query rows a block of 128 threads, 8 x 4, 7 or 8
-// logits a thread, panels of 32 dimensions through three stages of asynchronous copies, two blocks an SM. A logit is kept as
-// a pair, the sums over its even and its odd dimensions, so that packed FMAs take their operands as they lie in shared
-// memory: per four dimensions a thread reads 8 + 7 16-byte pieces (15 cycles of shared memory a warp) for 112 packed FMAs. (With
-// scalar FMAs on 8 x 7 single sums the pipe was 49 % busy, held up by dispatch stalls of three-operand reads: 139 us for
-// a chunk of 16 heads at 4096 keys.) The 64 x 64 tiles of 4 x 4 logits that were here first, with the tile's logits through
-// shared memory and the product done twice, took 1487 + 1234 us on that shape.
+// The product is a register-tiled matrix product, 8 keys x 4, 7 or 8 query rows a thread. The tile's keys lie transposed in shared
+// memory for as long as the tile lasts, two neighbouring keys make a packed pair of accumulators, and the query rows
+// come in panels of 32 dimensions by asynchronous copies, the next one under the arithmetic of this one, across row tiles.
+// 128 registers, 16 warps an SM: 191 us for 28 heads at 4096 keys (the FMA pipe 61 % busy by its counter, its throttle the
+// first stall). What was tried on the way on that launch: scalar FMAs in this layout 217 us, in rows of either side 240 us, held up by
+// dispatch stalls of three-operand reads; pairs of even and odd dimensions 218 us, and 201 us with half the address
+// arithmetic: twice the accumulators leave two warps a scheduler, which do not cover their latencies. The 64 x 64 tiles of 4 x 4
+// logits that were here first, with the logits through shared memory and the product done twice, took 1487 + 1234 us for 112 heads.
 // Logits are kept in base 2 (scale * log2 e folded into one multiply).
 #include "common.cuh"
 
 namespace akv {
 namespace {
 
-constexpr int kKeys = 64;            // keys per tile
-constexpr int kTileThreads = 128;    // 8 x 16 threads: keys x rows
-constexpr int kThreads = 256;        // of the merge and the sum kernel
-constexpr int kPanel = 32;     // dimensions per stage
-constexpr int kStages = 3;
+constexpr int kThreads = 256;  // of the merge and the sum kernel
+constexpr int kPanel = 32;     // dimensions per stage of query rows
+constexpr int kStages = 2;
+// Keys per tile: 64 KB of shared memory (32 KB at head_dim 64) with two blocks an SM.
+__host__ __device__ constexpr int tile_keys(int head_dim) { return head_dim == 256 ? 64 : 128; }
 
 struct HeadCoord {
   int r, l, h;
@@ -40,63 +41,60 @@ __device__ __forceinline__ HeadCoord head_coord(const Shape& sh, int u) {
   return c;
 }
 
-// A panel row in shared memory: 32 elements and 16 bytes of padding, which puts eight neighbouring rows' 16-byte pieces
-// on different banks.
-template <typename T>
-struct PanelRow {
-  static constexpr int kBytes = kPanel * static_cast<int>(sizeof(T)) + 16;
-};
 typedef unsigned long long f32x2;
-struct Piece {
-  f32x2 lo, hi;  // dimensions t, t + 1 and t + 2, t + 3
-};
-__device__ __forceinline__ f32x2 pair_of(uint32_t a, uint32_t b) {
+__device__ __forceinline__ f32x2 pair_of(float a, float b) {
   f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
   return r;
 }
+__device__ __forceinline__ void unpack(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   f32x2 d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-__device__ __forceinline__ float pair_sum(f32x2 v) {
-  float a, b;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-  return a + b;
+// Four elements as fp32, from shared or global memory.
+__device__ __forceinline__ float4 four(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 four(const __nv_bfloat16* p) {
+  const uint2 raw = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u), __uint_as_float(raw.y << 16),
+                     __uint_as_float(raw.y & 0xffff0000u));
 }
-__device__ __forceinline__ Piece piece(const unsigned char* row, int t, float) {
-  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(row + t * 4);
-  return Piece{v.x, v.y};
+// 16 bytes to shared memory without passing through registers.
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-__device__ __forceinline__ Piece piece(const unsigned char* row, int t, __nv_bfloat16) {
-  const uint2 raw = *reinterpret_cast<const uint2*>(row + t * 2);
-  return Piece{pair_of(raw.x << 16, raw.x & 0xffff0000u), pair_of(raw.y << 16, raw.y & 0xffff0000u)};
-}
-// 16 bytes to shared memory without passing through registers; zeros when `ok` is false (nothing is read then).
-__device__ __forceinline__ void copy16(void* dst, const void* src, bool ok) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src),
-               "r"(ok ? 16 : 0)
-               : "memory");
+// 2^x; arguments are at most 0, and what lies below 2^-126 of a row's maximum counts as nothing
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 enum { kStore = 0, kStats = 1, kColsum = 2 };
 
-constexpr int tile_smem_bytes(int rpt, int esize) {
-  return kStages * (kKeys + 16 * rpt) * (kPanel * esize + 16) + (kKeys + 16 * rpt) * static_cast<int>(sizeof(long long));
+// A panel row in shared memory: 32 elements and 16 bytes of padding, which puts neighbouring rows' 16-byte pieces on
+// different banks.
+constexpr int panel_row_bytes(int esize) { return kPanel * esize + 16; }
+constexpr int tile_smem_bytes(int d, int rpt, int esize, int rows) {
+  return tile_keys(d) * d * 4 + kStages * 16 * rpt * panel_row_bytes(esize) + (rows + 16 * rpt) * static_cast<int>(sizeof(void*));
 }
 
 // MODE kStore: one tile of keys per slab; its exponentials and row statistics. kStats: row statistics of a slab. kColsum: column
 // sums of a slab's prefix keys, the rows' c given (see merge_kernel). Heads u0, u0 + 1, ...; statistics of head u at u - u0.
 template <typename T, int D, int RPT, int MODE>
-__global__ void __launch_bounds__(kTileThreads, 2)
+__global__ void __launch_bounds__(2 * tile_keys(D), 2)
 score_tile_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const T* __restrict__ q, const T* __restrict__ k,
                   float* __restrict__ scores, float2* __restrict__ stats, float* __restrict__ exps, int n_slab, int slab_keys,
                   int u0) {
-  constexpr int kRows = 16 * RPT, kRowBytes = PanelRow<T>::kBytes, kStage = (kKeys + kRows) * kRowBytes;
+  constexpr int kKeys = tile_keys(D), kThr = 2 * kKeys, kTx = kKeys / 8, kRows = 16 * RPT;
+  constexpr int kRowBytes = panel_row_bytes(static_cast<int>(sizeof(T))), kStage = kRows * kRowBytes;
   constexpr int kPieces = kPanel * static_cast<int>(sizeof(T)) / 16;  // 16-byte pieces of a panel row
+  constexpr int kPanels = D / kPanel;
   extern __shared__ __align__(16) unsigned char smem[];
-  long long* off = reinterpret_cast<long long*>(smem + kStages * kStage);  // element offsets of the tile's rows, -1: zeros
+  float* kt_s = reinterpret_cast<float*>(smem);               // [D][kKeys]: the tile's keys, transposed
+  unsigned char* q_s = smem + kKeys * D * 4;                  // kStages panels of query rows
+  const T** rows = reinterpret_cast<const T**>(q_s + kStages * kStage);  // the head's query rows, whole row tiles
 
   chain_release();
   chain_wait();  // the request table may be the work of the kernel before
@@ -104,97 +102,125 @@ score_tile_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const T* __restric
   const HeadCoord hc = head_coord(sh, u);
   const ReqDesc rq = reqs[hc.r];
   const int R = sh.window * sh.group, G = sh.group;
-  const int ty = threadIdx.x >> 3, tx = threadIdx.x & 7;  // this thread's rows ty + 16 a and keys tx + 8 b
+  const int ty = threadIdx.x / kTx, tx = threadIdx.x % kTx;  // rows ty + 16 a; keys 4 tx .. + 3 of either half of the tile
   const int j0 = slab * slab_keys;
   const int j1 = min(MODE == kColsum ? rq.P : rq.L, j0 + slab_keys);  // column sums: prefix keys only
   float2* my_stats = stats + (static_cast<int64_t>(uc) * n_slab + slab) * R;
   const T* kbase = k + hc.l * sh.kv_stride_layer + hc.h * sh.kv_stride_head;  // the token term: kv_token_offset
   const T* qbase = q + rq.q_offset + hc.l * sh.q_stride_layer + static_cast<int64_t>(hc.h) * G * sh.q_stride_head;
+  if (j0 >= j1) {  // no keys of this request here
+    if (MODE != kColsum)
+      for (int r = threadIdx.x; r < R; r += kThr) my_stats[r] = make_float2(-INFINITY, 0.f);
+    return;
+  }
+  const int n_rt = (R + kRows - 1) / kRows;  // row tiles; rows past the end repeat the last one, their logits are dropped
+  for (int i = threadIdx.x; i < n_rt * kRows; i += kThr) {
+    const int rr = min(i, R - 1), w = rr / G;
+    rows[i] = qbase + w * sh.q_stride_tok + (rr - w * G) * sh.q_stride_head;
+  }
 
-  // acc[a][b] = <Q row rc + ty + 16 a, K row kt + tx + 8 b>
-  auto product = [&](float (&acc)[RPT][8], int kt, int rc) {
-    __syncthreads();  // the panels and offsets of the product before are free
-    for (int i = threadIdx.x; i < kKeys + kRows; i += kTileThreads) {
-      long long o = -1;
-      if (i < kKeys) {
-        if (kt + i < j1) o = kv_token_offset(sh, rq, hc.r, kt + i);
-      } else {
-        const int rr = rc + i - kKeys;
-        if (rr < R) o = rr / G * sh.q_stride_tok + rr % G * sh.q_stride_head;
+  const uint32_t q_smem = static_cast<uint32_t>(__cvta_generic_to_shared(q_s));
+  // Panel g of the query rows (row tile g / kPanels, dimensions 32 (g % kPanels) ..) into stage g % 2.
+  auto load_q = [&](int g) {
+    const int rt = g / kPanels, p = g - rt * kPanels;
+    const int my_row = threadIdx.x / kPieces, from = p * (kPanel * static_cast<int>(sizeof(T))) + threadIdx.x % kPieces * 16;
+    const uint32_t to = q_smem + (g & 1) * kStage + my_row * kRowBytes + threadIdx.x % kPieces * 16;
+    constexpr int kStep = kThr / kPieces;  // rows per turn
+#pragma unroll
+    for (int i = 0; i < (kRows + kStep - 1) / kStep; ++i)
+      if (kRows % kStep == 0 || my_row + i * kStep < kRows)
+        copy16(to + i * kStep * kRowBytes, reinterpret_cast<const unsigned char*>(rows[rt * kRows + my_row + i * kStep]) + from);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // Keys kt .. of the tile into shared memory, transposed: a lane holds a key, so that the stores run along the banks.
+  // Keys past the end repeat the last one: their logits are masked or dropped.
+  auto load_k = [&](int kt) {
+    const int key = threadIdx.x % kKeys, c0 = threadIdx.x / kKeys;  // pieces of four dimensions: c0, c0 + 2, ...
+    const T* src = kbase + kv_token_offset(sh, rq, hc.r, min(kt + key, j1 - 1));
+#pragma unroll 1
+    for (int c = c0; c < D / 4; c += 16) {
+      float4 v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = four(src + 4 * (c + 2 * i));
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float* dst = kt_s + 4 * (c + 2 * i) * kKeys + key;
+        dst[0] = v[i].x;
+        dst[kKeys] = v[i].y;
+        dst[2 * kKeys] = v[i].z;
+        dst[3 * kKeys] = v[i].w;
       }
-      off[i] = o;
     }
-    __syncthreads();
-    auto load = [&](int p) {  // panel p into stage p % kStages
-      unsigned char* st = smem + p % kStages * kStage;
-#pragma unroll 4
-      for (int i = threadIdx.x; i < (kKeys + kRows) * kPieces; i += kTileThreads) {
-        const int row = i / kPieces, c = i - row * kPieces;
-        const long long o = off[row];
-        const T* src = (row < kKeys ? kbase : qbase) + (o < 0 ? 0 : o) + p * kPanel + c * (16 / static_cast<int>(sizeof(T)));
-        copy16(st + row * kRowBytes + c * 16, src, o >= 0);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    f32x2 sum[RPT][8];
+  };
+  // acc[a][b] = <Q row ty + 16 a of row tile rt, key b of this thread>; the first panel of the row tile is on its way, and the
+  // first of row tile `next` (if not negative) is when this returns.
+  f32x2 sum[RPT][4];
+  float acc[8];
+  auto product = [&](int rt, int next) {
 #pragma unroll
     for (int a = 0; a < RPT; ++a)
 #pragma unroll
-      for (int b = 0; b < 8; ++b) sum[a][b] = 0ull;
-    constexpr int kPanels = D / kPanel;
-    load(0);
-    load(1);
+      for (int b = 0; b < 4; ++b) sum[a][b] = 0ull;
 #pragma unroll 1
     for (int p = 0; p < kPanels; ++p) {
-      if (p + 1 < kPanels) asm volatile("cp.async.wait_group 1;" ::: "memory");
-      else asm volatile("cp.async.wait_group 0;" ::: "memory");
-      __syncthreads();  // panel p is complete; everybody is done with panel p - 1
-      if (p + 2 < kPanels) load(p + 2);
-      const unsigned char* st = smem + p % kStages * kStage;
-      const unsigned char* kr = st + tx * kRowBytes;
-      const unsigned char* qr = st + (kKeys + ty) * kRowBytes;
-#pragma unroll(sizeof(T) == 4 ? 2 : 1)
+      const int g = rt * kPanels + p;
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();  // panel g (and the keys) are in place; everybody is done with panel g - 1
+      if (p + 1 < kPanels) load_q(g + 1);
+      else if (next >= 0) load_q(next * kPanels);  // the stages alternate: kPanels is even
+      const unsigned char* qr = q_s + (g & 1) * kStage + ty * kRowBytes;
+      const float* kr = kt_s + p * kPanel * kKeys + 4 * tx;
+#pragma unroll 1
       for (int t = 0; t < kPanel; t += 4) {
-        Piece kv[8];
+        float4 qv[RPT];
 #pragma unroll
-        for (int b = 0; b < 8; ++b) kv[b] = piece(kr + 8 * b * kRowBytes, t, T());
+        for (int a = 0; a < RPT; ++a) qv[a] = four(reinterpret_cast<const T*>(qr + 16 * a * kRowBytes) + t);
 #pragma unroll
-        for (int a = 0; a < RPT; ++a) {
-          const Piece qv = piece(qr + 16 * a * kRowBytes, t, T());
+        for (int i = 0; i < 4; ++i) {
+          const ulonglong2 k0 = *reinterpret_cast<const ulonglong2*>(kr + (t + i) * kKeys);
+          const ulonglong2 k1 = *reinterpret_cast<const ulonglong2*>(kr + (t + i) * kKeys + kKeys / 2);
 #pragma unroll
-          for (int b = 0; b < 8; ++b) {
-            sum[a][b] = fma2(qv.lo, kv[b].lo, sum[a][b]);
-            sum[a][b] = fma2(qv.hi, kv[b].hi, sum[a][b]);
+          for (int a = 0; a < RPT; ++a) {
+            const float s = i == 0 ? qv[a].x : i == 1 ? qv[a].y : i == 2 ? qv[a].z : qv[a].w;
+            const f32x2 s2 = pair_of(s, s);
+            sum[a][0] = fma2(s2, k0.x, sum[a][0]);
+            sum[a][1] = fma2(s2, k0.y, sum[a][1]);
+            sum[a][2] = fma2(s2, k1.x, sum[a][2]);
+            sum[a][3] = fma2(s2, k1.y, sum[a][3]);
           }
         }
       }
     }
-#pragma unroll
-    for (int a = 0; a < RPT; ++a)
-#pragma unroll
-      for (int b = 0; b < 8; ++b) acc[a][b] = pair_sum(sum[a][b]);
   };
-  float acc[RPT][8];
+  auto row_logits = [&](int a) {
+#pragma unroll
+    for (int b = 0; b < 4; ++b) unpack(sum[a][b], acc[2 * b], acc[2 * b + 1]);
+  };
+  auto key_of = [&](int b) { return (b >> 2) * (kKeys / 2) + 4 * tx + (b & 3); };
+  __syncthreads();  // the row pointers are in place
+  load_q(0);
   if constexpr (MODE == kColsum) {
     const float2* hs = stats + static_cast<int64_t>(uc) * n_slab * R;  // c of row r: .y of the head's first slab
     for (int kt = j0; kt < j1; kt += kKeys) {
+      load_k(kt);
       float col[8];
 #pragma unroll
       for (int b = 0; b < 8; ++b) col[b] = 0.f;
-      for (int rc = 0; rc < R; rc += kRows) {
-        product(acc, kt, rc);
+      for (int rt = 0; rt < n_rt; ++rt) {
+        product(rt, rt + 1 < n_rt ? rt + 1 : kt + kKeys < j1 ? 0 : -1);
 #pragma unroll
         for (int a = 0; a < RPT; ++a) {
-          const int rr = rc + ty + 16 * a;
+          const int rr = rt * kRows + ty + 16 * a;
           const float c = rr < R ? hs[rr].y : -INFINITY;
+          row_logits(a);
 #pragma unroll
-          for (int b = 0; b < 8; ++b) col[b] += exp2f(fmaf(acc[a][b], sh.scale_log2e, c));
+          for (int b = 0; b < 8; ++b) col[b] += ex2(fmaf(acc[b], sh.scale_log2e, c));
         }
       }
-      __syncthreads();  // the panels make room for the sums of the 16 thread rows
-      float* red = reinterpret_cast<float*>(smem);
+      __syncthreads();  // the keys make room for the sums of the 16 thread rows
+      float* red = kt_s;
 #pragma unroll
-      for (int b = 0; b < 8; ++b) red[ty * kKeys + tx + 8 * b] = col[b];
+      for (int b = 0; b < 8; ++b) red[ty * kKeys + key_of(b)] = col[b];
       __syncthreads();
       if (threadIdx.x < kKeys && kt + static_cast<int>(threadIdx.x) < j1) {
         float s = 0.f;
@@ -202,9 +228,11 @@ score_tile_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const T* __restric
         for (int y = 0; y < 16; ++y) s += red[y * kKeys + threadIdx.x];
         scores[rq.score_offset + (static_cast<int64_t>(hc.l) * sh.n_kv_heads + hc.h) * rq.P + kt + threadIdx.x] = s;
       }
+      __syncthreads();  // and the sums for the next keys
     }
   } else {
-    for (int rc = 0; rc < R; rc += kRows) {
+    if (MODE == kStore) load_k(j0);
+    for (int rt = 0; rt < n_rt; ++rt) {
       float m[RPT], Z[RPT];
 #pragma unroll
       for (int a = 0; a < RPT; ++a) {
@@ -212,54 +240,60 @@ score_tile_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const T* __restric
         Z[a] = 0.f;
       }
       for (int kt = j0; kt < j1; kt += kKeys) {
-        product(acc, kt, rc);
+        if (MODE == kStats) {
+          __syncthreads();  // everybody is done with the keys before
+          load_k(kt);
+        }
+        product(rt, kt + kKeys < j1 ? rt : rt + 1 < n_rt ? rt + 1 : -1);
+        const bool masked = kt + kKeys > min(j1, rq.P + 1);  // the tile reaches past the keys or into the window: causal mask
 #pragma unroll
         for (int a = 0; a < RPT; ++a) {
-          const int rr = rc + ty + 16 * a;
-          const int last = min(j1 - 1, rq.P + rr / G) - kt;  // last visible key of this row in the tile
-          float top = -INFINITY;
+          const int rr = rt * kRows + ty + 16 * a;
+          row_logits(a);
+          if (masked) {
+            const int last = min(j1 - 1, rq.P + rr / G) - kt;  // last visible key of this row
 #pragma unroll
-          for (int b = 0; b < 8; ++b) {
-            acc[a][b] = tx + 8 * b <= last ? acc[a][b] * sh.scale_log2e : -INFINITY;
-            top = fmaxf(top, acc[a][b]);
+            for (int b = 0; b < 8; ++b) acc[b] = key_of(b) <= last ? acc[b] : -INFINITY;
           }
+          float top = acc[0];
+#pragma unroll
+          for (int b = 1; b < 8; ++b) top = fmaxf(top, acc[b]);
           if (MODE == kStore) {  // one reference for the row's keys of the tile
 #pragma unroll
-            for (int o = 1; o < 8; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+            for (int o = 1; o < kTx; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
           }
-          const float ref = fmaxf(m[a], top);
+          const float ref = fmaxf(m[a], top * sh.scale_log2e);
           const float safe = ref == -INFINITY ? 0.f : ref;  // nothing visible yet: the exponentials are zeros
           float s = 0.f;
 #pragma unroll
           for (int b = 0; b < 8; ++b) {
-            acc[a][b] = exp2f(acc[a][b] - safe);
-            s += acc[a][b];
+            acc[b] = ex2(fmaf(acc[b], sh.scale_log2e, -safe));
+            s += acc[b];
           }
-          Z[a] = Z[a] * exp2f(m[a] - safe) + s;
+          Z[a] = MODE == kStore ? s : Z[a] * ex2(m[a] - safe) + s;  // kStore: one tile
           m[a] = ref;
-        }
-        if (MODE == kStore) {
-          float* e = exps + ((static_cast<int64_t>(uc) * n_slab + slab) * R) * kKeys;
-#pragma unroll
-          for (int a = 0; a < RPT; ++a) {
-            const int rr = rc + ty + 16 * a;
-            if (rr < R) {
-#pragma unroll
-              for (int b = 0; b < 8; ++b) e[static_cast<int64_t>(rr) * kKeys + tx + 8 * b] = acc[a][b];
-            }
+          if (MODE == kStore && rr < R) {
+            float* e = exps + ((static_cast<int64_t>(uc) * n_slab + slab) * R + rr) * kKeys + 4 * tx;
+            *reinterpret_cast<float4*>(e) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+            *reinterpret_cast<float4*>(e + kKeys / 2) = make_float4(acc[4], acc[5], acc[6], acc[7]);
           }
         }
       }
 #pragma unroll
       for (int a = 0; a < RPT; ++a) {
 #pragma unroll
-        for (int o = 1; o < 8; o <<= 1) {
-          const float mo = __shfl_xor_sync(0xffffffffu, m[a], o), zo = __shfl_xor_sync(0xffffffffu, Z[a], o);
-          const float mn = fmaxf(m[a], mo), safe = mn == -INFINITY ? 0.f : mn;
-          Z[a] = Z[a] * exp2f(m[a] - safe) + zo * exp2f(mo - safe);
-          m[a] = mn;
+        for (int o = 1; o < kTx; o <<= 1) {
+          const float zo = __shfl_xor_sync(0xffffffffu, Z[a], o);
+          if (MODE == kStore) {
+            Z[a] += zo;
+          } else {
+            const float mo = __shfl_xor_sync(0xffffffffu, m[a], o);
+            const float mn = fmaxf(m[a], mo), safe = mn == -INFINITY ? 0.f : mn;
+            Z[a] = Z[a] * ex2(m[a] - safe) + zo * ex2(mo - safe);
+            m[a] = mn;
+          }
         }
-        const int rr = rc + ty + 16 * a;
+        const int rr = rt * kRows + ty + 16 * a;
         if (tx == 0 && rr < R) my_stats[rr] = make_float2(m[a], Z[a]);
       }
     }
@@ -293,52 +327,53 @@ __global__ void __launch_bounds__(kThreads) merge_kernel(float2* __restrict__ st
   }
 }
 
-// Column sums from the stored exponentials: one block per tile. Half a warp reads one row (256 bytes) at a time.
+// Column sums from the stored exponentials: one block per tile; KEYS / 4 lanes read one row at a time.
+template <int KEYS>
 __global__ void __launch_bounds__(kThreads)
 colsum_kernel(Shape sh, const ReqDesc* __restrict__ reqs, float* __restrict__ scores, const float2* __restrict__ stats,
               const float* __restrict__ exps, int n_slab, int u0) {
   extern __shared__ __align__(16) unsigned char smem[];
   float* f = reinterpret_cast<float*>(smem);                   // [R] factor of every row
-  constexpr int kHalves = kThreads / 16;
-  __shared__ float4 red[kHalves][16];
+  constexpr int kLanes = KEYS / 4, kTurn = kThreads / kLanes;  // rows at a time
+  __shared__ float4 red[kTurn][kLanes];
   chain_release();
   chain_wait();
   const int uc = blockIdx.x / n_slab, slab = blockIdx.x - uc * n_slab, u = u0 + uc;
   const HeadCoord hc = head_coord(sh, u);
   const ReqDesc rq = reqs[hc.r];
-  const int R = sh.window * sh.group, j0 = slab * kKeys;
-  const int lane = threadIdx.x & 15, half = threadIdx.x >> 4;
+  const int R = sh.window * sh.group, j0 = slab * KEYS;
+  const int lane = threadIdx.x % kLanes, first = threadIdx.x / kLanes;
   if (j0 >= rq.P) return;
   const float2* hs = stats + static_cast<int64_t>(uc) * n_slab * R;
-  const float4* e = reinterpret_cast<const float4*>(exps + (static_cast<int64_t>(uc) * n_slab + slab) * R * kKeys) + lane;
+  const float4* e = reinterpret_cast<const float4*>(exps + (static_cast<int64_t>(uc) * n_slab + slab) * R * KEYS) + lane;
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   float4 v[8];
   auto fetch = [&](int r0) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = __ldcs(e + static_cast<int64_t>(min(r0 + i * kHalves, R - 1)) * (kKeys / 4));
+    for (int i = 0; i < 8; ++i) v[i] = __ldcs(e + static_cast<int64_t>(min(r0 + i * kTurn, R - 1)) * kLanes);
   };
-  fetch(half);  // the first rows run beside the factors' loads
+  fetch(first);  // the first rows run beside the factors' loads
   for (int r = threadIdx.x; r < R; r += kThreads) f[r] = exp2f(hs[static_cast<int64_t>(slab) * R + r].x + hs[r].y);
   __syncthreads();
-  for (int r0 = half; r0 < R;) {
+  for (int r0 = first; r0 < R;) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const float w = r0 + i * kHalves < R ? f[r0 + i * kHalves] : 0.f;
+      const float w = r0 + i * kTurn < R ? f[r0 + i * kTurn] : 0.f;
       s.x = fmaf(v[i].x, w, s.x);
       s.y = fmaf(v[i].y, w, s.y);
       s.z = fmaf(v[i].z, w, s.z);
       s.w = fmaf(v[i].w, w, s.w);
     }
-    r0 += 8 * kHalves;
+    r0 += 8 * kTurn;
     if (r0 < R) fetch(r0);
   }
-  red[half][lane] = s;
+  red[first][lane] = s;
   __syncthreads();
-  if (threadIdx.x < kKeys && j0 + static_cast<int>(threadIdx.x) < rq.P) {
+  if (threadIdx.x < KEYS && j0 + static_cast<int>(threadIdx.x) < rq.P) {
     const float* col = reinterpret_cast<const float*>(red) + threadIdx.x;
     float t = 0.f;
 #pragma unroll
-    for (int w = 0; w < kHalves; ++w) t += col[w * kKeys];
+    for (int w = 0; w < kTurn; ++w) t += col[w * KEYS];
     scores[rq.score_offset + (static_cast<int64_t>(hc.l) * sh.n_kv_heads + hc.h) * rq.P + j0 + threadIdx.x] = t;
   }
 }
@@ -347,24 +382,45 @@ template <typename T, int D, int RPT, int MODE>
 cudaError_t launch_tile(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
                         float* exps, int n_slab, int slab_keys, int u0, int heads, Launch ln) {
   auto kern = score_tile_kernel<T, D, RPT, MODE>;
-  const int smem = tile_smem_bytes(RPT, static_cast<int>(sizeof(T)));
+  const int smem = tile_smem_bytes(D, RPT, static_cast<int>(sizeof(T)), sh.window * sh.group);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  e = launch_chained(kern, dim3(static_cast<unsigned>(n_slab) * heads), dim3(kTileThreads), smem, ln.stream, sh, d_reqs,
+  e = launch_chained(kern, dim3(static_cast<unsigned>(n_slab) * heads), dim3(2 * tile_keys(D)), smem, ln.stream, sh, d_reqs,
                      static_cast<const T*>(q), static_cast<const T*>(k), scores, stats, exps, n_slab, slab_keys, u0);
   ln.done(MODE == kStore ? "score_simt_exps" : MODE == kStats ? "score_simt_stats" : "score_simt_colsum");
   return e;
 }
 
+// Heads of a chunk, at most `most`: as few waves of blocks over all chunks as possible, two blocks an SM, a chunk's three
+// launches counted as a third of a wave. (112 heads of 32 tiles: 28 heads a chunk are 3.03 waves, so four chunks of four,
+// 0.77 ms; 36 heads are 3.9, three chunks of four and one of one.)
+int heads_per_chunk(int most, int total, int tiles) {
+  const int64_t slots = 2LL * device_sm_count();
+  int best = most;
+  double cost = 1e30;
+  for (int h = most; h >= 1 && (h > most / 2 || h > most - 64); --h) {
+    const int full = total / h, rest = total - full * h;
+    const double c = full * (static_cast<double>((static_cast<int64_t>(h) * tiles + slots - 1) / slots) + 0.33) +
+                     (rest ? static_cast<double>((static_cast<int64_t>(rest) * tiles + slots - 1) / slots) + 0.33 : 0.0);
+    if (c < cost) {
+      cost = c;
+      best = h;
+    }
+  }
+  return best;
+}
+
 template <typename T, int D, int RPT>
 cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
                          int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln) {
+  constexpr int kKeys = tile_keys(D);
   const int R = sh.window * sh.group, n_tile = (max_L + kKeys - 1) / kKeys;
   const int64_t per_head = static_cast<int64_t>(n_tile) * R * kKeys;
   const bool store = exps != nullptr && per_head <= exps_len;
   const int slabs = store ? n_tile : n_slab;
   const int64_t room = store ? exps_len / per_head : 0x7fffffffLL / slabs;
-  const int chunk = static_cast<int>(room < sh.total_heads ? room : sh.total_heads);
+  const int chunk = store ? heads_per_chunk(static_cast<int>(room < sh.total_heads ? room : sh.total_heads), sh.total_heads, slabs)
+                          : static_cast<int>(room < sh.total_heads ? room : sh.total_heads);
   cudaError_t e = cudaSuccess;
   for (int u0 = 0; u0 < sh.total_heads && e == cudaSuccess; u0 += chunk) {
     const int heads = sh.total_heads - u0 < chunk ? sh.total_heads - u0 : chunk;
@@ -375,7 +431,7 @@ cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, 
     ln.done("score_simt_merge");
     if (e != cudaSuccess) return e;
     if (store) {
-      e = launch_chained(colsum_kernel, dim3(static_cast<unsigned>(slabs) * heads), dim3(kThreads), sizeof(float) * R, ln.stream, sh,
+      e = launch_chained(colsum_kernel<kKeys>, dim3(static_cast<unsigned>(slabs) * heads), dim3(kThreads), sizeof(float) * R, ln.stream, sh,
                          d_reqs, scores, stats, exps, slabs, u0);
       ln.done("score_simt_colsum");
     } else {
@@ -398,16 +454,15 @@ cudaError_t launch_rows(const Shape& sh, const ReqDesc* d_reqs, const void* q, c
 
 }  // namespace
 
-int64_t score_simt_exps_len(int total_heads, int max_L, int rows) {
+int score_simt_tile_keys(int head_dim) { return tile_keys(head_dim); }
+int64_t score_simt_exps_len(int total_heads, int max_L, int rows, int head_dim) {
   constexpr int64_t kRoom = (128LL << 20) / sizeof(float);
-  const int64_t per_head = static_cast<int64_t>((max_L + kKeys - 1) / kKeys) * kKeys * rows;
+  const int keys = tile_keys(head_dim);
+  const int64_t per_head = static_cast<int64_t>((max_L + keys - 1) / keys) * keys * rows;
   if (per_head > kRoom) return 0;
   const int64_t heads = kRoom / per_head < total_heads ? kRoom / per_head : total_heads;
-  // chunks of equal size
-  const int64_t n_chunks = (total_heads + heads - 1) / heads;
-  return (total_heads + n_chunks - 1) / n_chunks * per_head;
+  return heads * per_head;
 }
-int score_simt_tile_keys() { return kKeys; }
 
 cudaError_t launch_score_simt(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores,
                               float2* stats_ws, int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln) {
