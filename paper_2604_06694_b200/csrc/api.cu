@@ -18,16 +18,18 @@ constexpr size_t kAlign = 256;
 constexpr int kSlabKeys = 256;          // keys per slab of the softmax statistics (two K tiles of the tensor-core kernel)
 constexpr int kMaxRows = 1024;          // W * G
 constexpr int kMaxHeadsPerReq = 2048;
+constexpr size_t kStageBytes = 256 << 10;  // pinned staging of one plan upload
 constexpr int kHostChunks = 8;          // the host-buffer call evicts one request in at most this many runs of layers
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
-struct Layout {  // byte offsets inside the workspace
-  size_t status, reqs, plans, tables, units, ctas, order, stats, exps, fft_scratch, scores, kstar, aux, end;
+struct Layout {  // byte offsets inside the workspace; status .. order, up to blob_end, are uploaded as one piece with a plan
+  size_t status, reqs, plans, units, ctas, order, blob_end, tables, stats, exps, fft_scratch, scores, kstar, aux, end;
 };
 
 struct Plan {
   bool valid = false;
+  bool host_call = false;       // has the schedules of audiokv_evict_host
   audiokv_params p{};
   std::vector<int32_t> seq_len;
   std::vector<int64_t> kv_off, q_off;
@@ -67,6 +69,12 @@ struct audiokv_ctx {
   uint64_t plan_id = 0;      // counts plan rebuilds
   ScoreMapCache score_maps;
   cudaEvent_t plan_ready = nullptr;
+  cudaStream_t plan_stream = nullptr;     // where the plan went up
+  bool plan_settled = false;              // the upload was seen complete
+  static constexpr int kStageSlots = 4;
+  char* stage = nullptr;                  // pinned: kStageSlots x kStageBytes
+  cudaEvent_t stage_free[kStageSlots] = {};
+  std::vector<char> big_blob;
   cudaStream_t side = nullptr;            // audiokv_evict runs the allocation here, beside the scoring
   cudaEvent_t fork = nullptr, join = nullptr;
   // audiokv_evict_host: copies in on `side`, kernels on the caller's stream, copies out on `out`, chunk by chunk
@@ -214,14 +222,13 @@ void build_fft_plan(int n, FftPlan* fp, int64_t* table_len) {
     // convolution length: the smallest 2^a 3^b 5^c 7^d (a >= 2) that holds `need` points; close to it
     // instead of up to twice that for a power of two, which also keeps more transforms in shared memory
     int M = 0;
-    for (int64_t p7 = 1; p7 < 4LL * N; p7 *= 7)
-      for (int64_t p5 = p7; p5 < 4LL * N; p5 *= 5)
-        for (int64_t p3 = p5; p3 < 4LL * N; p3 *= 3)
-          for (int64_t p2 = p3 * 4; p2 < 8LL * N; p2 *= 2)
-            if (p2 >= need) {
-              if (M == 0 || p2 < M) M = static_cast<int>(p2);
-              break;
-            }
+    for (int64_t p7 = 4; M == 0 || p7 < M; p7 *= 7)
+      for (int64_t p5 = p7; M == 0 || p5 < M; p5 *= 5)
+        for (int64_t p3 = p5; M == 0 || p3 < M; p3 *= 3) {
+          int64_t p2 = p3;
+          while (p2 < need) p2 *= 2;
+          if (M == 0 || p2 < M) M = static_cast<int>(p2);
+        }
     fp->M = M;
     factor_len(M, &fp->seq);
   }
@@ -264,7 +271,7 @@ int host_chunk_layer(int n_layers, int c) { return static_cast<int>(static_cast<
 // runs of consecutive tiles of one head. Sweep 1 walks the heads in order over all L keys (the runs of a head number
 // its statistics slots); sweep 2 walks them backwards over the prefix keys (the heads sweep 1 touched last are the
 // ones still in L2).
-void build_score_schedules(const audiokv_params* p, Plan* pl) {
+void build_score_schedules(const audiokv_params* p, bool host_call, Plan* pl) {
   const Shape& sh = pl->sh;
   pl->units.clear();
   pl->score_ctas.clear();
@@ -348,7 +355,7 @@ void build_score_schedules(const audiokv_params* p, Plan* pl) {
   };
   const int cap = score_map_chunk(p->n_req);
   for (int r0 = 0; r0 < p->n_req; r0 += cap) add(true, r0, r0 + cap < p->n_req ? r0 + cap : p->n_req, 0, 0);
-  if (p->n_req == 1 && p->n_layers > 1) {
+  if (host_call && p->n_req == 1 && p->n_layers > 1) {
     // the host-buffer call evicts one request in chunks of layers
     const int n_chunks = host_chunks(p->n_layers);
     for (int c = 0; c < n_chunks; ++c)
@@ -356,7 +363,9 @@ void build_score_schedules(const audiokv_params* p, Plan* pl) {
   }
 }
 
-int build_plan(const audiokv_params* p, Plan* pl) {
+// host_call: with the schedules by chunks of layers that audiokv_evict_host runs through (eight more schedules of one request;
+// a serving loop whose every prompt brings a new length builds a plan a call, so the others go without).
+int build_plan(const audiokv_params* p, bool host_call, Plan* pl) {
   int rc = check_params(p);
   if (rc) return rc;
   pl->valid = false;
@@ -433,7 +442,8 @@ int build_plan(const audiokv_params* p, Plan* pl) {
     d.fft_plan = it->second;
   }
   pl->n_slab = (pl->max_L + kSlabKeys - 1) / kSlabKeys;
-  build_score_schedules(p, pl);
+  pl->host_call = host_call;
+  build_score_schedules(p, host_call, pl);
   // one block per head at a time, as many blocks as the planning SM count (the plan, and with it the workspace size,
   // does not depend on the device)
   pl->sss_grid = sh.total_heads < kScoreCtas ? sh.total_heads : kScoreCtas;
@@ -441,18 +451,20 @@ int build_plan(const audiokv_params* p, Plan* pl) {
     // Block b of the smoothing kernel takes entries b, b + grid, b + 2 grid, ... of this list. Heads are sorted by an
     // estimate of their transform's cost and dealt out in a snake (left to right, then right to left), so that
     // a ragged batch with a few expensive lengths (chirp-z in global scratch) does not leave them to one block.
-    auto cost = [&](int u) -> double {
-      const FftPlan& fp = pl->fft[pl->reqs[u / sh.heads_per_req].fft_plan];
+    auto cost = [&](int r) -> double {
+      const FftPlan& fp = pl->fft[pl->reqs[r].fft_plan];
       return seq_cost(fp.seq) * (fp.bluestein ? 2.0 : 1.0) * (fp.in_smem ? 1.0 : 1.5) + 8.0 * fp.n;
     };
-    std::vector<int32_t> by_cost(sh.total_heads);
-    for (int u = 0; u < sh.total_heads; ++u) by_cost[u] = u;
-    std::stable_sort(by_cost.begin(), by_cost.end(), [&](int a, int b) { return cost(a) > cost(b); });
+    // the heads of a request cost the same: the requests are sorted, and their heads follow in order
+    std::vector<std::pair<double, int32_t>> by_cost(p->n_req);
+    for (int r = 0; r < p->n_req; ++r) by_cost[r] = {cost(r), r};
+    std::stable_sort(by_cost.begin(), by_cost.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
     const int g = pl->sss_grid, tiers = (sh.total_heads + g - 1) / g;
     pl->sss_order.assign(static_cast<size_t>(tiers) * g, -1);
     for (int i = 0; i < sh.total_heads; ++i) {
       const int tier = i / g, j = i - tier * g;
-      pl->sss_order[static_cast<size_t>(tier) * g + ((tier & 1) ? g - 1 - j : j)] = by_cost[i];
+      pl->sss_order[static_cast<size_t>(tier) * g + ((tier & 1) ? g - 1 - j : j)] =
+          pl->reqs[by_cost[i / sh.heads_per_req].second].head_base + i % sh.heads_per_req;
     }
   }
   int smem_c = 64;
@@ -469,10 +481,11 @@ int build_plan(const audiokv_params* p, Plan* pl) {
   L.status = off;      off = align_up(off + 64);
   L.reqs = off;        off = align_up(off + sizeof(ReqDesc) * pl->reqs.size());
   L.plans = off;       off = align_up(off + sizeof(FftPlan) * pl->fft.size());
-  L.tables = off;      off = align_up(off + sizeof(float2) * static_cast<size_t>(pl->table_len));
   L.units = off;       off = align_up(off + sizeof(ScoreUnit) * pl->units.size());
   L.ctas = off;        off = align_up(off + sizeof(int32_t) * pl->score_ctas.size());
   L.order = off;       off = align_up(off + sizeof(int32_t) * pl->sss_order.size());
+  L.blob_end = off;
+  L.tables = off;      off = align_up(off + sizeof(float2) * static_cast<size_t>(pl->table_len));
   {
     // softmax statistics: [head][slab][row] for the FMA kernels, [head][part][group][row] for the tensor-core ones
     const int rows = sh.window * sh.group;
@@ -498,12 +511,12 @@ int cuda_fail(audiokv_ctx* ctx, cudaError_t e) {
 }
 
 // Makes ctx->plan match p and its tables resident on the device (stream-ordered).
-int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream) {
+int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool host_call = false) {
   if (!ctx) return AUDIOKV_EINVAL;
   cudaError_t e = cudaSetDevice(ctx->device);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
-  if (!same_plan(ctx->plan, p)) {
-    int rc = build_plan(p, &ctx->plan);
+  if (!same_plan(ctx->plan, p) || (host_call && !ctx->plan.host_call)) {
+    int rc = build_plan(p, host_call, &ctx->plan);
     ctx->plan_id += 1;
     if (rc) return rc;
     ctx->plan_uploaded = false;
@@ -521,33 +534,52 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream) {
       ctx->cuda_error = "the plan of these params is not on the device yet: make one call outside stream capture first";
       return AUDIOKV_ECUDA;
     }
-    // earlier calls on other streams may still read the old tables
-    if ((e = cudaStreamWaitEvent(stream, ctx->plan_ready, 0)) != cudaSuccess) return cuda_fail(ctx, e);
-    if ((e = cudaMemsetAsync(ctx->ws + pl.lay.status, 0, 64, stream)) != cudaSuccess) return cuda_fail(ctx, e);
-    if ((e = cudaMemcpyAsync(ctx->ws + pl.lay.reqs, pl.reqs.data(), sizeof(ReqDesc) * pl.reqs.size(),
-                             cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-      return cuda_fail(ctx, e);
-    if ((e = cudaMemcpyAsync(ctx->ws + pl.lay.plans, pl.fft.data(), sizeof(FftPlan) * pl.fft.size(),
-                             cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-      return cuda_fail(ctx, e);
-    if (!pl.units.empty() &&
-        ((e = cudaMemcpyAsync(ctx->ws + pl.lay.units, pl.units.data(), sizeof(ScoreUnit) * pl.units.size(),
-                              cudaMemcpyHostToDevice, stream)) != cudaSuccess ||
-         (e = cudaMemcpyAsync(ctx->ws + pl.lay.ctas, pl.score_ctas.data(), sizeof(int32_t) * pl.score_ctas.size(),
-                              cudaMemcpyHostToDevice, stream)) != cudaSuccess))
-      return cuda_fail(ctx, e);
-    if ((e = cudaMemcpyAsync(ctx->ws + pl.lay.order, pl.sss_order.data(), sizeof(int32_t) * pl.sss_order.size(),
-                             cudaMemcpyHostToDevice, stream)) != cudaSuccess)
-      return cuda_fail(ctx, e);
+    // The request table, FFT plans, schedules and order go up in one copy, and the status word starts clean with it. From
+    // pinned staging the host does not wait for it (a prompt of a new length then costs no round trip); a plan larger than
+    // a staging slot goes up from pageable memory, which does.
+    const size_t blob = pl.lay.blob_end;
+    const bool staged = blob <= kStageBytes;
+    char* src;
+    const int slot = static_cast<int>(ctx->plan_id % audiokv_ctx::kStageSlots);
+    if (staged) {
+      src = ctx->stage + slot * kStageBytes;
+      if ((e = cudaEventSynchronize(ctx->stage_free[slot])) != cudaSuccess) return cuda_fail(ctx, e);  // four plans ago
+    } else {
+      ctx->big_blob.resize(blob);
+      src = ctx->big_blob.data();
+    }
+    memset(src, 0, 64);
+    auto put = [&](size_t at, const void* data, size_t bytes) {
+      if (bytes) memcpy(src + at, data, bytes);
+    };
+    put(pl.lay.reqs, pl.reqs.data(), sizeof(ReqDesc) * pl.reqs.size());
+    put(pl.lay.plans, pl.fft.data(), sizeof(FftPlan) * pl.fft.size());
+    put(pl.lay.units, pl.units.data(), sizeof(ScoreUnit) * pl.units.size());
+    put(pl.lay.ctas, pl.score_ctas.data(), sizeof(int32_t) * pl.score_ctas.size());
+    put(pl.lay.order, pl.sss_order.data(), sizeof(int32_t) * pl.sss_order.size());
+    if ((e = cudaMemcpyAsync(ctx->ws, src, blob, cudaMemcpyHostToDevice, stream)) != cudaSuccess) return cuda_fail(ctx, e);
+    if (staged && (e = cudaEventRecord(ctx->stage_free[slot], stream)) != cudaSuccess) return cuda_fail(ctx, e);
     Launch ln{stream, &ctx->launches, &ctx->prof};
     e = launch_fft_tables(static_cast<int>(pl.fft.size()), reinterpret_cast<float2*>(ctx->ws + pl.lay.tables),
                           reinterpret_cast<const FftPlan*>(ctx->ws + pl.lay.plans), pl.sss_smem, ln);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
-    // The host waits until the plan is resident (once per shape): calls that follow, on any stream or inside a
-    // capture, then need no ordering against the upload.
     if ((e = cudaEventRecord(ctx->plan_ready, stream)) != cudaSuccess) return cuda_fail(ctx, e);
-    if ((e = cudaEventSynchronize(ctx->plan_ready)) != cudaSuccess) return cuda_fail(ctx, e);
+    ctx->plan_stream = stream;
+    ctx->plan_settled = false;
     ctx->plan_uploaded = true;
+  } else if (!ctx->plan_settled) {
+    // Calls on the stream of the upload are ordered behind it. On another stream, or inside a capture (which must not wait for
+    // an event from outside), the upload has to be complete: seen so once, no later call asks again.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if ((e = cudaStreamIsCapturing(stream, &cap)) != cudaSuccess) return cuda_fail(ctx, e);
+    if (stream != ctx->plan_stream || cap != cudaStreamCaptureStatusNone) {
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // the event is not the capture's: waiting for it is safe
+      if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return cuda_fail(ctx, e);
+      e = cudaEventSynchronize(ctx->plan_ready);
+      const cudaError_t e2 = cudaThreadExchangeStreamCaptureMode(&mode);
+      if (e != cudaSuccess || e2 != cudaSuccess) return cuda_fail(ctx, e != cudaSuccess ? e : e2);
+      ctx->plan_settled = true;
+    }
   }
   return AUDIOKV_OK;
 }
@@ -646,6 +678,30 @@ int do_select_gather(audiokv_ctx* ctx, const float* smoothed, const int32_t* bud
   return do_gather(ctx, cu_kept, kept_idx, k, v, k_out, v_out, stream);
 }
 
+// Where audiokv_evict_host keeps the device copies of its buffers: byte offsets behind the plan's own part of the workspace.
+struct HostStaging {
+  size_t q, k, v, head_scores, k_out, v_out, kept_idx, budgets, cu_kept, end;
+  int64_t rows;
+};
+HostStaging host_staging(const Plan& pl, int64_t q_elems, int64_t kv_elems, const int64_t* total_budget) {
+  HostStaging h{};
+  const size_t es = esize(pl.sh.dtype), TH = static_cast<size_t>(pl.sh.total_heads);
+  for (int r = 0; r < pl.sh.n_req; ++r) h.rows += total_budget[r];
+  const size_t row_bytes = static_cast<size_t>(h.rows) * pl.sh.head_dim * es;
+  size_t off = pl.lay.end;
+  h.q = off;           off = align_up(off + q_elems * es);
+  h.k = off;           off = align_up(off + kv_elems * es);
+  h.v = off;           off = align_up(off + kv_elems * es);
+  h.head_scores = off; off = align_up(off + sizeof(float) * TH);
+  h.k_out = off;       off = align_up(off + row_bytes);
+  h.v_out = off;       off = align_up(off + row_bytes);
+  h.kept_idx = off;    off = align_up(off + h.rows * sizeof(int32_t));
+  h.budgets = off;     off = align_up(off + sizeof(int32_t) * TH);
+  h.cu_kept = off;     off = align_up(off + sizeof(int32_t) * (TH + 1));
+  h.end = off;
+  return h;
+}
+
 }  // namespace
 
 extern "C" {
@@ -684,28 +740,15 @@ int64_t audiokv_scores_len(const audiokv_params* p) {
 
 size_t audiokv_workspace_bytes(const audiokv_params* p) {
   Plan pl;
-  if (build_plan(p, &pl)) return 0;
+  if (build_plan(p, true, &pl)) return 0;
   return pl.lay.end;
 }
 
 size_t audiokv_workspace_bytes_host(const audiokv_params* p, int64_t q_elems, int64_t kv_elems,
                                     const int64_t* total_budget) {
   Plan pl;
-  if (build_plan(p, &pl) || !total_budget || q_elems < 0 || kv_elems < 0) return 0;
-  const size_t es = esize(p->dtype);
-  int64_t rows = 0;
-  for (int r = 0; r < p->n_req; ++r) rows += total_budget[r];
-  size_t off = pl.lay.end;
-  off = align_up(off + q_elems * es);
-  off = align_up(off + kv_elems * es) ;
-  off = align_up(off + kv_elems * es);
-  off = align_up(off + sizeof(float) * pl.sh.total_heads);
-  off = align_up(off + rows * p->head_dim * es);
-  off = align_up(off + rows * p->head_dim * es);
-  off = align_up(off + rows * sizeof(int32_t));
-  off = align_up(off + sizeof(int32_t) * pl.sh.total_heads);
-  off = align_up(off + sizeof(int32_t) * (pl.sh.total_heads + 1));
-  return off;
+  if (build_plan(p, true, &pl) || !total_budget || q_elems < 0 || kv_elems < 0) return 0;
+  return host_staging(pl, q_elems, kv_elems, total_budget).end;
 }
 
 int audiokv_create(audiokv_ctx** out, int device, size_t workspace_bytes) {
@@ -736,7 +779,10 @@ int audiokv_create(audiokv_ctx** out, int device, size_t workspace_bytes) {
     return AUDIOKV_ECUDA;
   }
   bool ok = cudaStreamCreateWithFlags(&c->out, cudaStreamNonBlocking) == cudaSuccess &&
-            cudaEventCreateWithFlags(&c->copies_out, cudaEventDisableTiming) == cudaSuccess;
+            cudaEventCreateWithFlags(&c->copies_out, cudaEventDisableTiming) == cudaSuccess &&
+            cudaMallocHost(&c->stage, audiokv_ctx::kStageSlots * kStageBytes) == cudaSuccess;
+  for (int i = 0; i < audiokv_ctx::kStageSlots && ok; ++i)
+    ok = cudaEventCreateWithFlags(&c->stage_free[i], cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < audiokv_ctx::kMaxChunks && ok; ++i)
     ok = cudaEventCreateWithFlags(&c->chunk_in[i], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&c->chunk_done[i], cudaEventDisableTiming) == cudaSuccess;
@@ -763,6 +809,12 @@ int audiokv_destroy(audiokv_ctx* ctx) {
   }
   for (cudaEvent_t e : ctx->prof.ev)
     if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : ctx->stage_free)
+    if (e) {
+      cudaEventSynchronize(e);  // the copy out of the staging may still be on its way
+      cudaEventDestroy(e);
+    }
+  if (ctx->stage) cudaFreeHost(ctx->stage);
   cudaFree(ctx->ws);
   delete ctx;
   return AUDIOKV_OK;
@@ -1043,24 +1095,19 @@ int audiokv_evict_host(audiokv_ctx* ctx, const audiokv_params* p, const void* q_
     return AUDIOKV_EINVAL;
   if (p && p->page_size != 0) return AUDIOKV_EUNSUPPORTED;  // a page table is device data: use audiokv_evict
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int rc = prepare(ctx, p, s);
+  int rc = prepare(ctx, p, s, true);
   if (rc) return rc;
   Plan& pl = ctx->plan;
-  if (audiokv_workspace_bytes_host(p, q_elems, kv_elems, total_budget) > ctx->ws_bytes) return AUDIOKV_EWORKSPACE;
+  if (q_elems < 0 || kv_elems < 0) return AUDIOKV_EINVAL;
+  const HostStaging hs = host_staging(pl, q_elems, kv_elems, total_budget);
+  if (hs.rows < 0) return AUDIOKV_EINVAL;
+  if (hs.end > ctx->ws_bytes) return AUDIOKV_EWORKSPACE;
   const size_t es = esize(p->dtype);
-  int64_t rows = 0;
-  for (int r = 0; r < p->n_req; ++r) rows += total_budget[r];
+  const int64_t rows = hs.rows;
   const int TH = pl.sh.total_heads;
-  size_t off = pl.lay.end;
-  char* dq = ctx->ws + off;   off = align_up(off + q_elems * es);
-  char* dk = ctx->ws + off;   off = align_up(off + kv_elems * es);
-  char* dv = ctx->ws + off;   off = align_up(off + kv_elems * es);
-  char* dS = ctx->ws + off;   off = align_up(off + sizeof(float) * TH);
-  char* dko = ctx->ws + off;  off = align_up(off + rows * p->head_dim * es);
-  char* dvo = ctx->ws + off;  off = align_up(off + rows * p->head_dim * es);
-  char* dki = ctx->ws + off;  off = align_up(off + rows * sizeof(int32_t));
-  char* db = ctx->ws + off;   off = align_up(off + sizeof(int32_t) * TH);
-  char* dcu = ctx->ws + off;
+  char *dq = ctx->ws + hs.q, *dk = ctx->ws + hs.k, *dv = ctx->ws + hs.v, *dS = ctx->ws + hs.head_scores;
+  char *dko = ctx->ws + hs.k_out, *dvo = ctx->ws + hs.v_out, *dki = ctx->ws + hs.kept_idx, *db = ctx->ws + hs.budgets;
+  char* dcu = ctx->ws + hs.cu_kept;
   cudaError_t e;
 #define AKV_CP_ON(st, dst, src, n, kind) \
   if ((e = cudaMemcpyAsync(dst, src, n, kind, st)) != cudaSuccess) return cuda_fail(ctx, e)
