@@ -40,7 +40,7 @@ struct Plan {
   std::vector<int32_t> score_ctas;       // per-CTA run offsets of every (schedule, sweep)
   std::vector<ScoreSchedule> schedules;  // one per run of requests, plus one per chunk of layers of a single request
   int score_parts = 1;                   // statistics slots per head of the tensor-core scoring
-  std::vector<int32_t> sss_order;  // heads in the order the smoothing blocks take them (see build_plan); -1 = none
+  std::vector<int32_t> sss_order;  // heads in the order the smoothing blocks take them (see build_plan)
   int64_t table_len = 0;        // float2 elements
   int64_t scores_len = 0;
   int max_L = 0, max_P = 0;
@@ -448,9 +448,8 @@ int build_plan(const audiokv_params* p, bool host_call, Plan* pl) {
   // does not depend on the device)
   pl->sss_grid = sh.total_heads < kScoreCtas ? sh.total_heads : kScoreCtas;
   {
-    // Block b of the smoothing kernel takes entries b, b + grid, b + 2 grid, ... of this list. Heads are sorted by an
-    // estimate of their transform's cost and dealt out in a snake (left to right, then right to left), so that
-    // a ragged batch with a few expensive lengths (chirp-z in global scratch) does not leave them to one block.
+    // The smoothing blocks take the heads from a queue, in this order: by an estimate of their transform's cost, so that the
+    // last ones to be taken are cheap.
     auto cost = [&](int r) -> double {
       const FftPlan& fp = pl->fft[pl->reqs[r].fft_plan];
       return seq_cost(fp.seq) * (fp.bluestein ? 2.0 : 1.0) * (fp.in_smem ? 1.0 : 1.5) + 8.0 * fp.n;
@@ -459,13 +458,9 @@ int build_plan(const audiokv_params* p, bool host_call, Plan* pl) {
     std::vector<std::pair<double, int32_t>> by_cost(p->n_req);
     for (int r = 0; r < p->n_req; ++r) by_cost[r] = {cost(r), r};
     std::stable_sort(by_cost.begin(), by_cost.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-    const int g = pl->sss_grid, tiers = (sh.total_heads + g - 1) / g;
-    pl->sss_order.assign(static_cast<size_t>(tiers) * g, -1);
-    for (int i = 0; i < sh.total_heads; ++i) {
-      const int tier = i / g, j = i - tier * g;
-      pl->sss_order[static_cast<size_t>(tier) * g + ((tier & 1) ? g - 1 - j : j)] =
-          pl->reqs[by_cost[i / sh.heads_per_req].second].head_base + i % sh.heads_per_req;
-    }
+    pl->sss_order.resize(sh.total_heads);
+    for (int i = 0; i < sh.total_heads; ++i)
+      pl->sss_order[i] = pl->reqs[by_cost[i / sh.heads_per_req].second].head_base + i % sh.heads_per_req;
   }
   int smem_c = 64;
   pl->scratch_per_block = 0;
@@ -595,6 +590,7 @@ void profile_begin(audiokv_ctx* ctx, cudaStream_t stream) {
 }
 
 const ReqDesc* d_reqs(audiokv_ctx* c) { return reinterpret_cast<const ReqDesc*>(c->ws + c->plan.lay.reqs); }
+// The first 64 bytes of the workspace: the status word, and from int 4 on the queue of the smoothing kernel.
 int* d_status(audiokv_ctx* c) { return reinterpret_cast<int*>(c->ws + c->plan.lay.status); }
 
 // head_end >= 0 (one request, tensor-core path only): the heads [head_begin, head_end) alone.
@@ -636,7 +632,7 @@ int do_smooth(audiokv_ctx* ctx, const float* scores, float* smoothed, int32_t* k
                              reinterpret_cast<float2*>(ctx->ws + pl.lay.fft_scratch), pl.scratch_per_block,
                              all ? pl.sss_grid : (count < pl.sss_grid ? count : pl.sss_grid), pl.sss_smem,
                              all ? reinterpret_cast<const int32_t*>(ctx->ws + pl.lay.order) : nullptr, count,
-                             head_begin, budgets, cu_kept, kept_idx, d_status(ctx), ln);
+                             head_begin, budgets, cu_kept, kept_idx, d_status(ctx), d_status(ctx) + 4, ln);
   return e == cudaSuccess ? AUDIOKV_OK : cuda_fail(ctx, e);
 }
 

@@ -136,7 +136,7 @@ struct SssShared {
   int32_t *out, *kstar_out;
   int k_keep;
   double sums[3];      // sum x, sum x^2, alternating sum
-  int kstar;
+  int kstar, slot;
   int loaded;          // plan whose roots lie in shared memory
   uint32_t kmin, kmax;
   int pre[kPreInts];
@@ -1189,7 +1189,8 @@ sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict
            const float2* __restrict__ tables, const float* scores, float* smoothed /* may alias scores */,
            int32_t* __restrict__ kstar_out, float2* __restrict__ scratch, int64_t scratch_per_block,
            const int32_t* __restrict__ order, int n_order, int first_head, const int32_t* __restrict__ budgets,
-           const int32_t* __restrict__ cu_kept, int32_t* __restrict__ kept_idx, int* __restrict__ status) {
+           const int32_t* __restrict__ cu_kept, int32_t* __restrict__ kept_idx, int* __restrict__ status,
+           int* __restrict__ queue) {
   // Launched as a programmatic dependent: the block is brought in while the kernel before it drains, reads its plan
   // (written when the plan was made, not by the kernels of the pass), and waits for that kernel only where it first
   // touches the scores.
@@ -1198,9 +1199,18 @@ sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict
   if (threadIdx.x == 0) S.loaded = -1;
   const bool sel = budgets != nullptr;
 
-  for (int slot = blockIdx.x; slot < n_order; slot += gridDim.x) {
+  // A block's first head is its own; after that it takes the next one nobody has. Whether a head needs transforms shows only in
+  // its scores, so a deal beforehand leaves some blocks with transforms and others with few bins to evaluate. queue[0] counts the heads taken, queue[1]
+  // the blocks that are through; the last of them leaves both at zero for the next launch.
+  auto next_slot = [&]() -> int {
+    if (n_order <= static_cast<int>(gridDim.x)) return n_order;
+    __syncthreads();
+    if (threadIdx.x == 0) S.slot = gridDim.x + atomicAdd(queue, 1);
+    __syncthreads();
+    return S.slot;
+  };
+  for (int slot = blockIdx.x; slot < n_order; slot = next_slot()) {
     const int u = order ? order[slot] : first_head + slot;  // no list: heads first_head, first_head + 1, ...
-    if (u < 0) continue;
     const int r = u / sh.heads_per_req;
     const ReqDesc rq = reqs[r];
     __syncthreads();
@@ -1281,6 +1291,12 @@ sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict
     }
     if (S.pl.in_smem) smooth_head<false>(sh, tables, sel, status);
     else smooth_head<true>(sh, tables, sel, status);
+  }
+  if (n_order > static_cast<int>(gridDim.x) && threadIdx.x == 0) {
+    if (atomicAdd(queue + 1, 1) == static_cast<int>(gridDim.x) - 1) {
+      atomicExch(queue, 0);
+      atomicExch(queue + 1, 0);
+    }
   }
 }
 
@@ -1397,12 +1413,12 @@ cudaError_t launch_sss(const Shape& sh, const ReqDesc* d_reqs, const FftPlan* d_
                        const float* scores, float* smoothed, int32_t* kstar, float2* scratch,
                        int64_t scratch_per_block, int grid, size_t smem_bytes, const int32_t* order, int n_order,
                        int first_head, const int32_t* budgets, const int32_t* cu_kept, int32_t* kept_idx, int* status,
-                       Launch ln) {
+                       int* queue, Launch ln) {
   cudaError_t e = cudaFuncSetAttribute(sss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   if (e != cudaSuccess) return e;
   e = launch_chained(sss_kernel, dim3(grid), dim3(kT), smem_bytes, ln.stream, sh, d_reqs, d_plans, d_tables, scores,
                      smoothed, kstar, scratch, scratch_per_block, order, n_order, first_head, budgets, cu_kept, kept_idx,
-                     status);
+                     status, queue);
   ln.done(budgets ? "sss_select" : "sss");
   return e;
 }
