@@ -18,6 +18,8 @@
 // radix-4 passes than on arithmetic), every access to shared memory is a compile-time LDS / STS through a swizzle
 // that keeps the power-of-two strides of the passes and the digit-reversed reads of the spectrum off the same banks,
 // and twiddles come from per-pass tables whose reads are contiguous over the threads.
+#include <type_traits>
+
 #include "common.cuh"
 #include "select.cuh"
 
@@ -269,6 +271,74 @@ __device__ __forceinline__ void pass_small(const In& in, const Out& out, int tot
   __syncthreads();
 }
 
+// Two passes of small radices in one trip through shared memory: R1 on sub-transforms of length ns, then R2 on the R1 pieces
+// of each. A thread holds the R1 x R2 elements that meet; operations and roundings are those of the two passes one after
+// the other, so only the number of barriers and of loads and stores changes.
+template <int R1, int R2, bool INV>
+__device__ __forceinline__ void pass_pair(int total, int ns, int N, const Roots& root) {
+  const SmemBuf buf;
+  const int m1 = ns / R1, m2 = m1 / R2, step = N / ns;
+  const FastDiv dm(m2);
+#pragma unroll 1
+  for (int t = threadIdx.x; t < total / (R1 * R2); t += kT) {
+    const int b = dm.div(t), j = t - b * m2;
+    const int e0 = b * ns + j;
+    float2 x[R2][R1];
+#pragma unroll
+    for (int s2 = 0; s2 < R2; ++s2)
+#pragma unroll
+      for (int s1 = 0; s1 < R1; ++s1) x[s2][s1] = buf.ld(e0 + s1 * m1 + s2 * m2);
+    const double2 w2 = root.exact(R1 * j * step);
+    auto outer = [&]() {  // the pass of radix R1
+#pragma unroll
+      for (int s2 = 0; s2 < R2; ++s2) {
+        const double2 w1 = root.exact((j + s2 * m2) * step);
+        if (INV) twiddle<R1, true>(x[s2], w1);
+        dft_small<R1, INV>(x[s2]);
+        if (!INV) twiddle<R1, false>(x[s2], w1);
+      }
+    };
+    if (!INV) outer();
+#pragma unroll
+    for (int c = 0; c < R1; ++c) {
+      float2 u[R2];
+#pragma unroll
+      for (int s2 = 0; s2 < R2; ++s2) u[s2] = x[s2][c];
+      if (INV && m2 > 1) twiddle<R2, true>(u, w2);
+      dft_small<R2, INV>(u);
+      if (!INV && m2 > 1) twiddle<R2, false>(u, w2);
+#pragma unroll
+      for (int s2 = 0; s2 < R2; ++s2) x[s2][c] = u[s2];
+    }
+    if (INV) outer();
+#pragma unroll
+    for (int s2 = 0; s2 < R2; ++s2)
+#pragma unroll
+      for (int s1 = 0; s1 < R1; ++s1) buf.st(e0 + s1 * m1 + s2 * m2, x[s2][s1]);
+  }
+  __syncthreads();
+}
+// Whether two passes of these radices go through pass_pair. Only in a chirp-z, which runs every pass four times: a direct
+// transform runs it once a direction, mostly from a cold instruction cache, and the pair's longer code costs what its
+// shorter way saves (N = 496: 41 -> 44 us; 11985: 122 -> 127). And only where half the threads get a share. The smoothing kernel
+// at n = 12170 (M = 12288): 121 -> 100 us; at 8564: 98 -> 88.
+__device__ __forceinline__ bool pairable(int r1, int r2, int total) {
+  if (!S.pl.bluestein || total < kT / 2 * r1 * r2) return false;
+  return (r1 == 4 && r2 == 4) || (r1 == 4 && r2 == 2) || (r1 == 3 && r2 == 4) || (r1 == 3 && r2 == 3) || (r1 == 5 && r2 == 3);
+}
+// The pair at pass i (sub-transforms of length ns there).
+template <bool INV>
+__device__ __forceinline__ void one_pair(int total, int ns, const FftSeq& sq, int i, const Roots& root) {
+  const int N = sq.N;
+  switch (sq.radix[i] * 8 + sq.radix[i + 1]) {
+    case 4 * 8 + 4: pass_pair<4, 4, INV>(total, ns, N, root); break;
+    case 4 * 8 + 2: pass_pair<4, 2, INV>(total, ns, N, root); break;
+    case 3 * 8 + 4: pass_pair<3, 4, INV>(total, ns, N, root); break;
+    case 3 * 8 + 3: pass_pair<3, 3, INV>(total, ns, N, root); break;
+    default: pass_pair<5, 3, INV>(total, ns, N, root); break;
+  }
+}
+
 // The same pass for an odd prime radix p, 17 <= p <= kMaxPrime. With inputs s and p - s folded into P_s = a_s + a_{p-s}
 // and Q_s = a_s - a_{p-s}, outputs c and p - c come from the same real-by-complex sums, X_c = A_c -/+ i B_c,
 // A_c = a_0 + sum_s P_s cos(2 pi s c / p), B_c = sum_s Q_s sin(2 pi s c / p): a product of a small matrix with as many
@@ -418,6 +488,14 @@ __device__ __noinline__ void passes_fwd(const Buf buf, int total, int ns, const 
                                         const float2* __restrict__ tables) {
 #pragma unroll 1
   for (int i = i0; i < i1; ++i) {
+    if constexpr (std::is_same<Buf, SmemBuf>::value) {
+      if (i + 1 < i1 && pairable(sq.radix[i], sq.radix[i + 1], total)) {
+        one_pair<false>(total, ns, sq, i, root);
+        ns /= sq.radix[i] * sq.radix[i + 1];
+        ++i;
+        continue;
+      }
+    }
     one_pass<false>(buf, total, ns, sq, i, root, tables);
     ns /= sq.radix[i];
   }
@@ -429,6 +507,14 @@ __device__ __noinline__ void passes_inv(const Buf buf, int total, int ns, const 
 #pragma unroll 1
   for (int i = i1 - 1; i >= i0; --i) {
     ns *= sq.radix[i];
+    if constexpr (std::is_same<Buf, SmemBuf>::value) {
+      if (i > i0 && pairable(sq.radix[i - 1], sq.radix[i], total)) {
+        --i;
+        ns *= sq.radix[i];
+        one_pair<true>(total, ns, sq, i, root);
+        continue;
+      }
+    }
     one_pass<true>(buf, total, ns, sq, i, root, tables);
   }
 }
