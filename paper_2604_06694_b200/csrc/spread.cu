@@ -10,9 +10,10 @@ namespace akv {
 namespace {
 
 constexpr int kSpreadThreads = 256;
+constexpr int kHistThreads = 1024;  // a head's few thousand indices in one or two turns
 constexpr int kSpreadMaxBins = 4096;
 
-__global__ void __launch_bounds__(kSpreadThreads)
+__global__ void __launch_bounds__(kHistThreads)
 spread_hist_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const int32_t* __restrict__ kept_idx,
                    const int32_t* __restrict__ cu_kept, int n_bins, int32_t* __restrict__ hist,
                    int* __restrict__ status) {
@@ -20,19 +21,30 @@ spread_hist_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const int32_t* __
   const int u = blockIdx.x;
   const int r = u / sh.heads_per_req;
   const int P = reqs[r].P;
-  for (int b = threadIdx.x; b < n_bins; b += kSpreadThreads) h[b] = 0;
+  for (int b = threadIdx.x; b < n_bins; b += kHistThreads) h[b] = 0;
   __syncthreads();
-  const int a = cu_kept[u], e = cu_kept[u + 1];
-  for (int i = a + threadIdx.x; i < e; i += kSpreadThreads) {
-    const int j = kept_idx[i];
-    if (j < 0 || j >= reqs[r].L) {
-      atomicExch(status, AUDIOKV_EDEVICE);  // not an index of this head: skipped
-      continue;
+  const int a = cu_kept[u], e = cu_kept[u + 1], L = reqs[r].L;
+  // Indices come in ascending order, so the lanes of a warp mostly share a stretch: one add per stretch and warp. (One atomic
+  // and one 64-bit division per index took 21 us for 112 heads of 4800 kept tokens; j * n_bins is below 2^29.)
+  constexpr int kUnroll = 4;
+  const int lane = threadIdx.x & 31;
+  for (int i0 = a + static_cast<int>(threadIdx.x); i0 - lane < e; i0 += kUnroll * kHistThreads) {
+    int j[kUnroll];
+#pragma unroll
+    for (int q = 0; q < kUnroll; ++q) j[q] = i0 + q * kHistThreads < e ? __ldg(kept_idx + i0 + q * kHistThreads) : P;
+#pragma unroll
+    for (int q = 0; q < kUnroll; ++q) {
+      if (j[q] < 0 || j[q] >= L) {
+        atomicExch(status, AUDIOKV_EDEVICE);  // not an index of this head: skipped
+        j[q] = P;
+      }
+      const int bin = j[q] < P ? static_cast<int>(static_cast<uint32_t>(j[q]) * static_cast<uint32_t>(n_bins) / static_cast<uint32_t>(P)) : -1;
+      const uint32_t same = __match_any_sync(0xffffffffu, bin);
+      if (bin >= 0 && lane == __ffs(same) - 1) atomicAdd(&h[bin], __popc(same));
     }
-    if (j < P) atomicAdd(&h[static_cast<long long>(j) * n_bins / P], 1);
   }
   __syncthreads();
-  for (int b = threadIdx.x; b < n_bins; b += kSpreadThreads)
+  for (int b = threadIdx.x; b < n_bins; b += kHistThreads)
     if (h[b]) atomicAdd(hist + static_cast<int64_t>(r) * n_bins + b, h[b]);
 }
 
@@ -95,7 +107,7 @@ cudaError_t launch_selection_spread(const Shape& sh, const ReqDesc* d_reqs, cons
   if (n_bins < 1 || n_bins > kSpreadMaxBins) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int32_t) * static_cast<size_t>(sh.n_req) * n_bins, ln.stream);
   if (e != cudaSuccess) return e;
-  spread_hist_kernel<<<sh.total_heads, kSpreadThreads, 0, ln.stream>>>(sh, d_reqs, kept_idx, cu_kept, n_bins, hist,
+  spread_hist_kernel<<<sh.total_heads, kHistThreads, 0, ln.stream>>>(sh, d_reqs, kept_idx, cu_kept, n_bins, hist,
                                                                        status);
   ln.done("spread_hist");
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
