@@ -88,8 +88,8 @@ allocate_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const float* __restr
     long long lover = 0;
     for (int h = threadIdx.x; h < N; h += kAllocThreads)
       if (active[h]) {
-        const long long prod = R * Sq[h];  // R < 2^31 and S_q <= 2^31: no overflow
-        const long long sh_ = prod / sum;
+        const unsigned long long prod = static_cast<unsigned long long>(R) * Sq[h];  // R < 2^31 and S_q <= 2^31: no overflow
+        const long long sh_ = prod / static_cast<unsigned long long>(sum);
         tk[h] = sh_;
         rem[h] = prod - sh_ * sum;
         if (sh_ > cap) ++lover;
@@ -116,15 +116,22 @@ allocate_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const float* __restr
         if (active[h] && tk[h] < cap) ++lelig;
       const long long n_elig = block_sum_ll(lelig, red);
       if (n_elig == 0) break;
+      // the remainders of the heads that can take a row, -1 for the others: one array to rank against
       for (int h = threadIdx.x; h < N; h += kAllocThreads)
-        if (active[h] && tk[h] < cap) {
-          long long rank = 0;
-          for (int g = 0; g < N; ++g)
-            if (active[g] && tk[g] < cap && (rem[g] > rem[h] || (rem[g] == rem[h] && g < h))) ++rank;
-          give[h] = rank < left ? 1 : 0;
-        } else {
-          give[h] = 0;
+        if (!(active[h] && tk[h] < cap)) rem[h] = -1;
+      __syncthreads();
+      for (int h = threadIdx.x; h < N; h += kAllocThreads) {
+        const long long mine = rem[h];
+        int rank = 0;
+        if (mine >= 0) {
+#pragma unroll 8
+          for (int g = 0; g < N; ++g) {
+            const long long other = rem[g];
+            rank += other > mine || (other == mine && g < h);
+          }
         }
+        give[h] = mine >= 0 && rank < left ? 1 : 0;
+      }
       __syncthreads();  // the increments are applied after every thread has ranked against the old shares
       for (int h = threadIdx.x; h < N; h += kAllocThreads)
         if (give[h]) tk[h] += 1;
