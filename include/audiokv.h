@@ -142,9 +142,9 @@ int audiokv_create(audiokv_ctx** ctx, int device, size_t workspace_bytes);
  * Use one context per stream; contexts are independent of one another.
  *
  * Stream capture: every device-buffer entry point may be recorded into a CUDA graph, once the
- * context has seen its params in a call OUTSIDE capture (the first call with a new shape copies
- * the plan up from pageable memory and waits for it; inside a capture it returns AUDIOKV_ECUDA
- * and says so in audiokv_last_cuda_error). Every kernel of audiokv_evict goes to the caller's stream
+ * context has seen its params in a call OUTSIDE capture (the first call with a new shape brings
+ * the plan to the device, which a graph must not do over again at every replay; inside a capture it
+ * returns AUDIOKV_ECUDA and says so in audiokv_last_cuda_error). Every kernel of audiokv_evict goes to the caller's stream
  * (some as programmatic dependents of the one before). The host-buffer call waits on the host and
  * cannot be captured. */
 

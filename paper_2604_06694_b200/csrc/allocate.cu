@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(kAllocThreads)
 allocate_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const float* __restrict__ head_scores, BudgetArgs args,
                 int32_t* __restrict__ budgets, int32_t* __restrict__ cu_kept, int* __restrict__ status) {
   extern __shared__ long long sm[];
+  chain_wait();     // the request table may be the work of the kernel before
   chain_release();  // the first scoring sweep, which needs nothing from here, may start beside this kernel
   const int N = sh.heads_per_req;
   long long* Sq = sm;            // [N] quantised scores
@@ -223,7 +224,7 @@ cudaError_t launch_budget_prefix(const Shape& sh, const ReqDesc* d_reqs, const i
 
 cudaError_t launch_allocate(const Shape& sh, const ReqDesc* d_reqs, const float* head_scores,
                             const int64_t* h_total_budget, int32_t* budgets, int32_t* cu_kept, int* status,
-                            Launch ln) {
+                            Launch ln, bool chained) {
   int64_t all = 0;
   for (int r = 0; r < sh.n_req; ++r) all += h_total_budget[r];
   if (all > 0x7fffffffLL) return cudaErrorInvalidValue;  // cu_kept is int32
@@ -240,9 +241,15 @@ cudaError_t launch_allocate(const Shape& sh, const ReqDesc* d_reqs, const float*
       args.cu_base[i] = rows;
       rows += h_total_budget[r0 + i];
     }
-    allocate_kernel<<<n, kAllocThreads, smem, ln.stream>>>(sh, d_reqs, head_scores, args, budgets, cu_kept, status);
+    // the first launch of a pass is an ordinary one, so that everything earlier on the stream is complete when it starts
+    if (chained) {
+      e = launch_chained(allocate_kernel, dim3(n), dim3(kAllocThreads), smem, ln.stream, sh, d_reqs, head_scores, args, budgets, cu_kept, status);
+    } else {
+      allocate_kernel<<<n, kAllocThreads, smem, ln.stream>>>(sh, d_reqs, head_scores, args, budgets, cu_kept, status);
+      e = cudaGetLastError();
+    }
     ln.done("allocate");
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

@@ -23,8 +23,8 @@ constexpr int kHostChunks = 8;          // the host-buffer call evicts one reque
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
-struct Layout {  // byte offsets inside the workspace; status .. order, up to blob_end, are uploaded as one piece with a plan
-  size_t status, reqs, plans, units, ctas, order, blob_end, tables, stats, exps, fft_scratch, scores, kstar, aux, end;
+struct Layout {  // byte offsets inside the workspace; status .. ctas, up to blob_end, are uploaded as one piece with a plan
+  size_t status, reqs, plans, order, units, ctas, blob_end, tables, stats, exps, fft_scratch, scores, kstar, aux, end;
 };
 
 struct Plan {
@@ -66,6 +66,7 @@ struct audiokv_ctx {
   size_t ws_bytes = 0;
   Plan plan;
   bool plan_uploaded = false;
+  bool plan_fresh = false;                // the call at hand put the plan on the device: its last launch was launch_fft_tables
   uint64_t plan_id = 0;      // counts plan rebuilds
   ScoreMapCache score_maps;
   cudaEvent_t plan_ready = nullptr;
@@ -74,7 +75,7 @@ struct audiokv_ctx {
   static constexpr int kStageSlots = 4;
   char* stage = nullptr;                  // pinned: kStageSlots x kStageBytes
   cudaEvent_t stage_free[kStageSlots] = {};
-  std::vector<char> big_blob;
+  std::vector<char> blob;
   cudaStream_t side = nullptr;            // audiokv_evict runs the allocation here, beside the scoring
   cudaEvent_t fork = nullptr, join = nullptr;
   // audiokv_evict_host: copies in on `side`, kernels on the caller's stream, copies out on `out`, chunk by chunk
@@ -476,9 +477,9 @@ int build_plan(const audiokv_params* p, bool host_call, Plan* pl) {
   L.status = off;      off = align_up(off + 64);
   L.reqs = off;        off = align_up(off + sizeof(ReqDesc) * pl->reqs.size());
   L.plans = off;       off = align_up(off + sizeof(FftPlan) * pl->fft.size());
+  L.order = off;       off = align_up(off + sizeof(int32_t) * pl->sss_order.size());
   L.units = off;       off = align_up(off + sizeof(ScoreUnit) * pl->units.size());
   L.ctas = off;        off = align_up(off + sizeof(int32_t) * pl->score_ctas.size());
-  L.order = off;       off = align_up(off + sizeof(int32_t) * pl->sss_order.size());
   L.blob_end = off;
   L.tables = off;      off = align_up(off + sizeof(float2) * static_cast<size_t>(pl->table_len));
   {
@@ -520,28 +521,31 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
   if (pl.lay.end > ctx->ws_bytes) return AUDIOKV_EWORKSPACE;
   pl.sh.page_table = p->page_size ? p->page_table : nullptr;  // device data of this call, not part of the plan
   pl.sh.page_status = reinterpret_cast<int*>(ctx->ws + pl.lay.status);
+  ctx->plan_fresh = !ctx->plan_uploaded;
   if (!ctx->plan_uploaded) {
-    // A new plan goes up with copies from pageable memory, which a stream capture cannot hold: the first call with
-    // a given shape has to run outside capture (later ones add nothing but kernels and may be captured).
+    // A graph that held the upload would bring this plan back at every replay, over the one the context then has: the first
+    // call with a given shape has to run outside capture (later ones add nothing but the kernels of the pass).
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if ((e = cudaStreamIsCapturing(stream, &cap)) != cudaSuccess) return cuda_fail(ctx, e);
     if (cap != cudaStreamCaptureStatusNone) {
       ctx->cuda_error = "the plan of these params is not on the device yet: make one call outside stream capture first";
       return AUDIOKV_ECUDA;
     }
-    // The request table, FFT plans, schedules and order go up in one copy, and the status word starts clean with it. From
-    // pinned staging the host does not wait for it (a prompt of a new length then costs no round trip); a plan larger than
-    // a staging slot goes up from pageable memory, which does.
+    // The request table, FFT plans, order and schedules go up as one piece, and the status word starts clean with it. A plan
+    // of some tens of heads travels as arguments of the table kernels. A larger one goes up from pinned staging, for which the host
+    // does not wait either (a prompt of a new length then costs no round trip), one that is larger than a staging
+    // slot from pageable memory, for which it does.
     const size_t blob = pl.lay.blob_end;
-    const bool staged = blob <= kStageBytes;
+    const bool inlined = blob <= 2 * kPlanPartBytes && pl.lay.units <= kPlanPartBytes;
+    const bool staged = !inlined && blob <= kStageBytes;
     char* src;
     const int slot = static_cast<int>(ctx->plan_id % audiokv_ctx::kStageSlots);
     if (staged) {
       src = ctx->stage + slot * kStageBytes;
       if ((e = cudaEventSynchronize(ctx->stage_free[slot])) != cudaSuccess) return cuda_fail(ctx, e);  // four plans ago
     } else {
-      ctx->big_blob.resize(blob);
-      src = ctx->big_blob.data();
+      ctx->blob.resize(blob);
+      src = ctx->blob.data();
     }
     memset(src, 0, 64);
     auto put = [&](size_t at, const void* data, size_t bytes) {
@@ -552,11 +556,11 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
     put(pl.lay.units, pl.units.data(), sizeof(ScoreUnit) * pl.units.size());
     put(pl.lay.ctas, pl.score_ctas.data(), sizeof(int32_t) * pl.score_ctas.size());
     put(pl.lay.order, pl.sss_order.data(), sizeof(int32_t) * pl.sss_order.size());
-    if ((e = cudaMemcpyAsync(ctx->ws, src, blob, cudaMemcpyHostToDevice, stream)) != cudaSuccess) return cuda_fail(ctx, e);
+    if (!inlined && (e = cudaMemcpyAsync(ctx->ws, src, blob, cudaMemcpyHostToDevice, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     if (staged && (e = cudaEventRecord(ctx->stage_free[slot], stream)) != cudaSuccess) return cuda_fail(ctx, e);
     Launch ln{stream, &ctx->launches, &ctx->prof};
-    e = launch_fft_tables(static_cast<int>(pl.fft.size()), reinterpret_cast<float2*>(ctx->ws + pl.lay.tables),
-                          reinterpret_cast<const FftPlan*>(ctx->ws + pl.lay.plans), pl.sss_smem, ln);
+    e = launch_fft_tables(static_cast<int>(pl.fft.size()), inlined ? src : nullptr, blob, ctx->ws, pl.lay.plans,
+                          reinterpret_cast<float2*>(ctx->ws + pl.lay.tables), pl.sss_smem, ln);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     if ((e = cudaEventRecord(ctx->plan_ready, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     ctx->plan_stream = stream;
@@ -656,12 +660,13 @@ int check_budgets(const Plan& pl, const int64_t* total_budget) {
 }
 
 int do_allocate(audiokv_ctx* ctx, const float* head_scores, const int64_t* total_budget, int32_t* budgets,
-                int32_t* cu_kept, cudaStream_t stream) {
+                int32_t* cu_kept, cudaStream_t stream, bool chained = false) {
   Plan& pl = ctx->plan;
   int rc = check_budgets(pl, total_budget);
   if (rc) return rc;
   Launch ln{stream, &ctx->launches, &ctx->prof};
-  cudaError_t e = launch_allocate(pl.sh, d_reqs(ctx), head_scores, total_budget, budgets, cu_kept, d_status(ctx), ln);
+  cudaError_t e = launch_allocate(pl.sh, d_reqs(ctx), head_scores, total_budget, budgets, cu_kept, d_status(ctx), ln,
+                                  chained);
   return e == cudaSuccess ? AUDIOKV_OK : cuda_fail(ctx, e);
 }
 
@@ -929,7 +934,7 @@ int audiokv_evict(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, 
   // own end, so that the smoothing and selection, two chained kernels later, find the budgets complete. With per-kernel
   // timing on, every kernel waits for the one before it.
   const bool beside = !ctx->prof.on && score_umma_takes(pl.sh);
-  rc = do_allocate(ctx, head_scores, total_budget, budgets, cu_kept, s);
+  rc = do_allocate(ctx, head_scores, total_budget, budgets, cu_kept, s, ctx->plan_fresh && !ctx->prof.on);
   if (!rc) rc = do_score(ctx, q_win, k, ws_scores, s, 0, -1, beside);
   if (rc) return rc;
   // the pooling variants hand their result to the selection through the score buffer itself

@@ -238,7 +238,12 @@ cudaError_t launch_score_umma(const Shape& sh, const ReqDesc* h_reqs, const Scor
 // sss.cu
 int sss_static_smem();  // bytes of shared memory a smoothing block uses beside its work buffer
 // smem_bytes: the dynamic shared memory launch_sss is given for these plans.
-cudaError_t launch_fft_tables(int n_plans, float2* d_tables, const FftPlan* d_plans, size_t smem_bytes, Launch ln);
+// h_blob: the first blob_bytes of the workspace (a multiple of 16), at most two parts' worth, which the launch itself takes to
+// the device; what is read before a chain_wait (request table, transform plans, order) has to lie in the first part. Null: it
+// is all there already. plans_at: where the transform plans lie in the workspace.
+constexpr size_t kPlanPartBytes = 30 << 10;  // kernel arguments end at 32764 bytes
+cudaError_t launch_fft_tables(int n_plans, const char* h_blob, size_t blob_bytes, char* ws, size_t plans_at, float2* d_tables,
+                              size_t smem_bytes, Launch ln);
 // order: the heads, the ones that can cost most first; a null order stands for the n_order heads first_head, first_head + 1, ... .
 // The blocks take them from a queue (two ints, zero before and after). smoothed may be null when budgets, cu_kept and kept_idx
 // are given: the kernel then goes on to the top-k selection of each head from the smoothed scores it holds on chip (step
@@ -249,10 +254,10 @@ cudaError_t launch_sss(const Shape& sh, const ReqDesc* d_reqs, const FftPlan* d_
                        int first_head, const int32_t* budgets, const int32_t* cu_kept, int32_t* kept_idx, int* status,
                        int* queue, Launch ln);
 
-// allocate.cu (h_total_budget: host array [n_req])
+// allocate.cu (h_total_budget: host array [n_req]). chained: what was launched just before is launch_fft_tables.
 cudaError_t launch_allocate(const Shape& sh, const ReqDesc* d_reqs, const float* head_scores,
                             const int64_t* h_total_budget, int32_t* budgets, int32_t* cu_kept, int* status,
-                            Launch ln);
+                            Launch ln, bool chained);
 
 // given: device int32 [total heads], budgets chosen by the caller; budgets: their checked copy; cu_kept: prefix sums.
 cudaError_t launch_budget_prefix(const Shape& sh, const ReqDesc* d_reqs, const int32_t* given, int32_t* budgets,

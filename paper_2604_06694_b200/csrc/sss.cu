@@ -18,6 +18,8 @@
 // radix-4 passes than on arithmetic), every access to shared memory is a compile-time LDS / STS through a swizzle
 // that keeps the power-of-two strides of the passes and the digit-reversed reads of the spectrum off the same banks,
 // and twiddles come from per-pass tables whose reads are contiguous over the threads.
+#include <algorithm>
+#include <cstring>
 #include <type_traits>
 
 #include "common.cuh"
@@ -1393,8 +1395,30 @@ __device__ __forceinline__ float2 root_of_unity(int64_t num, int den) {  // exp(
   return make_float2(static_cast<float>(c), static_cast<float>(-s));
 }
 
-__global__ void fft_table_kernel(const FftPlan* __restrict__ plans, int n_plans, float2* __restrict__ tables) {
-  const FftPlan& pl = plans[blockIdx.y];
+// A plan's bytes travel to the device as arguments of the two table kernels: 4 us for the two together, whatever they hold,
+// where a copy out of pinned memory takes 5 us up to 16 KB and 12 above, in front of the table kernel (28 layers of 4 heads
+// make 36 KB; reading the pinned memory from the kernel took 40 us). Each thread then reads its own 16 bytes of the
+// argument bank, so the copy is spread over blocks.
+struct PlanPart {
+  uint4 v[kPlanPartBytes / 16];
+};
+__device__ __forceinline__ void put_part(const PlanPart& part, uint4* to, int n16, int block, int blocks) {
+  for (int i = block * blockDim.x + threadIdx.x; i < n16; i += blocks * blockDim.x) to[i] = part.v[i];
+}
+
+// Writes the tables of every transform plan, 32 blocks each, and the first n16 x 16 bytes of the workspace from `part`. The
+// transform plans, at byte plans_at of the workspace, are read from `part` when they travel in it.
+__global__ void __launch_bounds__(256)
+fft_table_kernel(const __grid_constant__ PlanPart part, int n16, char* ws, size_t plans_at, float2* __restrict__ tables) {
+  chain_release();
+  __shared__ FftPlan pl;
+  {
+    const char* from = (n16 ? reinterpret_cast<const char*>(part.v) : ws) + plans_at + sizeof(FftPlan) * blockIdx.y;
+    for (int i = threadIdx.x; i < static_cast<int>(sizeof(FftPlan) / 4); i += blockDim.x)
+      reinterpret_cast<int*>(&pl)[i] = reinterpret_cast<const int*>(from)[i];
+  }
+  put_part(part, reinterpret_cast<uint4*>(ws), n16, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+  __syncthreads();
   const int gid = blockIdx.x * blockDim.x + threadIdx.x, gsz = gridDim.x * blockDim.x;
   // roots: 256 fine entries and the coarse ones, of the order the passes want and, for a chirp-z, of order 2N
   for (int t = gid; t < pl.root_count + pl.root_count2; t += gsz) {
@@ -1454,10 +1478,16 @@ __global__ void fft_table_kernel(const FftPlan* __restrict__ plans, int n_plans,
   }
 }
 
-// Transforms each chirp-z filter in place and folds in the 1/M of the inverse: one block per plan and filter.
+// Transforms each chirp-z filter in place and folds in the 1/M of the inverse: one block per plan and filter. The blocks from
+// y = 2 on write the rest of the plan (n16 x 16 bytes) from `part`.
 __global__ void __launch_bounds__(kT, 1)
-fft_filter_kernel(const FftPlan* __restrict__ plans, float2* __restrict__ tables) {
+fft_filter_kernel(const __grid_constant__ PlanPart part, int n16, uint4* rest, const FftPlan* __restrict__ plans, float2* __restrict__ tables) {
   const FftPlan& pl = S.pl;
+  chain_wait();
+  if (blockIdx.y >= 2) {
+    put_part(part, rest, n16, (blockIdx.y - 2) * gridDim.x + blockIdx.x, (gridDim.y - 2) * gridDim.x);
+    return;
+  }
   for (int i = threadIdx.x; i < static_cast<int>(sizeof(FftPlan) / 4); i += kT)
     reinterpret_cast<int*>(&S.pl)[i] = reinterpret_cast<const int*>(plans + blockIdx.x)[i];
   __syncthreads();
@@ -1485,14 +1515,22 @@ fft_filter_kernel(const FftPlan* __restrict__ plans, float2* __restrict__ tables
 
 int sss_static_smem() { return static_cast<int>(sizeof(SssShared)); }
 
-cudaError_t launch_fft_tables(int n_plans, float2* d_tables, const FftPlan* d_plans, size_t smem_bytes, Launch ln) {
-  fft_table_kernel<<<dim3(32, n_plans), 256, 0, ln.stream>>>(d_plans, n_plans, d_tables);
-  ln.done("fft_table");
+cudaError_t launch_fft_tables(int n_plans, const char* h_blob, size_t blob_bytes, char* ws, size_t plans_at, float2* d_tables,
+                              size_t smem_bytes, Launch ln) {
   cudaError_t e = cudaFuncSetAttribute(fft_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   if (e != cudaSuccess) return e;
-  fft_filter_kernel<<<dim3(n_plans, 2), kT, smem_bytes, ln.stream>>>(d_plans, d_tables);
+  const size_t first = h_blob ? std::min(blob_bytes, kPlanPartBytes) : 0, rest = h_blob ? blob_bytes - first : 0;
+  PlanPart part;
+  if (first) memcpy(part.v, h_blob, first);
+  fft_table_kernel<<<dim3(32, n_plans), 256, 0, ln.stream>>>(part, static_cast<int>(first / 16), ws, plans_at, d_tables);
+  ln.done("fft_table");
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (rest) memcpy(part.v, h_blob + first, rest);
+  e = launch_chained(fft_filter_kernel, dim3(n_plans, rest ? 2 + (8 + n_plans - 1) / n_plans : 2), dim3(kT), smem_bytes, ln.stream, part,
+                     static_cast<int>(rest / 16), reinterpret_cast<uint4*>(ws + first),
+                     reinterpret_cast<const FftPlan*>(ws + plans_at), d_tables);
   ln.done("fft_filter");
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_sss(const Shape& sh, const ReqDesc* d_reqs, const FftPlan* d_plans, const float2* d_tables,
