@@ -618,7 +618,8 @@ int do_score(audiokv_ctx* ctx, const void* q, const void* k, float* scores, cuda
     // engine cannot take; audiokv_last_score_path tells the caller which route ran
     ctx->score_path = 2;
     float* exps = pl.exps_len ? reinterpret_cast<float*>(ctx->ws + pl.lay.exps) : nullptr;
-    e = launch_score_simt(pl.sh, d_reqs(ctx), q, k, scores, stats, pl.n_slab, kSlabKeys, exps, pl.exps_len, pl.max_L, ln);
+    e = launch_score_simt(pl.sh, d_reqs(ctx), q, k, scores, stats, pl.n_slab, kSlabKeys, exps, pl.exps_len, pl.max_L, ln,
+                          beside && !score_umma_takes(pl.sh));
   }
   return e == cudaSuccess ? AUDIOKV_OK : cuda_fail(ctx, e);
 }
@@ -933,7 +934,7 @@ int audiokv_evict(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, 
   // dependents in at once; the first scoring sweep, a programmatic dependent, runs beside it and waits for it at its
   // own end, so that the smoothing and selection, two chained kernels later, find the budgets complete. With per-kernel
   // timing on, every kernel waits for the one before it.
-  const bool beside = !ctx->prof.on && score_umma_takes(pl.sh);
+  const bool beside = !ctx->prof.on;
   rc = do_allocate(ctx, head_scores, total_budget, budgets, cu_kept, s, ctx->plan_fresh && !ctx->prof.on);
   if (!rc) rc = do_score(ctx, q_win, k, ws_scores, s, 0, -1, beside);
   if (rc) return rc;
@@ -970,7 +971,7 @@ int audiokv_evict_budgeted(audiokv_ctx* ctx, const audiokv_params* p, const void
   Launch ln{s, &ctx->launches, &ctx->prof};
   cudaError_t e = launch_budget_prefix(pl.sh, d_reqs(ctx), budgets, ws_budgets, cu_kept, d_status(ctx), ln);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
-  if ((rc = do_score(ctx, q_win, k, ws_scores, s, 0, -1, !ctx->prof.on && score_umma_takes(pl.sh)))) return rc;
+  if ((rc = do_score(ctx, q_win, k, ws_scores, s, 0, -1, !ctx->prof.on))) return rc;
   float* ws_smoothed = pl.sh.smooth_mode >= AUDIOKV_SMOOTH_AVG_POOL ? ws_scores : nullptr;
   if ((rc = do_smooth(ctx, ws_scores, ws_smoothed, ws_kstar, ws_budgets, cu_kept, kept_idx, s))) return rc;
   return do_gather(ctx, cu_kept, kept_idx, k, v, k_out, v_out, s);

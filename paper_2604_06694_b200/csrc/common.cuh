@@ -168,7 +168,7 @@ cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t
 // exps (a workspace of exps_len floats that holds one head's exponentials at least) the product is done once and
 // the statistics take [heads of a chunk][tiles of score_simt_tile_keys keys][rows] instead.
 cudaError_t launch_score_simt(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores,
-                              float2* stats_ws, int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln);
+                              float2* stats_ws, int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln, bool beside = false);
 // Floats of workspace the single-product scoring is given: a chunk of heads, at most 128 MB; 0 when one head alone is longer.
 int64_t score_simt_exps_len(int total_heads, int max_L, int rows, int head_dim);
 int score_simt_tile_keys(int head_dim);

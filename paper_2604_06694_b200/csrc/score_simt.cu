@@ -86,7 +86,7 @@ template <typename T, int D, int RPT, int MODE>
 __global__ void __launch_bounds__(2 * tile_keys(D), 2)
 score_tile_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const T* __restrict__ q, const T* __restrict__ k,
                   float* __restrict__ scores, float2* __restrict__ stats, float* __restrict__ exps, int n_slab, int slab_keys,
-                  int u0) {
+                  int u0, int beside) {
   constexpr int kKeys = tile_keys(D), kThr = 2 * kKeys, kTx = kKeys / 8, kRows = 16 * RPT;
   constexpr int kRowBytes = panel_row_bytes(static_cast<int>(sizeof(T))), kStage = kRows * kRowBytes;
   constexpr int kPieces = kPanel * static_cast<int>(sizeof(T)) / 16;  // 16-byte pieces of a panel row
@@ -96,8 +96,11 @@ score_tile_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const T* __restric
   unsigned char* q_s = smem + kKeys * D * 4;                  // kStages panels of query rows
   const T** rows = reinterpret_cast<const T**>(q_s + kStages * kStage);  // the head's query rows, whole row tiles
 
+  // The budget kernel launched just before (see launch_score_umma's `beside`) lets this one in when everything earlier on the
+  // stream is complete, and computes nothing that is read here: the two run side by side, and every block waits for it at its
+  // end, which the kernels behind then need not do (6 us of a pass over 2 heads of 1024 keys, 59 in all).
   chain_release();
-  chain_wait();  // the request table may be the work of the kernel before
+  if (!beside) chain_wait();  // the request table may be the work of the kernel before
   const int uc = blockIdx.x / n_slab, slab = blockIdx.x - uc * n_slab, u = u0 + uc;
   const HeadCoord hc = head_coord(sh, u);
   const ReqDesc rq = reqs[hc.r];
@@ -111,6 +114,7 @@ score_tile_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const T* __restric
   if (j0 >= j1) {  // no keys of this request here
     if (MODE != kColsum)
       for (int r = threadIdx.x; r < R; r += kThr) my_stats[r] = make_float2(-INFINITY, 0.f);
+    if (beside) chain_wait();
     return;
   }
   const int n_rt = (R + kRows - 1) / kRows;  // row tiles; rows past the end repeat the last one, their logits are dropped
@@ -298,6 +302,7 @@ score_tile_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const T* __restric
       }
     }
   }
+  if (beside) chain_wait();
 }
 
 // c = -(max + log2 sum) of every row over its head's slabs, into .y of the row's entry of the first slab (whose sum is no
@@ -380,13 +385,13 @@ colsum_kernel(Shape sh, const ReqDesc* __restrict__ reqs, float* __restrict__ sc
 
 template <typename T, int D, int RPT, int MODE>
 cudaError_t launch_tile(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
-                        float* exps, int n_slab, int slab_keys, int u0, int heads, Launch ln) {
+                        float* exps, int n_slab, int slab_keys, int u0, int heads, Launch ln, bool beside) {
   auto kern = score_tile_kernel<T, D, RPT, MODE>;
   const int smem = tile_smem_bytes(D, RPT, static_cast<int>(sizeof(T)), sh.window * sh.group);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   e = launch_chained(kern, dim3(static_cast<unsigned>(n_slab) * heads), dim3(2 * tile_keys(D)), smem, ln.stream, sh, d_reqs,
-                     static_cast<const T*>(q), static_cast<const T*>(k), scores, stats, exps, n_slab, slab_keys, u0);
+                     static_cast<const T*>(q), static_cast<const T*>(k), scores, stats, exps, n_slab, slab_keys, u0, beside ? 1 : 0);
   ln.done(MODE == kStore ? "score_simt_exps" : MODE == kStats ? "score_simt_stats" : "score_simt_colsum");
   return e;
 }
@@ -412,7 +417,7 @@ int heads_per_chunk(int most, int total, int tiles) {
 
 template <typename T, int D, int RPT>
 cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
-                         int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln) {
+                         int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln, bool beside) {
   constexpr int kKeys = tile_keys(D);
   const int R = sh.window * sh.group, n_tile = (max_L + kKeys - 1) / kKeys;
   const int64_t per_head = static_cast<int64_t>(n_tile) * R * kKeys;
@@ -424,8 +429,8 @@ cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, 
   cudaError_t e = cudaSuccess;
   for (int u0 = 0; u0 < sh.total_heads && e == cudaSuccess; u0 += chunk) {
     const int heads = sh.total_heads - u0 < chunk ? sh.total_heads - u0 : chunk;
-    if (store) e = launch_tile<T, D, RPT, kStore>(sh, d_reqs, q, k, scores, stats, exps, slabs, kKeys, u0, heads, ln);
-    else e = launch_tile<T, D, RPT, kStats>(sh, d_reqs, q, k, scores, stats, exps, slabs, slab_keys, u0, heads, ln);
+    if (store) e = launch_tile<T, D, RPT, kStore>(sh, d_reqs, q, k, scores, stats, exps, slabs, kKeys, u0, heads, ln, beside && u0 == 0);
+    else e = launch_tile<T, D, RPT, kStats>(sh, d_reqs, q, k, scores, stats, exps, slabs, slab_keys, u0, heads, ln, beside && u0 == 0);
     if (e != cudaSuccess) return e;
     e = launch_chained(merge_kernel, dim3(heads, (R + 31) / 32), dim3(kThreads), 0, ln.stream, stats, slabs, R);
     ln.done("score_simt_merge");
@@ -435,7 +440,7 @@ cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, 
                          d_reqs, scores, stats, exps, slabs, u0);
       ln.done("score_simt_colsum");
     } else {
-      e = launch_tile<T, D, RPT, kColsum>(sh, d_reqs, q, k, scores, stats, exps, slabs, slab_keys, u0, heads, ln);
+      e = launch_tile<T, D, RPT, kColsum>(sh, d_reqs, q, k, scores, stats, exps, slabs, slab_keys, u0, heads, ln, false);
     }
   }
   return e;
@@ -444,12 +449,12 @@ cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, 
 // Rows per thread: the tile height that leaves the fewest padding rows, the larger one on a tie.
 template <typename T, int D>
 cudaError_t launch_rows(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
-                        int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln) {
+                        int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln, bool beside) {
   const int R = sh.window * sh.group;
   auto padded = [R](int rows) { return (R + rows - 1) / rows * rows; };
-  if (R <= 64) return launch_typed<T, D, 4>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln);
-  if (padded(112) < padded(128)) return launch_typed<T, D, 7>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln);
-  return launch_typed<T, D, 8>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln);
+  if (R <= 64) return launch_typed<T, D, 4>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln, beside);
+  if (padded(112) < padded(128)) return launch_typed<T, D, 7>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln, beside);
+  return launch_typed<T, D, 8>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln, beside);
 }
 
 }  // namespace
@@ -465,8 +470,8 @@ int64_t score_simt_exps_len(int total_heads, int max_L, int rows, int head_dim) 
 }
 
 cudaError_t launch_score_simt(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores,
-                              float2* stats_ws, int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln) {
-#define AKV_CASE(T, D) return launch_rows<T, D>(sh, d_reqs, q, k, scores, stats_ws, n_slab, slab_keys, exps, exps_len, max_L, ln)
+                              float2* stats_ws, int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln, bool beside) {
+#define AKV_CASE(T, D) return launch_rows<T, D>(sh, d_reqs, q, k, scores, stats_ws, n_slab, slab_keys, exps, exps_len, max_L, ln, beside)
   if (sh.dtype == AUDIOKV_F32) {
     if (sh.head_dim == 64) AKV_CASE(float, 64);
     if (sh.head_dim == 128) AKV_CASE(float, 128);
