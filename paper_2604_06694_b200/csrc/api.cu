@@ -76,7 +76,7 @@ struct audiokv_ctx {
   char* stage = nullptr;                  // pinned: kStageSlots x kStageBytes
   cudaEvent_t stage_free[kStageSlots] = {};
   std::vector<char> blob;
-  cudaStream_t side = nullptr;            // audiokv_evict runs the allocation here, beside the scoring
+  cudaStream_t side = nullptr;            // audiokv_evict_host copies in here
   cudaEvent_t fork = nullptr, join = nullptr;
   // audiokv_evict_host: copies in on `side`, kernels on the caller's stream, copies out on `out`, chunk by chunk
   static constexpr int kMaxChunks = kHostChunks;

@@ -17,7 +17,9 @@
 // flight each (128 registers; the earlier 1024 threads with 64 registers spent more cycles on the barriers and on
 // radix-4 passes than on arithmetic), every access to shared memory is a compile-time LDS / STS through a swizzle
 // that keeps the power-of-two strides of the passes and the digit-reversed reads of the spectrum off the same banks,
-// and twiddles come from per-pass tables whose reads are contiguous over the threads.
+// and twiddles come from a two-level table of roots of unity in shared memory. Heads are taken from a queue, since what a
+// head costs shows only in its scores. 112 heads of 8160 tokens, no transform: 27 us; 192 heads of 16352 tokens, two
+// transforms each of 16 * 7 * 73 points: 195 us (two turns on 148 SMs).
 #include <algorithm>
 #include <cstring>
 #include <type_traits>
