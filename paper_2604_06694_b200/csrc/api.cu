@@ -75,9 +75,10 @@ struct audiokv_ctx {
   static constexpr int kStageSlots = 4;
   char* stage = nullptr;                  // pinned: kStageSlots x kStageBytes
   cudaEvent_t stage_free[kStageSlots] = {};
+  uint64_t large_plans = 0;               // plans too large for the kernels' arguments
   std::vector<char> blob;
   cudaStream_t side = nullptr;            // audiokv_evict_host copies in here
-  cudaEvent_t fork = nullptr, join = nullptr;
+  cudaEvent_t fork = nullptr;
   // audiokv_evict_host: copies in on `side`, kernels on the caller's stream, copies out on `out`, chunk by chunk
   static constexpr int kMaxChunks = kHostChunks;
   cudaStream_t out = nullptr;
@@ -506,6 +507,22 @@ int cuda_fail(audiokv_ctx* ctx, cudaError_t e) {
   return AUDIOKV_ECUDA;
 }
 
+// The ring of pinned staging slots; false when it cannot be had (the plans then go up from pageable memory).
+bool make_stage(audiokv_ctx* ctx) {
+  if (ctx->stage) return true;
+  for (cudaEvent_t& ev : ctx->stage_free)
+    if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+  if (cudaMallocHost(&ctx->stage, audiokv_ctx::kStageSlots * kStageBytes) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->stage = nullptr;
+    return false;
+  }
+  return true;
+}
+
 // Makes ctx->plan match p and its tables resident on the device (stream-ordered).
 int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool host_call = false) {
   if (!ctx) return AUDIOKV_EINVAL;
@@ -537,7 +554,8 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
     // slot from pageable memory, for which it does.
     const size_t blob = pl.lay.blob_end;
     const bool inlined = blob <= 2 * kPlanPartBytes && pl.lay.units <= kPlanPartBytes;
-    const bool staged = !inlined && blob <= kStageBytes;
+    // (The staging is made when a context brings its second plan of that size: pinning costs about a millisecond.)
+    const bool staged = !inlined && blob <= kStageBytes && ctx->large_plans++ > 0 && make_stage(ctx);
     char* src;
     const int slot = static_cast<int>(ctx->plan_id % audiokv_ctx::kStageSlots);
     if (staged) {
@@ -771,20 +789,15 @@ int audiokv_create(audiokv_ctx** out, int device, size_t workspace_bytes) {
   }
   if (cudaEventCreateWithFlags(&c->plan_ready, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) != cudaSuccess ||
       cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) {
     if (c->plan_ready) cudaEventDestroy(c->plan_ready);
     if (c->fork) cudaEventDestroy(c->fork);
-    if (c->join) cudaEventDestroy(c->join);
     cudaFree(c->ws);
     delete c;
     return AUDIOKV_ECUDA;
   }
   bool ok = cudaStreamCreateWithFlags(&c->out, cudaStreamNonBlocking) == cudaSuccess &&
-            cudaEventCreateWithFlags(&c->copies_out, cudaEventDisableTiming) == cudaSuccess &&
-            cudaMallocHost(&c->stage, audiokv_ctx::kStageSlots * kStageBytes) == cudaSuccess;
-  for (int i = 0; i < audiokv_ctx::kStageSlots && ok; ++i)
-    ok = cudaEventCreateWithFlags(&c->stage_free[i], cudaEventDisableTiming) == cudaSuccess;
+            cudaEventCreateWithFlags(&c->copies_out, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < audiokv_ctx::kMaxChunks && ok; ++i)
     ok = cudaEventCreateWithFlags(&c->chunk_in[i], cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&c->chunk_done[i], cudaEventDisableTiming) == cudaSuccess;
@@ -801,7 +814,6 @@ int audiokv_destroy(audiokv_ctx* ctx) {
   cudaSetDevice(ctx->device);
   cudaEventDestroy(ctx->plan_ready);
   cudaEventDestroy(ctx->fork);
-  cudaEventDestroy(ctx->join);
   cudaStreamDestroy(ctx->side);
   if (ctx->out) cudaStreamDestroy(ctx->out);
   if (ctx->copies_out) cudaEventDestroy(ctx->copies_out);
