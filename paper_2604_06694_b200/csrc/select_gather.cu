@@ -73,8 +73,9 @@ gather_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const int32_t* __restr
               const int32_t* __restrict__ kept_idx, const uint4* __restrict__ k, const uint4* __restrict__ v,
               uint4* __restrict__ k_out, uint4* __restrict__ v_out, int log2_chunks, int elems_per_chunk,
               int head_begin, int head_end) {
-  // Launched the ordinary way, after the smoothing kernel has finished: brought in early (programmatic dependent
-  // launch) its blocks only sat on the SMs that finished their heads first, and a ragged batch ran 7 % slower.
+  // The smoothing kernel lets this one in at its end. (Let in at its start, the blocks here only sat on the SMs that finished their
+  // heads first, and a ragged batch ran 7 % slower.)
+  chain_wait();
   chain_release();  // the next pass's first scoring sweep may be set up while this kernel drains
   const int64_t first_row = cu_kept[head_begin];  // the rows of heads [head_begin, head_end)
   const int64_t total_rows = cu_kept[head_end];
@@ -145,10 +146,9 @@ cudaError_t launch_gather(const Shape& sh, const ReqDesc* d_reqs, const int32_t*
   const int chunks_per_row = sh.head_dim / elems_per_chunk;  // 8 .. 64: head_dim is 64, 128 or 256
   int log2_chunks = 0;
   while ((1 << log2_chunks) < chunks_per_row) ++log2_chunks;
-  gather_kernel<<<dim3(device_sm_count() * 8), dim3(256), 0, ln.stream>>>(sh, d_reqs, cu_kept, kept_idx, (const uint4*)k, (const uint4*)v,
-                                                         (uint4*)k_out, (uint4*)v_out, log2_chunks, elems_per_chunk,
-                                                         head_begin, head_end);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_chained(gather_kernel, dim3(device_sm_count() * 8), dim3(256), 0, ln.stream, sh, d_reqs, cu_kept, kept_idx,
+                                 (const uint4*)k, (const uint4*)v, (uint4*)k_out, (uint4*)v_out, log2_chunks, elems_per_chunk,
+                                 head_begin, head_end);
   ln.done("gather");
   return e;
 }

@@ -1284,7 +1284,6 @@ sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict
   // Launched as a programmatic dependent: the block is brought in while the kernel before it drains, reads its plan
   // (written when the plan was made, not by the kernels of the pass), and waits for that kernel only where it first
   // touches the scores.
-  chain_release();
   bool waited = false;
   if (threadIdx.x == 0) S.loaded = -1;
   const bool sel = budgets != nullptr;
@@ -1382,6 +1381,9 @@ sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict
     if (S.pl.in_smem) smooth_head<false>(sh, tables, sel, status);
     else smooth_head<true>(sh, tables, sel, status);
   }
+  // Only now: the gather, whose blocks would sit on the SMs that are through and keep the others' places, is brought in when the
+  // last block ends, and its launch is hidden behind that.
+  chain_release();
   if (n_order > static_cast<int>(gridDim.x) && threadIdx.x == 0) {
     if (atomicAdd(queue + 1, 1) == static_cast<int>(gridDim.x) - 1) {
       atomicExch(queue, 0);
