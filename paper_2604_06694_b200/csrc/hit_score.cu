@@ -193,10 +193,12 @@ hit_count_kernel(const float* __restrict__ attn, int n_steps, int n_heads, int64
     }
     if (lane == 0 && c) atomicAdd(counts + a, c);
   }
+  chain_release();  // the ratios are launched under the last rows
 }
 
 __global__ void hit_ratio_kernel(const int32_t* __restrict__ counts, int n_heads, int n_steps, int top_k,
                                  float* __restrict__ s_hit) {
+  chain_wait();
   const int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a < n_heads)
     s_hit[a] = static_cast<float>(static_cast<double>(counts[a]) / (static_cast<double>(top_k) * n_steps));
@@ -213,9 +215,10 @@ cudaError_t launch_hit_score(const float* attn, int n_steps, int n_heads, int64_
   const int grid = static_cast<int>(n_blocks < max_grid ? n_blocks : max_grid);
   hit_count_kernel<<<grid, kHitThreads, 0, ln.stream>>>(attn, n_steps, n_heads, row_stride, row_len, span, top_k, counts);
   ln.done("hit_count");
-  hit_ratio_kernel<<<(n_heads + 255) / 256, 256, 0, ln.stream>>>(counts, n_heads, n_steps, top_k, s_hit);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = launch_chained(hit_ratio_kernel, dim3((n_heads + 255) / 256), dim3(256), 0, ln.stream, counts, n_heads, n_steps, top_k, s_hit);
   ln.done("hit_ratio");
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace akv

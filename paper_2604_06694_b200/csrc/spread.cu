@@ -44,6 +44,7 @@ spread_hist_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const int32_t* __
     }
   }
   __syncthreads();
+  chain_release();  // the summaries are launched under the last heads
   for (int b = threadIdx.x; b < n_bins; b += kHistThreads)
     if (h[b]) atomicAdd(hist + static_cast<int64_t>(r) * n_bins + b, h[b]);
 }
@@ -53,6 +54,7 @@ spread_stats_kernel(const int32_t* __restrict__ hist, int n_bins, float* __restr
   __shared__ long long s_tot[kSpreadThreads / 32];
   __shared__ int s_top[kSpreadThreads / 32];
   __shared__ double s_ent[kSpreadThreads / 32];
+  chain_wait();
   const int32_t* hr = hist + static_cast<int64_t>(blockIdx.x) * n_bins;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   long long tot = 0;
@@ -111,9 +113,9 @@ cudaError_t launch_selection_spread(const Shape& sh, const ReqDesc* d_reqs, cons
                                                                        status);
   ln.done("spread_hist");
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  spread_stats_kernel<<<sh.n_req, kSpreadThreads, 0, ln.stream>>>(hist, n_bins, stats);
+  e = launch_chained(spread_stats_kernel, dim3(sh.n_req), dim3(kSpreadThreads), 0, ln.stream, hist, n_bins, stats);
   ln.done("spread_stats");
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace akv
