@@ -1314,6 +1314,7 @@ sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict
       waited = true;
     }
     if (threadIdx.x == 0) {
+      if (S.loaded != rq.fft_plan) S.loaded = -1;  // this head's work buffer may run over the roots of the plan before
       S.x = scores + base;
       S.y = smoothed ? smoothed + base : nullptr;
       S.g = scratch + static_cast<int64_t>(blockIdx.x) * scratch_per_block;
