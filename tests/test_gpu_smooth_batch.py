@@ -47,3 +47,38 @@ def test_roots_of_one_plan_survive_the_heads_of_another(B, outer, inner):
         assert torch.equal(ks[r * heads:(r + 1) * heads], ks_alone)
         assert torch.equal(y[at:at + p.numel()], alone), f"request {r}"
         at += p.numel()
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+@pytest.mark.parametrize("n", [1000, 3001, 8160, 8161, 40000])
+def test_cutoff_close_to_all_of_the_energy(B, n, mode):
+    """rho near 1 on spectra that fall off: many bins share what is left above the cut-off. It is found against the transform's
+    own total, so it may be off only by bins that hold less than a thousandth of that rest: a bin of the transform is off by
+    some 1e-7 of the root mean square of all of them, one near these cut-offs is 1e-2 to 1e-3 of it. (Against
+    a total of another source, 1e-7 of the whole energy away, the rest would be off by a tenth.)"""
+    heads, gen = 32, torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    f = torch.fft.rfft(torch.randn((heads, n), generator=gen, device="cuda").double(), dim=1)
+    x = torch.fft.irfft(f / (1 + (torch.arange(n // 2 + 1, device="cuda") / 20) ** 2), n=n, dim=1)
+    x = (x - x.amin() + 0.1 * x.std()).float().contiguous()
+    e = torch.fft.rfft(x.double(), dim=1).abs() ** 2
+    if mode == B.AUDIOKV_SMOOTH_ENERGY_NO_MEAN:
+        e[:, 0] = 0
+    cum = torch.cumsum(e, 1)
+    rest = torch.flip(torch.cumsum(torch.flip(e, [1]), 1), [1]) - e      # energy above bin k
+    for rho in (0.999, 0.9999, 0.99999, 0.999999):
+        prob = _problem(B, heads, [n], rho=rho, smooth_mode=mode)
+        _, ks = _smooth(B, prob, x.reshape(-1))
+        left = (1 - float(prob.p.rho)) * cum[:, -1:]
+        k = ks.long()[:, None]
+        assert (rest.gather(1, k) <= left * 1.001).all(), rho
+        assert (rest.gather(1, k - 1) > left * 0.999).all(), rho
+
+
+@pytest.mark.parametrize("n", [500, 1001, 1021, 2042])
+def test_cutoff_at_rho_one(B, n):
+    """All of the energy is reached at the last bin, or at once where there is none."""
+    x = torch.rand((2, n), device="cuda")
+    x[1] = 0
+    y, ks = _smooth(B, _problem(B, 2, [n], rho=1.0), x.reshape(-1))
+    assert ks.tolist() == [n // 2, 0] and bool((y[n:] == 0).all())
