@@ -321,9 +321,10 @@ int audiokv_selection_spread(audiokv_ctx* ctx, const audiokv_params* p, const in
  *   c = |S intersect span|,  r = c / top_k,  s_hit[a] = mean over the steps of r.
  * attn: device fp32 [n_steps][n_heads][row_stride], row t holds row_len[t] <= row_stride tokens (a row
  * shorter than top_k contributes all of them). row_len: device int32 [n_steps]. span: device int32
- * [n_steps][2]. top_k in 1..1024 (the paper uses 24). hit_counts: device int32 [n_heads], receives the
- * integer totals sum_t c. s_hit: device fp32 [n_heads]. The paper records the rows with hooks on a real
- * model and takes the spans from a word aligner; neither is part of this library. */
+ * [n_steps][2]. top_k in 1..1024 (the paper uses 24). A NaN ranks above every number (below them with its
+ * sign bit set). hit_counts: device int32 [n_heads], receives the integer totals sum_t c. s_hit: device fp32
+ * [n_heads]. The paper records the rows with hooks on a real model and takes the spans from a word aligner;
+ * neither is part of this library. */
 int audiokv_hit_score(audiokv_ctx* ctx, const float* attn, int32_t n_steps, int32_t n_heads, int64_t row_stride,
                       const int32_t* row_len, const int32_t* span, int32_t top_k, int32_t* hit_counts, float* s_hit,
                       audiokv_stream stream);

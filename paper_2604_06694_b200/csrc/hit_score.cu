@@ -28,9 +28,16 @@ struct HitSmem {
   uint16_t entry[kHitGroups * 32];           // groups that reach the bound: group * 32 + lane
 };
 
+// The larger value, NaN if either is NaN.
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // Exact count for a row the list cannot serve (many equal values, NaN, a large K): the k-th largest key by a search over its
 // bits, two bits a pass over the row (L2), then the span's tokens against it; of the keys equal to it the lowest
-// indices count. One warp.
+// indices count. Keys order a NaN by its bits: above every number, or below with the sign bit set. One warp.
 __device__ __noinline__ int hits_by_search(const float* __restrict__ row, int L, int k, int lo, int hi) {
   const int lane = threadIdx.x & 31;
   uint32_t key = 0u;  // the largest key x with at least k keys >= x
@@ -109,7 +116,7 @@ hit_count_kernel(const float* __restrict__ attn, int n_steps, int n_heads, int64
             v[g] = m < nvec ? __ldg(rv + m) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
           }
 #pragma unroll
-          for (int g = 0; g < 8; ++g) gm[g0 + g] = fmaxf(fmaxf(gm[g0 + g], fmaxf(v[g].x, v[g].y)), fmaxf(v[g].z, v[g].w));
+          for (int g = 0; g < 8; ++g) gm[g0 + g] = max_nan(max_nan(gm[g0 + g], max_nan(v[g].x, v[g].y)), max_nan(v[g].z, v[g].w));
         }
       }
       // Lower bound of the k-th largest value: the k-th largest of the 32 lanes' maxima (of 64, one for the even and one for
@@ -117,9 +124,10 @@ hit_count_kernel(const float* __restrict__ attn, int n_steps, int n_heads, int64
       float me = -INFINITY, mo = -INFINITY;
 #pragma unroll
       for (int g = 0; g < kHitGroups; g += 2) {
-        me = fmaxf(me, gm[g]);
-        mo = fmaxf(mo, gm[g + 1]);
+        me = max_nan(me, gm[g]);
+        mo = max_nan(mo, gm[g + 1]);
       }
+      const bool nan = isnan(me) || isnan(mo);
       const bool two = k > 32;
       if (!two) me = fmaxf(me, mo);
       int re = 0, ro = 0;  // ranks, ties to the lower lane, the even half first
@@ -169,7 +177,9 @@ hit_count_kernel(const float* __restrict__ attn, int n_steps, int n_heads, int64
       }
       const int single = lane < 3 ? lane : tail + lane - 3;  // the values before and after the pieces
       const bool have = lane < 3 ? lane < j0 : (lane < 6 && single < L);
-      take(have, have ? __ldg(row + single) : 0.f, single);
+      const float xs = have ? __ldg(row + single) : 0.f;
+      take(have, xs, single);
+      if (__any_sync(0xffffffffu, nan || isnan(xs))) n = 0;  // a NaN compares with nothing: its row is left to the search
       __syncwarp();
     }
     int c = 0;

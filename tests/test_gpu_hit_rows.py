@@ -44,3 +44,28 @@ def test_hit_score_row_shapes(B, lens, K, kind):
     assert np.array_equal(counts.cpu().numpy(), want)
     assert np.array_equal(s.cpu().numpy(), want_s.astype(np.float32))
     assert ctx.last_device_status() == 0
+
+
+@pytest.mark.parametrize("K", [24, 65])
+def test_hit_score_nan(B, K):
+    """A NaN ranks above every number (below with its sign bit set), whichever way its row takes: among the 16-byte pieces
+    or the single values before and after them, inside the span or pushing a number of the span out of the K largest."""
+    rng = np.random.default_rng(K)
+    L, places = 1003, (0, 2, 500, 1000, 1002)
+    attn = np.exp(rng.standard_normal((1, 2 * len(places) + 1, L))).astype(np.float32)
+    for i, j in enumerate(places):
+        attn[0, 2 * i, j] = np.nan
+        attn[0, 2 * i + 1, j] = -np.float32(np.nan)
+    attn[0, -1, 100:140] = np.nan                   # more of them than the smaller K
+    bits = attn.view(np.uint32)
+    key = np.where(bits >> 31, ~bits, bits | 0x80000000).astype(np.uint32)
+    for span in ((0, 120), (495, 510), (900, 1002)):
+        order = np.argsort(-key[0].astype(np.int64), axis=1, kind="stable")[:, :K]
+        want = ((order >= span[0]) & (order <= span[1])).sum(axis=1)
+        ctx = B.Context(B.Problem(B.AUDIOKV_BF16, 1, 4, 4, 64, [64], 8, (0, 0, 0, 0), (0, 64, 0)))
+        H = attn.shape[1]
+        counts, s = torch.full((H,), -1, dtype=torch.int32, device="cuda"), torch.zeros(H, device="cuda")
+        B.audiokv_hit_score(ctx, torch.from_numpy(attn).cuda(), torch.tensor([L], dtype=torch.int32, device="cuda"),
+                            torch.tensor([span], dtype=torch.int32, device="cuda"), K, counts, s)
+        torch.cuda.synchronize()
+        assert np.array_equal(counts.cpu().numpy(), want)
