@@ -144,9 +144,11 @@ int audiokv_create(audiokv_ctx** ctx, int device, size_t workspace_bytes);
  * Stream capture: every device-buffer entry point may be recorded into a CUDA graph, once the
  * context has seen its params in a call OUTSIDE capture (the first call with a new shape brings
  * the plan to the device, which a graph must not do over again at every replay; inside a capture it
- * returns AUDIOKV_ECUDA and says so in audiokv_last_cuda_error). Every kernel of audiokv_evict goes to the caller's stream
- * (some as programmatic dependents of the one before). The host-buffer call waits on the host and
- * cannot be captured. */
+ * returns AUDIOKV_ECUDA and says so in audiokv_last_cuda_error). The graph reads the plan where that
+ * call put it, so it may be replayed until the context is given other params; audiokv_evict_host with
+ * the same ones leaves it as it is. Every kernel of audiokv_evict goes to the caller's stream (some as
+ * programmatic dependents of the one before). The host-buffer call waits on the host and cannot be
+ * captured. */
 
 /* Frees the workspace. The caller makes sure no call on this context is still running. */
 int audiokv_destroy(audiokv_ctx* ctx);

@@ -23,23 +23,32 @@ constexpr int kHostChunks = 8;          // the host-buffer call evicts one reque
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
-struct Layout {  // byte offsets inside the workspace; status .. ctas, up to blob_end, are uploaded as one piece with a plan
+// Byte offsets inside the workspace; status .. ctas, up to blob_end, are uploaded as one piece with a plan. What only
+// audiokv_evict_host needs lies behind the rest, so that the rest stays where a captured graph has it.
+struct Layout {
   size_t status, reqs, plans, order, units, ctas, blob_end, tables, stats, exps, fft_scratch, scores, kstar, aux, end;
+  size_t host_units, host_ctas, host_stats, host_end;
+};
+
+// Runs of the tensor-core scoring: both sweeps of every schedule.
+struct ScoreTables {
+  std::vector<ScoreUnit> units;
+  std::vector<int32_t> ctas;             // per-CTA run offsets of every (schedule, sweep)
+  std::vector<ScoreSchedule> schedules;
+  int parts = 1;                         // statistics slots per head
 };
 
 struct Plan {
   bool valid = false;
-  bool host_call = false;       // has the schedules of audiokv_evict_host
+  bool host_call = false;       // has the schedules of audiokv_evict_host, in host_score
   audiokv_params p{};
   std::vector<int32_t> seq_len;
   std::vector<int64_t> kv_off, q_off;
   Shape sh{};
   std::vector<ReqDesc> reqs;
   std::vector<FftPlan> fft;
-  std::vector<ScoreUnit> units;          // runs of the tensor-core scoring: both sweeps of every schedule
-  std::vector<int32_t> score_ctas;       // per-CTA run offsets of every (schedule, sweep)
-  std::vector<ScoreSchedule> schedules;  // one per run of requests, plus one per chunk of layers of a single request
-  int score_parts = 1;                   // statistics slots per head of the tensor-core scoring
+  ScoreTables score;            // one schedule per run of requests
+  ScoreTables host_score;       // one per chunk of layers of a single request
   std::vector<int32_t> sss_order;  // heads in the order the smoothing blocks take them (see build_plan)
   int64_t table_len = 0;        // float2 elements
   int64_t scores_len = 0;
@@ -66,6 +75,7 @@ struct audiokv_ctx {
   size_t ws_bytes = 0;
   Plan plan;
   bool plan_uploaded = false;
+  bool host_uploaded = false;             // plan.host_score too
   bool plan_fresh = false;                // the call at hand put the plan on the device: its last launch was launch_fft_tables
   uint64_t plan_id = 0;      // counts plan rebuilds
   ScoreMapCache score_maps;
@@ -273,16 +283,14 @@ int host_chunk_layer(int n_layers, int c) { return static_cast<int>(static_cast<
 // runs of consecutive tiles of one head. Sweep 1 walks the heads in order over all L keys (the runs of a head number
 // its statistics slots); sweep 2 walks them backwards over the prefix keys (the heads sweep 1 touched last are the
 // ones still in L2).
-void build_score_schedules(const audiokv_params* p, bool host_call, Plan* pl) {
-  const Shape& sh = pl->sh;
-  pl->units.clear();
-  pl->score_ctas.clear();
-  pl->schedules.clear();
-  pl->score_parts = 1;
+// chunks: not the schedules of whole requests but those of audiokv_evict_host, which evicts one request in chunks of layers
+void build_score_schedules(const Plan& pl, bool chunks, ScoreTables* tab) {
+  const Shape& sh = pl.sh;
+  *tab = ScoreTables{};
   if (!score_umma_takes(sh)) return;
   // a head whose W * G query rows exceed the kernel's Q tile is scored in chunks of window rows (runs of their own)
   const int w_chunk = score_window_chunk(sh);
-  const int n_wchunks = (p->window + w_chunk - 1) / w_chunk;
+  const int n_wchunks = (sh.window + w_chunk - 1) / w_chunk;
   std::vector<int32_t> parts_of(static_cast<size_t>(sh.total_heads) * n_wchunks, 0);
   auto add = [&](bool whole, int r_begin, int r_end, int head_begin, int head_end) {
     ScoreSchedule sc{};
@@ -297,24 +305,24 @@ void build_score_schedules(const audiokv_params* p, bool host_call, Plan* pl) {
     std::vector<Q> qs;  // the (head, window chunk) pairs of this schedule, in sweep-1 order
     for (int r = r_begin; r < r_end; ++r)
       for (int hr = whole ? 0 : head_begin; hr < (whole ? sh.heads_per_req : head_end); ++hr)
-        for (int ch = 0; ch < n_wchunks; ++ch) qs.push_back(Q{pl->reqs[r].head_base + hr, r, hr, ch});
+        for (int ch = 0; ch < n_wchunks; ++ch) qs.push_back(Q{pl.reqs[r].head_base + hr, r, hr, ch});
     for (int sweep = 1; sweep <= 2; ++sweep) {
       if (sweep == 2) std::reverse(qs.begin(), qs.end());
       int64_t total = 0;
       for (const Q& x : qs) {
-        const int range = sweep == 1 ? pl->reqs[x.r].L : pl->reqs[x.r].P;
+        const int range = sweep == 1 ? pl.reqs[x.r].L : pl.reqs[x.r].P;
         total += (range + 127) / 128;
       }
       const int grid = static_cast<int>(total < kScoreCtas ? total : kScoreCtas);
-      sc.unit_off[sweep - 1] = static_cast<int32_t>(pl->units.size());
-      sc.cta_off[sweep - 1] = static_cast<int32_t>(pl->score_ctas.size());
+      sc.unit_off[sweep - 1] = static_cast<int32_t>(tab->units.size());
+      sc.cta_off[sweep - 1] = static_cast<int32_t>(tab->ctas.size());
       sc.grid[sweep - 1] = grid;
-      const size_t first = pl->units.size();
+      const size_t first = tab->units.size();
       int64_t tile = 0;  // tiles before the current head in the sweep's sequence
       int c = 0;         // CTA whose range holds the next tile
-      pl->score_ctas.push_back(0);
+      tab->ctas.push_back(0);
       for (const Q& x : qs) {
-        const ReqDesc& d = pl->reqs[x.r];
+        const ReqDesc& d = pl.reqs[x.r];
         const int range = sweep == 1 ? d.L : d.P;
         const int n_tiles = (range + 127) / 128;
         int t = 0, part = 0;
@@ -322,52 +330,55 @@ void build_score_schedules(const audiokv_params* p, bool host_call, Plan* pl) {
           // the CTA that owns tile `tile + t`, and how far its range reaches into this head
           while (c + 1 < grid && (static_cast<int64_t>(c + 1) * total) / grid <= tile + t) {
             ++c;
-            pl->score_ctas.push_back(static_cast<int32_t>(pl->units.size() - first));
+            tab->ctas.push_back(static_cast<int32_t>(tab->units.size() - first));
           }
           const int64_t c_end = (static_cast<int64_t>(c + 1) * total) / grid;
           const int take = static_cast<int>(std::min<int64_t>(n_tiles - t, c_end - (tile + t)));
           ScoreUnit un{};
           un.u = x.u;
           un.r = x.r;
-          un.l = x.hr / p->n_kv_heads;
-          un.h = x.hr % p->n_kv_heads;
+          un.l = x.hr / sh.n_kv_heads;
+          un.h = x.hr % sh.n_kv_heads;
           un.part = part++;
           un.kt0 = t * 128;
           un.n_tiles = take;
           un.P = d.P;
           un.score_base = d.score_offset + static_cast<int64_t>(x.hr) * d.P;
           un.w0 = x.ch * w_chunk;
-          un.wn = p->window - un.w0 < w_chunk ? p->window - un.w0 : w_chunk;
+          un.wn = sh.window - un.w0 < w_chunk ? sh.window - un.w0 : w_chunk;
           un.qid = x.u * n_wchunks + x.ch;
           un.head_parts = 0;  // set below
-          pl->units.push_back(un);
+          tab->units.push_back(un);
           t += take;
         }
         if (sweep == 1) {
           parts_of[static_cast<size_t>(x.u) * n_wchunks + x.ch] = part;
-          pl->score_parts = part > pl->score_parts ? part : pl->score_parts;
+          tab->parts = part > tab->parts ? part : tab->parts;
         }
         tile += n_tiles;
       }
-      while (static_cast<int>(pl->score_ctas.size()) - sc.cta_off[sweep - 1] < grid + 1)
-        pl->score_ctas.push_back(static_cast<int32_t>(pl->units.size() - first));
-      for (size_t i = first; i < pl->units.size(); ++i) pl->units[i].head_parts = parts_of[pl->units[i].qid];
+      while (static_cast<int>(tab->ctas.size()) - sc.cta_off[sweep - 1] < grid + 1)
+        tab->ctas.push_back(static_cast<int32_t>(tab->units.size() - first));
+      for (size_t i = first; i < tab->units.size(); ++i) tab->units[i].head_parts = parts_of[tab->units[i].qid];
     }
-    pl->schedules.push_back(sc);
+    tab->schedules.push_back(sc);
   };
-  const int cap = score_map_chunk(p->n_req);
-  for (int r0 = 0; r0 < p->n_req; r0 += cap) add(true, r0, r0 + cap < p->n_req ? r0 + cap : p->n_req, 0, 0);
-  if (host_call && p->n_req == 1 && p->n_layers > 1) {
-    // the host-buffer call evicts one request in chunks of layers
-    const int n_chunks = host_chunks(p->n_layers);
+  if (!chunks) {
+    const int cap = score_map_chunk(sh.n_req);
+    for (int r0 = 0; r0 < sh.n_req; r0 += cap) add(true, r0, r0 + cap < sh.n_req ? r0 + cap : sh.n_req, 0, 0);
+  } else if (sh.n_req == 1 && sh.n_layers > 1) {
+    const int n_chunks = host_chunks(sh.n_layers);
     for (int c = 0; c < n_chunks; ++c)
-      add(false, 0, 1, host_chunk_layer(p->n_layers, c) * p->n_kv_heads, host_chunk_layer(p->n_layers, c + 1) * p->n_kv_heads);
+      add(false, 0, 1, host_chunk_layer(sh.n_layers, c) * sh.n_kv_heads, host_chunk_layer(sh.n_layers, c + 1) * sh.n_kv_heads);
   }
 }
 
-// host_call: with the schedules by chunks of layers that audiokv_evict_host runs through (eight more schedules of one request;
-// a serving loop whose every prompt brings a new length builds a plan a call, so the others go without).
-int build_plan(const audiokv_params* p, bool host_call, Plan* pl) {
+// Softmax statistics of the tensor-core kernels: [head][part][group][row].
+size_t stat_entries(const Plan& pl, const ScoreTables& tab) {
+  return static_cast<size_t>(pl.sh.total_heads) * tab.parts * score_stat_sets() * pl.sh.window * pl.sh.group;
+}
+
+int build_plan(const audiokv_params* p, Plan* pl) {
   int rc = check_params(p);
   if (rc) return rc;
   pl->valid = false;
@@ -444,8 +455,9 @@ int build_plan(const audiokv_params* p, bool host_call, Plan* pl) {
     d.fft_plan = it->second;
   }
   pl->n_slab = (pl->max_L + kSlabKeys - 1) / kSlabKeys;
-  pl->host_call = host_call;
-  build_score_schedules(p, host_call, pl);
+  build_score_schedules(*pl, false, &pl->score);
+  pl->host_score = ScoreTables{};
+  pl->host_call = false;
   // one block per head at a time, as many blocks as the planning SM count (the plan, and with it the workspace size,
   // does not depend on the device)
   pl->sss_grid = sh.total_heads < kScoreCtas ? sh.total_heads : kScoreCtas;
@@ -479,14 +491,14 @@ int build_plan(const audiokv_params* p, bool host_call, Plan* pl) {
   L.reqs = off;        off = align_up(off + sizeof(ReqDesc) * pl->reqs.size());
   L.plans = off;       off = align_up(off + sizeof(FftPlan) * pl->fft.size());
   L.order = off;       off = align_up(off + sizeof(int32_t) * pl->sss_order.size());
-  L.units = off;       off = align_up(off + sizeof(ScoreUnit) * pl->units.size());
-  L.ctas = off;        off = align_up(off + sizeof(int32_t) * pl->score_ctas.size());
+  L.units = off;       off = align_up(off + sizeof(ScoreUnit) * pl->score.units.size());
+  L.ctas = off;        off = align_up(off + sizeof(int32_t) * pl->score.ctas.size());
   L.blob_end = off;
   L.tables = off;      off = align_up(off + sizeof(float2) * static_cast<size_t>(pl->table_len));
   {
-    // softmax statistics: [head][slab][row] for the FMA kernels, [head][part][group][row] for the tensor-core ones
+    // softmax statistics: [head][slab][row] for the FMA kernels
     const int rows = sh.window * sh.group;
-    size_t entries = static_cast<size_t>(sh.total_heads) * std::max<size_t>(pl->n_slab, static_cast<size_t>(pl->score_parts) * score_stat_sets()) * rows;
+    size_t entries = std::max(static_cast<size_t>(sh.total_heads) * pl->n_slab * rows, stat_entries(*pl, pl->score));
     // the FMA kernels keep a chunk's exponentials when they are the ones that score (see score_simt.cu)
     pl->exps_len = score_umma_takes(sh) ? 0 : score_simt_exps_len(sh.total_heads, pl->max_L, rows, sh.head_dim);
     entries = std::max(entries, static_cast<size_t>(pl->exps_len / score_simt_tile_keys(sh.head_dim)));
@@ -497,9 +509,24 @@ int build_plan(const audiokv_params* p, bool host_call, Plan* pl) {
   L.scores = off;      off = align_up(off + sizeof(float) * static_cast<size_t>(pl->scores_len));
   L.kstar = off;       off = align_up(off + sizeof(int32_t) * static_cast<size_t>(sh.total_heads));
   L.aux = off;         off = align_up(off + 2 * sizeof(int32_t) * static_cast<size_t>(sh.total_heads));  // audiokv_reevict
-  L.end = off;
+  L.end = L.host_end = off;
   pl->valid = true;
   return AUDIOKV_OK;
+}
+
+// The schedules by chunks of layers that audiokv_evict_host runs through, and their place in the workspace (a serving loop whose
+// every prompt brings a new length builds a plan a call, so the others go without).
+void add_host_part(Plan* pl) {
+  build_score_schedules(*pl, true, &pl->host_score);
+  Layout& L = pl->lay;
+  size_t off = L.end;
+  if (!pl->host_score.units.empty()) {
+    L.host_units = off;  off = align_up(off + sizeof(ScoreUnit) * pl->host_score.units.size());
+    L.host_ctas = off;   off = align_up(off + sizeof(int32_t) * pl->host_score.ctas.size());
+    L.host_stats = off;  off = align_up(off + sizeof(float2) * stat_entries(*pl, pl->host_score));
+  }
+  L.host_end = off;
+  pl->host_call = true;
 }
 
 int cuda_fail(audiokv_ctx* ctx, cudaError_t e) {
@@ -528,14 +555,15 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
   if (!ctx) return AUDIOKV_EINVAL;
   cudaError_t e = cudaSetDevice(ctx->device);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
-  if (!same_plan(ctx->plan, p) || (host_call && !ctx->plan.host_call)) {
-    int rc = build_plan(p, host_call, &ctx->plan);
+  if (!same_plan(ctx->plan, p)) {
+    int rc = build_plan(p, &ctx->plan);
     ctx->plan_id += 1;
     if (rc) return rc;
-    ctx->plan_uploaded = false;
+    ctx->plan_uploaded = ctx->host_uploaded = false;
   }
   Plan& pl = ctx->plan;
-  if (pl.lay.end > ctx->ws_bytes) return AUDIOKV_EWORKSPACE;
+  if (host_call && !pl.host_call) add_host_part(&pl);
+  if ((host_call ? pl.lay.host_end : pl.lay.end) > ctx->ws_bytes) return AUDIOKV_EWORKSPACE;
   pl.sh.page_table = p->page_size ? p->page_table : nullptr;  // device data of this call, not part of the plan
   pl.sh.page_status = reinterpret_cast<int*>(ctx->ws + pl.lay.status);
   ctx->plan_fresh = !ctx->plan_uploaded;
@@ -571,8 +599,8 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
     };
     put(pl.lay.reqs, pl.reqs.data(), sizeof(ReqDesc) * pl.reqs.size());
     put(pl.lay.plans, pl.fft.data(), sizeof(FftPlan) * pl.fft.size());
-    put(pl.lay.units, pl.units.data(), sizeof(ScoreUnit) * pl.units.size());
-    put(pl.lay.ctas, pl.score_ctas.data(), sizeof(int32_t) * pl.score_ctas.size());
+    put(pl.lay.units, pl.score.units.data(), sizeof(ScoreUnit) * pl.score.units.size());
+    put(pl.lay.ctas, pl.score.ctas.data(), sizeof(int32_t) * pl.score.ctas.size());
     put(pl.lay.order, pl.sss_order.data(), sizeof(int32_t) * pl.sss_order.size());
     if (!inlined && (e = cudaMemcpyAsync(ctx->ws, src, blob, cudaMemcpyHostToDevice, stream)) != cudaSuccess) return cuda_fail(ctx, e);
     if (staged && (e = cudaEventRecord(ctx->stage_free[slot], stream)) != cudaSuccess) return cuda_fail(ctx, e);
@@ -598,6 +626,17 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
       ctx->plan_settled = true;
     }
   }
+  if (host_call && !ctx->host_uploaded) {
+    // from pageable memory: this call waits on the host in any case
+    const ScoreTables& t = pl.host_score;
+    if (!t.units.empty() &&
+        ((e = cudaMemcpyAsync(ctx->ws + pl.lay.host_units, t.units.data(), sizeof(ScoreUnit) * t.units.size(),
+                              cudaMemcpyHostToDevice, stream)) != cudaSuccess ||
+         (e = cudaMemcpyAsync(ctx->ws + pl.lay.host_ctas, t.ctas.data(), sizeof(int32_t) * t.ctas.size(),
+                              cudaMemcpyHostToDevice, stream)) != cudaSuccess))
+      return cuda_fail(ctx, e);
+    ctx->host_uploaded = true;
+  }
   return AUDIOKV_OK;
 }
 
@@ -615,18 +654,20 @@ const ReqDesc* d_reqs(audiokv_ctx* c) { return reinterpret_cast<const ReqDesc*>(
 // The first 64 bytes of the workspace: the status word, and from int 4 on the queue of the smoothing kernel.
 int* d_status(audiokv_ctx* c) { return reinterpret_cast<int*>(c->ws + c->plan.lay.status); }
 
-// head_end >= 0 (one request, tensor-core path only): the heads [head_begin, head_end) alone.
+// head_end >= 0 (one request, tensor-core path only): the heads [head_begin, head_end) alone, a chunk of audiokv_evict_host.
 int do_score(audiokv_ctx* ctx, const void* q, const void* k, float* scores, cudaStream_t stream, int head_begin = 0,
              int head_end = -1, bool beside = false) {
   Plan& pl = ctx->plan;
   Launch ln{stream, &ctx->launches, &ctx->prof};
   float2* stats = reinterpret_cast<float2*>(ctx->ws + pl.lay.stats);
   cudaError_t e = cudaErrorNotSupported;
-  if (score_umma_takes(pl.sh))
-  {
-    e = launch_score_umma(pl.sh, pl.reqs.data(), reinterpret_cast<const ScoreUnit*>(ctx->ws + pl.lay.units),
-                          reinterpret_cast<const int32_t*>(ctx->ws + pl.lay.ctas), pl.schedules.data(),
-                          static_cast<int>(pl.schedules.size()), q, k, scores, stats, pl.score_parts, d_status(ctx), ln,
+  if (score_umma_takes(pl.sh)) {
+    const bool chunk = head_end >= 0;
+    const ScoreTables& t = chunk ? pl.host_score : pl.score;
+    e = launch_score_umma(pl.sh, pl.reqs.data(), reinterpret_cast<const ScoreUnit*>(ctx->ws + (chunk ? pl.lay.host_units : pl.lay.units)),
+                          reinterpret_cast<const int32_t*>(ctx->ws + (chunk ? pl.lay.host_ctas : pl.lay.ctas)), t.schedules.data(),
+                          static_cast<int>(t.schedules.size()), q, k, scores,
+                          chunk ? reinterpret_cast<float2*>(ctx->ws + pl.lay.host_stats) : stats, t.parts, d_status(ctx), ln,
                           head_begin, head_end, &ctx->score_maps, ctx->plan_id, beside);
   }
   if (head_end >= 0 && e != cudaSuccess) return cuda_fail(ctx, e);  // no head ranges in the FMA kernel
@@ -708,7 +749,7 @@ HostStaging host_staging(const Plan& pl, int64_t q_elems, int64_t kv_elems, cons
   const size_t es = esize(pl.sh.dtype), TH = static_cast<size_t>(pl.sh.total_heads);
   for (int r = 0; r < pl.sh.n_req; ++r) h.rows += total_budget[r];
   const size_t row_bytes = static_cast<size_t>(h.rows) * pl.sh.head_dim * es;
-  size_t off = pl.lay.end;
+  size_t off = pl.lay.host_end;
   h.q = off;           off = align_up(off + q_elems * es);
   h.k = off;           off = align_up(off + kv_elems * es);
   h.v = off;           off = align_up(off + kv_elems * es);
@@ -760,14 +801,15 @@ int64_t audiokv_scores_len(const audiokv_params* p) {
 
 size_t audiokv_workspace_bytes(const audiokv_params* p) {
   Plan pl;
-  if (build_plan(p, true, &pl)) return 0;
+  if (build_plan(p, &pl)) return 0;
   return pl.lay.end;
 }
 
 size_t audiokv_workspace_bytes_host(const audiokv_params* p, int64_t q_elems, int64_t kv_elems,
                                     const int64_t* total_budget) {
   Plan pl;
-  if (build_plan(p, true, &pl) || !total_budget || q_elems < 0 || kv_elems < 0) return 0;
+  if (build_plan(p, &pl) || !total_budget || q_elems < 0 || kv_elems < 0) return 0;
+  add_host_part(&pl);
   return host_staging(pl, q_elems, kv_elems, total_budget).end;
 }
 

@@ -1,7 +1,6 @@
 """audiokv_evict under CUDA graph capture: a serving loop records the pass once and replays it. The first call (which
 uploads the plan and builds the tables) runs outside the capture; the captured call must launch the same kernels
-(the allocation forks to the context's side stream and joins back) and a replay must reproduce the eager result on
-new contents of the same buffers."""
+and a replay must reproduce the eager result on new contents of the same buffers."""
 import dataclasses
 
 import numpy as np
@@ -87,3 +86,35 @@ def test_capture_before_the_first_call_is_refused(B):
     graph.replay()
     torch.cuda.synchronize()
     assert float(sc[0]) == 1.0
+
+
+def test_graph_outlives_a_host_call_with_the_same_params(B):
+    """audiokv_evict_host needs more schedules than the captured pass: they must not move what the graph points to."""
+    spec = dataclasses.replace(wl.config(1), seq_lens=[1301], audio_frac=[0.9])
+    w = wl.generate(spec, seed=5, layers=3)
+    prob = B.Problem.from_workload(w)
+    TH, rows = prob.total_heads, int(w.total_budget.sum())
+    tb = [int(x) for x in w.total_budget]
+    host = [w.as_torch(a) for a in (w.q, w.k, w.v)] + [torch.from_numpy(w.head_scores)]
+    dev = [t.cuda() for t in host]
+    ctx = B.Context(prob, workspace_bytes=B.audiokv_workspace_bytes_host(prob, host[0].numel(), host[1].numel(), tb))
+
+    def mk(device):
+        return (*(torch.zeros((rows, spec.head_dim), dtype=torch.bfloat16, device=device) for _ in range(2)),
+                *(torch.zeros(n, dtype=torch.int32, device=device) for n in (rows, TH, TH + 1)))
+
+    eager, out, back = mk("cuda"), mk("cuda"), mk("cpu")
+    B.audiokv_evict(ctx, prob, *dev, tb, *eager)
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=side):
+        B.audiokv_evict(ctx, prob, *dev, tb, *out)
+    for turn in range(2):
+        B.audiokv_evict_host(ctx, prob, *host, tb, *back)
+        for t in out:
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert ctx.last_device_status() == 0
+        for a, b, c in zip(eager, out, back):
+            assert torch.equal(a, b) and torch.equal(a.cpu(), c), turn
