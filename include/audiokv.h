@@ -127,7 +127,10 @@ int64_t audiokv_budget_from_ratio(double c, int32_t n_heads_total, int32_t seq_l
 int64_t audiokv_scores_len(const audiokv_params* p);
 
 /* Bytes of workspace audiokv_create must be given so that every call below works for
- * these params (0 on invalid params). Grows with sum_r L_r; a few MB per 100k tokens. */
+ * these params (0 on invalid params): a few MB per 100k tokens, scratch for transforms of lengths that
+ * do not fit on chip, and, where the FMA kernels score (see audiokv_last_score_path), up to 130 MB to keep
+ * exponentials in instead of computing them twice. Without that last part, or with some of it, every call works
+ * as well, only slower. A context for several problems takes the largest of their sizes. */
 size_t audiokv_workspace_bytes(const audiokv_params* p);
 
 /* ---- context ------------------------------------------------------------------------- */

@@ -26,7 +26,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // Byte offsets inside the workspace; status .. ctas, up to blob_end, are uploaded as one piece with a plan. What only
 // audiokv_evict_host needs lies behind the rest, so that the rest stays where a captured graph has it.
 struct Layout {
-  size_t status, reqs, plans, order, units, ctas, blob_end, tables, stats, exps, fft_scratch, scores, kstar, aux, end;
+  size_t status, reqs, plans, order, units, ctas, blob_end, tables, stats, fft_scratch, scores, kstar, aux, end;
   size_t host_units, host_ctas, host_stats, host_end;
 };
 
@@ -54,7 +54,7 @@ struct Plan {
   int64_t scores_len = 0;
   int max_L = 0, max_P = 0;
   int n_slab = 0;
-  int64_t exps_len = 0;         // floats
+  size_t score_room = 0;        // bytes of workspace behind everything else that the FMA scoring puts to use
   int sss_grid = 0;
   size_t sss_smem = 0;
   int64_t scratch_per_block = 0;  // float2 elements
@@ -498,13 +498,10 @@ int build_plan(const audiokv_params* p, Plan* pl) {
   {
     // softmax statistics: [head][slab][row] for the FMA kernels
     const int rows = sh.window * sh.group;
-    size_t entries = std::max(static_cast<size_t>(sh.total_heads) * pl->n_slab * rows, stat_entries(*pl, pl->score));
-    // the FMA kernels keep a chunk's exponentials when they are the ones that score (see score_simt.cu)
-    pl->exps_len = score_umma_takes(sh) ? 0 : score_simt_exps_len(sh.total_heads, pl->max_L, rows, sh.head_dim);
-    entries = std::max(entries, static_cast<size_t>(pl->exps_len / score_simt_tile_keys(sh.head_dim)));
+    const size_t entries = std::max(static_cast<size_t>(sh.total_heads) * pl->n_slab * rows, stat_entries(*pl, pl->score));
     L.stats = off;     off = align_up(off + sizeof(float2) * entries);
+    pl->score_room = score_umma_takes(sh) ? 0 : score_simt_room(sh.total_heads, pl->max_L, rows, sh.head_dim);
   }
-  L.exps = off;        off = align_up(off + sizeof(float) * static_cast<size_t>(pl->exps_len));
   L.fft_scratch = off; off = align_up(off + sizeof(float2) * static_cast<size_t>(pl->scratch_per_block) * pl->sss_grid);
   L.scores = off;      off = align_up(off + sizeof(float) * static_cast<size_t>(pl->scores_len));
   L.kstar = off;       off = align_up(off + sizeof(int32_t) * static_cast<size_t>(sh.total_heads));
@@ -654,8 +651,9 @@ const ReqDesc* d_reqs(audiokv_ctx* c) { return reinterpret_cast<const ReqDesc*>(
 // The first 64 bytes of the workspace: the status word, and from int 4 on the queue of the smoothing kernel.
 int* d_status(audiokv_ctx* c) { return reinterpret_cast<int*>(c->ws + c->plan.lay.status); }
 
-// head_end >= 0 (one request, tensor-core path only): the heads [head_begin, head_end) alone, a chunk of audiokv_evict_host.
-int do_score(audiokv_ctx* ctx, const void* q, const void* k, float* scores, cudaStream_t stream, int head_begin = 0,
+// used: bytes at the front of the workspace that the call needs; the FMA scoring may have the rest. head_end >= 0 (one request,
+// tensor-core path only): the heads [head_begin, head_end) alone, a chunk of audiokv_evict_host.
+int do_score(audiokv_ctx* ctx, const void* q, const void* k, float* scores, cudaStream_t stream, size_t used, int head_begin = 0,
              int head_end = -1, bool beside = false) {
   Plan& pl = ctx->plan;
   Launch ln{stream, &ctx->launches, &ctx->prof};
@@ -676,9 +674,8 @@ int do_score(audiokv_ctx* ctx, const void* q, const void* k, float* scores, cuda
     // fp32 inputs (which must not be rounded to TF32), a GQA group above 256 query heads, or strides the copy
     // engine cannot take; audiokv_last_score_path tells the caller which route ran
     ctx->score_path = 2;
-    float* exps = pl.exps_len ? reinterpret_cast<float*>(ctx->ws + pl.lay.exps) : nullptr;
-    e = launch_score_simt(pl.sh, d_reqs(ctx), q, k, scores, stats, pl.n_slab, kSlabKeys, exps, pl.exps_len, pl.max_L, ln,
-                          beside && !score_umma_takes(pl.sh));
+    e = launch_score_simt(pl.sh, d_reqs(ctx), q, k, scores, stats, pl.n_slab, kSlabKeys, ctx->ws + used,
+                          std::min(pl.score_room, ctx->ws_bytes - used), pl.max_L, ln, beside && !score_umma_takes(pl.sh));
   }
   return e == cudaSuccess ? AUDIOKV_OK : cuda_fail(ctx, e);
 }
@@ -802,7 +799,7 @@ int64_t audiokv_scores_len(const audiokv_params* p) {
 size_t audiokv_workspace_bytes(const audiokv_params* p) {
   Plan pl;
   if (build_plan(p, &pl)) return 0;
-  return pl.lay.end;
+  return pl.lay.end + pl.score_room;
 }
 
 size_t audiokv_workspace_bytes_host(const audiokv_params* p, int64_t q_elems, int64_t kv_elems,
@@ -810,7 +807,7 @@ size_t audiokv_workspace_bytes_host(const audiokv_params* p, int64_t q_elems, in
   Plan pl;
   if (build_plan(p, &pl) || !total_budget || q_elems < 0 || kv_elems < 0) return 0;
   add_host_part(&pl);
-  return host_staging(pl, q_elems, kv_elems, total_budget).end;
+  return host_staging(pl, q_elems, kv_elems, total_budget).end + pl.score_room;
 }
 
 int audiokv_create(audiokv_ctx** out, int device, size_t workspace_bytes) {
@@ -937,7 +934,7 @@ int audiokv_score(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int rc = prepare(ctx, p, s);
   if (rc) return rc;
-  return do_score(ctx, q_win, k, scores, s);
+  return do_score(ctx, q_win, k, scores, s, ctx->plan.lay.end);
 }
 
 int audiokv_smooth(audiokv_ctx* ctx, const audiokv_params* p, const float* scores, float* smoothed,
@@ -969,9 +966,12 @@ int audiokv_select_gather(audiokv_ctx* ctx, const audiokv_params* p, const float
   return do_select_gather(ctx, smoothed, budgets, cu_kept, k, v, k_out, v_out, kept_idx, s);
 }
 
-int audiokv_evict(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, const void* k, const void* v,
-                  const float* head_scores, const int64_t* total_budget, void* k_out, void* v_out,
-                  int32_t* kept_idx, int32_t* budgets, int32_t* cu_kept, audiokv_stream stream) {
+namespace {
+
+// audiokv_evict; used: bytes at the front of the workspace that the caller needs, if more than the plan's.
+int evict_pass(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, const void* k, const void* v,
+               const float* head_scores, const int64_t* total_budget, void* k_out, void* v_out,
+               int32_t* kept_idx, int32_t* budgets, int32_t* cu_kept, audiokv_stream stream, size_t used) {
   if (!q_win || !k || !v || !head_scores || !total_budget || !k_out || !v_out || !kept_idx || !budgets || !cu_kept)
     return AUDIOKV_EINVAL;
   if (!aligned16(q_win) || !aligned16(k) || !aligned16(v) || !aligned16(k_out) || !aligned16(v_out))
@@ -990,12 +990,20 @@ int audiokv_evict(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, 
   // timing on, every kernel waits for the one before it.
   const bool beside = !ctx->prof.on;
   rc = do_allocate(ctx, head_scores, total_budget, budgets, cu_kept, s, ctx->plan_fresh && !ctx->prof.on);
-  if (!rc) rc = do_score(ctx, q_win, k, ws_scores, s, 0, -1, beside);
+  if (!rc) rc = do_score(ctx, q_win, k, ws_scores, s, std::max(used, pl.lay.end), 0, -1, beside);
   if (rc) return rc;
   // the pooling variants hand their result to the selection through the score buffer itself
   float* ws_smoothed = pl.sh.smooth_mode >= AUDIOKV_SMOOTH_AVG_POOL ? ws_scores : nullptr;
   if ((rc = do_smooth(ctx, ws_scores, ws_smoothed, ws_kstar, budgets, cu_kept, kept_idx, s))) return rc;
   return do_gather(ctx, cu_kept, kept_idx, k, v, k_out, v_out, s);
+}
+
+}  // namespace
+
+int audiokv_evict(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, const void* k, const void* v,
+                  const float* head_scores, const int64_t* total_budget, void* k_out, void* v_out,
+                  int32_t* kept_idx, int32_t* budgets, int32_t* cu_kept, audiokv_stream stream) {
+  return evict_pass(ctx, p, q_win, k, v, head_scores, total_budget, k_out, v_out, kept_idx, budgets, cu_kept, stream, 0);
 }
 
 int audiokv_evict_kstar(audiokv_ctx* ctx, int32_t* kstar, audiokv_stream stream) {
@@ -1025,7 +1033,7 @@ int audiokv_evict_budgeted(audiokv_ctx* ctx, const audiokv_params* p, const void
   Launch ln{s, &ctx->launches, &ctx->prof};
   cudaError_t e = launch_budget_prefix(pl.sh, d_reqs(ctx), budgets, ws_budgets, cu_kept, d_status(ctx), ln);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
-  if ((rc = do_score(ctx, q_win, k, ws_scores, s, 0, -1, !ctx->prof.on))) return rc;
+  if ((rc = do_score(ctx, q_win, k, ws_scores, s, pl.lay.end, 0, -1, !ctx->prof.on))) return rc;
   float* ws_smoothed = pl.sh.smooth_mode >= AUDIOKV_SMOOTH_AVG_POOL ? ws_scores : nullptr;
   if ((rc = do_smooth(ctx, ws_scores, ws_smoothed, ws_kstar, ws_budgets, cu_kept, kept_idx, s))) return rc;
   return do_gather(ctx, cu_kept, kept_idx, k, v, k_out, v_out, s);
@@ -1213,7 +1221,7 @@ int audiokv_evict_host(audiokv_ctx* ctx, const audiokv_params* p, const void* q_
       if ((e = cudaEventRecord(ctx->chunk_in[c], ctx->side)) != cudaSuccess) return cuda_fail(ctx, e);
       if ((e = cudaStreamWaitEvent(s, ctx->chunk_in[c], 0)) != cudaSuccess) return cuda_fail(ctx, e);
       const int u0 = l0 * Hkv, u1 = l1 * Hkv;
-      if ((rc = do_score(ctx, dq, dk, ws_scores, s, u0, u1))) return rc;
+      if ((rc = do_score(ctx, dq, dk, ws_scores, s, hs.end, u0, u1))) return rc;
       if ((rc = do_smooth(ctx, ws_scores, ws_smoothed, ws_kstar, d_budgets, d_cu, reinterpret_cast<int32_t*>(dki), s, u0, u1)))
         return rc;
       if ((rc = do_gather(ctx, d_cu, reinterpret_cast<int32_t*>(dki), dk, v_src, dko, dvo, s, u0, u1))) return rc;
@@ -1237,8 +1245,8 @@ int audiokv_evict_host(audiokv_ctx* ctx, const audiokv_params* p, const void* q_
   AKV_CP(dk, k, kv_elems * es, cudaMemcpyHostToDevice);
   AKV_CP(dv, v, kv_elems * es, cudaMemcpyHostToDevice);
   AKV_CP(dS, head_scores, sizeof(float) * TH, cudaMemcpyHostToDevice);
-  rc = audiokv_evict(ctx, p, dq, dk, dv, reinterpret_cast<float*>(dS), total_budget, dko, dvo,
-                     reinterpret_cast<int32_t*>(dki), reinterpret_cast<int32_t*>(db), reinterpret_cast<int32_t*>(dcu), s);
+  rc = evict_pass(ctx, p, dq, dk, dv, reinterpret_cast<float*>(dS), total_budget, dko, dvo, reinterpret_cast<int32_t*>(dki),
+                  reinterpret_cast<int32_t*>(db), reinterpret_cast<int32_t*>(dcu), s, hs.end);
   if (rc) return rc;
   AKV_CP(k_out, dko, rows * p->head_dim * es, cudaMemcpyDeviceToHost);
   AKV_CP(v_out, dvo, rows * p->head_dim * es, cudaMemcpyDeviceToHost);

@@ -164,14 +164,13 @@ cudaError_t launch_chained(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
-// score_simt.cu: fp32-FMA scoring for any dtype. stats_ws: float2 [total_heads][n_slab][rows], slabs of slab_keys keys; with
-// exps (a workspace of exps_len floats that holds one head's exponentials at least) the product is done once and
-// the statistics take [heads of a chunk][tiles of score_simt_tile_keys keys][rows] instead.
+// score_simt.cu: fp32-FMA scoring for any dtype. stats_ws: float2 [total_heads][n_slab][rows], slabs of slab_keys keys. With
+// room (16-byte aligned workspace) for one head's exponentials at least, the product is done once, a chunk of heads at a time.
 cudaError_t launch_score_simt(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores,
-                              float2* stats_ws, int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln, bool beside = false);
-// Floats of workspace the single-product scoring is given: a chunk of heads, at most 128 MB; 0 when one head alone is longer.
-int64_t score_simt_exps_len(int total_heads, int max_L, int rows, int head_dim);
-int score_simt_tile_keys(int head_dim);
+                              float2* stats_ws, int n_slab, int slab_keys, void* room, size_t room_bytes, int max_L, Launch ln,
+                              bool beside = false);
+// The room that is put to use; grows with every argument.
+size_t score_simt_room(int total_heads, int max_L, int rows, int head_dim);
 
 // One run of work of the tensor-core scoring kernel: consecutive key tiles of one head (of one chunk of its window
 // rows) that one CTA processes. The schedule of each sweep is a table of these, built on the host in processing

@@ -7,8 +7,8 @@
 // they are done once. So where there is room they are done once: the product kernel writes exp2(z - m) of its tile, m the
 // row's maximum over the tile's keys, and (m, sum) per row; a merge gives every row c = -(max + log2 sum) over all keys;
 // the sum kernel adds exp2(m + c) exp2(z - m) over the rows of every key, a stream at memory speed. Heads go through in
-// chunks of up to 128 MB of exponentials. A head too long for the chunk's room, and the entry point with fixed
-// scratch, run the product twice: statistics, merge, column sums.
+// chunks of up to 128 MB of exponentials, or what room the caller has. A head too long for it, and the entry point with
+// fixed scratch, run the product twice: statistics, merge, column sums.
 // The product is a register-tiled matrix product, 8 keys x 4, 7 or 8 query rows a thread. The tile's keys lie transposed in shared
 // memory for as long as the tile lasts, two neighbouring keys make a packed pair of accumulators, and the query rows
 // come in panels of 32 dimensions by asynchronous copies, the next one under the arithmetic of this one, across row tiles.
@@ -18,6 +18,8 @@
 // arithmetic: twice the accumulators leave two warps a scheduler, which do not cover their latencies. The 64 x 64 tiles of 4 x 4
 // logits that were here first, with the logits through shared memory and the product done twice, took 1487 + 1234 us for 112 heads.
 // Logits are kept in base 2 (scale * log2 e folded into one multiply).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace akv {
@@ -415,17 +417,27 @@ int heads_per_chunk(int most, int total, int tiles) {
   return best;
 }
 
+// Exponentials of one head, in floats, and their row statistics, in float2.
+int64_t head_exps(int max_L, int rows, int head_dim) {
+  const int keys = tile_keys(head_dim);
+  return static_cast<int64_t>((max_L + keys - 1) / keys) * keys * rows;
+}
+constexpr int64_t kMaxExps = (128LL << 20) / sizeof(float);  // of a chunk
+
+// room: where the exponentials of a chunk of heads and then their statistics may go.
 template <typename T, int D, int RPT>
 cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
-                         int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln, bool beside) {
+                         int n_slab, int slab_keys, void* room, size_t room_bytes, int max_L, Launch ln, bool beside) {
   constexpr int kKeys = tile_keys(D);
   const int R = sh.window * sh.group, n_tile = (max_L + kKeys - 1) / kKeys;
-  const int64_t per_head = static_cast<int64_t>(n_tile) * R * kKeys;
-  const bool store = exps != nullptr && per_head <= exps_len;
+  const int64_t per_head = head_exps(max_L, R, D);
+  const int64_t fit = std::min<int64_t>(room_bytes / (per_head / kKeys * (kKeys * sizeof(float) + sizeof(float2))), kMaxExps / per_head);
+  const bool store = fit >= 1;
   const int slabs = store ? n_tile : n_slab;
-  const int64_t room = store ? exps_len / per_head : 0x7fffffffLL / slabs;
-  const int chunk = store ? heads_per_chunk(static_cast<int>(room < sh.total_heads ? room : sh.total_heads), sh.total_heads, slabs)
-                          : static_cast<int>(room < sh.total_heads ? room : sh.total_heads);
+  const int most = static_cast<int>(std::min<int64_t>(store ? fit : 0x7fffffffLL / slabs, sh.total_heads));
+  const int chunk = store ? heads_per_chunk(most, sh.total_heads, slabs) : most;
+  float* exps = static_cast<float*>(room);
+  if (store) stats = reinterpret_cast<float2*>(exps + chunk * per_head);
   cudaError_t e = cudaSuccess;
   for (int u0 = 0; u0 < sh.total_heads && e == cudaSuccess; u0 += chunk) {
     const int heads = sh.total_heads - u0 < chunk ? sh.total_heads - u0 : chunk;
@@ -449,29 +461,25 @@ cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, 
 // Rows per thread: the tile height that leaves the fewest padding rows, the larger one on a tie.
 template <typename T, int D>
 cudaError_t launch_rows(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores, float2* stats,
-                        int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln, bool beside) {
+                        int n_slab, int slab_keys, void* room, size_t room_bytes, int max_L, Launch ln, bool beside) {
   const int R = sh.window * sh.group;
   auto padded = [R](int rows) { return (R + rows - 1) / rows * rows; };
-  if (R <= 64) return launch_typed<T, D, 4>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln, beside);
-  if (padded(112) < padded(128)) return launch_typed<T, D, 7>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln, beside);
-  return launch_typed<T, D, 8>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, exps, exps_len, max_L, ln, beside);
+  if (R <= 64) return launch_typed<T, D, 4>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, room, room_bytes, max_L, ln, beside);
+  if (padded(112) < padded(128)) return launch_typed<T, D, 7>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, room, room_bytes, max_L, ln, beside);
+  return launch_typed<T, D, 8>(sh, d_reqs, q, k, scores, stats, n_slab, slab_keys, room, room_bytes, max_L, ln, beside);
 }
 
 }  // namespace
 
-int score_simt_tile_keys(int head_dim) { return tile_keys(head_dim); }
-int64_t score_simt_exps_len(int total_heads, int max_L, int rows, int head_dim) {
-  constexpr int64_t kRoom = (128LL << 20) / sizeof(float);
+size_t score_simt_room(int total_heads, int max_L, int rows, int head_dim) {
   const int keys = tile_keys(head_dim);
-  const int64_t per_head = static_cast<int64_t>((max_L + keys - 1) / keys) * keys * rows;
-  if (per_head > kRoom) return 0;
-  const int64_t heads = kRoom / per_head < total_heads ? kRoom / per_head : total_heads;
-  return heads * per_head;
+  const int64_t exps = std::min(head_exps(max_L, rows, head_dim) * total_heads, kMaxExps);
+  return static_cast<size_t>(exps / keys) * (keys * sizeof(float) + sizeof(float2));
 }
 
 cudaError_t launch_score_simt(const Shape& sh, const ReqDesc* d_reqs, const void* q, const void* k, float* scores,
-                              float2* stats_ws, int n_slab, int slab_keys, float* exps, int64_t exps_len, int max_L, Launch ln, bool beside) {
-#define AKV_CASE(T, D) return launch_rows<T, D>(sh, d_reqs, q, k, scores, stats_ws, n_slab, slab_keys, exps, exps_len, max_L, ln, beside)
+                              float2* stats_ws, int n_slab, int slab_keys, void* room, size_t room_bytes, int max_L, Launch ln, bool beside) {
+#define AKV_CASE(T, D) return launch_rows<T, D>(sh, d_reqs, q, k, scores, stats_ws, n_slab, slab_keys, room, room_bytes, max_L, ln, beside)
   if (sh.dtype == AUDIOKV_F32) {
     if (sh.head_dim == 64) AKV_CASE(float, 64);
     if (sh.head_dim == 128) AKV_CASE(float, 128);

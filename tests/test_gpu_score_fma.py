@@ -1,6 +1,7 @@
-"""The fp32 scoring kernels at the sizes where they can go wrong: key tiles of 64 and their remainders, every height of the row
-tile and its remainders, requests of different lengths in one launch, both element types, and both routes: exponentials
-kept (chunks of heads), and the product done twice (a head too long to be kept; the entry point with fixed scratch).
+"""The fp32 scoring kernels at the sizes where they can go wrong: key tiles of 128 (64 at head_dim 256) and their remainders,
+every height of the row tile and its remainders, requests of different lengths in one launch, both element types, and both
+routes: exponentials kept (chunks of heads), and the product done twice (no room; a head too long to be kept; the entry
+point with fixed scratch).
 
 Bound: a logit is a sum of d products in fp32, off by at most d 2^-24 of sum_t |q_t k_t| scale, about 0.64 sqrt(d) for normal
 q and k; half as much again for the fluctuation of that sum, and twice (the row's normaliser is as far off). The exponentials
@@ -47,7 +48,7 @@ ROWS = [(1, 1), (5, 3), (16, 1), (9, 7), (32, 2), (13, 5), (16, 7), (113, 1), (3
 @pytest.mark.parametrize("W,G", ROWS)
 @pytest.mark.parametrize("d", [64, 128, 256])
 def test_score_f32_rows(B, W, G, d):
-    lens = [W + 1, W + 63, W + 64, 65, 128, 129, 300]
+    lens = [W + 1, W + 63, W + 64, 65, 128, 129, 300]      # a tile less, full and one key more; several
     lens = [max(W + 1, L) for L in lens]
     w = wl.generate(wl.WorkloadSpec("fma", "f32", 1, 2 * G, 2, d, lens, [0.8] * len(lens), 0, window=W), seed=W * G + d)
     prob = B.Problem.from_workload(w)
@@ -60,14 +61,34 @@ def test_score_f32_rows(B, W, G, d):
 
 
 def test_score_f32_chunks_of_heads(B):
-    """Seven heads of 13 MB of exponentials each fit the room of one launch; forty take several."""
+    """Forty heads of 3.4 MB of exponentials and statistics each go through at once where the workspace has room for them, in
+    chunks of seven and one of five where it has room for seven, and with the product done twice where it has none. What
+    is kept does not depend on the chunks to the last bit."""
     w = wl.generate(wl.WorkloadSpec("fma", "f32", 10, 28, 4, 64, [3700], [0.8], 0, window=32), seed=4)
     prob = B.Problem.from_workload(w)
-    ctx = B.Context(prob)
-    scores = torch.full((B.audiokv_scores_len(prob),), float("nan"), device="cuda")
-    B.audiokv_score(ctx, prob, to_dev(w, w.q), to_dev(w, w.k), scores)
-    torch.cuda.synchronize()
-    _check(w, scores.cpu().numpy())
+    head = 29 * 224 * (128 * 4 + 8)                 # 29 tiles of 128 keys, 224 rows
+    need = B.audiokv_workspace_bytes(prob) - 40 * head
+    q, k = to_dev(w, w.q), to_dev(w, w.k)
+    S, tb = torch.from_numpy(w.head_scores).cuda(), [int(x) for x in w.total_budget]
+    results = []
+    for heads, launches in ((40, 3), (7, 18), (0, 3)):
+        ctx = B.Context(prob, workspace_bytes=need + heads * head)
+        scores = torch.full((B.audiokv_scores_len(prob),), float("nan"), device="cuda")
+        for _ in range(2):                          # the first call brings the plan
+            before = ctx.launch_count()
+            B.audiokv_score(ctx, prob, q, k, scores)
+        assert ctx.launch_count() - before == launches
+        kept = [torch.zeros((tb[0], 64), device="cuda"), torch.zeros((tb[0], 64), device="cuda"),
+                *(torch.zeros(n, dtype=torch.int32, device="cuda") for n in (tb[0], 40, 41))]
+        B.audiokv_evict(ctx, prob, q, k, k, S, tb, *kept)  # scoring beside the allocation
+        torch.cuda.synchronize()
+        assert ctx.last_device_status() == 0
+        _check(w, scores.cpu().numpy())
+        results.append((scores, kept[2]))
+    assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
+    with pytest.raises(B.AudioKVError) as e:
+        B.audiokv_score(B.Context(prob, workspace_bytes=need - 256), prob, q, k, scores)
+    assert e.value.status == B.AUDIOKV_EWORKSPACE
 
 
 def test_score_f32_head_too_long_to_keep(B):

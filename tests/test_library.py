@@ -52,6 +52,15 @@ def _prob(B, **kw):
     return B.Problem(**base)
 
 
+def test_fp32_workspace_grows_with_the_prompt(B):
+    """A context sized for its longest fp32 prompt has what a shorter one asks for (prefixes that are transformed on chip)."""
+    for hq, hkv, window in ((8, 1, 128), (28, 4, 32)):
+        sizes = [B.audiokv_workspace_bytes(_prob(B, dtype=B.AUDIOKV_F32, n_q_heads=hq, n_kv_heads=hkv, window=window,
+                                                 seq_lens=[P + window], kv_req_offset=None))
+                 for P in (256, 1024, 4096, 8192, 16384, 20480, 32768, 40960)]
+        assert sizes[0] > 0 and sizes == sorted(sizes), (hq, sizes)
+
+
 def test_sizes_and_param_checks(B):
     p = _prob(B)
     assert B.audiokv_scores_len(p) == 2 * 2 * (968 + 301)
