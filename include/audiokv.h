@@ -164,7 +164,8 @@ int audiokv_last_device_status(audiokv_ctx* ctx, audiokv_stream stream);
 /* Text of the last CUDA error a call on this context met (empty string if none). */
 const char* audiokv_last_cuda_error(const audiokv_ctx* ctx);
 
-/* Kernels launched by calls on this context since it was created (for accounting). */
+/* Kernels launched by calls on this context since it was created (for accounting; the transfer of a plan
+ * to the device, whatever form it takes, is not counted). */
 int64_t audiokv_launch_count(const audiokv_ctx* ctx);
 
 /* Which kernels the last scoring on this context ran on (audiokv_score, or step 1 inside audiokv_evict and

@@ -18,7 +18,6 @@ constexpr size_t kAlign = 256;
 constexpr int kSlabKeys = 256;          // keys per slab of the softmax statistics (two K tiles of the tensor-core kernel)
 constexpr int kMaxRows = 1024;          // W * G
 constexpr int kMaxHeadsPerReq = 2048;
-constexpr size_t kStageBytes = 256 << 10;  // pinned staging of one plan upload
 constexpr int kHostChunks = 8;          // the host-buffer call evicts one request in at most this many runs of layers
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -82,11 +81,7 @@ struct audiokv_ctx {
   cudaEvent_t plan_ready = nullptr;
   cudaStream_t plan_stream = nullptr;     // where the plan went up
   bool plan_settled = false;              // the upload was seen complete
-  static constexpr int kStageSlots = 4;
-  char* stage = nullptr;                  // pinned: kStageSlots x kStageBytes
-  cudaEvent_t stage_free[kStageSlots] = {};
-  uint64_t large_plans = 0;               // plans too large for the kernels' arguments
-  std::vector<char> blob;
+  std::vector<char> blob;                 // the plan as it goes up
   cudaStream_t side = nullptr;            // audiokv_evict_host copies in here
   cudaEvent_t fork = nullptr;
   // audiokv_evict_host: copies in on `side`, kernels on the caller's stream, copies out on `out`, chunk by chunk
@@ -531,22 +526,6 @@ int cuda_fail(audiokv_ctx* ctx, cudaError_t e) {
   return AUDIOKV_ECUDA;
 }
 
-// The ring of pinned staging slots; false when it cannot be had (the plans then go up from pageable memory).
-bool make_stage(audiokv_ctx* ctx) {
-  if (ctx->stage) return true;
-  for (cudaEvent_t& ev : ctx->stage_free)
-    if (!ev && cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-  if (cudaMallocHost(&ctx->stage, audiokv_ctx::kStageSlots * kStageBytes) != cudaSuccess) {
-    cudaGetLastError();
-    ctx->stage = nullptr;
-    return false;
-  }
-  return true;
-}
-
 // Makes ctx->plan match p and its tables resident on the device (stream-ordered).
 int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool host_call = false) {
   if (!ctx) return AUDIOKV_EINVAL;
@@ -573,23 +552,13 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
       ctx->cuda_error = "the plan of these params is not on the device yet: make one call outside stream capture first";
       return AUDIOKV_ECUDA;
     }
-    // The request table, FFT plans, order and schedules go up as one piece, and the status word starts clean with it. A plan
-    // of some tens of heads travels as arguments of the table kernels. A larger one goes up from pinned staging, for which the host
-    // does not wait either (a prompt of a new length then costs no round trip), one that is larger than a staging
-    // slot from pageable memory, for which it does.
+    // The request table, FFT plans, order and schedules go up as one piece, and the status word starts clean with it. It travels
+    // as arguments of kernels, for which the host does not wait (a prompt of a new length then costs no round trip); a
+    // plan too large for some of these, thousands of heads or requests, goes up from pageable memory, for which it does.
     const size_t blob = pl.lay.blob_end;
-    const bool inlined = blob <= 2 * kPlanPartBytes && pl.lay.units <= kPlanPartBytes;
-    // (The staging is made when a context brings its second plan of that size: pinning costs about a millisecond.)
-    const bool staged = !inlined && blob <= kStageBytes && ctx->large_plans++ > 0 && make_stage(ctx);
-    char* src;
-    const int slot = static_cast<int>(ctx->plan_id % audiokv_ctx::kStageSlots);
-    if (staged) {
-      src = ctx->stage + slot * kStageBytes;
-      if ((e = cudaEventSynchronize(ctx->stage_free[slot])) != cudaSuccess) return cuda_fail(ctx, e);  // four plans ago
-    } else {
-      ctx->blob.resize(blob);
-      src = ctx->blob.data();
-    }
+    const bool inlined = blob <= kPlanParts * kPlanPartBytes;
+    ctx->blob.resize(blob);
+    char* src = ctx->blob.data();
     memset(src, 0, 64);
     auto put = [&](size_t at, const void* data, size_t bytes) {
       if (bytes) memcpy(src + at, data, bytes);
@@ -600,9 +569,8 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
     put(pl.lay.ctas, pl.score.ctas.data(), sizeof(int32_t) * pl.score.ctas.size());
     put(pl.lay.order, pl.sss_order.data(), sizeof(int32_t) * pl.sss_order.size());
     if (!inlined && (e = cudaMemcpyAsync(ctx->ws, src, blob, cudaMemcpyHostToDevice, stream)) != cudaSuccess) return cuda_fail(ctx, e);
-    if (staged && (e = cudaEventRecord(ctx->stage_free[slot], stream)) != cudaSuccess) return cuda_fail(ctx, e);
     Launch ln{stream, &ctx->launches, &ctx->prof};
-    e = launch_fft_tables(static_cast<int>(pl.fft.size()), inlined ? src : nullptr, blob, ctx->ws, pl.lay.plans,
+    e = launch_fft_tables(static_cast<int>(pl.fft.size()), inlined ? src : nullptr, blob, pl.lay.units, ctx->ws, pl.lay.plans,
                           reinterpret_cast<float2*>(ctx->ws + pl.lay.tables), pl.sss_smem, ln);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     if ((e = cudaEventRecord(ctx->plan_ready, stream)) != cudaSuccess) return cuda_fail(ctx, e);
@@ -862,12 +830,6 @@ int audiokv_destroy(audiokv_ctx* ctx) {
   }
   for (cudaEvent_t e : ctx->prof.ev)
     if (e) cudaEventDestroy(e);
-  for (cudaEvent_t e : ctx->stage_free)
-    if (e) {
-      cudaEventSynchronize(e);  // the copy out of the staging may still be on its way
-      cudaEventDestroy(e);
-    }
-  if (ctx->stage) cudaFreeHost(ctx->stage);
   cudaFree(ctx->ws);
   delete ctx;
   return AUDIOKV_OK;

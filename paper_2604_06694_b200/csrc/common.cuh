@@ -237,12 +237,13 @@ cudaError_t launch_score_umma(const Shape& sh, const ReqDesc* h_reqs, const Scor
 // sss.cu
 int sss_static_smem();  // bytes of shared memory a smoothing block uses beside its work buffer
 // smem_bytes: the dynamic shared memory launch_sss is given for these plans.
-// h_blob: the first blob_bytes of the workspace (a multiple of 16), at most two parts' worth, which the launch itself takes to
-// the device; what is read before a chain_wait (request table, transform plans, order) has to lie in the first part. Null: it
-// is all there already. plans_at: where the transform plans lie in the workspace.
+// h_blob: the first blob_bytes of the workspace (a multiple of 16, at most kPlanParts parts), which the launches themselves take
+// to the device; its first early_bytes are what kernels read before a chain_wait (request table, transform plans, order).
+// Null: it is all there already. plans_at: where the transform plans lie in the workspace.
 constexpr size_t kPlanPartBytes = 30 << 10;  // kernel arguments end at 32764 bytes
-cudaError_t launch_fft_tables(int n_plans, const char* h_blob, size_t blob_bytes, char* ws, size_t plans_at, float2* d_tables,
-                              size_t smem_bytes, Launch ln);
+constexpr size_t kPlanParts = 8;
+cudaError_t launch_fft_tables(int n_plans, const char* h_blob, size_t blob_bytes, size_t early_bytes, char* ws, size_t plans_at,
+                              float2* d_tables, size_t smem_bytes, Launch ln);
 // order: the heads, the ones that can cost most first; a null order stands for the n_order heads first_head, first_head + 1, ... .
 // The blocks take them from a queue (two ints, zero before and after). smoothed may be null when budgets, cu_kept and kept_idx
 // are given: the kernel then goes on to the top-k selection of each head from the smoothed scores it holds on chip (step

@@ -1427,15 +1427,19 @@ __device__ __forceinline__ float2 root_of_unity(int64_t num, int den) {  // exp(
   return make_float2(static_cast<float>(c), static_cast<float>(-s));
 }
 
-// A plan's bytes travel to the device as arguments of the two table kernels: 4 us for the two together, whatever they hold,
+// A plan's bytes travel to the device as arguments: of the two table kernels, 4 us for the two together, whatever they hold,
 // where a copy out of pinned memory takes 5 us up to 16 KB and 12 above, in front of the table kernel (28 layers of 4 heads
-// make 36 KB; reading the pinned memory from the kernel took 40 us). Each thread then reads its own 16 bytes of the
-// argument bank, so the copy is spread over blocks.
+// make 36 KB; reading the pinned memory from the kernel took 40 us). What does not fit these two goes ahead in kernels of
+// its own. Each thread reads its own 16 bytes of the argument bank, so the copy is spread over blocks.
 struct PlanPart {
   uint4 v[kPlanPartBytes / 16];
 };
 __device__ __forceinline__ void put_part(const PlanPart& part, uint4* to, int n16, int block, int blocks) {
   for (int i = block * blockDim.x + threadIdx.x; i < n16; i += blocks * blockDim.x) to[i] = part.v[i];
+}
+
+__global__ void __launch_bounds__(256) plan_part_kernel(const __grid_constant__ PlanPart part, int n16, uint4* to) {
+  put_part(part, to, n16, blockIdx.x, gridDim.x);
 }
 
 // Writes the tables of every transform plan, 32 blocks each, and the first n16 x 16 bytes of the workspace from `part`. The
@@ -1547,12 +1551,24 @@ fft_filter_kernel(const __grid_constant__ PlanPart part, int n16, uint4* rest, c
 
 int sss_static_smem() { return static_cast<int>(sizeof(SssShared)); }
 
-cudaError_t launch_fft_tables(int n_plans, const char* h_blob, size_t blob_bytes, char* ws, size_t plans_at, float2* d_tables,
-                              size_t smem_bytes, Launch ln) {
+cudaError_t launch_fft_tables(int n_plans, const char* h_blob, size_t blob_bytes, size_t early_bytes, char* ws, size_t plans_at,
+                              float2* d_tables, size_t smem_bytes, Launch ln) {
   cudaError_t e = cudaFuncSetAttribute(fft_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   if (e != cudaSuccess) return e;
-  const size_t first = h_blob ? std::min(blob_bytes, kPlanPartBytes) : 0, rest = h_blob ? blob_bytes - first : 0;
   PlanPart part;
+  // two parts go with the table kernels, the second with the one that kernels behind may not have waited for
+  size_t first = 0, rest = 0;
+  if (h_blob && blob_bytes <= 2 * kPlanPartBytes && early_bytes <= kPlanPartBytes) {
+    first = std::min(blob_bytes, kPlanPartBytes);
+    rest = blob_bytes - first;
+  } else if (h_blob) {
+    for (size_t at = 0; at < blob_bytes; at += kPlanPartBytes) {  // a transfer: not counted as a launch
+      const size_t bytes = std::min(blob_bytes - at, kPlanPartBytes);
+      memcpy(part.v, h_blob + at, bytes);
+      plan_part_kernel<<<8, 256, 0, ln.stream>>>(part, static_cast<int>(bytes / 16), reinterpret_cast<uint4*>(ws + at));
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+  }
   if (first) memcpy(part.v, h_blob, first);
   fft_table_kernel<<<dim3(32, n_plans), 256, 0, ln.stream>>>(part, static_cast<int>(first / 16), ws, plans_at, d_tables);
   ln.done("fft_table");

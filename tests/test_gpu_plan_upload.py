@@ -1,7 +1,7 @@
-"""New plans, on every way they travel to the device: in the arguments of one table kernel or of both, from pinned staging and
-from pageable memory (8 to 2280 heads). One context takes a new length call after call with no wait in between, more often than there
-are staging slots, then on a second stream, then inside a capture that follows the upload at once. Every result has to equal
-that of a context made for the length, and that one the oracle's."""
+"""New plans, on every way they travel to the device: in the arguments of one table kernel, of both, of kernels ahead of them, and
+from pageable memory (8 to 2280 heads). One context takes a new length call after call with no wait in between, then on a
+second stream, then inside a capture that follows the upload at once. Every result has to equal that of a context made
+for the length, and that one the oracle's."""
 import dataclasses
 
 import numpy as np
