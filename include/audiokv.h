@@ -184,10 +184,10 @@ const char* audiokv_last_score_path(const audiokv_ctx* ctx);
 int64_t audiokv_set_wait_limit(int64_t cycles);
 
 /* Per-kernel timing of audiokv_evict, for benchmarks. While enabled, every audiokv_evict call
- * on this context records a CUDA event on its stream after each kernel it launches (creating
- * the events on the first enable). After the call, kernel i of the call (0 <= i <
- * audiokv_profile_count) has the name audiokv_profile_name(ctx, i) and took
- * audiokv_profile_ms(ctx, i) milliseconds from the end of the kernel before it (blocks until
+ * on this context records a CUDA event on its stream after each kernel it launches (the events are
+ * created on the first enable, and more when a call launches more kernels than any before). After the
+ * call, kernel i of the call (0 <= i < audiokv_profile_count) has the name audiokv_profile_name(ctx, i)
+ * and took audiokv_profile_ms(ctx, i) milliseconds from the end of the kernel before it (blocks until
  * that kernel has finished; -1 on error). Off by default. */
 int audiokv_profile_enable(audiokv_ctx* ctx, int on);
 int audiokv_profile_count(const audiokv_ctx* ctx);

@@ -605,15 +605,17 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
   return AUDIOKV_OK;
 }
 
-// Starts the per-kernel timing of one call (event 0), when profiling is on.
-void profile_begin(audiokv_ctx* ctx, cudaStream_t stream) {
-  Profiler& pf = ctx->prof;
-  if (!pf.on) return;
-  pf.n = 0;
-  cudaEventRecord(pf.ev[0], stream);
-  pf.name[0] = "begin";
-  pf.n = 1;
-}
+// The per-kernel timing of one call, from here (event 0) to its end, when profiling is on.
+struct ProfiledCall {
+  Profiler& pf;
+  ProfiledCall(audiokv_ctx* ctx, cudaStream_t stream) : pf(ctx->prof) {
+    if (!pf.on) return;
+    pf.n = 0;
+    pf.recording = true;
+    pf.mark("begin", stream);
+  }
+  ~ProfiledCall() { pf.recording = false; }
+};
 
 const ReqDesc* d_reqs(audiokv_ctx* c) { return reinterpret_cast<const ReqDesc*>(c->ws + c->plan.lay.reqs); }
 // The first 64 bytes of the workspace: the status word, and from int 4 on the queue of the smoothing kernel.
@@ -828,8 +830,7 @@ int audiokv_destroy(audiokv_ctx* ctx) {
     if (ctx->chunk_in[i]) cudaEventDestroy(ctx->chunk_in[i]);
     if (ctx->chunk_done[i]) cudaEventDestroy(ctx->chunk_done[i]);
   }
-  for (cudaEvent_t e : ctx->prof.ev)
-    if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : ctx->prof.ev) cudaEventDestroy(e);
   cudaFree(ctx->ws);
   delete ctx;
   return AUDIOKV_OK;
@@ -865,10 +866,7 @@ int audiokv_profile_enable(audiokv_ctx* ctx, int on) {
   if (!ctx) return AUDIOKV_EINVAL;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return AUDIOKV_ECUDA;
   Profiler& pf = ctx->prof;
-  if (on && !pf.ev[0]) {
-    for (cudaEvent_t& e : pf.ev)
-      if (cudaEventCreate(&e) != cudaSuccess) return AUDIOKV_ECUDA;
-  }
+  if (on && !pf.reserve(32)) return AUDIOKV_ECUDA;  // enough for a pass of one request; longer ones add theirs
   pf.on = on != 0;
   pf.n = 0;
   return AUDIOKV_OK;
@@ -944,7 +942,7 @@ int evict_pass(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, con
   Plan& pl = ctx->plan;
   float* ws_scores = reinterpret_cast<float*>(ctx->ws + pl.lay.scores);
   int32_t* ws_kstar = reinterpret_cast<int32_t*>(ctx->ws + pl.lay.kstar);
-  profile_begin(ctx, s);
+  const ProfiledCall timed(ctx, s);
   // The budgets depend on nothing the GPU computes, and only the selection needs them. The allocation kernel is
   // launched the ordinary way (everything earlier on the stream is then complete when it starts) and lets its
   // dependents in at once; the first scoring sweep, a programmatic dependent, runs beside it and waits for it at its
@@ -991,7 +989,7 @@ int audiokv_evict_budgeted(audiokv_ctx* ctx, const audiokv_params* p, const void
   float* ws_scores = reinterpret_cast<float*>(ctx->ws + pl.lay.scores);
   int32_t* ws_kstar = reinterpret_cast<int32_t*>(ctx->ws + pl.lay.kstar);
   int32_t* ws_budgets = reinterpret_cast<int32_t*>(ctx->ws + pl.lay.aux);  // the checked copy the selection reads
-  profile_begin(ctx, s);
+  const ProfiledCall timed(ctx, s);
   Launch ln{s, &ctx->launches, &ctx->prof};
   cudaError_t e = launch_budget_prefix(pl.sh, d_reqs(ctx), budgets, ws_budgets, cu_kept, d_status(ctx), ln);
   if (e != cudaSuccess) return cuda_fail(ctx, e);

@@ -118,13 +118,31 @@ inline int device_sm_count() {
 }
 
 // ---- launchers (one per source file) ---------------------------------------------------
-// Optional per-kernel timing: an event after every kernel launch of one call.
+// Optional per-kernel timing: an event after every kernel launch of one call, as many as it takes.
 struct Profiler {
-  static constexpr int kMax = 32;
   bool on = false;
-  int n = 0;                 // events recorded in the current call (event 0 = start of the call)
-  cudaEvent_t ev[kMax] = {};
-  const char* name[kMax] = {};
+  bool recording = false;         // inside a call that is timed
+  int n = 0;                      // events recorded in the last such call (event 0 = its start)
+  std::vector<cudaEvent_t> ev;
+  std::vector<const char*> name;
+  bool reserve(size_t count) {
+    while (ev.size() < count) {
+      cudaEvent_t e;
+      if (cudaEventCreate(&e) != cudaSuccess) return false;
+      ev.push_back(e);
+      name.push_back("");
+    }
+    return true;
+  }
+  void mark(const char* what, cudaStream_t stream) {
+    if (!reserve(n + 1)) {  // no record rather than part of one
+      recording = false;
+      n = 0;
+      return;
+    }
+    cudaEventRecord(ev[n], stream);
+    name[n++] = what;
+  }
 };
 
 struct Launch {
@@ -134,11 +152,7 @@ struct Launch {
   // Counts one kernel launch and, when profiling, records the event that ends it.
   void done(const char* kernel_name) const {
     *launch_counter += 1;
-    if (prof && prof->on && prof->n < Profiler::kMax) {
-      cudaEventRecord(prof->ev[prof->n], stream);
-      prof->name[prof->n] = kernel_name;
-      prof->n += 1;
-    }
+    if (prof && prof->recording) prof->mark(kernel_name, stream);
   }
 };
 

@@ -91,6 +91,24 @@ def test_score_f32_chunks_of_heads(B):
     assert e.value.status == B.AUDIOKV_EWORKSPACE
 
 
+def test_profile_lists_every_kernel_of_a_long_pass(B):
+    """Chunks of three heads make some 42 launches of the scoring alone; the profile ends with the gather."""
+    w = wl.generate(wl.WorkloadSpec("fma", "f32", 10, 28, 4, 64, [3700], [0.8], 0, window=32), seed=4)
+    prob = B.Problem.from_workload(w)
+    head = 29 * 224 * (128 * 4 + 8)
+    ctx = B.Context(prob, workspace_bytes=B.audiokv_workspace_bytes(prob) - 37 * head)
+    q, k, tb = to_dev(w, w.q), to_dev(w, w.k), [int(x) for x in w.total_budget]
+    out = [torch.zeros((tb[0], 64), device="cuda"), torch.zeros((tb[0], 64), device="cuda"),
+           *(torch.zeros(n, dtype=torch.int32, device="cuda") for n in (tb[0], 40, 41))]
+    ctx.profile_enable(True)
+    for _ in range(2):                              # the first call brings the plan
+        before = ctx.launch_count()
+        B.audiokv_evict(ctx, prob, q, k, k, torch.from_numpy(w.head_scores).cuda(), tb, *out)
+    prof = ctx.profile_read()
+    assert len(prof) == ctx.launch_count() - before > 40
+    assert prof[0][0] == "allocate" and prof[-1][0] == "gather" and all(ms >= 0 for _, ms in prof)
+
+
 def test_score_f32_head_too_long_to_keep(B):
     """W * G = 1024 and 33000 keys: 135 MB of exponentials for one head, so the product is done twice."""
     w = wl.generate(wl.WorkloadSpec("fma", "f32", 1, 8, 1, 64, [33000], [0.8], 0, window=128), seed=6)
