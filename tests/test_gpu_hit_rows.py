@@ -1,6 +1,7 @@
 """The head-score kernel at the row shapes where its paths part ways: rows shorter than a warp's worth of 16-byte pieces,
-remainders before and after them, rows longer than what a block holds in registers, top_k around the limit of the
-list, and rows of so many equal values that the list overflows. Counts are whole numbers: they equal the oracle's."""
+remainders before and after them, long rows, top_k around the limit of a warp's list and far above it, rows of so many
+equal values that the list overflows, and more rows than one turn of the grid. Counts are whole numbers: they equal
+the oracle's."""
 import numpy as np
 import pytest
 import torch
@@ -19,7 +20,8 @@ def B():
 
 
 @pytest.mark.parametrize("lens,K", [((1, 2, 31, 65), 1), ((66, 127, 128, 129, 133), 64), ((1025, 1026, 1027), 65),
-                                    ((8191, 8192, 8193, 9001), 24), ((20011, 16384), 8), ((5000,), 63)])
+                                    ((8191, 8192, 8193, 9001), 24), ((20011, 16384), 8), ((5000,), 63),
+                                    ((2049, 31, 300, 33), 32), ((259, 4100), 33), ((8190, 1003), 1000)])
 @pytest.mark.parametrize("kind", ["softmax", "steps"])
 def test_hit_score_row_shapes(B, lens, K, kind):
     rng = np.random.default_rng(sum(lens) + K)
@@ -69,3 +71,20 @@ def test_hit_score_nan(B, K):
                             torch.tensor([span], dtype=torch.int32, device="cuda"), K, counts, s)
         torch.cuda.synchronize()
         assert np.array_equal(counts.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("K", [8, 33])
+def test_hit_score_many_short_rows(B, K):
+    """100000 rows of 47 values are more than every block takes in one turn; a third of them are constant and left to the block."""
+    rng = np.random.default_rng(K)
+    T, H, L = 100, 1000, 47
+    attn = rng.random((T, H, L), dtype=np.float32)
+    attn[:, ::3] = 0.5
+    row_len = np.full(T, L, dtype=np.int32)
+    span = np.stack([np.arange(T) % 30, np.arange(T) % 30 + 12], axis=1).astype(np.int32)
+    ctx = B.Context(B.Problem(B.AUDIOKV_BF16, 1, 4, 4, 64, [64], 8, (0, 0, 0, 0), (0, 64, 0)))
+    counts, s = torch.full((H,), -1, dtype=torch.int32, device="cuda"), torch.zeros(H, device="cuda")
+    B.audiokv_hit_score(ctx, torch.from_numpy(attn).cuda(), torch.from_numpy(row_len).cuda(),
+                        torch.from_numpy(span).cuda(), K, counts, s)
+    torch.cuda.synchronize()
+    assert np.array_equal(counts.cpu().numpy(), oracle.hit_score(attn, row_len, span, K)[1])
