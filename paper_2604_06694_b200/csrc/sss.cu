@@ -711,6 +711,16 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Inclusive prefix of v over the warp.
+__device__ __forceinline__ double warp_prefix(double v) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double t = __shfl_up_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) >= o) v += t;
+  }
+  return v;
+}
+
 // ---- low cut-offs without a transform ---------------------------------------------------------------------------
 // Attention scores are positive, so where a head attends evenly their mean carries most of the energy and k* is a
 // handful of bins. The block then evaluates those bins directly, O(n (k* + T)) operations instead of two transforms of
@@ -994,14 +1004,11 @@ __device__ __noinline__ void transform_head(const Shape& sh, const float2* __res
   }
 
   // 2. The spectrum of the real sequence and the cut-off, the smallest k with E(k) = sum_{i<=k} |F_i|^2 >= rho E(Kb) (fp64).
-  //    E(Kb) is known from the sums over the scores (Parseval), so the bins are gone through in ascending order and only
-  //    until the threshold is reached; what lies above the cut-off and its band is masked away unseen. But the bins are
-  //    fp32: their own total is off from Parseval's, and near rho = 1 that would move the cut-off by many bins of a spectrum
-  //    that falls off. So a cut-off found this way counts only when it is clear of the threshold by more than the two totals can
-  //    differ; else all bins are summed and the search is done over against their total.
   //    packed: Z is turned into F pairwise in place (the slot of bin 0 holds (F_0, F_N), both real). Energies are summed by
   //    chunks of 32 neighbouring bins (one warp's share): chunk i of the low bins at energy[i], chunk i of their partners
-  //    N - k, which count downwards, at energy[2 nc - 1 - i]. After every 64 chunks each warp looks where the sum stands.
+  //    N - k, which count downwards, at energy[2 nc - 1 - i]. The threshold is taken from the sum of all bins, not from
+  //    Parseval's identity, though that would let the sums end at the cut-off: the bins are fp32 and their total is off by
+  //    1e-7 of the energy, which near rho = 1 is many bins of a spectrum that falls off.
   const bool no_mean = sh.smooth_mode == AUDIOKV_SMOOTH_ENERGY_NO_MEAN;  // variant: bin 0 adds no energy
   const int n_low = packed ? N / 2 + 1 : Kb + 1;
   const int nc = (n_low + 31) / 32, n_chunk = packed ? 2 * nc : nc;
@@ -1014,128 +1021,79 @@ __device__ __noinline__ void transform_head(const Shape& sh, const float2* __res
     fk = cadd(E, T);
     fq = cconj(csub(E, T));
   };
-  int kc = 0;  // packed: bins k < kc (and their partners) have been split
-  if (sh.smooth_mode == AUDIOKV_SMOOTH_FIXED_FRACTION) {
-    // variant: the cut-off sits at a fixed fraction of the spectrum, no energies needed
-    if (threadIdx.x == 0) S.kstar = min(static_cast<int>(floor(static_cast<double>(sh.smooth_kappa) * Kb)), Kb);
-  } else {
-    const double F0 = S.sums[0], FN = S.sums[2];
-    const double total = 0.5 * (static_cast<double>(n) * S.sums[1] + F0 * F0 + ((n & 1) ? 0.0 : FN * FN));
-    const double whole = no_mean ? fmax(total - F0 * F0, 0.0) : total;
-    // The transform is off by less than kOff of the spectrum's norm (33 roundings; a few are usual), the energies by this:
-    constexpr double kOff = 2e-6;
-    const double margin = 2.0 * kOff * sqrt(whole * total) + kOff * kOff * total;
-    const bool all = sh.rho >= 1.f && whole > 0.0;  // asks for everything: no bin short of the last will do
-    double thr = all ? INFINITY : static_cast<double>(sh.rho) * whole;
-    constexpr int U = 4;
-    static_assert(U * kWarps == 64, "two chunks per lane and round");
-    int stage = all ? 2 : 0;  // 0: against Parseval's total; 1: the sum of all bins; 2: against that
-    int summed = 0;           // chunks below this have their sums
+  const bool fixed = sh.smooth_mode == AUDIOKV_SMOOTH_FIXED_FRACTION;  // variant: no energies needed, step 3 splits the bins
+  constexpr int U = 4;
 #pragma unroll 1
-    for (;;) {
-      double run = 0.0;
-      int chunk = -1;  // the chunk that crosses the threshold, and the sum before it
-#pragma unroll 1
-      for (int c0 = 0; c0 < n_chunk && chunk < 0; c0 += U * kWarps) {
-        if (c0 < nc && c0 >= summed) {
-          uint2 at[U];
+  for (int c0 = 0; c0 < nc && !fixed; c0 += U * kWarps) {
+    uint2 at[U];
 #pragma unroll
-          for (int q = 0; q < U; ++q) at[q] = slots_of(min(32 * (c0 + q * kWarps + warp) + lane, n_low - 1));
+    for (int q = 0; q < U; ++q) at[q] = slots_of(min(32 * (c0 + q * kWarps + warp) + lane, n_low - 1));
 #pragma unroll
-          for (int q = 0; q < U; ++q) {
-            const int c = c0 + q * kWarps + warp, k = 32 * c + lane;
-            double el = 0.0, eh = 0.0;
-            if (k < n_low) {
-              float2 fk = buf.ld(at[q].x);
-              if (packed) {
-                float2 fq;
-                split(k, fk, buf.ld(at[q].y), fk, fq);
-                buf.st(at[q].x, k == 0 ? make_float2(fk.x, fq.x) : fk);
-                if (k > 0) buf.st(at[q].y, fq);
-                eh = 2 * k == N ? 0.0 : sq_abs(fq);
-              }
-              el = k == 0 && no_mean ? 0.0 : sq_abs(fk);
-            }
-            // both sums in one tree: the lower half of the warp goes on with the low bins, the upper half with the others
-            const double ol = __shfl_xor_sync(0xffffffffu, el, 16), oh = __shfl_xor_sync(0xffffffffu, eh, 16);
-            double v = (lane & 16) ? eh + oh : el + ol;
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (c < nc) {
-              if (lane == 0) S.energy[c] = v;
-              if (lane == 16 && packed) S.energy[2 * nc - 1 - c] = v;
-            }
-          }
-          summed = c0 + U * kWarps;
-          kc = min(n_low, 32 * summed);
-          __syncthreads();
+    for (int q = 0; q < U; ++q) {
+      const int c = c0 + q * kWarps + warp, k = 32 * c + lane;
+      double el = 0.0, eh = 0.0;
+      if (k < n_low) {
+        float2 fk = buf.ld(at[q].x);
+        if (packed) {
+          float2 fq;
+          split(k, fk, buf.ld(at[q].y), fk, fq);
+          buf.st(at[q].x, k == 0 ? make_float2(fk.x, fq.x) : fk);
+          if (k > 0) buf.st(at[q].y, fq);
+          eh = 2 * k == N ? 0.0 : sq_abs(fq);
         }
-        // chunks c0 .. c0 + 63: in the last round of the low bins the chunks of the upper bins follow at once
-        const int ca = c0 + 2 * lane;
-        const double ea = ca < n_chunk && (ca < nc || c0 + U * kWarps > nc) ? S.energy[ca] : 0.0;
-        const double eb = ca + 1 < n_chunk && (ca + 1 < nc || c0 + U * kWarps > nc) ? S.energy[ca + 1] : 0.0;
-        double inc = ea + eb;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const double t = __shfl_up_sync(0xffffffffu, inc, o);
-          if (lane >= o) inc += t;
-        }
-        const uint32_t hit = __ballot_sync(0xffffffffu, run + inc >= thr);
-        if (hit) {
-          const int at_lane = __ffs(hit) - 1;
-          const double before = run + __shfl_sync(0xffffffffu, inc - (ea + eb), at_lane);
-          const double first = __shfl_sync(0xffffffffu, ea, at_lane);
-          const bool second = !(before + first >= thr);
-          chunk = min(c0 + 2 * at_lane + (second ? 1 : 0), n_chunk - 1);
-          run = second ? before + first : before;
-        } else {
-          run += __shfl_sync(0xffffffffu, inc, 31);
-        }
+        el = k == 0 && no_mean ? 0.0 : sq_abs(fk);
       }
-      if (stage == 1) {
-        thr = static_cast<double>(sh.rho) * run;
-        stage = 2;
-        continue;
-      }
-      if (warp == 0) {
-        int ks = Kb;
-        bool clear = false;
-        if (chunk >= 0) {
-          // the chunk's bins in ascending order, one per lane
-          const bool upper = packed && chunk >= nc;
-          const int k = upper ? N - (32 * (2 * nc - 1 - chunk) + 31 - lane) : 32 * chunk + lane;
-          const bool in = upper ? (k >= N - N / 2 && 2 * k != N && k <= N) : k < n_low;
-          double own = 0.0;
-          if (in) {
-            if (packed && (k == N || k == 0)) {
-              const float2 f = buf.ld(0);
-              own = k == N ? static_cast<double>(f.y) * f.y : no_mean ? 0.0 : static_cast<double>(f.x) * f.x;
-            } else if (!(k == 0 && no_mean)) {
-              const uint2 at = slots_of(upper ? N - k : k);
-              own = sq_abs(buf.ld(upper ? at.y : at.x));
-            }
-          }
-          double e = own;
+      // both sums in one tree: the lower half of the warp goes on with the low bins, the upper half with the others
+      const double ol = __shfl_xor_sync(0xffffffffu, el, 16), oh = __shfl_xor_sync(0xffffffffu, eh, 16);
+      double v = (lane & 16) ? eh + oh : el + ol;
 #pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const double t = __shfl_up_sync(0xffffffffu, e, o);
-            if (lane >= o) e += t;
-          }
-          const uint32_t hit = __ballot_sync(0xffffffffu, in && run + e >= thr);
-          const uint32_t any = __ballot_sync(0xffffffffu, in);
-          const int at_lane = hit ? __ffs(hit) - 1 : 31 - __clz(any | 1u);  // rounding of the two sums: the chunk's last bin
-          ks = min(max(__shfl_sync(0xffffffffu, k, at_lane), 0), Kb);
-          const bool mine = run + e >= thr + margin && (ks == 0 || run + (e - own) <= thr - margin);
-          clear = hit && __shfl_sync(0xffffffffu, mine, at_lane);
-        }
-        if (lane == 0) S.kstar = stage == 2 || clear ? ks : -1;
+      for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (c < nc) {
+        if (lane == 0) S.energy[c] = v;
+        if (lane == 16 && packed) S.energy[2 * nc - 1 - c] = v;
       }
-      __syncthreads();
-      if (S.kstar >= 0) break;
-      __syncthreads();
-      stage = 1;
-      thr = INFINITY;
     }
+  }
+  __syncthreads();
+  if (fixed) {
+    if (threadIdx.x == 0) S.kstar = min(static_cast<int>(floor(static_cast<double>(sh.smooth_kappa) * Kb)), Kb);
+  } else if (warp == 0) {
+    // every lane sums a run of chunks; then the lane, the chunk and the bin that reach the threshold
+    const int per = (n_chunk + 31) / 32, c0 = min(n_chunk, lane * per), c1 = min(n_chunk, c0 + per);
+    double own = 0.0;
+    for (int c = c0; c < c1; ++c) own += S.energy[c];
+    const double inc = warp_prefix(own), total = __shfl_sync(0xffffffffu, inc, 31);
+    // all of a total above zero is reached at the last bin, whatever the rounding of the sums
+    const double thr = sh.rho < 1.f || !(total > 0.0) ? static_cast<double>(sh.rho) * total : INFINITY;
+    const uint32_t hit = __ballot_sync(0xffffffffu, inc >= thr);
+    int ks = Kb;
+    if (hit) {
+      double run = inc - own;
+      int chunk = c0;
+      while (chunk + 1 < c1 && !(run + S.energy[chunk] >= thr)) run += S.energy[chunk++];
+      chunk = __shfl_sync(0xffffffffu, chunk, __ffs(hit) - 1);
+      run = __shfl_sync(0xffffffffu, run, __ffs(hit) - 1);
+      // the chunk's bins in ascending order, one per lane
+      const bool upper = packed && chunk >= nc;
+      const int k = upper ? N - (32 * (2 * nc - 1 - chunk) + 31 - lane) : 32 * chunk + lane;
+      const bool in = upper ? (k >= N - N / 2 && 2 * k != N && k <= N) : k < n_low;
+      double e = 0.0;
+      if (in) {
+        if (packed && (k == N || k == 0)) {
+          const float2 f = buf.ld(0);
+          e = k == N ? static_cast<double>(f.y) * f.y : no_mean ? 0.0 : static_cast<double>(f.x) * f.x;
+        } else if (!(k == 0 && no_mean)) {
+          const uint2 at = slots_of(upper ? N - k : k);
+          e = sq_abs(buf.ld(upper ? at.y : at.x));
+        }
+      }
+      e = warp_prefix(e);
+      const uint32_t reach = __ballot_sync(0xffffffffu, in && run + e >= thr);
+      const uint32_t any = __ballot_sync(0xffffffffu, in);
+      const int at_lane = reach ? __ffs(reach) - 1 : 31 - __clz(any | 1u);  // rounding of the two sums: the chunk's last bin
+      ks = min(max(__shfl_sync(0xffffffffu, k, at_lane), 0), Kb);
+    }
+    if (lane == 0) S.kstar = ks;
   }
   __syncthreads();
   const int kstar = S.kstar;
@@ -1152,7 +1110,7 @@ __device__ __noinline__ void transform_head(const Shape& sh, const float2* __res
       float2 ok = make_float2(0.f, 0.f), oq = ok;
       if (k <= k_hi) {  // else its partner, further up, is masked away as well
         float2 fk = buf.ld(at.x), fq = buf.ld(at.y);
-        if (k >= kc) {
+        if (fixed) {
           split(k, fk, fq, fk, fq);
         } else if (k == 0) {
           fq = make_float2(fk.y, 0.f);
