@@ -208,7 +208,7 @@ void seq_tables(FftSeq* sq, int64_t* table_len) {
   int off = 0;
   for (int i = 0; i < sq->n_pass; ++i) {
     sq->mat[i] = off;
-    if (sq->radix[i] > 13) off += (sq->radix[i] - 1) / 2 * fft_mat_cols(sq->radix[i]);
+    if (sq->radix[i] > kMaxSmall) off += (sq->radix[i] - 1) / 2 * fft_mat_cols(sq->radix[i]);
   }
   *table_len += off;
 }

@@ -62,6 +62,7 @@ __device__ __forceinline__ int find_req(const ReqDesc* __restrict__ reqs, int n_
 
 // ---- FFT plans -------------------------------------------------------------------------
 constexpr int kMaxRadices = 20;   // passes of one transform
+constexpr int kMaxSmall = 19;     // largest radix of a butterfly in one thread's registers
 constexpr int kMaxPrime = 127;    // largest radix of a pass; lengths with a larger prime factor go through a chirp-z
 constexpr int kSssThreads = 512;  // threads of a smoothing block: 128 registers each
 
@@ -71,7 +72,7 @@ struct FftSeq {
   int32_t N;
   int32_t n_pass;
   int32_t radix[kMaxRadices];
-  int32_t mat[kMaxRadices];  // radices above 13: (cos, sin)(2 pi s c / p), [s = 1 .. H][c = 0 .. fft_mat_cols - 1], from `base`
+  int32_t mat[kMaxRadices];  // radices above kMaxSmall: (cos, sin)(2 pi s c / p), [s = 1 .. H][c = 0 .. fft_mat_cols - 1], from `base`
   int64_t base;              // float2 index of the first of these matrices inside the table area
 };
 __host__ __device__ inline int fft_mat_cols(int p) { return ((p - 1) / 2 + 1 + 7) / 8 * 8; }

@@ -2,7 +2,7 @@
 //
 // A real sequence of even length n is packed into a complex one of length N = n/2
 // (odd n: length N = n with zero imaginary part). The complex transform is an in-place
-// mixed-radix decimation-in-frequency FFT: radices 2 to 13 one butterfly per thread, larger primes
+// mixed-radix decimation-in-frequency FFT: radices 2 to 19 one butterfly per thread, larger primes
 // as a product with the p x p cosine and sine matrices, register-tiled. Its output is left in digit-reversed order
 // and addressed through a table, and the inverse is the matching decimation-in-time chain, so no reordering pass
 // and no second buffer is needed. Lengths with a large prime factor go through a chirp-z
@@ -169,8 +169,14 @@ __device__ __forceinline__ constexpr float rcos(int t) {
                             -0.95949297361449737f};
   constexpr float c13[7] = {1.f, 0.88545602565320991f, 0.56806474673115592f, 0.12053668025532301f,
                             -0.35460488704253545f, -0.74851074817110119f, -0.97094181742605201f};
+  constexpr float c17[9] = {1.f, 0.9324722294043558f, 0.73900891722065912f, 0.44573835577653827f, 0.092268359463302f,
+                            -0.27366299007208286f, -0.60263463637925639f, -0.85021713572961415f, -0.98297309968390178f};
+  constexpr float c19[10] = {1.f, 0.94581724170063468f, 0.7891405093963936f, 0.54694815812242687f, 0.24548548714079915f,
+                             -0.08257934547233232f, -0.40169542465296946f, -0.67728157162574107f, -0.87947375120648907f,
+                             -0.98636130340272237f};
   const int i = 2 * t > R ? R - t : t;
-  return R == 3 ? c3[i < 2 ? i : 0] : R == 5 ? c5[i < 3 ? i : 0] : R == 7 ? c7[i < 4 ? i : 0] : R == 11 ? c11[i < 6 ? i : 0] : c13[i];
+  return R == 3 ? c3[i < 2 ? i : 0] : R == 5 ? c5[i < 3 ? i : 0] : R == 7 ? c7[i < 4 ? i : 0] : R == 11 ? c11[i < 6 ? i : 0]
+         : R == 13 ? c13[i < 7 ? i : 0] : R == 17 ? c17[i < 9 ? i : 0] : c19[i];
 }
 template <int R>
 __device__ __forceinline__ constexpr float rsin(int t) {
@@ -181,8 +187,14 @@ __device__ __forceinline__ constexpr float rsin(int t) {
                             0.28173255684142967f};
   constexpr float s13[7] = {0.f, 0.46472317204376851f, 0.82298386589365635f, 0.99270887409805397f, 0.93501624268541483f,
                             0.66312265824079519f, 0.23931566428755768f};
+  constexpr float s17[9] = {0.f, 0.36124166618715295f, 0.67369564364655721f, 0.89516329135506232f, 0.99573417629503452f,
+                            0.96182564317281907f, 0.7980172272802395f, 0.5264321628773558f, 0.18374951781657033f};
+  constexpr float s19[10] = {0.f, 0.32469946920468349f, 0.61421271268966782f, 0.83716647826252857f, 0.96940026593933042f,
+                             0.99658449300666985f, 0.91577332665505744f, 0.73572391067313162f, 0.47594739303707354f,
+                             0.16459459028073389f};
   const int i = 2 * t > R ? R - t : t;
-  const float v = R == 3 ? s3[i < 2 ? i : 0] : R == 5 ? s5[i < 3 ? i : 0] : R == 7 ? s7[i < 4 ? i : 0] : R == 11 ? s11[i < 6 ? i : 0] : s13[i];
+  const float v = R == 3 ? s3[i < 2 ? i : 0] : R == 5 ? s5[i < 3 ? i : 0] : R == 7 ? s7[i < 4 ? i : 0]
+                : R == 11 ? s11[i < 6 ? i : 0] : R == 13 ? s13[i < 7 ? i : 0] : R == 17 ? s17[i < 9 ? i : 0] : s19[i];
   return 2 * t > R ? -v : v;
 }
 
@@ -275,6 +287,12 @@ __device__ __forceinline__ void pass_small(const In& in, const Out& out, int tot
   __syncthreads();
 }
 
+// The same for the two radices that want most of a thread's registers, out of the way of the others.
+template <int R, bool INV, class Buf>
+__device__ __noinline__ void pass_mid(const Buf buf, int total, int ns, int N, const Roots root) {
+  pass_small<R, INV>(buf, buf, total, ns, N, root);
+}
+
 // Two passes of small radices in one trip through shared memory: R1 on sub-transforms of length ns, then R2 on the R1 pieces
 // of each. A thread holds the R1 x R2 elements that meet; operations and roundings are those of the two passes one after
 // the other, so only the number of barriers and of loads and stores changes.
@@ -343,7 +361,7 @@ __device__ __forceinline__ void one_pair(int total, int ns, const FftSeq& sq, in
   }
 }
 
-// The same pass for an odd prime radix p, 17 <= p <= kMaxPrime. With inputs s and p - s folded into P_s = a_s + a_{p-s}
+// The same pass for an odd prime radix p, kMaxSmall < p <= kMaxPrime. With inputs s and p - s folded into P_s = a_s + a_{p-s}
 // and Q_s = a_s - a_{p-s}, outputs c and p - c come from the same real-by-complex sums, X_c = A_c -/+ i B_c,
 // A_c = a_0 + sum_s P_s cos(2 pi s c / p), B_c = sum_s Q_s sin(2 pi s c / p): a product of a small matrix with as many
 // columns as there are butterflies. A thread computes a tile of TO outputs x TC butterflies in registers: per s it reads TC
@@ -450,6 +468,11 @@ __device__ __forceinline__ void prime_product(const Buf& buf, int ns, int p, int
 template <bool INV, class Buf>
 __device__ __noinline__ void pass_prime(const Buf buf, int total, int ns, int N, int p, const Roots root,
                                         const float2* __restrict__ mat) {
+  if (p <= kMaxSmall) {  // asked here and not with the smaller radices, which would make every transform 0.3 to 1 us longer
+    if (p == 17) pass_mid<17, INV, Buf>(buf, total, ns, N, root);
+    else pass_mid<19, INV, Buf>(buf, total, ns, N, root);
+    return;
+  }
   const int m = ns / p, nb = total / p, H = (p - 1) / 2, step = N / ns;
   const FastDiv dm(m), dn(nb);
 #pragma unroll 2
@@ -1424,7 +1447,7 @@ fft_table_kernel(const __grid_constant__ PlanPart part, int n16, char* ws, size_
   }
   for (int i = 0; i < pl.seq.n_pass; ++i) {
     const int R = pl.seq.radix[i];
-    if (R > 13) {
+    if (R > kMaxSmall) {
       const int H = (R - 1) / 2, Cp = fft_mat_cols(R);
       for (int t = gid; t < H * Cp; t += gsz) {
         const int s = t / Cp + 1, c = t - (s - 1) * Cp;

@@ -82,3 +82,22 @@ def test_cutoff_at_rho_one(B, n):
     x[1] = 0
     y, ks = _smooth(B, _problem(B, 2, [n], rho=1.0), x.reshape(-1))
     assert ks.tolist() == [n // 2, 0] and bool((y[n:] == 0).all())
+
+
+@pytest.mark.parametrize("n", [17, 19, 51, 76, 323, 646, 4 * 17 * 19, 17 ** 3, 2 * 19 ** 3, 34 * 2048, 38 * 2048])
+def test_radix_17_and_19(B, n):
+    """One pass or several of either radix, on chip and (the longest two) on the global buffer, against the filter in 64 bits."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    x = torch.exp(torch.randn((2, n), generator=gen, device="cuda"))
+    prob = _problem(B, 2, [n], rho=0.9, alpha=1.0, transition_bins=2)
+    y, ks = _smooth(B, prob, x.reshape(-1))
+    f = torch.fft.rfft(x.double(), dim=1)
+    e = torch.cumsum(f.abs() ** 2, 1)
+    i, k = torch.arange(n // 2 + 1, device="cuda"), ks.long()[:, None]
+    thr = float(prob.p.rho) * e[:, -1:]
+    assert (e.gather(1, k) >= thr * (1 - 1e-6)).all() and (e.gather(1, (k - 1).clamp_min(0)) < thr * (1 + 1e-6)).all()
+    band = 0.5 * (1 + torch.cos(torch.pi * (i - k) / 3))
+    want = torch.fft.irfft(f * torch.where(i <= k, 1.0, torch.where(i <= k + 2, band, 0.0)), n=n, dim=1)
+    # a transform is off by some sqrt(passes) roundings of the norm, two transforms by 1e-6
+    assert float((y.view(2, n) - want).norm() / want.norm()) < 1e-6
