@@ -70,8 +70,7 @@ __device__ __forceinline__ void for_row(const float* __restrict__ row, int L, Us
 // Exact count for one row of any kind, by the whole block: a histogram of 2048 equal steps between the smallest and the largest
 // key (equal steps of the float's bits), again inside the bin of the k-th key while that holds too many, then a comparison
 // of its keys; of the keys equal to the k-th the lowest indices count. Keys order a NaN by its bits: above every
-// number, or below with the sign bit set. Eight rows of 8192
-// take 18 us, 1792 of them 50, whatever top_k is.
+// number, or below with the sign bit set. Eight rows of 8192 take 18 us, 1792 of them 50, whatever top_k is.
 __device__ __noinline__ int hits_by_block(const float* __restrict__ row, int L, int k, int lo_tok, int hi_tok, HitBlock& sm) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int kOwn = kHitBins / kHitThreads;
@@ -243,7 +242,7 @@ hit_count_kernel(const float* __restrict__ attn, int n_steps, int n_heads, int64
         int n_ent = 0;
 #pragma unroll
         for (int g = 0; g < kHitGroups; ++g) {
-          const bool in = gm[g] >= bound;
+          const bool in = lane + 32 * (g * gs) < nvec && gm[g] >= bound;  // a short row leaves most groups empty
           const uint32_t b = __ballot_sync(0xffffffffu, in);
           if (in) sm.entry[n_ent + __popc(b & lt)] = static_cast<uint16_t>(g * 32 + lane);
           n_ent += __popc(b);
