@@ -1282,6 +1282,103 @@ __device__ __noinline__ void smooth_head(const Shape& sh, const float2* __restri
   else select_head<BIG, false>(sh.window, status);
 }
 
+// Variant: local pooling instead of the spectral filter: pooled over |i - j| <= pool_kernel / 2 (average: zero padding counts in
+// the divisor; maximum: padding never wins), mixed with alpha and written out; the selection then reads it back. The
+// sequence goes through shared memory, in stretches when it is longer; scores and smoothed may be the same array, so what a
+// stretch needs from before its start comes from the stretch before.
+__device__ __noinline__ void pool_head(const Shape& sh, bool sel, int* status) {
+  const int n = S.pl.n;
+  const float* x = S.x;
+  float* y = S.y;
+  float* st = reinterpret_cast<float*>(g_sbuf);  // st[i - base] = x[i]
+  if (threadIdx.x == 0) {
+    S.kmin = 0xffffffffu;
+    S.kmax = 0u;
+  }
+  const int hw = sh.pool_kernel / 2;  // at most 511
+  static_assert(kT > 511, "a thread per value carried over");
+  const bool is_max = sh.smooth_mode == AUDIOKV_SMOOTH_MAX_POOL;
+  const float inv_pool = 1.f / static_cast<float>(sh.pool_kernel), al = sh.alpha, om = 1.f - sh.alpha;
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+  const int room = 2 * S.pl.root_at, stretch = n <= room ? n : room - 2 * hw;
+  int base = 0;
+#pragma unroll 1
+  for (int c0 = 0; c0 < n; c0 += stretch) {
+    const int c1 = min(n, c0 + stretch), end = min(n, c1 + hw);
+    if (c0 > 0) {
+      const int t = threadIdx.x;
+      const float keep = t < hw ? st[c0 - hw + t - base] : 0.f;
+      __syncthreads();
+      if (t < hw) st[t] = keep;
+      base = c0 - hw;
+    }
+    batched<8>(end - c0, [&](int t) { return x[c0 + t]; }, [&](int t, float v) { st[c0 + t - base] = v; });
+    __syncthreads();
+    auto mix = [&](int j, float acc) {
+      const float v = fmaf(al, is_max ? acc : acc * inv_pool, om * st[j - base]);
+      if (y) y[j] = v;
+      kmin = min(kmin, score_key(v));
+      kmax = max(kmax, score_key(v));
+    };
+    // Four tokens of a thread at a time, their reads in flight together, where no window reaches over an end.
+    constexpr int Q = 4;
+    for (int j0 = c0 + threadIdx.x; j0 < c1; j0 += Q * kT) {
+      if (j0 >= hw && j0 + (Q - 1) * kT < c1 && j0 + (Q - 1) * kT + hw < n) {
+        const float* p = st + j0 - hw - base;
+        float acc[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) acc[q] = is_max ? -INFINITY : 0.f;
+        if (is_max) {
+#pragma unroll 4
+          for (int i = 0; i < sh.pool_kernel; ++i)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) acc[q] = fmaxf(acc[q], p[i + q * kT]);
+        } else {
+#pragma unroll 4
+          for (int i = 0; i < sh.pool_kernel; ++i)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) acc[q] += p[i + q * kT];
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) mix(j0 + q * kT, acc[q]);
+      } else {
+#pragma unroll 1
+        for (int j = j0; j < min(c1, j0 + Q * kT); j += kT) {
+          const float* p = st - base;
+          const int lo = max(0, j - hw), hi = min(n - 1, j + hw);
+          float acc = is_max ? -INFINITY : 0.f;
+          if (is_max) {
+#pragma unroll 8
+            for (int i = lo; i <= hi; ++i) acc = fmaxf(acc, p[i]);
+          } else {
+#pragma unroll 8
+            for (int i = lo; i <= hi; ++i) acc += p[i];
+          }
+          mix(j, acc);
+        }
+      }
+    }
+    __syncthreads();  // everybody is done with the stretch
+  }
+  if (threadIdx.x == 0 && S.kstar_out) *S.kstar_out = 0;
+  if (!sel) return;
+  if (y == nullptr) {
+    if (threadIdx.x == 0) atomicExch(status, AUDIOKV_EDEVICE);
+    return;
+  }
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&S.kmin, kmin);
+    atomicMax(&S.kmax, kmax);
+  }
+  __syncthreads();  // y is complete; the sequence makes room for the masks
+  int* words = reinterpret_cast<int*>(g_sbuf);
+  select_entries<kT, false>([&](int j) -> float2 { return make_float2(__uint_as_float(score_key(y[j])), 0.f); }, n, n, sh.window,
+                            S.k_keep, S.kmin, S.kmax, S.out, &S.sel, reinterpret_cast<uint32_t*>(words),
+                            words + select_words(n, false), status);
+}
+
 __global__ void __launch_bounds__(kT, 1)
 sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict__ plans,
            const float2* __restrict__ tables, const float* scores, float* smoothed /* may alias scores */,
@@ -1339,52 +1436,7 @@ sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict
     }
     __syncthreads();
     if (sh.smooth_mode >= AUDIOKV_SMOOTH_AVG_POOL) {
-      // Variant: local pooling instead of the spectral filter. The sequence is staged first (scores and smoothed
-      // may be the same array), pooled over |i - j| <= pool_kernel / 2 (average: zero padding counts in the
-      // divisor; maximum: padding never wins), mixed with alpha and written out; the selection then reads it back.
-      const int n = P;
-      const float* x = S.x;
-      float* y = S.y;
-      float* st = S.pl.in_smem ? reinterpret_cast<float*>(g_sbuf) : reinterpret_cast<float*>(S.g);
-      if (threadIdx.x == 0) {
-        S.kmin = 0xffffffffu;
-        S.kmax = 0u;
-      }
-#pragma unroll 4
-      for (int j = threadIdx.x; j < n; j += kT) st[j] = x[j];
-      __syncthreads();
-      const int hw = sh.pool_kernel / 2;
-      const bool is_max = sh.smooth_mode == AUDIOKV_SMOOTH_MAX_POOL;
-      const float inv_pool = 1.f / static_cast<float>(sh.pool_kernel), al = sh.alpha, om = 1.f - sh.alpha;
-      uint32_t kmin = 0xffffffffu, kmax = 0u;
-      for (int j = threadIdx.x; j < n; j += kT) {
-        const int lo = max(0, j - hw), hi = min(n - 1, j + hw);
-        float acc = is_max ? -INFINITY : 0.f;
-        for (int i = lo; i <= hi; ++i) acc = is_max ? fmaxf(acc, st[i]) : acc + st[i];
-        const float pooled = is_max ? acc : acc * inv_pool;
-        const float v = fmaf(al, pooled, om * st[j]);
-        if (y) y[j] = v;
-        kmin = min(kmin, score_key(v));
-        kmax = max(kmax, score_key(v));
-      }
-      if (threadIdx.x == 0 && S.kstar_out) *S.kstar_out = 0;
-      if (sel) {
-        if (y == nullptr) {
-          if (threadIdx.x == 0) atomicExch(status, AUDIOKV_EDEVICE);
-          continue;
-        }
-        kmin = __reduce_min_sync(0xffffffffu, kmin);
-        kmax = __reduce_max_sync(0xffffffffu, kmax);
-        if ((threadIdx.x & 31) == 0) {
-          atomicMin(&S.kmin, kmin);
-          atomicMax(&S.kmax, kmax);
-        }
-        __syncthreads();  // the staged sequence makes room for the masks; y is complete
-        int* words = reinterpret_cast<int*>(g_sbuf);
-        select_entries<kT, false>([&](int j) -> float2 { return make_float2(__uint_as_float(score_key(y[j])), 0.f); }, n, P, W,
-                                  S.k_keep, S.kmin, S.kmax, S.out, &S.sel, reinterpret_cast<uint32_t*>(words),
-                                  words + select_words(n, false), status);
-      }
+      pool_head(sh, sel, status);
       continue;
     }
     if (S.pl.in_smem) smooth_head<false>(sh, tables, sel, status);

@@ -101,3 +101,25 @@ def test_radix_17_and_19(B, n):
     want = torch.fft.irfft(f * torch.where(i <= k, 1.0, torch.where(i <= k + 2, band, 0.0)), n=n, dim=1)
     # a transform is off by some sqrt(passes) roundings of the norm, two transforms by 1e-6
     assert float((y.view(2, n) - want).norm() / want.norm()) < 1e-6
+
+
+@pytest.mark.parametrize("n,window", [(600, 1023), (2047, 1), (8160, 7), (50000, 1023), (50001, 255), (131040, 7)])
+@pytest.mark.parametrize("mode", [3, 4])
+def test_pooling_in_stretches(B, n, window, mode):
+    """Sequences shorter than the window, on chip, and in several stretches, into another array and in place: the sum of a window
+    in 32 bits is off by at most its length in roundings of it, a maximum by none."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n)
+    x = torch.rand((2, n), generator=gen, device="cuda")
+    prob = _problem(B, 2, [n], smooth_mode=mode, pool_kernel=window, alpha=1.0)
+    y, ks = _smooth(B, prob, x.reshape(-1))
+    if mode == B.AUDIOKV_SMOOTH_AVG_POOL:
+        want = torch.nn.functional.avg_pool1d(x.double()[:, None], window, 1, window // 2)[:, 0]
+        assert float((y.view(2, n) - want).abs().max()) <= window * 2.0 ** -24
+    else:
+        want = torch.nn.functional.max_pool1d(torch.nn.functional.pad(x, (window // 2, window // 2))[:, None], window, 1)
+        assert torch.equal(y.view(2, n), want[:, 0])     # the values are positive: zeros never win
+    ctx = B.Context(prob)
+    B.audiokv_smooth(ctx, prob, x, x)
+    torch.cuda.synchronize()
+    assert torch.equal(x.reshape(-1), y) and ks.tolist() == [0, 0]
