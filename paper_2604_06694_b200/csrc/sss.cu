@@ -14,8 +14,7 @@
 // What bounds it: a head is a chain of short phases with a barrier between them, each a few thousand cycles of
 // shared-memory traffic and index arithmetic on one SM; HBM sees only the scores coming in and the indices going out.
 // So the block reads the scores once into shared memory, 512 threads keep eight or more independent accesses in
-// flight each (128 registers; the earlier 1024 threads with 64 registers spent more cycles on the barriers and on
-// radix-4 passes than on arithmetic), every access to shared memory is a compile-time LDS / STS through a swizzle
+// flight each (128 registers), every access to shared memory is a compile-time LDS / STS through a swizzle
 // that keeps the power-of-two strides of the passes and the digit-reversed reads of the spectrum off the same banks,
 // and twiddles come from a two-level table of roots of unity in shared memory. Heads are taken from a queue, since what a
 // head costs shows only in its scores. 112 heads of 8160 tokens, no transform: 27 us; 192 heads of 16352 tokens, two
@@ -366,8 +365,8 @@ __device__ __forceinline__ void one_pair(int total, int ns, const FftSeq& sq, in
 // A_c = a_0 + sum_s P_s cos(2 pi s c / p), B_c = sum_s Q_s sin(2 pi s c / p): a product of a small matrix with as many
 // columns as there are butterflies. A thread computes a tile of TO outputs x TC butterflies in registers: per s it reads TC
 // values of P and of Q and TO (cos, sin) pairs, the latter the same for most of a warp and staged in shared memory, for 4 TO TC
-// FMAs. 8 x 2 where that gives enough tiles to go round, 2 x 1 for few butterflies (which are latency: a length of 7 x 167
-// has 44 tiles of 8 x 2, two warps' worth). The folding sweep (inverse) and the write-back (forward) carry the
+// FMAs. 8 x 2 or 8 x 1 where that makes tiles for five warps, in one round (4815 = 45 x 107: 71 -> 59 us against three rounds of
+// 2 x 1), 2 x 1 for few butterflies (which are latency: a length of 7 x 167 has 44 tiles of 8 x 2, two warps' worth). The folding sweep (inverse) and the write-back (forward) carry the
 // pass twiddles. (An earlier version gave a thread 5 outputs of one butterfly and looked the cosines up by (s c mod p): the
 // radix-73 pass of N = 8176 took 45-55 k cycles, seven loads and their index arithmetic for every 20 FMAs.)
 template <bool INV, class Buf, int TO, int TC>
@@ -489,6 +488,7 @@ __device__ __noinline__ void pass_prime(const Buf buf, int total, int ns, int N,
     buf.st(e1, csub(x, y));
   }
   if (nb * fft_mat_cols(p) >= 16 * 160) prime_product<INV, Buf, 8, 2>(buf, ns, p, m, nb, step, root, mat);
+  else if (nb * fft_mat_cols(p) >= 8 * 160) prime_product<INV, Buf, 8, 1>(buf, ns, p, m, nb, step, root, mat);
   else prime_product<INV, Buf, 2, 1>(buf, ns, p, m, nb, step, root, mat);
 }
 
