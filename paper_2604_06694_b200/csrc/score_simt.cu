@@ -12,11 +12,10 @@
 // The product is a register-tiled matrix product, 8 keys x 4, 7 or 8 query rows a thread. The tile's keys lie transposed in shared
 // memory for as long as the tile lasts, two neighbouring keys make a packed pair of accumulators, and the query rows
 // come in panels of 32 dimensions by asynchronous copies, the next one under the arithmetic of this one, across row tiles.
-// 128 registers, 16 warps an SM: 191 us for 28 heads at 4096 keys (the FMA pipe 61 % busy by its counter, its throttle the
+// 128 registers, 16 warps an SM: 180 to 191 us for 28 heads at 4096 keys (the FMA pipe 61 % busy by its counter, its throttle the
 // first stall). What was tried on the way on that launch: scalar FMAs in this layout 217 us, in rows of either side 240 us, held up by
 // dispatch stalls of three-operand reads; pairs of even and odd dimensions 218 us, and 201 us with half the address
-// arithmetic: twice the accumulators leave two warps a scheduler, which do not cover their latencies. The 64 x 64 tiles of 4 x 4
-// logits that were here first, with the logits through shared memory and the product done twice, took 1487 + 1234 us for 112 heads.
+// arithmetic: twice the accumulators leave two warps a scheduler, which do not cover their latencies.
 // Logits are kept in base 2 (scale * log2 e folded into one multiply).
 #include <algorithm>
 

@@ -1,4 +1,4 @@
-// Top-k of one head's scores by radix select, for one thread block.
+// Top-k of one head's scores by histograms of their keys, for one thread block.
 // Shared by the stand-alone selection kernel and by the smoothing kernel, which selects straight from the
 // smoothed scores it still holds on chip.
 #pragma once

@@ -1,4 +1,4 @@
-// Per-head top-k by radix select, ordered compaction of the kept indices, and the
+// Per-head top-k (see select.cuh), ordered compaction of the kept indices, and the
 // vectorised gather of the kept K and V rows into the compacted cache.
 #include "common.cuh"
 #include "select.cuh"
