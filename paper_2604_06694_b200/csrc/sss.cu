@@ -1029,9 +1029,11 @@ __device__ __noinline__ void transform_head(const Shape& sh, const float2* __res
   // 2. The spectrum of the real sequence and the cut-off, the smallest k with E(k) = sum_{i<=k} |F_i|^2 >= rho E(Kb) (fp64).
   //    packed: Z is turned into F pairwise in place (the slot of bin 0 holds (F_0, F_N), both real). Energies are summed by
   //    chunks of 32 neighbouring bins (one warp's share): chunk i of the low bins at energy[i], chunk i of their partners
-  //    N - k, which count downwards, at energy[2 nc - 1 - i]. The threshold is taken from the sum of all bins, not from
-  //    Parseval's identity, though that would let the sums end at the cut-off: the bins are fp32 and their total is off by
-  //    1e-7 of the energy, which near rho = 1 is many bins of a spectrum that falls off.
+  //    N - k, which count downwards, at energy[2 nc - 1 - i].
+  //    The threshold is taken from the sum of all bins. Parseval's identity gives a total before that, but the bins are
+  //    fp32 and their own sum is off from it by some 1e-7 of the energy, which near rho = 1 is many bins of a spectrum that falls
+  //    off. So it serves only to end the sums early, 2048 low bins at a time, and only for a cut-off that is clear of the
+  //    threshold by more than the two totals can differ.
   const bool no_mean = sh.smooth_mode == AUDIOKV_SMOOTH_ENERGY_NO_MEAN;  // variant: bin 0 adds no energy
   const int n_low = packed ? N / 2 + 1 : Kb + 1;
   const int nc = (n_low + 31) / 32, n_chunk = packed ? 2 * nc : nc;
@@ -1044,81 +1046,107 @@ __device__ __noinline__ void transform_head(const Shape& sh, const float2* __res
     fk = cadd(E, T);
     fq = cconj(csub(E, T));
   };
-  const bool fixed = sh.smooth_mode == AUDIOKV_SMOOTH_FIXED_FRACTION;  // variant: no energies needed, step 3 splits the bins
-  constexpr int U = 4;
-#pragma unroll 1
-  for (int c0 = 0; c0 < nc && !fixed; c0 += U * kWarps) {
-    uint2 at[U];
-#pragma unroll
-    for (int q = 0; q < U; ++q) at[q] = slots_of(min(32 * (c0 + q * kWarps + warp) + lane, n_low - 1));
-#pragma unroll
-    for (int q = 0; q < U; ++q) {
-      const int c = c0 + q * kWarps + warp, k = 32 * c + lane;
-      double el = 0.0, eh = 0.0;
-      if (k < n_low) {
-        float2 fk = buf.ld(at[q].x);
-        if (packed) {
-          float2 fq;
-          split(k, fk, buf.ld(at[q].y), fk, fq);
-          buf.st(at[q].x, k == 0 ? make_float2(fk.x, fq.x) : fk);
-          if (k > 0) buf.st(at[q].y, fq);
-          eh = 2 * k == N ? 0.0 : sq_abs(fq);
-        }
-        el = k == 0 && no_mean ? 0.0 : sq_abs(fk);
-      }
-      // both sums in one tree: the lower half of the warp goes on with the low bins, the upper half with the others
-      const double ol = __shfl_xor_sync(0xffffffffu, el, 16), oh = __shfl_xor_sync(0xffffffffu, eh, 16);
-      double v = (lane & 16) ? eh + oh : el + ol;
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (c < nc) {
-        if (lane == 0) S.energy[c] = v;
-        if (lane == 16 && packed) S.energy[2 * nc - 1 - c] = v;
-      }
-    }
-  }
-  __syncthreads();
+  const bool fixed = sh.smooth_mode == AUDIOKV_SMOOTH_FIXED_FRACTION;  // variant: no energies needed
+  int summed = 0;  // chunks of low bins that have their sums and, packed, have been split with their partners
   if (fixed) {
     if (threadIdx.x == 0) S.kstar = min(static_cast<int>(floor(static_cast<double>(sh.smooth_kappa) * Kb)), Kb);
-  } else if (warp == 0) {
-    // every lane sums a run of chunks; then the lane, the chunk and the bin that reach the threshold
-    const int per = (n_chunk + 31) / 32, c0 = min(n_chunk, lane * per), c1 = min(n_chunk, c0 + per);
-    double own = 0.0;
-    for (int c = c0; c < c1; ++c) own += S.energy[c];
-    const double inc = warp_prefix(own), total = __shfl_sync(0xffffffffu, inc, 31);
-    // all of a total above zero is reached at the last bin, whatever the rounding of the sums
-    const double thr = sh.rho < 1.f || !(total > 0.0) ? static_cast<double>(sh.rho) * total : INFINITY;
-    const uint32_t hit = __ballot_sync(0xffffffffu, inc >= thr);
-    int ks = Kb;
-    if (hit) {
-      double run = inc - own;
-      int chunk = c0;
-      while (chunk + 1 < c1 && !(run + S.energy[chunk] >= thr)) run += S.energy[chunk++];
-      chunk = __shfl_sync(0xffffffffu, chunk, __ffs(hit) - 1);
-      run = __shfl_sync(0xffffffffu, run, __ffs(hit) - 1);
-      // the chunk's bins in ascending order, one per lane
-      const bool upper = packed && chunk >= nc;
-      const int k = upper ? N - (32 * (2 * nc - 1 - chunk) + 31 - lane) : 32 * chunk + lane;
-      const bool in = upper ? (k >= N - N / 2 && 2 * k != N && k <= N) : k < n_low;
-      double e = 0.0;
-      if (in) {
-        if (packed && (k == N || k == 0)) {
-          const float2 f = buf.ld(0);
-          e = k == N ? static_cast<double>(f.y) * f.y : no_mean ? 0.0 : static_cast<double>(f.x) * f.x;
-        } else if (!(k == 0 && no_mean)) {
-          const uint2 at = slots_of(upper ? N - k : k);
-          e = sq_abs(buf.ld(upper ? at.y : at.x));
-        }
-      }
-      e = warp_prefix(e);
-      const uint32_t reach = __ballot_sync(0xffffffffu, in && run + e >= thr);
-      const uint32_t any = __ballot_sync(0xffffffffu, in);
-      const int at_lane = reach ? __ffs(reach) - 1 : 31 - __clz(any | 1u);  // rounding of the two sums: the chunk's last bin
-      ks = min(max(__shfl_sync(0xffffffffu, k, at_lane), 0), Kb);
+    __syncthreads();
+  } else {
+    double whole = 0.0, margin = 0.0, early = INFINITY;
+    if (nc > 64 && sh.rho < 1.f) {  // more than one turn of sums
+      const double F0 = S.sums[0], FN = S.sums[2];
+      const double total = 0.5 * (static_cast<double>(n) * S.sums[1] + F0 * F0 + ((n & 1) ? 0.0 : FN * FN));
+      // The transform is off by less than kOff of the spectrum's norm (33 roundings; six were the most seen), the energies by this:
+      constexpr double kOff = 2e-6;
+      whole = no_mean ? fmax(total - F0 * F0, 0.0) : total;
+      margin = 2.0 * kOff * sqrt(whole * total) + kOff * kOff * total;
+      early = static_cast<double>(sh.rho) * whole + margin;
     }
-    if (lane == 0) S.kstar = ks;
+    double run = 0.0;
+    constexpr int U = 4;
+    static_assert(U * kWarps == 64, "two chunks per lane and round");
+#pragma unroll 1
+    for (bool last = false;; last = true) {
+#pragma unroll 1
+      while (summed < nc && (last || !(run >= early))) {
+        uint2 at[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) at[q] = slots_of(min(32 * (summed + q * kWarps + warp) + lane, n_low - 1));
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+          const int c = summed + q * kWarps + warp, k = 32 * c + lane;
+          double el = 0.0, eh = 0.0;
+          if (k < n_low) {
+            float2 fk = buf.ld(at[q].x);
+            if (packed) {
+              float2 fq;
+              split(k, fk, buf.ld(at[q].y), fk, fq);
+              buf.st(at[q].x, k == 0 ? make_float2(fk.x, fq.x) : fk);
+              if (k > 0) buf.st(at[q].y, fq);
+              eh = 2 * k == N ? 0.0 : sq_abs(fq);
+            }
+            el = k == 0 && no_mean ? 0.0 : sq_abs(fk);
+          }
+          // both sums in one tree: the lower half of the warp goes on with the low bins, the upper half with the others
+          const double ol = __shfl_xor_sync(0xffffffffu, el, 16), oh = __shfl_xor_sync(0xffffffffu, eh, 16);
+          double v = (lane & 16) ? eh + oh : el + ol;
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (c < nc) {
+            if (lane == 0) S.energy[c] = v;
+            if (lane == 16 && packed) S.energy[2 * nc - 1 - c] = v;
+          }
+        }
+        summed += U * kWarps;
+        __syncthreads();
+        if (summed < nc && !last) run += warp_sum(S.energy[summed - 64 + lane] + S.energy[summed - 32 + lane]);
+      }
+      const bool exact = summed >= nc;
+      if (warp == 0) {
+        // every lane sums a run of chunks; then the lane, the chunk and the bin that reach the threshold
+        const int avail = exact ? n_chunk : summed, per = (avail + 31) / 32, c0 = min(avail, lane * per), c1 = min(avail, c0 + per);
+        double own = 0.0;
+        for (int c = c0; c < c1; ++c) own += S.energy[c];
+        const double inc = warp_prefix(own), all = __shfl_sync(0xffffffffu, inc, 31), sum = exact ? all : whole;
+        // all of a total above zero is reached at the last bin, whatever the rounding of the sums
+        const double thr = sh.rho < 1.f || !(sum > 0.0) ? static_cast<double>(sh.rho) * sum : INFINITY;
+        const uint32_t hit = __ballot_sync(0xffffffffu, inc >= thr);
+        int ks = exact ? Kb : -1;
+        if (hit) {
+          double before = inc - own;
+          int chunk = c0;
+          while (chunk + 1 < c1 && !(before + S.energy[chunk] >= thr)) before += S.energy[chunk++];
+          chunk = __shfl_sync(0xffffffffu, chunk, __ffs(hit) - 1);
+          before = __shfl_sync(0xffffffffu, before, __ffs(hit) - 1);
+          // the chunk's bins in ascending order, one per lane
+          const bool upper = packed && chunk >= nc;
+          const int k = upper ? N - (32 * (2 * nc - 1 - chunk) + 31 - lane) : 32 * chunk + lane;
+          const bool in = upper ? (k >= N - N / 2 && 2 * k != N && k <= N) : k < n_low;
+          double e = 0.0;
+          if (in) {
+            if (packed && (k == N || k == 0)) {
+              const float2 f = buf.ld(0);
+              e = k == N ? static_cast<double>(f.y) * f.y : no_mean ? 0.0 : static_cast<double>(f.x) * f.x;
+            } else if (!(k == 0 && no_mean)) {
+              const uint2 at = slots_of(upper ? N - k : k);
+              e = sq_abs(buf.ld(upper ? at.y : at.x));
+            }
+          }
+          const double up_to = before + warp_prefix(e);
+          const uint32_t reach = __ballot_sync(0xffffffffu, in && up_to >= thr);
+          const uint32_t any = __ballot_sync(0xffffffffu, in);
+          const int at_lane = reach ? __ffs(reach) - 1 : 31 - __clz(any | 1u);  // rounding of the two sums: the chunk's last bin
+          ks = min(max(__shfl_sync(0xffffffffu, k, at_lane), 0), Kb);
+          const int clear = up_to >= thr + margin && (ks == 0 || up_to - e <= thr - margin);
+          if (!__shfl_sync(0xffffffffu, clear, at_lane) && !exact) ks = -1;
+        }
+        if (lane == 0) S.kstar = ks;
+      }
+      __syncthreads();
+      if (S.kstar >= 0) break;  // else close: with the sums of all bins
+      __syncthreads();
+    }
   }
-  __syncthreads();
   const int kstar = S.kstar;
 
   // 3. mask (1 up to k*, raised-cosine tail of T bins, 0 beyond) and back to the packed transform
@@ -1133,7 +1161,7 @@ __device__ __noinline__ void transform_head(const Shape& sh, const float2* __res
       float2 ok = make_float2(0.f, 0.f), oq = ok;
       if (k <= k_hi) {  // else its partner, further up, is masked away as well
         float2 fk = buf.ld(at.x), fq = buf.ld(at.y);
-        if (fixed) {
+        if (k >= 32 * summed) {
           split(k, fk, fq, fk, fq);
         } else if (k == 0) {
           fq = make_float2(fk.y, 0.f);
