@@ -5,7 +5,7 @@
 // one warp, which streams it through registers and keeps the maxima of 32 groups of its values per lane; the k-th largest
 // of the lanes' maxima bounds the k-th largest value from below; the few groups that reach the bound are read once more
 // (from L2) and their values listed; the listed values inside the span are ranked against the list. No barrier joins
-// two warps, so that twenty rows an SM are in different phases and the loads never stop: 285 us, 88 % of the measured
+// two warps, so that twenty rows an SM are in different phases and the loads never stop: 289 us, 87 % of the measured
 // copy bandwidth. Rows a list cannot serve (top_k above 32, many values equal to the bound, NaN) are left to the
 // whole block, a histogram of the keys at a time.
 #include "common.cuh"
