@@ -221,6 +221,18 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// One lane of a converged warp, in a form from which the compiler knows that a single thread goes on.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "elect.sync _|p, 0xffffffff;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(one));
+  return one != 0;
+}
 // The mbarrier gets one arrival when every MMA issued so far by this thread has finished.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -660,62 +672,67 @@ score_umma_kernel(const __grid_constant__ TmapPack<CAP> tm, const UmmaArgs a) {
       }
     }
   } else if (warp == kMmaWarp || warp == kMmaWarp + 1) {
-    if (lane == 0) {
-      // ---- MMA issuer of group g ----
-      // Tile `it` of the CTA belongs to group it & 1 and sits in stage it % S of the K ring. Its parts go to the
-      // group's buffers in turn: part number qc of the group uses buffer qc & 1, in phase (qc >> 1) & 1 of the
-      // buffer's barriers.
-      const int g = warp - kMmaWarp;
-      int it = 0, heads = 0, prev_u = -1, qc = 0;
-      bool ok = true;
-      ScoreUnit Unext = a.units[unit_begin < unit_end ? unit_begin : 0];
-      for (int n = unit_begin; n < unit_end && ok; ++n) {
-        const ScoreUnit U = Unext;
-        if (n + 1 < unit_end) Unext = a.units[n + 1];  // the next descriptor arrives under this run's work
-        if (U.qid != prev_u) {
-          if (prev_u != -1) umma_commit(smem_u32(&sm->q_empty));  // this thread's MMAs on the old Q tile are done
-          ok = mbar_wait(smem_u32(&sm->q_full), heads & 1, abort, wl);
+    // ---- MMA issuer of group g ----
+    // Tile `it` of the CTA belongs to group it & 1 and sits in stage it % S of the K ring. Its parts go to the
+    // group's buffers in turn: part number qc of the group uses buffer qc & 1, in phase (qc >> 1) & 1 of the
+    // buffer's barriers.
+    // The whole warp walks the schedule and waits; one elected lane issues, in code that the compiler knows to be the
+    // warp's one thread. Under a plain `lane == 0` the descriptors cannot go to uniform registers, and an MMA
+    // takes about 200 cycles to issue instead of the 56 to 64 it needs to run.
+    const int g = warp - kMmaWarp;
+    const bool leader = elect_one();
+    int it = 0, heads = 0, prev_u = -1, qc = 0;
+    bool ok = true;
+    ScoreUnit Unext = a.units[unit_begin < unit_end ? unit_begin : 0];
+    for (int n = unit_begin; n < unit_end && ok; ++n) {
+      const ScoreUnit U = Unext;
+      if (n + 1 < unit_end) Unext = a.units[n + 1];  // the next descriptor arrives under this run's work
+      if (U.qid != prev_u) {
+        if (prev_u != -1 && leader) umma_commit(smem_u32(&sm->q_empty));  // this thread's MMAs on the old Q tile are done
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sm->q_full), heads & 1, abort, wl));
+        if (!ok) break;
+        tc_fence_after();
+        prev_u = U.qid;
+        ++heads;
+      }
+      for (int t = 0; t < U.n_tiles && ok; ++t, ++it) {
+        if ((it & 1) != g) continue;  // the other warp's tile
+        const int s = it % S;
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sm->k_full[s]), (it / S) & 1, abort, wl));
+        if (!ok) break;
+        const uint64_t dk = umma_desc(smem_u32(k_s + s * kKStage));
+        for (int p = 0; p < n_parts; ++p) {
+          const int b = qc & 1;
+          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sm->acc_empty[g][b]), ((qc >> 1) & 1) ^ 1, abort, wl));
           if (!ok) break;
+          ++qc;
           tc_fence_after();
-          prev_u = U.qid;
-          ++heads;
-        }
-        for (int t = 0; t < U.n_tiles && ok; ++t, ++it) {
-          if ((it & 1) != g) continue;  // the other thread's tile
-          const int s = it % S;
-          ok = mbar_wait(smem_u32(&sm->k_full[s]), (it / S) & 1, abort, wl);
-          if (!ok) break;
-          const uint32_t k_addr = smem_u32(k_s + s * kKStage);
-          const uint32_t q_addr = smem_u32(q_s);
-          for (int p = 0; p < n_parts; ++p) {
-            const int b = qc & 1;
-            ok = mbar_wait(smem_u32(&sm->acc_empty[g][b]), ((qc >> 1) & 1) ^ 1, abort, wl);
-            if (!ok) break;
-            ++qc;
-            tc_fence_after();
-            const uint32_t d_tmem = tmem_base + (2 * g + b) * 128;
-            // byte offset of the part inside the Q tile (a multiple of 1024: whole 8-row groups)
-            const uint32_t q_off = SWEEP == 1 ? p * (128 * 128) : (p == 0 ? 0 : cols0 * 128);
-            const uint32_t idesc = SWEEP == 1 ? umma_idesc(128, kTileKeys) : umma_idesc(kTileKeys, p == 0 ? cols0 : cols1);
+          const uint32_t d_tmem = tmem_base + (2 * g + b) * 128;
+          // byte offset of the part inside the Q tile (a multiple of 1024: whole 8-row groups)
+          const uint32_t q_off = SWEEP == 1 ? p * (128 * 128) : (p == 0 ? 0 : cols0 * 128);
+          const uint32_t idesc = SWEEP == 1 ? umma_idesc(128, kTileKeys) : umma_idesc(kTileKeys, p == 0 ? cols0 : cols1);
+          const uint64_t dq = umma_desc(smem_u32(q_s) + q_off);
+          if (leader) {
 #pragma unroll
             for (int kb = 0; kb < KB; ++kb) {
 #pragma unroll
-              for (int ks = 0; ks < 4; ++ks) {
-                const uint64_t dq = umma_desc(q_addr + kb * q_blk + q_off + ks * 32);
-                const uint64_t dk = umma_desc(k_addr + kb * kKBlk + ks * 32);
-                if (SWEEP == 1) umma_bf16(d_tmem, dq, dk, idesc, (kb | ks) != 0);
-                else umma_bf16(d_tmem, dk, dq, idesc, (kb | ks) != 0);
+              for (int ks = 0; ks < 4; ++ks) {  // the address field counts 16 bytes and does not run over: 227 KB
+                const uint64_t q_at = dq + static_cast<uint32_t>((kb * q_blk + ks * 32) >> 4);
+                const uint64_t k_at = dk + static_cast<uint32_t>((kb * kKBlk + ks * 32) >> 4);
+                if (SWEEP == 1) umma_bf16(d_tmem, q_at, k_at, idesc, (kb | ks) != 0);
+                else umma_bf16(d_tmem, k_at, q_at, idesc, (kb | ks) != 0);
               }
             }
             umma_commit(smem_u32(&sm->acc_full[g][b]));
+            if (p == n_parts - 1) umma_commit(smem_u32(&sm->k_empty[s]));
           }
-          if (ok) umma_commit(smem_u32(&sm->k_empty[s]));
+          __syncwarp();
         }
       }
-      if (*abort) {  // TMEM must not be released under MMAs that are still running
-        umma_commit(smem_u32(&sm->drain[g]));
-        mbar_wait_drain(smem_u32(&sm->drain[g]), 0);
-      }
+    }
+    if (*abort) {  // TMEM must not be released under MMAs that are still running
+      if (leader) umma_commit(smem_u32(&sm->drain[g]));
+      mbar_wait_drain(smem_u32(&sm->drain[g]), 0);
     }
   } else {
     // ---- epilogue: two groups of kSets sets of four warps; warp w reads TMEM lanes 32 (w % 4) .. +31 ----
