@@ -489,15 +489,17 @@ __device__ __forceinline__ void colsum_part(const uint32_t (&r)[32], const float
 // loop has no branch on chunk counts or on a half-filled last buffer. The part's buffer is handed back to the MMA
 // thread once this set's last chunk is in registers (at once when the set has no chunk in the part).
 template <int COLS, int SET>
-__device__ __forceinline__ void colsum_cols_set(uint32_t taddr, const float* __restrict__ ncp, f32x2 sl2, uint32_t ebar, int lane,
+__device__ __forceinline__ void colsum_cols_set(uint32_t taddr, const float* __restrict__ ncp, f32x2 sl2, uint32_t ebar, bool give, int lane,
                                                 uint32_t (&ra)[32], f32x2& a0, f32x2& a1, f32x2& a2, f32x2& a3) {
   constexpr int n_ch = (COLS + 31) / 32;
   constexpr bool tail = (COLS & 16) != 0;
   constexpr int c_lo = 2 * SET, c_hi = c_lo + 2 < n_ch ? c_lo + 2 : n_ch;  // chunks [c_lo, c_hi)
   if (c_lo >= n_ch) {
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(ebar);
+    if (give) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(ebar);
+    }
     return;
   }
 #pragma unroll
@@ -507,7 +509,7 @@ __device__ __forceinline__ void colsum_cols_set(uint32_t taddr, const float* __r
     else tmem_ld32_issue(taddr + c * 32, ra);
     if (half) tmem_wait_lo(ra);
     else tmem_wait(ra);
-    if (c == c_hi - 1) {
+    if (c == c_hi - 1 && give) {
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(ebar);
@@ -545,6 +547,9 @@ score_umma_kernel(const __grid_constant__ TmapPack<CAP> tm, const UmmaArgs a) {
   const int n_parts = SWEEP == 1 ? (R > 128 ? 2 : 1) : (a.r_pad > 128 ? 2 : 1);
   const int cols0 = SWEEP == 1 ? kTileKeys : (n_parts == 2 ? ((a.r_pad >> 4) + 1) / 2 * 16 : a.r_pad);
   const int cols1 = SWEEP == 1 ? kTileKeys : a.r_pad - cols0;
+  // Sweep 2 of more than 128 rows: one MMA over all of them, so that the K tile is read from shared memory once (128 x 112 x 16
+  // takes 90 cycles, bound by its operands, 128 x 224 x 16 takes 117). The parts then share one accumulator of the group's 256 columns.
+  const bool wide = SWEEP == 2 && n_parts == 2;
 
   // ---- set-up ----
   if (threadIdx.x == 0) {
@@ -701,16 +706,16 @@ score_umma_kernel(const __grid_constant__ TmapPack<CAP> tm, const UmmaArgs a) {
         ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sm->k_full[s]), (it / S) & 1, abort, wl));
         if (!ok) break;
         const uint64_t dk = umma_desc(smem_u32(k_s + s * kKStage));
-        for (int p = 0; p < n_parts; ++p) {
-          const int b = qc & 1;
-          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sm->acc_empty[g][b]), ((qc >> 1) & 1) ^ 1, abort, wl));
+        for (int p = 0; p < (wide ? 1 : n_parts); ++p) {
+          const int b = wide ? 0 : qc & 1;
+          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&sm->acc_empty[g][b]), ((wide ? qc : qc >> 1) & 1) ^ 1, abort, wl));
           if (!ok) break;
           ++qc;
           tc_fence_after();
           const uint32_t d_tmem = tmem_base + (2 * g + b) * 128;
           // byte offset of the part inside the Q tile (a multiple of 1024: whole 8-row groups)
-          const uint32_t q_off = SWEEP == 1 ? p * (128 * 128) : (p == 0 ? 0 : cols0 * 128);
-          const uint32_t idesc = SWEEP == 1 ? umma_idesc(128, kTileKeys) : umma_idesc(kTileKeys, p == 0 ? cols0 : cols1);
+          const uint32_t q_off = SWEEP == 1 ? p * (128 * 128) : 0;
+          const uint32_t idesc = SWEEP == 1 ? umma_idesc(128, kTileKeys) : umma_idesc(kTileKeys, wide ? a.r_pad : cols0);
           const uint64_t dq = umma_desc(smem_u32(q_s) + q_off);
           if (leader) {
 #pragma unroll
@@ -724,7 +729,7 @@ score_umma_kernel(const __grid_constant__ TmapPack<CAP> tm, const UmmaArgs a) {
               }
             }
             umma_commit(smem_u32(&sm->acc_full[g][b]));
-            if (p == n_parts - 1) umma_commit(smem_u32(&sm->k_empty[s]));
+            if (wide || p == n_parts - 1) umma_commit(smem_u32(&sm->k_empty[s]));
           }
           __syncwarp();
         }
@@ -807,13 +812,16 @@ score_umma_kernel(const __grid_constant__ TmapPack<CAP> tm, const UmmaArgs a) {
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
           if (p >= n_parts || !ok) continue;
-          const int b = qc & 1;
-          ok = mbar_wait(smem_u32(&sm->acc_full[g][b]), (qc >> 1) & 1, abort, wl);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) continue;
-          ++qc;
-          tc_fence_after();
-          const uint32_t taddr = lane_addr + b * 128;
+          const int b = wide ? 0 : qc & 1;
+          if (!wide || p == 0) {
+            ok = mbar_wait(smem_u32(&sm->acc_full[g][b]), (wide ? qc : qc >> 1) & 1, abort, wl);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) continue;
+            ++qc;
+            tc_fence_after();
+          }
+          const uint32_t taddr = lane_addr + (wide ? p * cols0 : b * 128);
+          const bool give = !wide || p == 1;  // the accumulator goes back to the MMA thread with this part
           const uint32_t ebar = smem_u32(&sm->acc_empty[g][b]);
           // Steps of 64 accumulator columns (two register buffers of 32; the last one may hold 16 in sweep 2): the loads of
           // a step land within tens of cycles, so nothing is prefetched, and the arithmetic of a step is one long block
@@ -838,8 +846,8 @@ score_umma_kernel(const __grid_constant__ TmapPack<CAP> tm, const UmmaArgs a) {
             switch (cols) {  // the shapes of a launch: one or two of these
 #define AKV_COLS_CASE(C)                                                                          \
   case C:                                                                                         \
-    if ((set ^ p) == 0) colsum_cols_set<C, 0>(taddr, ncp, sl2, ebar, lane, ra, a0, a1, a2, a3);   \
-    else colsum_cols_set<C, 1>(taddr, ncp, sl2, ebar, lane, ra, a0, a1, a2, a3);                  \
+    if ((set ^ p) == 0) colsum_cols_set<C, 0>(taddr, ncp, sl2, ebar, give, lane, ra, a0, a1, a2, a3); \
+    else colsum_cols_set<C, 1>(taddr, ncp, sl2, ebar, give, lane, ra, a0, a1, a2, a3);            \
     break;
               AKV_COLS_CASE(16) AKV_COLS_CASE(32) AKV_COLS_CASE(48) AKV_COLS_CASE(64)
               AKV_COLS_CASE(80) AKV_COLS_CASE(96) AKV_COLS_CASE(112) AKV_COLS_CASE(128)
