@@ -25,7 +25,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // Byte offsets inside the workspace; status .. ctas, up to blob_end, are uploaded as one piece with a plan. What only
 // audiokv_evict_host needs lies behind the rest, so that the rest stays where a captured graph has it.
 struct Layout {
-  size_t status, reqs, plans, order, units, ctas, blob_end, tables, stats, fft_scratch, scores, kstar, aux, end;
+  size_t status, reqs, plans, order, units, ctas, ready, blob_end, tables, stats, fft_scratch, scores, kstar, aux, end;
   size_t host_units, host_ctas, host_stats, host_end;
 };
 
@@ -54,6 +54,7 @@ struct Plan {
   int max_L = 0, max_P = 0;
   int n_slab = 0;
   size_t score_room = 0;        // bytes of workspace behind everything else that the FMA scoring puts to use
+  bool follow = false;          // the gather runs beside the smoothing, head by head
   int sss_grid = 0;
   size_t sss_smem = 0;
   int64_t scratch_per_block = 0;  // float2 elements
@@ -471,6 +472,11 @@ int build_plan(const audiokv_params* p, Plan* pl) {
     for (int i = 0; i < sh.total_heads; ++i)
       pl->sss_order[i] = pl->reqs[by_cost[i / sh.heads_per_req].second].head_base + i % sh.heads_per_req;
   }
+  // The gather beside the smoothing pays as soon as some heads can end well before others: when the blocks take a second turn
+  // (48 layers of 2048 tokens, 192 heads: 145.9 -> 133.0 us a pass) or when a transform takes long beside a head that needs none
+  // (28 layers, 30 % of heads with transforms: 8192 tokens 269.7 -> 247.8, 32768 908 -> 812). Its start costs 3 us more: at 700 tokens
+  // and one turn 58.5 -> 61.4, at 1500 76.2 -> 76.1.
+  pl->follow = sh.total_heads > pl->sss_grid || pl->max_P >= 1400;
   int smem_c = 64;
   pl->scratch_per_block = 0;
   for (const FftPlan& fp : pl->fft) {
@@ -488,6 +494,7 @@ int build_plan(const audiokv_params* p, Plan* pl) {
   L.order = off;       off = align_up(off + sizeof(int32_t) * pl->sss_order.size());
   L.units = off;       off = align_up(off + sizeof(ScoreUnit) * pl->score.units.size());
   L.ctas = off;        off = align_up(off + sizeof(int32_t) * pl->score.ctas.size());
+  L.ready = off;       off = align_up(off + sizeof(uint64_t) * static_cast<size_t>(sh.total_heads));  // goes up as zeros
   L.blob_end = off;
   L.tables = off;      off = align_up(off + sizeof(float2) * static_cast<size_t>(pl->table_len));
   {
@@ -560,6 +567,7 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
     ctx->blob.resize(blob);
     char* src = ctx->blob.data();
     memset(src, 0, 64);
+    memset(src + pl.lay.ready, 0, blob - pl.lay.ready);
     auto put = [&](size_t at, const void* data, size_t bytes) {
       if (bytes) memcpy(src + at, data, bytes);
     };
@@ -618,7 +626,8 @@ struct ProfiledCall {
 };
 
 const ReqDesc* d_reqs(audiokv_ctx* c) { return reinterpret_cast<const ReqDesc*>(c->ws + c->plan.lay.reqs); }
-// The first 64 bytes of the workspace: the status word, and from int 4 on the queue of the smoothing kernel.
+// The first 64 bytes of the workspace: the status word, from int 4 on the queue of the smoothing kernel, from int 8 on the
+// counters of the queue between smoothing and gather.
 int* d_status(audiokv_ctx* c) { return reinterpret_cast<int*>(c->ws + c->plan.lay.status); }
 
 // used: bytes at the front of the workspace that the call needs; the FMA scoring may have the rest. head_end >= 0 (one request,
@@ -653,7 +662,8 @@ int do_score(audiokv_ctx* ctx, const void* q, const void* k, float* scores, cuda
 // Smoothing; with budgets, cu_kept and kept_idx it also selects each head's kept tokens (smoothed may then be null).
 // head_end < 0: all heads, in the plan's cost-sorted order; else the heads [head_begin, head_end) in index order.
 int do_smooth(audiokv_ctx* ctx, const float* scores, float* smoothed, int32_t* kstar, const int32_t* budgets,
-              const int32_t* cu_kept, int32_t* kept_idx, cudaStream_t stream, int head_begin = 0, int head_end = -1) {
+              const int32_t* cu_kept, int32_t* kept_idx, cudaStream_t stream, int head_begin = 0, int head_end = -1,
+              HeadQueue hq = {}) {
   Plan& pl = ctx->plan;
   Launch ln{stream, &ctx->launches, &ctx->prof};
   const bool all = head_end < 0;
@@ -663,7 +673,7 @@ int do_smooth(audiokv_ctx* ctx, const float* scores, float* smoothed, int32_t* k
                              reinterpret_cast<float2*>(ctx->ws + pl.lay.fft_scratch), pl.scratch_per_block,
                              all ? pl.sss_grid : (count < pl.sss_grid ? count : pl.sss_grid), pl.sss_smem,
                              all ? reinterpret_cast<const int32_t*>(ctx->ws + pl.lay.order) : nullptr, count,
-                             head_begin, budgets, cu_kept, kept_idx, d_status(ctx), d_status(ctx) + 4, ln);
+                             head_begin, budgets, cu_kept, kept_idx, d_status(ctx), d_status(ctx) + 4, hq, ln);
   return e == cudaSuccess ? AUDIOKV_OK : cuda_fail(ctx, e);
 }
 
@@ -674,6 +684,25 @@ int do_gather(audiokv_ctx* ctx, const int32_t* cu_kept, const int32_t* kept_idx,
   cudaError_t e = launch_gather(pl.sh, d_reqs(ctx), cu_kept, kept_idx, k, v, k_out, v_out, head_begin,
                                 head_end < 0 ? pl.sh.total_heads : head_end, ln);
   return e == cudaSuccess ? AUDIOKV_OK : cuda_fail(ctx, e);
+}
+
+// Smoothing, selection and gather of all heads; kept_rows: about how many rows they keep.
+int do_smooth_gather(audiokv_ctx* ctx, const float* scores, float* smoothed, int32_t* kstar, const int32_t* budgets,
+                     const int32_t* cu_kept, int32_t* kept_idx, const void* k, const void* v, void* k_out, void* v_out,
+                     int64_t kept_rows, cudaStream_t stream) {
+  Plan& pl = ctx->plan;
+  const bool follow = pl.follow;
+  int* words = d_status(ctx);
+  const HeadQueue hq{reinterpret_cast<unsigned long long*>(words + 8), words + 10,
+                     follow ? reinterpret_cast<unsigned long long*>(ctx->ws + pl.lay.ready) : nullptr, gather_unit_rows(pl.sh)};
+  int rc = do_smooth(ctx, scores, smoothed, kstar, budgets, cu_kept, kept_idx, stream, 0, -1, hq);
+  if (rc || !follow) return rc ? rc : do_gather(ctx, cu_kept, kept_idx, k, v, k_out, v_out, stream);
+  Launch ln{stream, &ctx->launches, &ctx->prof};
+  cudaError_t e = launch_gather_stream(pl.sh, d_reqs(ctx), cu_kept, kept_idx, k, v, k_out, v_out, pl.sh.total_heads, kept_rows, hq,
+                                       d_status(ctx), ln);
+  if (e == cudaSuccess) return AUDIOKV_OK;
+  ctx->plan_uploaded = false;  // the queue keeps this call's heads: it goes up again, empty
+  return cuda_fail(ctx, e);
 }
 
 int check_budgets(const Plan& pl, const int64_t* total_budget) {
@@ -954,8 +983,9 @@ int evict_pass(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, con
   if (rc) return rc;
   // the pooling variants hand their result to the selection through the score buffer itself
   float* ws_smoothed = pl.sh.smooth_mode >= AUDIOKV_SMOOTH_AVG_POOL ? ws_scores : nullptr;
-  if ((rc = do_smooth(ctx, ws_scores, ws_smoothed, ws_kstar, budgets, cu_kept, kept_idx, s))) return rc;
-  return do_gather(ctx, cu_kept, kept_idx, k, v, k_out, v_out, s);
+  int64_t rows = 0;
+  for (int r = 0; r < pl.sh.n_req; ++r) rows += total_budget[r];
+  return do_smooth_gather(ctx, ws_scores, ws_smoothed, ws_kstar, budgets, cu_kept, kept_idx, k, v, k_out, v_out, rows, s);
 }
 
 }  // namespace
@@ -995,8 +1025,9 @@ int audiokv_evict_budgeted(audiokv_ctx* ctx, const audiokv_params* p, const void
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   if ((rc = do_score(ctx, q_win, k, ws_scores, s, pl.lay.end, 0, -1, !ctx->prof.on))) return rc;
   float* ws_smoothed = pl.sh.smooth_mode >= AUDIOKV_SMOOTH_AVG_POOL ? ws_scores : nullptr;
-  if ((rc = do_smooth(ctx, ws_scores, ws_smoothed, ws_kstar, ws_budgets, cu_kept, kept_idx, s))) return rc;
-  return do_gather(ctx, cu_kept, kept_idx, k, v, k_out, v_out, s);
+  // only the device knows the budgets: a guess
+  const int64_t rows = pl.scores_len / 3 + static_cast<int64_t>(pl.sh.total_heads) * pl.sh.window;
+  return do_smooth_gather(ctx, ws_scores, ws_smoothed, ws_kstar, ws_budgets, cu_kept, kept_idx, k, v, k_out, v_out, rows, s);
 }
 
 namespace {

@@ -42,17 +42,40 @@ struct Shape {
   int* page_status;           // status word that a page id outside the pool is reported to (may be null)
 };
 
-// Element offset of token j of request r inside K / V, without the layer and head terms. A page id outside the pool
-// is reported through the status word and read as page 0, so that no address leaves the pool.
-__device__ __forceinline__ int64_t kv_token_offset(const Shape& sh, const ReqDesc& rq, int r, int j) {
-  if (sh.page_size == 0) return rq.kv_offset + static_cast<int64_t>(j) * sh.kv_stride_tok;
+// Row of token j of request r, in rows of kv_stride_tok from the request's offset (contiguous) or from the pool's start (paged).
+// A page id outside the pool is reported through the status word and read as page 0, so that no address leaves the pool.
+__device__ __forceinline__ int kv_token_row(const Shape& sh, int r, int j) {
+  if (sh.page_size == 0) return j;
   int page = __ldg(sh.page_table + r * sh.page_table_stride + (j >> sh.page_shift));
   if (page < 0 || page >= sh.n_pages) {
     if (sh.page_status) atomicExch(sh.page_status, AUDIOKV_EDEVICE);
     page = 0;
   }
-  return ((static_cast<int64_t>(page) << sh.page_shift) + (j & (sh.page_size - 1))) * sh.kv_stride_tok;
+  return (page << sh.page_shift) + (j & (sh.page_size - 1));
 }
+// The same as an element offset inside K / V, without the layer and head terms.
+__device__ __forceinline__ int64_t kv_token_offset(const Shape& sh, const ReqDesc& rq, int r, int j) {
+  return (sh.page_size ? 0 : rq.kv_offset) + static_cast<int64_t>(kv_token_row(sh, r, j)) * sh.kv_stride_tok;
+}
+
+// The heads whose selection has ended, in that order, from the smoothing kernel to the gather beside it. All zero before a
+// pass; the gather's last block leaves it so. done == nullptr: the gather does not follow head by head.
+struct HeadQueue {
+  unsigned long long* listed;  // heads listed (upper half) and the units of rows that they have (lower half)
+  int* counters;               // units taken, gather blocks that are through
+  unsigned long long* done;    // [heads of the launch] head index + 1 (upper half), units before it (lower half)
+  int unit_rows;               // kept rows to a unit; the last unit of a head may be short
+  __device__ int* ticket() const { return counters; }
+  __device__ int* blocks() const { return counters + 1; }
+  // One thread, behind a block barrier that the writers of the head's indices have passed.
+  __device__ void finished(int u, int kept) const {
+    __threadfence();
+    const unsigned long long units = (kept + unit_rows - 1) / unit_rows;
+    const unsigned long long at = atomicAdd(listed, (1ull << 32) | units);
+    const unsigned long long e = (static_cast<unsigned long long>(u + 1) << 32) | (at & 0xffffffffull);
+    asm volatile("st.release.gpu.global.b64 [%0], %1;" ::"l"(done + (at >> 32)), "l"(e) : "memory");
+  }
+};
 
 // Maps a flat head index to (request, layer, kv head). n_req is small: linear search.
 __device__ __forceinline__ int find_req(const ReqDesc* __restrict__ reqs, int n_req, int heads_per_req, int u) {
@@ -267,7 +290,7 @@ cudaError_t launch_sss(const Shape& sh, const ReqDesc* d_reqs, const FftPlan* d_
                        const float* scores, float* smoothed, int32_t* kstar, float2* scratch,
                        int64_t scratch_per_block, int grid, size_t smem_bytes, const int32_t* order, int n_order,
                        int first_head, const int32_t* budgets, const int32_t* cu_kept, int32_t* kept_idx, int* status,
-                       int* queue, Launch ln);
+                       int* queue, HeadQueue hq, Launch ln);
 
 // allocate.cu (h_total_budget: host array [n_req]). chained: what was launched just before is launch_fft_tables.
 cudaError_t launch_allocate(const Shape& sh, const ReqDesc* d_reqs, const float* head_scores,
@@ -285,6 +308,11 @@ cudaError_t launch_select(const Shape& sh, const ReqDesc* d_reqs, const float* s
 cudaError_t launch_gather(const Shape& sh, const ReqDesc* d_reqs, const int32_t* cu_kept, const int32_t* kept_idx,
                           const void* k, const void* v, void* k_out, void* v_out, int head_begin, int head_end,
                           Launch ln);
+// The same for the n_heads heads that the launch_sss just before lists in hq as it goes. kept_rows: about how many rows they keep.
+int gather_unit_rows(const Shape& sh);
+cudaError_t launch_gather_stream(const Shape& sh, const ReqDesc* d_reqs, const int32_t* cu_kept, const int32_t* kept_idx,
+                                 const void* k, const void* v, void* k_out, void* v_out, int n_heads, int64_t kept_rows,
+                                 HeadQueue hq, int* status, Launch ln);
 
 // hit_score.cu: offline head score. counts: int32 [n_heads] (cleared here, then the hit totals).
 cudaError_t launch_hit_score(const float* attn, int n_steps, int n_heads, int64_t row_stride, const int32_t* row_len,

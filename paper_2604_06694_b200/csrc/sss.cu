@@ -1413,7 +1413,9 @@ sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict
            int32_t* __restrict__ kstar_out, float2* __restrict__ scratch, int64_t scratch_per_block,
            const int32_t* __restrict__ order, int n_order, int first_head, const int32_t* __restrict__ budgets,
            const int32_t* __restrict__ cu_kept, int32_t* __restrict__ kept_idx, int* __restrict__ status,
-           int* __restrict__ queue) {
+           int* __restrict__ queue, HeadQueue hq) {
+  // A gather that follows head by head is set up when every block here has started, on the SMs that come free.
+  if (hq.done) chain_release();
   // Launched as a programmatic dependent: the block is brought in while the kernel before it drains, reads its plan
   // (written when the plan was made, not by the kernels of the pass), and waits for that kernel only where it first
   // touches the scores.
@@ -1463,16 +1465,14 @@ sss_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const FftPlan* __restrict
       }
     }
     __syncthreads();
-    if (sh.smooth_mode >= AUDIOKV_SMOOTH_AVG_POOL) {
-      pool_head(sh, sel, status);
-      continue;
-    }
-    if (S.pl.in_smem) smooth_head<false>(sh, tables, sel, status);
+    if (sh.smooth_mode >= AUDIOKV_SMOOTH_AVG_POOL) pool_head(sh, sel, status);
+    else if (S.pl.in_smem) smooth_head<false>(sh, tables, sel, status);
     else smooth_head<true>(sh, tables, sel, status);
+    if (hq.done && threadIdx.x == 0) hq.finished(u, S.k_keep + W);  // the selection ends with a barrier
   }
-  // Only now: the gather, whose blocks would sit on the SMs that are through and keep the others' places, is brought in when the
-  // last block ends, and its launch is hidden behind that.
-  chain_release();
+  // Only now: the other gather, whose blocks would sit on the SMs that are through and keep the others' places, is brought in
+  // when the last block ends, and its launch is hidden behind that.
+  if (!hq.done) chain_release();
   if (n_order > static_cast<int>(gridDim.x) && threadIdx.x == 0) {
     if (atomicAdd(queue + 1, 1) == static_cast<int>(gridDim.x) - 1) {
       atomicExch(queue, 0);
@@ -1646,12 +1646,12 @@ cudaError_t launch_sss(const Shape& sh, const ReqDesc* d_reqs, const FftPlan* d_
                        const float* scores, float* smoothed, int32_t* kstar, float2* scratch,
                        int64_t scratch_per_block, int grid, size_t smem_bytes, const int32_t* order, int n_order,
                        int first_head, const int32_t* budgets, const int32_t* cu_kept, int32_t* kept_idx, int* status,
-                       int* queue, Launch ln) {
+                       int* queue, HeadQueue hq, Launch ln) {
   cudaError_t e = cudaFuncSetAttribute(sss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
   if (e != cudaSuccess) return e;
   e = launch_chained(sss_kernel, dim3(grid), dim3(kT), smem_bytes, ln.stream, sh, d_reqs, d_plans, d_tables, scores,
                      smoothed, kstar, scratch, scratch_per_block, order, n_order, first_head, budgets, cu_kept, kept_idx,
-                     status, queue);
+                     status, queue, hq);
   ln.done(budgets ? "sss_select" : "sss");
   return e;
 }
