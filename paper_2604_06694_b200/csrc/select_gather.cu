@@ -135,7 +135,7 @@ gather_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const int32_t* __restr
 constexpr int kCopyWarps = 8;
 constexpr int kStreamThreads = (kCopyWarps + 1) * 32;
 constexpr int kRing = 2 * kCopyWarps;  // batches of rows prepared ahead
-constexpr int kUnitChunks = 1024;      // rows of a unit times 16-byte chunks of a row of K
+constexpr int kUnitChunks = 512;       // rows of a unit times 16-byte chunks of a row of K
 constexpr int kTicketUnits = 4;        // units of a ticket at most
 constexpr long long kHeadWaitCycles = 8000000000LL;  // about four seconds without another head finished
 

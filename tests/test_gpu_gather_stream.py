@@ -19,8 +19,8 @@ def B():
 
 CASES = [  # layers, KV heads, head_dim, type, window, lengths, kept share, page
     (1, 1, 128, "bf16", 16, [1500], 0.4, 0),
-    (1, 1, 64, "bf16", 8, [1531], 128 / 1531, 0),      # one unit of 128 rows
-    (1, 1, 64, "bf16", 8, [1531], 129.5 / 1531, 0),    # one more
+    (1, 1, 64, "bf16", 8, [1531], 64 / 1531, 0),       # one unit of 64 rows
+    (1, 1, 64, "bf16", 8, [1531], 65.5 / 1531, 0),     # one more
     (40, 4, 64, "bf16", 8, [97], 0.3, 0),
     (75, 2, 128, "bf16", 8, [40], 0.0, 0),             # the windows alone
     (38, 4, 128, "bf16", 16, [200], 1.0, 0),           # everything
