@@ -7,7 +7,7 @@
 // they are done once. So where there is room they are done once: the product kernel writes exp2(z - m) of its tile, m the
 // row's maximum over the tile's keys, and (m, sum) per row; a merge gives every row c = -(max + log2 sum) over all keys;
 // the sum kernel adds exp2(m + c) exp2(z - m) over the rows of every key, a stream at memory speed. Heads go through in
-// chunks of up to 128 MB of exponentials, or what room the caller has. A head too long for it, and the entry point with
+// chunks of up to 512 MB of exponentials, or what room the caller has. A head too long for it, and the entry point with
 // fixed scratch, run the product twice: statistics, merge, column sums.
 // The product is a register-tiled matrix product, 8 keys x 4, 7 or 8 query rows a thread. The tile's keys lie transposed in shared
 // memory for as long as the tile lasts, two neighbouring keys make a packed pair of accumulators, and the query rows
@@ -398,8 +398,8 @@ cudaError_t launch_tile(const Shape& sh, const ReqDesc* d_reqs, const void* q, c
 }
 
 // Heads of a chunk, at most `most`: as few waves of blocks over all chunks as possible, two blocks an SM, a chunk's three
-// launches counted as a third of a wave. (112 heads of 32 tiles: 28 heads a chunk are 3.03 waves, so four chunks of four,
-// 0.77 ms; 36 heads are 3.9, three chunks of four and one of one.)
+// launches counted as a third of a wave. (112 heads of 32 tiles in room for 36: 28 heads a chunk are 3.03 waves, so four chunks
+// of four, 0.77 ms; 36 heads are 3.9, three chunks of four and one of one.)
 int heads_per_chunk(int most, int total, int tiles) {
   const int64_t slots = 2LL * device_sm_count();
   int best = most;
@@ -421,7 +421,11 @@ int64_t head_exps(int max_L, int rows, int head_dim) {
   const int keys = tile_keys(head_dim);
   return static_cast<int64_t>((max_L + keys - 1) / keys) * keys * rows;
 }
-constexpr int64_t kMaxExps = (128LL << 20) / sizeof(float);  // of a chunk
+// Of a chunk. Every chunk ends in a wave of blocks that is not full, a merge and a stream, so fewer are better, even though the
+// exponentials no longer stay in L2: 112 heads of 4096 keys, 224 rows (411 MB): 878 us a pass at 96 MB, 853 at 128 (four chunks), 805
+// at 256 (two), 788 in one.
+constexpr int64_t kMaxExps = (512LL << 20) / sizeof(float);
+constexpr int64_t kMaxHeadExps = (128LL << 20) / sizeof(float);  // a head with more has its product done twice
 
 // room: where the exponentials of a chunk of heads and then their statistics may go.
 template <typename T, int D, int RPT>
@@ -430,7 +434,7 @@ cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, 
   constexpr int kKeys = tile_keys(D);
   const int R = sh.window * sh.group, n_tile = (max_L + kKeys - 1) / kKeys;
   const int64_t per_head = head_exps(max_L, R, D);
-  const int64_t fit = std::min<int64_t>(room_bytes / (per_head / kKeys * (kKeys * sizeof(float) + sizeof(float2))), kMaxExps / per_head);
+  const int64_t fit = per_head > kMaxHeadExps ? 0 : std::min<int64_t>(room_bytes / (per_head / kKeys * (kKeys * sizeof(float) + sizeof(float2))), kMaxExps / per_head);
   const bool store = fit >= 1;
   const int slabs = store ? n_tile : n_slab;
   const int most = static_cast<int>(std::min<int64_t>(store ? fit : 0x7fffffffLL / slabs, sh.total_heads));
@@ -447,6 +451,10 @@ cudaError_t launch_typed(const Shape& sh, const ReqDesc* d_reqs, const void* q, 
     ln.done("score_simt_merge");
     if (e != cudaSuccess) return e;
     if (store) {
+      // The blocks follow the product's on the SM and would keep its shared memory: 40 % of it holds eight of them, the rest is L1 for
+      // their loads in flight (23 us for 36 heads of 4096 keys with what the product leaves, 18 so).
+      e = cudaFuncSetAttribute(colsum_kernel<kKeys>, cudaFuncAttributePreferredSharedMemoryCarveout, 40);
+      if (e != cudaSuccess) return e;
       e = launch_chained(colsum_kernel<kKeys>, dim3(static_cast<unsigned>(slabs) * heads), dim3(kThreads), sizeof(float) * R, ln.stream, sh,
                          d_reqs, scores, stats, exps, slabs, u0);
       ln.done("score_simt_colsum");
