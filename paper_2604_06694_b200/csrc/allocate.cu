@@ -224,7 +224,7 @@ cudaError_t launch_budget_prefix(const Shape& sh, const ReqDesc* d_reqs, const i
 
 cudaError_t launch_allocate(const Shape& sh, const ReqDesc* d_reqs, const float* head_scores,
                             const int64_t* h_total_budget, int32_t* budgets, int32_t* cu_kept, int* status,
-                            Launch ln, bool chained) {
+                            Launch ln) {
   int64_t all = 0;
   for (int r = 0; r < sh.n_req; ++r) all += h_total_budget[r];
   if (all > 0x7fffffffLL) return cudaErrorInvalidValue;  // cu_kept is int32
@@ -241,13 +241,9 @@ cudaError_t launch_allocate(const Shape& sh, const ReqDesc* d_reqs, const float*
       args.cu_base[i] = rows;
       rows += h_total_budget[r0 + i];
     }
-    // the first launch of a pass is an ordinary one, so that everything earlier on the stream is complete when it starts
-    if (chained) {
-      e = launch_chained(allocate_kernel, dim3(n), dim3(kAllocThreads), smem, ln.stream, sh, d_reqs, head_scores, args, budgets, cu_kept, status);
-    } else {
-      allocate_kernel<<<n, kAllocThreads, smem, ln.stream>>>(sh, d_reqs, head_scores, args, budgets, cu_kept, status);
-      e = cudaGetLastError();
-    }
+    // set up while the kernel before it drains (the gather of the pass before: 2 us a pass); everything earlier on the stream is
+    // complete when it lets the scoring in
+    e = launch_chained(allocate_kernel, dim3(n), dim3(kAllocThreads), smem, ln.stream, sh, d_reqs, head_scores, args, budgets, cu_kept, status);
     ln.done("allocate");
     if (e != cudaSuccess) return e;
   }

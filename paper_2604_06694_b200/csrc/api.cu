@@ -76,7 +76,6 @@ struct audiokv_ctx {
   Plan plan;
   bool plan_uploaded = false;
   bool host_uploaded = false;             // plan.host_score too
-  bool plan_fresh = false;                // the call at hand put the plan on the device: its last launch was launch_fft_tables
   uint64_t plan_id = 0;      // counts plan rebuilds
   ScoreMapCache score_maps;
   cudaEvent_t plan_ready = nullptr;
@@ -549,7 +548,6 @@ int prepare(audiokv_ctx* ctx, const audiokv_params* p, cudaStream_t stream, bool
   if ((host_call ? pl.lay.host_end : pl.lay.end) > ctx->ws_bytes) return AUDIOKV_EWORKSPACE;
   pl.sh.page_table = p->page_size ? p->page_table : nullptr;  // device data of this call, not part of the plan
   pl.sh.page_status = reinterpret_cast<int*>(ctx->ws + pl.lay.status);
-  ctx->plan_fresh = !ctx->plan_uploaded;
   if (!ctx->plan_uploaded) {
     // A graph that held the upload would bring this plan back at every replay, over the one the context then has: the first
     // call with a given shape has to run outside capture (later ones add nothing but the kernels of the pass).
@@ -716,13 +714,12 @@ int check_budgets(const Plan& pl, const int64_t* total_budget) {
 }
 
 int do_allocate(audiokv_ctx* ctx, const float* head_scores, const int64_t* total_budget, int32_t* budgets,
-                int32_t* cu_kept, cudaStream_t stream, bool chained = false) {
+                int32_t* cu_kept, cudaStream_t stream) {
   Plan& pl = ctx->plan;
   int rc = check_budgets(pl, total_budget);
   if (rc) return rc;
   Launch ln{stream, &ctx->launches, &ctx->prof};
-  cudaError_t e = launch_allocate(pl.sh, d_reqs(ctx), head_scores, total_budget, budgets, cu_kept, d_status(ctx), ln,
-                                  chained);
+  cudaError_t e = launch_allocate(pl.sh, d_reqs(ctx), head_scores, total_budget, budgets, cu_kept, d_status(ctx), ln);
   return e == cudaSuccess ? AUDIOKV_OK : cuda_fail(ctx, e);
 }
 
@@ -972,13 +969,12 @@ int evict_pass(audiokv_ctx* ctx, const audiokv_params* p, const void* q_win, con
   float* ws_scores = reinterpret_cast<float*>(ctx->ws + pl.lay.scores);
   int32_t* ws_kstar = reinterpret_cast<int32_t*>(ctx->ws + pl.lay.kstar);
   const ProfiledCall timed(ctx, s);
-  // The budgets depend on nothing the GPU computes, and only the selection needs them. The allocation kernel is
-  // launched the ordinary way (everything earlier on the stream is then complete when it starts) and lets its
-  // dependents in at once; the first scoring sweep, a programmatic dependent, runs beside it and waits for it at its
+  // The budgets depend on nothing the GPU computes, and only the selection needs them. The allocation kernel waits for
+  // everything earlier on the stream and then lets its dependents in; the first scoring sweep, a programmatic dependent, runs beside it and waits for it at its
   // own end, so that the smoothing and selection, two chained kernels later, find the budgets complete. With per-kernel
   // timing on, every kernel waits for the one before it.
   const bool beside = !ctx->prof.on;
-  rc = do_allocate(ctx, head_scores, total_budget, budgets, cu_kept, s, ctx->plan_fresh && !ctx->prof.on);
+  rc = do_allocate(ctx, head_scores, total_budget, budgets, cu_kept, s);
   if (!rc) rc = do_score(ctx, q_win, k, ws_scores, s, std::max(used, pl.lay.end), 0, -1, beside);
   if (rc) return rc;
   // the pooling variants hand their result to the selection through the score buffer itself

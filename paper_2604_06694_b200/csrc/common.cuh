@@ -265,8 +265,8 @@ struct ScoreMapCache {
 // d_units / d_cta: device tables of runs and per-CTA offsets (both sweeps of every schedule). scheds: host.
 // head_end < 0: every whole-request schedule in turn; else the schedule made for heads [head_begin, head_end).
 // stats_ws: float2 [total heads][max_parts][score_stat_sets()][W * G].
-// beside: the kernel launched just before on the stream is the library's own budget kernel (ordinary launch, calls
-// chain_release at once): the first sweep then runs beside it instead of after it.
+// beside: the kernel launched just before on the stream is the library's own budget kernel, which calls chain_release when
+// everything before it is complete: the first sweep then runs beside it instead of after it.
 cudaError_t launch_score_umma(const Shape& sh, const ReqDesc* h_reqs, const ScoreUnit* d_units, const int32_t* d_cta,
                               const ScoreSchedule* scheds, int n_sched, const void* q, const void* k, float* scores,
                               float2* stats_ws, int max_parts, int* status, Launch ln, int head_begin = 0,
@@ -292,10 +292,10 @@ cudaError_t launch_sss(const Shape& sh, const ReqDesc* d_reqs, const FftPlan* d_
                        int first_head, const int32_t* budgets, const int32_t* cu_kept, int32_t* kept_idx, int* status,
                        int* queue, HeadQueue hq, Launch ln);
 
-// allocate.cu (h_total_budget: host array [n_req]). chained: what was launched just before is launch_fft_tables.
+// allocate.cu (h_total_budget: host array [n_req])
 cudaError_t launch_allocate(const Shape& sh, const ReqDesc* d_reqs, const float* head_scores,
                             const int64_t* h_total_budget, int32_t* budgets, int32_t* cu_kept, int* status,
-                            Launch ln, bool chained);
+                            Launch ln);
 
 // given: device int32 [total heads], budgets chosen by the caller; budgets: their checked copy; cu_kept: prefix sums.
 cudaError_t launch_budget_prefix(const Shape& sh, const ReqDesc* d_reqs, const int32_t* given, int32_t* budgets,

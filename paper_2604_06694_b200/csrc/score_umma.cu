@@ -590,8 +590,8 @@ score_umma_kernel(const __grid_constant__ TmapPack<CAP> tm, const UmmaArgs a) {
   // and Q) and only then lets sweep 2 be brought in. A CTA of sweep 2 therefore starts on inputs that are
   // final: its copies and MMAs begin as soon as a CTA of sweep 1 has left the SM, and only its epilogue waits
   // (below) for sweep 1 to finish, since only the statistics come from there.
-  // When the kernel before sweep 1 is the library's own budget kernel, launched the ordinary way (so that everything
-  // earlier on the stream is complete) and needing nothing sweep 1 touches, sweep 1 runs beside it and waits for it
+  // When the kernel before sweep 1 is the library's own budget kernel, which lets it in when everything earlier on the
+  // stream is complete and computes nothing that sweep 1 touches, sweep 1 runs beside it and waits for it
   // only at its end: the kernels after it then find the budgets complete through the chain of waits.
   if (SWEEP == 1 && !a.beside) chain_wait();
   chain_release();

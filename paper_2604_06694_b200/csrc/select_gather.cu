@@ -15,6 +15,7 @@ __global__ void __launch_bounds__(kSelThreads, 1)
 select_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const float* __restrict__ smoothed,
               const int32_t* __restrict__ budgets, const int32_t* __restrict__ cu_kept,
               int32_t* __restrict__ kept_idx, int smem_keys, int* __restrict__ status) {
+  chain_wait();
   extern __shared__ uint32_t skeys[];  // smem_keys keys, then the masks and prefix sums of the longest head
   __shared__ SelectSmem ssm;
   __shared__ uint32_t s_min, s_max;
@@ -60,6 +61,7 @@ select_kernel(Shape sh, const ReqDesc* __restrict__ reqs, const float* __restric
       select_entries<kSelThreads, false>([&](int j) { return make_float2(__uint_as_float(score_key(s[j])), 0.f); }, P, P,
                                          W, k, s_min, s_max, out, &ssm, words, pre, status);
   }
+  chain_release();  // at the end: see the gather
 }
 
 // Copies the kept rows. A warp takes eight output rows at a time: lanes 0-7 look up the head of one row each
@@ -328,10 +330,10 @@ cudaError_t launch_select(const Shape& sh, const ReqDesc* d_reqs, const float* s
   if (e != cudaSuccess) return e;
   const int max_grid = device_sm_count() * 4;
   const int grid = sh.total_heads < max_grid ? sh.total_heads : max_grid;
-  select_kernel<<<grid, kSelThreads, smem, ln.stream>>>(sh, d_reqs, smoothed, budgets, cu_kept, kept_idx, smem_keys,
-                                                        status);
+  e = launch_chained(select_kernel, dim3(grid), dim3(kSelThreads), smem, ln.stream, sh, d_reqs, smoothed, budgets, cu_kept, kept_idx,
+                     smem_keys, status);
   ln.done("select");
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_gather(const Shape& sh, const ReqDesc* d_reqs, const int32_t* cu_kept, const int32_t* kept_idx,
