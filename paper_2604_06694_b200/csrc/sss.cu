@@ -1507,6 +1507,7 @@ __global__ void __launch_bounds__(256) plan_part_kernel(const __grid_constant__ 
 // transform plans, at byte plans_at of the workspace, are read from `part` when they travel in it.
 __global__ void __launch_bounds__(256)
 fft_table_kernel(const __grid_constant__ PlanPart part, int n16, char* ws, size_t plans_at, float2* __restrict__ tables) {
+  chain_wait();  // set up while the pass before drains, which reads what is overwritten here
   chain_release();
   __shared__ FftPlan pl;
   {
@@ -1631,9 +1632,10 @@ cudaError_t launch_fft_tables(int n_plans, const char* h_blob, size_t blob_bytes
     }
   }
   if (first) memcpy(part.v, h_blob, first);
-  fft_table_kernel<<<dim3(32, n_plans), 256, 0, ln.stream>>>(part, static_cast<int>(first / 16), ws, plans_at, d_tables);
+  e = launch_chained(fft_table_kernel, dim3(32, n_plans), dim3(256), 0, ln.stream, part, static_cast<int>(first / 16), ws, plans_at,
+                     d_tables);
   ln.done("fft_table");
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   if (rest) memcpy(part.v, h_blob + first, rest);
   e = launch_chained(fft_filter_kernel, dim3(n_plans, rest ? 2 + (8 + n_plans - 1) / n_plans : 2), dim3(kT), smem_bytes, ln.stream, part,
                      static_cast<int>(rest / 16), reinterpret_cast<uint4*>(ws + first),
