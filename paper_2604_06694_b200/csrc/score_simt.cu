@@ -7,7 +7,7 @@
 // they are done once. So where there is room they are done once: the product kernel writes exp2(z - m) of its tile, m the
 // row's maximum over the tile's keys, and (m, sum) per row; a merge gives every row c = -(max + log2 sum) over all keys;
 // the sum kernel adds exp2(m + c) exp2(z - m) over the rows of every key, a stream at memory speed. Heads go through in
-// chunks of up to 512 MB of exponentials, or what room the caller has. A head too long for it, and the entry point with
+// chunks of up to 256 MB of exponentials, or what room the caller has. A head too long for it, and the entry point with
 // fixed scratch, run the product twice: statistics, merge, column sums.
 // The product is a register-tiled matrix product, 8 keys x 4, 7 or 8 query rows a thread. The tile's keys lie transposed in shared
 // memory for as long as the tile lasts, two neighbouring keys make a packed pair of accumulators, and the query rows
@@ -423,8 +423,8 @@ int64_t head_exps(int max_L, int rows, int head_dim) {
 }
 // Of a chunk. Every chunk ends in a wave of blocks that is not full, a merge and a stream, so fewer are better, even though the
 // exponentials no longer stay in L2: 112 heads of 4096 keys, 224 rows (411 MB): 878 us a pass at 96 MB, 853 at 128 (four chunks), 805
-// at 256 (two), 788 in one.
-constexpr int64_t kMaxExps = (512LL << 20) / sizeof(float);
+// at 256 (two), 788 in one, which would make a context 1.5 ms longer to create.
+constexpr int64_t kMaxExps = (256LL << 20) / sizeof(float);
 constexpr int64_t kMaxHeadExps = (128LL << 20) / sizeof(float);  // a head with more has its product done twice
 
 // room: where the exponentials of a chunk of heads and then their statistics may go.

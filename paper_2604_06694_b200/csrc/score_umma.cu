@@ -17,13 +17,14 @@
 //               nothing is exchanged through shared memory, and while one group waits, loads or stores, the other
 //               keeps the special-function unit busy. The two sets of a group split the columns of every part;
 //   warp 16     TMA producer: the Q tile of a head once, K tiles of 128 keys through a ring;
-//   warps 17-18 MMA issuers, one thread per epilogue group: tcgen05.mma, bf16 x bf16 -> fp32 in TMEM. With one issuer
+//   warps 17-18 MMA issuers, one elected lane per epilogue group: tcgen05.mma, bf16 x bf16 -> fp32 in TMEM. With one issuer
 //               for both groups the tiles were issued in order, and a group that had handed its buffers back waited
 //               for the MMAs of the other group's tile to be let in first.
 // A tile is processed in one or two parts (sweep 1: blocks of 128 query rows; sweep 2: halves of
-// the query rows), each with an accumulator buffer of 128 TMEM columns that goes back to the MMA
-// thread as soon as its last chunk is in registers: the MMAs of the group's next tile run under
-// the arithmetic of this one.
+// the query rows). In sweep 1, and in sweep 2 up to 128 rows, a part has an accumulator buffer of 128 TMEM columns
+// that goes back to the MMA thread as soon as its last chunk is in registers: the MMAs of the group's next
+// tile run under the arithmetic of this one. In sweep 2 with more rows both parts lie in one accumulator of the group's 256
+// columns, and the group's next MMAs run under the arithmetic of the other group.
 // The work of a launch is dealt out tile by tile: CTA c takes the tiles [c T / grid, (c + 1) T / grid)
 // of the launch's tile sequence, as a few runs of consecutive tiles of one head (host-built table).
 // Q and K tiles are K-major with the 128-byte swizzle, so the same shared-memory tile is
