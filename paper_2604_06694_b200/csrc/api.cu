@@ -54,7 +54,6 @@ struct Plan {
   int max_L = 0, max_P = 0;
   int n_slab = 0;
   size_t score_room = 0;        // bytes of workspace behind everything else that the FMA scoring puts to use
-  bool follow = false;          // the gather runs beside the smoothing, head by head
   int sss_grid = 0;
   size_t sss_smem = 0;
   int64_t scratch_per_block = 0;  // float2 elements
@@ -471,11 +470,6 @@ int build_plan(const audiokv_params* p, Plan* pl) {
     for (int i = 0; i < sh.total_heads; ++i)
       pl->sss_order[i] = pl->reqs[by_cost[i / sh.heads_per_req].second].head_base + i % sh.heads_per_req;
   }
-  // The gather beside the smoothing pays as soon as some heads can end well before others: when the blocks take a second turn
-  // (48 layers of 2048 tokens, 192 heads: 145.9 -> 133.0 us a pass) or when a transform takes long beside a head that needs none
-  // (28 layers, 30 % of heads with transforms: 8192 tokens 269.7 -> 247.8, 32768 908 -> 812). Its start costs 3 us more: at 700 tokens
-  // and one turn 58.5 -> 61.4, at 1500 76.2 -> 76.1.
-  pl->follow = sh.total_heads > pl->sss_grid || pl->max_P >= 1400;
   int smem_c = 64;
   pl->scratch_per_block = 0;
   for (const FftPlan& fp : pl->fft) {
@@ -689,7 +683,13 @@ int do_smooth_gather(audiokv_ctx* ctx, const float* scores, float* smoothed, int
                      const int32_t* cu_kept, int32_t* kept_idx, const void* k, const void* v, void* k_out, void* v_out,
                      int64_t kept_rows, cudaStream_t stream) {
   Plan& pl = ctx->plan;
-  const bool follow = pl.follow;
+  // The gather beside the smoothing pays as soon as some heads can end well before others: when the blocks take a second turn
+  // (48 layers of 2048 tokens, 192 heads: 145.9 -> 133.0 us a pass) or when a transform takes long beside a head that needs none
+  // (28 layers, 30 % of heads with transforms: 8192 tokens 269.7 -> 247.8, 32768 908 -> 812). It costs 2 to 3 us more where no
+  // head needs one, which its own work has to be long against: with less than 80 MB to read and write (14 layers of 1500 tokens,
+  // half kept: 42 MB) 64.6 -> 67.7, above (2500 tokens: 70 MB; 5000: 140 MB) 75.4 -> 74.3 and 107.1 -> 103.7.
+  const int64_t moved = kept_rows * pl.sh.head_dim * esize(pl.sh.dtype) * 4;
+  const bool follow = pl.sh.total_heads > pl.sss_grid || (pl.max_P >= 1400 && moved >= (80LL << 20));
   int* words = d_status(ctx);
   const HeadQueue hq{reinterpret_cast<unsigned long long*>(words + 8), words + 10,
                      follow ? reinterpret_cast<unsigned long long*>(ctx->ws + pl.lay.ready) : nullptr, gather_unit_rows(pl.sh)};

@@ -73,7 +73,8 @@ struct HeadQueue {
     const unsigned long long units = (kept + unit_rows - 1) / unit_rows;
     const unsigned long long at = atomicAdd(listed, (1ull << 32) | units);
     const unsigned long long e = (static_cast<unsigned long long>(u + 1) << 32) | (at & 0xffffffffull);
-    asm volatile("st.release.gpu.global.b64 [%0], %1;" ::"l"(done + (at >> 32)), "l"(e) : "memory");
+    // the fence above orders it behind the head's indices; a release here would be a second fence
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(done + (at >> 32)), "l"(e) : "memory");
   }
 };
 

@@ -18,16 +18,17 @@ def B():
 
 
 CASES = [  # layers, KV heads, head_dim, type, window, lengths, kept share, page
-    (1, 1, 128, "bf16", 16, [1500], 0.4, 0),
-    (1, 1, 64, "bf16", 8, [1531], 64 / 1531, 0),       # one unit of 64 rows
-    (1, 1, 64, "bf16", 8, [1531], 65.5 / 1531, 0),     # one more
+    (1, 1, 256, "bf16", 16, [90001], 0.6, 0),
+    (150, 1, 64, "bf16", 8, [1531], 64 / 1531, 0),     # units of 64 rows
+    (150, 1, 64, "bf16", 8, [1531], 65.5 / 1531, 0),   # one more
     (40, 4, 64, "bf16", 8, [97], 0.3, 0),
     (75, 2, 128, "bf16", 8, [40], 0.0, 0),             # the windows alone
     (38, 4, 128, "bf16", 16, [200], 1.0, 0),           # everything
-    (3, 2, 256, "bf16", 16, [33, 3001, 1444], 0.37, 0),
-    (2, 2, 256, "f32", 8, [1999], 0.5, 0),
+    (25, 2, 256, "bf16", 16, [33, 3001, 1444], 0.37, 0),
+    (20, 4, 256, "f32", 8, [1999], 0.5, 0),
     (30, 4, 64, "f32", 8, [131, 64], 0.25, 0),
-    (4, 2, 128, "bf16", 16, [1407, 2050], 0.4, 16),
+    (40, 2, 128, "bf16", 16, [1407, 2050], 0.4, 16),
+    (4, 2, 128, "bf16", 16, [1407, 2050], 0.4, 16),    # small: behind the selection
 ]
 
 
